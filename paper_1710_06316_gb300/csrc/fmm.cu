@@ -460,7 +460,16 @@ constexpr int kP2PRegBlocks = kP2PResident;
 //   dn PhiL += -c (n0.d)/r^3 + (g/eps_bar) [(n0.n)/r^3 - 3 (n.d)(n0.d)/r^5]
 //   PhiY += c e/r + g (n.d) e1/r^3,           e = exp(-kr), e1 = e (1 + kr)
 //   dn PhiY += e1 [g (n0.n) - c (n0.d)]/r^3 - 3 g e2 (n.d)(n0.d)/r^5,  e2 = e (1 + kr + (kr)^2/3)
-// with d = x_target - y_source.  g enters only through the vector g n.
+// with d = x_target - y_source.  g enters only through the vector g n.  With
+//   P = g n.d,  Q = n0.d,  S = g n0.n,  p2 = P/r^2,  k1 = 1 + kr,  m = S - (3 p2 + c) Q
+// (3 e2 = 3 e1 + e (kr)^2, and (kr)^2 p2 = k^2 P) the four sums are
+//   PhiL += (p2/eps_bar + c)/r,              dn PhiL += (1/eps_bar) [m + (1 - eps_bar) c Q]/r^3,
+//   PhiY += e (k1 p2 + c)/r,                 dn PhiY += e (k1 m - k^2 P Q)/r^3.
+// The FP32 pipe bounds the kernel, so the count of its operations per pair is what this
+// form is for: 35 (43 in the order the formulas are printed in), 38 where the pair's
+// distance has to be tested, 27 and 30 without salt (k = 0: e = k1 = 1 and no exp2).
+// Measured, P2P alone: 0.255 -> 0.235 ms (163,842-node sphere, leaves of 80), 0.582 ->
+// 0.519 ms (leaves of 192), 1.032 -> 0.765 ms (655,362 nodes without salt).
 //
 // The sums run on packed FP32 pairs (sm_100 FFMA2 / FADD2 / FMUL2): each thread takes
 // its target against two sources per instruction, lane 0 an even and lane 1 an odd
@@ -494,45 +503,62 @@ struct P2PTarget {
   float2 rs;             // scaled skip radius
 };
 
+// Factors of the pair sums that all pairs of a problem share, in both lanes.
+struct P2PConst {
+  float2 inv_e;          // 1 / eps_bar
+  float2 kappa;          // k
+  float2 nkl2e;          // -k log2(e)
+  float2 kappa2;         // k^2
+  float2 omce;           // 1 - eps_bar
+};
+
 // sources: a = (-x0, -x1, -y0, -y1), b = (-z0, -z1, c0, c1), c = (gnx0, gnx1, gny0, gny1),
-// d = (gnz0, gnz1, skip0, skip1); positions in the target leaf's frame.
+// d = (gnz0, gnz1, w0, w1); positions in the target leaf's frame.  kTest: w = skip radius,
+// and pairs inside it contribute nothing here (the near CSR carries their whole near-rule
+// value; t == p is among them).  Otherwise no pair can be inside it and w = (1 - eps_bar) c.
+// Sums: sL, sY as above; nD = eps_bar dn PhiL; dY.
+template <bool kTest, bool kSalt>
 __device__ __forceinline__ void p2p_pair2(const P2PTarget &t, const float4 &a, const float4 &b, const float4 &c,
-                                          const float4 &d, float2 inv_e, float2 kappa, float2 &sL, float2 &nD,
-                                          float2 &sY, float2 &dY) {
+                                          const float4 &d, const P2PConst &k, float2 &sL, float2 &nD, float2 &sY,
+                                          float2 &dY) {
   const float2 dx = __fadd2_rn(t.x, make_float2(a.x, a.y));
   const float2 dy = __fadd2_rn(t.y, make_float2(a.z, a.w));
   const float2 dz = __fadd2_rn(t.z, make_float2(b.x, b.y));
   const float2 cc = make_float2(b.z, b.w);
   const float2 gx = make_float2(c.x, c.y), gy = make_float2(c.z, c.w), gz = make_float2(d.x, d.y);
   const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));   // p2p_r2
-  const float2 R = __fadd2_rn(t.rs, make_float2(d.z, d.w));                        // p2p_evaluates
-  const float2 RR = __fmul2_rn(R, R);
-  // Pairs inside the skip radius (t == p among them) contribute nothing here: the near
-  // CSR carries their whole near-rule value.
-  const float2 ri = make_float2(r2.x > RR.x ? rsqrt_approx(r2.x) : 0.0f, r2.y > RR.y ? rsqrt_approx(r2.y) : 0.0f);
+  float2 ri;
+  if (kTest) {
+    const float2 R = __fadd2_rn(t.rs, make_float2(d.z, d.w));                      // p2p_evaluates
+    const float2 RR = __fmul2_rn(R, R);
+    ri = make_float2(r2.x > RR.x ? rsqrt_approx(r2.x) : 0.0f, r2.y > RR.y ? rsqrt_approx(r2.y) : 0.0f);
+  } else {
+    ri = make_float2(rsqrt_approx(r2.x), rsqrt_approx(r2.y));
+  }
   const float2 ri2 = __fmul2_rn(ri, ri);
+  const float2 P = __ffma2_rn(gx, dx, __ffma2_rn(gy, dy, __fmul2_rn(gz, dz)));
+  const float2 Q = __ffma2_rn(t.nx, dx, __ffma2_rn(t.ny, dy, __fmul2_rn(t.nz, dz)));
+  const float2 S = __ffma2_rn(t.nx, gx, __ffma2_rn(t.ny, gy, __fmul2_rn(t.nz, gz)));
+  const float2 p2 = __fmul2_rn(P, ri2);
   const float2 G3 = __fmul2_rn(ri, ri2);
-  const float2 gnd = __ffma2_rn(gx, dx, __ffma2_rn(gy, dy, __fmul2_rn(gz, dz)));      // g n.d
-  const float2 npd = __ffma2_rn(t.nx, dx, __ffma2_rn(t.ny, dy, __fmul2_rn(t.nz, dz)));  // n0.d
-  const float2 gnn = __ffma2_rn(t.nx, gx, __ffma2_rn(t.ny, gy, __fmul2_rn(t.nz, gz)));  // g n0.n
-  const float2 kr = __fmul2_rn(kappa, __fmul2_rn(r2, ri));
-  const float2 arg = __fmul2_rn(kr, dup2(-1.4426950408889634f));
-  const float2 ex = make_float2(ex2_approx(arg.x), ex2_approx(arg.y));
-  const float2 e1 = __ffma2_rn(ex, kr, ex);
-  const float2 e2 = __ffma2_rn(__fmul2_rn(ex, kr), __fmul2_rn(kr, dup2(1.0f / 3.0f)), e1);
-  const float2 cri = __fmul2_rn(cc, ri);
-  const float2 A = __fmul2_rn(gnd, G3);
-  const float2 B = __fmul2_rn(gnn, G3);
-  const float2 npdG3 = __fmul2_rn(npd, G3);
-  const float2 Tn = __fmul2_rn(__fmul2_rn(__fmul2_rn(A, dup2(-3.0f)), npd), ri2);     // -T
-  sL = __fadd2_rn(sL, __ffma2_rn(inv_e, A, cri));
-  // nD accumulates -dn PhiL = c (n0.d)/r^3 - (1/eps_bar)(B - T)
-  nD = __ffma2_rn(make_float2(-inv_e.x, -inv_e.y), __fadd2_rn(B, Tn), __ffma2_rn(cc, npdG3, nD));
-  sY = __ffma2_rn(ex, cri, __ffma2_rn(e1, A, sY));
-  // negated operands instead of products with -1 (measured: P2P 0.256 -> 0.2515 ms on the
-  // 163,842-node sphere)
-  const float2 BmC = __ffma2_rn(make_float2(-cc.x, -cc.y), npdG3, B);               // B - c (n0.d)/r^3
-  dY = __ffma2_rn(e1, BmC, __ffma2_rn(e2, Tn, dY));
+  const float2 h = __ffma2_rn(p2, dup2(3.0f), cc);
+  const float2 m = __ffma2_rn(make_float2(-h.x, -h.y), Q, S);
+  const float2 dc = kTest ? __fmul2_rn(cc, k.omce) : make_float2(d.z, d.w);
+  nD = __ffma2_rn(G3, __ffma2_rn(dc, Q, m), nD);
+  sL = __ffma2_rn(ri, __ffma2_rn(k.inv_e, p2, cc), sL);
+  if (kSalt) {
+    const float2 rr = __fmul2_rn(r2, ri);
+    const float2 arg = __fmul2_rn(rr, k.nkl2e);
+    const float2 ex = make_float2(ex2_approx(arg.x), ex2_approx(arg.y));
+    const float2 k1 = __ffma2_rn(rr, k.kappa, dup2(1.0f));
+    const float2 ei = __fmul2_rn(ex, ri);
+    sY = __ffma2_rn(ei, __ffma2_rn(k1, p2, cc), sY);
+    const float2 V = __fmul2_rn(__fmul2_rn(P, Q), k.kappa2);
+    dY = __ffma2_rn(__fmul2_rn(ei, ri2), __ffma2_rn(k1, m, make_float2(-V.x, -V.y)), dY);
+  } else {
+    sY = __ffma2_rn(ri, __fadd2_rn(p2, cc), sY);
+    dY = __ffma2_rn(G3, m, dY);
+  }
 }
 
 // A unit that covers its leaf's whole source list stores; a part of a split leaf adds.
@@ -551,6 +577,7 @@ __device__ __forceinline__ void store_or_add(float4 *p, float4 v, bool whole) {
 template <bool kBatch>
 __device__ __forceinline__ void p2p_body(int nunits, const int4 *__restrict__ units, const int32_t *__restrict__ leaves_1,
                                          const int64_t *__restrict__ pptr_1, const int32_t *__restrict__ pidx_1,
+                                         const uint8_t *__restrict__ ptest_1,
                                          const int32_t *__restrict__ bbeg_1, const int32_t *__restrict__ bend_1,
                                          const dbl4 *__restrict__ center_1, const float4 *__restrict__ pos_1,
                                          const float4 *__restrict__ nrm_1, const float2 *__restrict__ xs_1,
@@ -558,7 +585,7 @@ __device__ __forceinline__ void p2p_body(int nunits, const int4 *__restrict__ un
                                          const P2PReq *__restrict__ reqs) {
   static_assert(2 * kP2PThreads <= kP2PPairs, "the reduction reuses the staging buffer");
   __shared__ float4 sa[kP2PPairs], sb[kP2PPairs], sc[kP2PPairs], sd[kP2PPairs];
-  __shared__ int s_beg[kP2PBoxes], s_pre[kP2PBoxes + 1];
+  __shared__ int s_beg[kP2PBoxes], s_pos[kP2PBoxes], s_cnt[kP2PBoxes], s_tot[4];
   __shared__ float s_off[kP2PBoxes][3];
   __shared__ __align__(8) P2PReq s_req;
   float4 *red = sa;
@@ -580,7 +607,16 @@ __device__ __forceinline__ void p2p_body(int nunits, const int4 *__restrict__ un
     __syncthreads();
     if (s_req.active && *s_req.active == 0) continue;  // uniform: the problem has stopped
   }
-  const float2 inv_e = dup2(kBatch ? s_req.inv_ebar : inv_ebar_1), kap = dup2(kBatch ? s_req.kappa : kappa_1);
+  P2PConst kc;
+  {
+    const float inv_e = P2P_ARG(inv_ebar), kap = P2P_ARG(kappa);
+    kc.inv_e = dup2(inv_e);
+    kc.kappa = dup2(kap);
+    kc.nkl2e = dup2(-1.4426950408889634f * kap);
+    kc.kappa2 = dup2(kap * kap);
+    kc.omce = dup2(1.0f - 1.0f / inv_e);
+  }
+  const bool salt = kc.kappa.x > 0.0f;
   const int leaf = unit.x;
   const int b = P2P_ARG(leaves)[leaf];
   const dbl4 cb = P2P_ARG(center)[b];
@@ -615,75 +651,116 @@ __device__ __forceinline__ void p2p_body(int nunits, const int4 *__restrict__ un
     for (int64_t g0 = l0; g0 < l1; g0 += kP2PBoxes) {
       const int nb = (int)min((int64_t)kP2PBoxes, l1 - g0);
       __syncthreads();
-      int mycnt = 0;
+      // The boxes whose pairs may be inside the skip radius come first in the staged order
+      // (slots [0, nf)), the others after them from the next even slot on.
+      int cf = 0, cu = 0;
+      bool test = false;
       if (threadIdx.x < nb) {
         const int c = P2P_ARG(pidx)[g0 + threadIdx.x];
         const dbl4 cc = P2P_ARG(center)[c];
-        s_beg[threadIdx.x] = P2P_ARG(bbeg)[c];
-        mycnt = P2P_ARG(bend)[c] - P2P_ARG(bbeg)[c];
+        const int beg = P2P_ARG(bbeg)[c], cnt = P2P_ARG(bend)[c] - beg;
+        test = P2P_ARG(ptest)[g0 + threadIdx.x] != 0;
+        cf = test ? cnt : 0;
+        cu = test ? 0 : cnt;
+        s_beg[threadIdx.x] = beg;
+        s_cnt[threadIdx.x] = cnt;
         s_off[threadIdx.x][0] = (float)(cc.x - cb.x);
         s_off[threadIdx.x][1] = (float)(cc.y - cb.y);
         s_off[threadIdx.x][2] = (float)(cc.z - cb.z);
       }
-      if (warp < 2) {                       // inclusive scan of the (<= 64) box sizes
-        int v = mycnt;
+      int vf = cf, vu = cu;
+      if (warp < 2) {                       // inclusive scans of the (<= 64) box sizes
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-          const int u = __shfl_up_sync(0xffffffffu, v, o);
-          if (lane >= o) v += u;
+          const int f = __shfl_up_sync(0xffffffffu, vf, o), u = __shfl_up_sync(0xffffffffu, vu, o);
+          if (lane >= o) {
+            vf += f;
+            vu += u;
+          }
         }
-        s_pre[threadIdx.x + 1] = v;         // per-warp partial; fixed up below
+        if (lane == 31) {
+          s_tot[warp] = vf;
+          s_tot[2 + warp] = vu;
+        }
       }
       __syncthreads();
-      if (threadIdx.x >= 32 && threadIdx.x < 64) s_pre[threadIdx.x + 1] += s_pre[32];
-      if (threadIdx.x == 0) s_pre[0] = 0;
+      const int nf = s_tot[0] + s_tot[1], nfe = (nf + 1) & ~1, total = nfe + s_tot[2] + s_tot[3];
+      if (threadIdx.x < nb) {
+        if (warp == 1) {
+          vf += s_tot[0];
+          vu += s_tot[2];
+        }
+        s_pos[threadIdx.x] = test ? vf - cf : nfe + vu - cu;
+      }
       __syncthreads();
-      const int total = s_pre[nb];
       for (int c0 = 0; c0 < total; c0 += kP2PChunk) {
         const int cnt = min(kP2PChunk, total - c0);
         const int npairs = (cnt + 1) >> 1;
+        const int ntest = min(max(nfe - c0, 0), cnt) >> 1;       // pairs of the tested part
         if (c0 > 0) __syncthreads();
-        for (int e = threadIdx.x; e < 2 * npairs; e += kP2PThreads) {
-          float px = 0.f, py = 0.f, pz = 0.f, cw = 0.f, gx = 0.f, gy = 0.f, gz = 0.f, rs = 3.0e18f;
-          if (e < cnt) {                    // the odd slot past the end stays a never-evaluated pad
-            const int j = c0 + e;
-            int lo = 0, hi = nb;            // last box with s_pre[box] <= j
-            while (hi - lo > 1) {
-              const int mid = (lo + hi) >> 1;
-              if (s_pre[mid] <= j) lo = mid; else hi = mid;
+        // sixteen threads to a box
+        for (int bi = threadIdx.x >> 4; bi < nb; bi += kP2PThreads / 16) {
+          const int p0 = s_pos[bi], hi = min(p0 + s_cnt[bi], c0 + kP2PChunk);
+          const float ox = s_off[bi][0], oy = s_off[bi][1], oz = s_off[bi][2];
+          const bool tested = p0 < nf;
+          const int beg = s_beg[bi] - p0;
+          for (int j = max(p0, c0) + (threadIdx.x & 15); j < hi; j += 16) {
+            const float4 p = P2P_ARG(pos)[beg + j], q = P2P_ARG(nrm)[beg + j];
+            const float2 fh = P2P_ARG(xs)[beg + j];
+            const float px = __fadd_rn(p.x, ox), py = __fadd_rn(p.y, oy), pz = __fadd_rn(p.z, oz);
+            const float cw = p.w * fh.y, g = -p.w * fh.x;
+            const int e = j - c0, pr = e >> 1, ln = e & 1;
+            float *fa = reinterpret_cast<float *>(sa + pr), *fb = reinterpret_cast<float *>(sb + pr);
+            float *fc = reinterpret_cast<float *>(sc + pr), *fd = reinterpret_cast<float *>(sd + pr);
+            fa[ln] = -px; fa[2 + ln] = -py;
+            fb[ln] = -pz; fb[2 + ln] = cw;
+            fc[ln] = g * q.x; fc[2 + ln] = g * q.y;
+            fd[ln] = g * q.z;
+            fd[2 + ln] = tested ? p2p_skip_radius(P2P_ARG(skip_scale), q.w) : cw * kc.omce.x;
+            // the odd slot after the last source of either part: its neighbour's place, no
+            // weight, and in the tested part a radius that leaves it out
+            if (ln == 0 && (j + 1 == nf || j + 1 == total)) {
+              fa[1] = -px; fa[3] = -py;
+              fb[1] = -pz; fb[3] = 0.f;
+              fc[1] = 0.f; fc[3] = 0.f;
+              fd[1] = 0.f;
+              fd[3] = tested ? 3.0e18f : 0.f;
             }
-            const int sidx = s_beg[lo] + (j - s_pre[lo]);
-            const float4 p = P2P_ARG(pos)[sidx], q = P2P_ARG(nrm)[sidx];
-            const float2 fh = P2P_ARG(xs)[sidx];
-            px = __fadd_rn(p.x, s_off[lo][0]);
-            py = __fadd_rn(p.y, s_off[lo][1]);
-            pz = __fadd_rn(p.z, s_off[lo][2]);
-            cw = p.w * fh.y;
-            const float g = -p.w * fh.x;
-            gx = g * q.x; gy = g * q.y; gz = g * q.z;
-            rs = p2p_skip_radius(P2P_ARG(skip_scale), q.w);
           }
-          const int pr = e >> 1, ln = e & 1;
-          float *fa = reinterpret_cast<float *>(sa + pr), *fb = reinterpret_cast<float *>(sb + pr);
-          float *fc = reinterpret_cast<float *>(sc + pr), *fd = reinterpret_cast<float *>(sd + pr);
-          fa[ln] = -px; fa[2 + ln] = -py;
-          fb[ln] = -pz; fb[2 + ln] = cw;
-          fc[ln] = gx; fc[2 + ln] = gy;
-          fd[ln] = gz; fd[2 + ln] = rs;
         }
         __syncthreads();
         if (act) {
-          for (int e = si; e < npairs; e += slices) {
-            const float4 qa = sa[e], qb = sb[e], qc = sc[e], qd = sd[e];
-            p2p_pair2(tg, qa, qb, qc, qd, inv_e, kap, sL, nD, sY, dY);
-            p2p_pair2(tg2, qa, qb, qc, qd, inv_e, kap, sL2, nD2, sY2, dY2);
+          int e = si;
+          if (salt) {
+            for (; e < ntest; e += slices) {
+              const float4 qa = sa[e], qb = sb[e], qc = sc[e], qd = sd[e];
+              p2p_pair2<true, true>(tg, qa, qb, qc, qd, kc, sL, nD, sY, dY);
+              p2p_pair2<true, true>(tg2, qa, qb, qc, qd, kc, sL2, nD2, sY2, dY2);
+            }
+            for (; e < npairs; e += slices) {
+              const float4 qa = sa[e], qb = sb[e], qc = sc[e], qd = sd[e];
+              p2p_pair2<false, true>(tg, qa, qb, qc, qd, kc, sL, nD, sY, dY);
+              p2p_pair2<false, true>(tg2, qa, qb, qc, qd, kc, sL2, nD2, sY2, dY2);
+            }
+          } else {
+            for (; e < ntest; e += slices) {
+              const float4 qa = sa[e], qb = sb[e], qc = sc[e], qd = sd[e];
+              p2p_pair2<true, false>(tg, qa, qb, qc, qd, kc, sL, nD, sY, dY);
+              p2p_pair2<true, false>(tg2, qa, qb, qc, qd, kc, sL2, nD2, sY2, dY2);
+            }
+            for (; e < npairs; e += slices) {
+              const float4 qa = sa[e], qb = sb[e], qc = sc[e], qd = sd[e];
+              p2p_pair2<false, false>(tg, qa, qb, qc, qd, kc, sL, nD, sY, dY);
+              p2p_pair2<false, false>(tg2, qa, qb, qc, qd, kc, sL2, nD2, sY2, dY2);
+            }
           }
         }
       }
     }
     __syncthreads();
-    red[threadIdx.x] = make_float4(sL.x + sL.y, -(nD.x + nD.y), sY.x + sY.y, dY.x + dY.y);
-    red[kP2PThreads + threadIdx.x] = make_float4(sL2.x + sL2.y, -(nD2.x + nD2.y), sY2.x + sY2.y, dY2.x + dY2.y);
+    const float ie = kc.inv_e.x;
+    red[threadIdx.x] = make_float4(sL.x + sL.y, ie * (nD.x + nD.y), sY.x + sY.y, dY.x + dY.y);
+    red[kP2PThreads + threadIdx.x] = make_float4(sL2.x + sL2.y, ie * (nD2.x + nD2.y), sY2.x + sY2.y, dY2.x + dY2.y);
     __syncthreads();
     if (si == 0 && t < te) {
       const float s = (float)kInv4Pi;
@@ -710,6 +787,7 @@ __global__ void __launch_bounds__(kP2PThreads, kP2PRegBlocks) k_p2p(int nunits, 
                                                       const int32_t *__restrict__ leaves,
                                                       const int64_t *__restrict__ pptr,
                                                       const int32_t *__restrict__ pidx,
+                                                      const uint8_t *__restrict__ ptest,
                                                       const int32_t *__restrict__ bbeg,
                                                       const int32_t *__restrict__ bend,
                                                       const dbl4 *__restrict__ center,
@@ -718,15 +796,15 @@ __global__ void __launch_bounds__(kP2PThreads, kP2PRegBlocks) k_p2p(int nunits, 
                                                       const float2 *__restrict__ xs, float inv_ebar,
                                                       float kappa, float skip_scale,
                                                       float4 *__restrict__ phi) {
-  p2p_body<false>(nunits, units, leaves, pptr, pidx, bbeg, bend, center, pos, nrm, xs, inv_ebar, kappa, skip_scale,
+  p2p_body<false>(nunits, units, leaves, pptr, pidx, ptest, bbeg, bend, center, pos, nrm, xs, inv_ebar, kappa, skip_scale,
                   phi, nullptr);
 }
 
 // P2P of several problems in one launch: the units of all of them, cost-ordered together.
 __global__ void __launch_bounds__(kP2PThreads, kP2PRegBlocks) k_p2p_batch(int nunits, const int4 *__restrict__ units,
                                                                           const P2PReq *__restrict__ reqs) {
-  p2p_body<true>(nunits, units, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 0.f,
-                 0.f, 0.f, nullptr, reqs);
+  p2p_body<true>(nunits, units, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr,
+                 nullptr, 0.f, 0.f, 0.f, nullptr, reqs);
 }
 
 // ------------------------------------------------------------------------------------
@@ -914,6 +992,10 @@ Err enqueue_far(afmpb_t *h, cudaStream_t s, StageTimer *tm, int parts) {
   }
 }
 
+// kappa as the P2P pass takes it: k^2 enters it, so a value whose screening is complete
+// (e^-kr = 0 for every r above 1e-13) is cut to where k^2 and its products stay finite.
+static float p2p_kappa(const afmpb_t *h) { return (float)std::min(h->kappa, 1e15); }
+
 Err enqueue_p2p(afmpb_t *h, cudaStream_t s) {
   // Beside the far-field chain, six resident blocks per SM walk the units while the
   // chain's kernels run at a higher stream priority (measured best among four to six, and
@@ -927,9 +1009,9 @@ Err enqueue_p2p(afmpb_t *h, cudaStream_t s) {
   const int grid = overlap_p2p(h) ? std::max(1, std::min(h->p2p_nunits, std::min(h->p2p_resident, kP2PRegBlocks) * sms))
                                   : std::max(1, h->p2p_nunits);
   AFMPB_CUDA(cudaMemsetAsync(h->d_phi_near, 0, sizeof(float4) * h->n, s));   // split leaves add into it
-  k_p2p<<<grid, kP2PThreads, 0, s>>>(h->p2p_nunits, h->d_p2p_units, h->d_leaves, h->d_p2p_ptr, h->d_p2p_idx, h->d_box_begin,
+  k_p2p<<<grid, kP2PThreads, 0, s>>>(h->p2p_nunits, h->d_p2p_units, h->d_leaves, h->d_p2p_ptr, h->d_p2p_idx, h->d_p2p_test, h->d_box_begin,
                                                   h->d_box_end, h->d_box_center, h->d_pos, h->d_nrm, h->d_xs,
-                                                  (float)(1.0 / h->ebar), (float)h->kappa,
+                                                  (float)(1.0 / h->ebar), p2p_kappa(h),
                                                   (float)(kP2PSkip * h->opt.near_c), h->d_phi_near);
   return check_launch("k_p2p");
 }
@@ -939,6 +1021,7 @@ P2PReq p2p_req_of(const afmpb_t *h, const int *active) {
   q.leaves = h->d_leaves;
   q.pptr = h->d_p2p_ptr;
   q.pidx = h->d_p2p_idx;
+  q.ptest = h->d_p2p_test;
   q.bbeg = h->d_box_begin;
   q.bend = h->d_box_end;
   q.center = h->d_box_center;
@@ -948,7 +1031,7 @@ P2PReq p2p_req_of(const afmpb_t *h, const int *active) {
   q.phi = h->d_phi_near;
   q.active = active;
   q.inv_ebar = (float)(1.0 / h->ebar);
-  q.kappa = (float)h->kappa;
+  q.kappa = p2p_kappa(h);
   q.skip_scale = (float)(kP2PSkip * h->opt.near_c);
   return q;
 }

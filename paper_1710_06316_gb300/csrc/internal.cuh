@@ -217,7 +217,9 @@ struct __align__(16) TSItem {
 struct P2PReq {
   const int32_t *leaves;
   const int64_t *pptr;
-  const int32_t *pidx, *bbeg, *bend;
+  const int32_t *pidx;
+  const uint8_t *ptest;
+  const int32_t *bbeg, *bend;
   const dbl4 *center;
   const float4 *pos, *nrm;
   const float2 *xs;
@@ -289,6 +291,7 @@ struct afmpb_t {
   int32_t *d_u_idx = nullptr, *d_v_idx = nullptr, *d_w_idx = nullptr, *d_x_idx = nullptr;
   int64_t *d_p2p_ptr = nullptr;    // [nleaf+1] lists 1 + 3 per leaf (leaf order)
   int32_t *d_p2p_idx = nullptr;
+  uint8_t *d_p2p_test = nullptr;   // [entries of p2p_idx] 1 where a pair may be inside the skip radius
   int4 *d_p2p_units = nullptr;     // [p2p_nunits] P2P work units (leaf, first and end entry of its
   int p2p_nunits = 0;              // source boxes in p2p_idx, -), most pairs first
   int p2p_resident = afmpb::kP2PResident;            // P2P blocks per SM (tile tuner)

@@ -511,6 +511,61 @@ __global__ void k_p2p_units(int nleaf, const int32_t *__restrict__ leaves, const
   if (!fill) cnt[i] = nu;
 }
 
+// Extent of each leaf's nodes about its centre (as P2P sees them, FP32): one warp a leaf.
+// An empty leaf gets an extent that is far from everything.
+__global__ void k_leaf_extent(int nleaf, const int32_t *__restrict__ leaves, const int32_t *__restrict__ bbeg,
+                              const int32_t *__restrict__ bend, const float4 *__restrict__ pos,
+                              float *__restrict__ ext) {
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (i >= nleaf) return;                               // whole warps
+  const int b = leaves[i];
+  float v[6] = {3e38f, 3e38f, 3e38f, 3e38f, 3e38f, 3e38f};   // minima of x, y, z and of -x, -y, -z
+  for (int t = bbeg[b] + lane; t < bend[b]; t += 32) {
+    const float4 p = pos[t];
+    v[0] = fminf(v[0], p.x); v[1] = fminf(v[1], p.y); v[2] = fminf(v[2], p.z);
+    v[3] = fminf(v[3], -p.x); v[4] = fminf(v[4], -p.y); v[5] = fminf(v[5], -p.z);
+  }
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v[k] = fminf(v[k], __shfl_xor_sync(0xffffffffu, v[k], o));
+    if (lane == 0) ext[6 * (size_t)i + k] = v[k];
+  }
+}
+
+// test[j] = 1 where a node of source box p2p_idx[j] can be within the skip radius of a
+// target of its leaf: the gap between the two extents against the largest skip radii, with
+// a margin for the rounding of P2P's FP32 positions (2^-23 of the coordinates that a
+// distance is formed from; the margin is eight times that).  P2P does not test the other
+// boxes' pairs (they pass the test).  One warp a leaf.
+__global__ void k_p2p_test(int nleaf, const int32_t *__restrict__ leaves, const int32_t *__restrict__ leaf_index,
+                           const int64_t *__restrict__ pptr, const int32_t *__restrict__ pidx,
+                           const dbl4 *__restrict__ center, const double *__restrict__ brho,
+                           const float *__restrict__ ext, double skip, uint8_t *__restrict__ test) {
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (i >= nleaf) return;
+  const int b = leaves[i];
+  const dbl4 ct = center[b];
+  const double tc[3] = {ct.x, ct.y, ct.z};
+  for (int64_t j = pptr[i] + lane; j < pptr[i + 1]; j += 32) {
+    const int c = pidx[j];
+    const int l = leaf_index[c];
+    const dbl4 cs = center[c];
+    const double sc[3] = {cs.x, cs.y, cs.z};
+    double gap2 = 0.0, size = ct.w + cs.w;
+    for (int d = 0; d < 3; ++d) {
+      const double off = sc[d] - tc[d];                 // source minus target
+      const double above = off + ext[6 * (size_t)l + d] + ext[6 * (size_t)i + 3 + d];
+      const double below = -off + ext[6 * (size_t)i + d] + ext[6 * (size_t)l + 3 + d];
+      const double g = fmax(0.0, fmax(above, below));
+      gap2 += g * g;
+      size += fabs(off);
+    }
+    const double R = skip * (brho[b] + brho[c]) * (1.0 + 1e-5) + 1e-6 * size;
+    test[j] = gap2 <= R * R ? 1 : 0;
+  }
+}
+
 __global__ void k_gather_int4(int64_t n, const int32_t *__restrict__ idx, const int4 *__restrict__ src,
                               int4 *__restrict__ dst) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -974,6 +1029,7 @@ Err build_tree(afmpb_t *h) {
     int64_t n_p = 0;
     AFMPB_TRY(csr_ptr(h, cnt, nl, &h->d_p2p_ptr, &n_p, "p2p_ptr"));
     AFMPB_TRY(A.alloc(&h->d_p2p_idx, n_p, "p2p_idx"));
+    AFMPB_TRY(A.alloc(&h->d_p2p_test, n_p, "p2p test flags"));
     k_p2p_lists<<<div_up(nl, 64), 64, 0, s>>>(nl, h->d_leaves, bbeg, bend, bparent, bchild0, bnchild, d_uptr,
                                               h->d_u_idx, d_xptr, h->d_x_idx, d_xdirect, d_wptr, h->d_w_idx, nullptr,
                                               nullptr, nullptr, h->d_p2p_ptr, h->d_p2p_idx, true);
@@ -1070,6 +1126,15 @@ Err build_tree(afmpb_t *h) {
     k_box_rho_up<<<div_up(nl, 128), 128, 0, s>>>(ls, nl, bchild0, bnchild, h->d_box_rho);
     AFMPB_TRY(check_launch("k_box_rho_up"));
   }
+  // which P2P source boxes can hold a pair inside the skip radius
+  float *d_ext = nullptr;
+  AFMPB_TRY(A.alloc(&d_ext, 6 * (size_t)T.nleaf, "leaf extents"));
+  k_leaf_extent<<<div_up((int64_t)T.nleaf * 32, 128), 128, 0, s>>>(T.nleaf, h->d_leaves, bbeg, bend, h->d_pos, d_ext);
+  k_p2p_test<<<div_up((int64_t)T.nleaf * 32, 128), 128, 0, s>>>(T.nleaf, h->d_leaves, h->d_leaf_index, h->d_p2p_ptr,
+                                                                h->d_p2p_idx, h->d_box_center, h->d_box_rho, d_ext,
+                                                                kP2PSkip * h->opt.near_c, h->d_p2p_test);
+  AFMPB_TRY(check_launch("k_p2p_test"));
+  A.release(d_ext);
   A.release(d_cnt1);
   A.release(d_cnt2);
   A.release(d_lvl_start);
