@@ -3,8 +3,8 @@
 //
 // The product (one GMRES matvec, Sec. 2 step 3) is captured once per parts mask into a
 // CUDA graph: the far-field chain (P2M, M2M per level, M2L, P2L, L2L per level, L2P) runs
-// on the handle's capture stream while the point-to-point kernel runs beside it on a
-// second stream; the combine kernel (near correction + Eq. 5 assembly) joins them.
+// on the handle's capture stream while the point-to-point kernel and the near
+// correction run beside it on a second stream; its last kernel joins them (Eq. 5).
 // Replaying the graph replaces the paper's per-iteration DAG execution (Sec. 3.3:
 // create the DAG once, execute it many times).
 #include <algorithm>
@@ -75,6 +75,48 @@ void destroy_handle(afmpb_t *h) {
 // working sets far above it).
 constexpr int64_t kOverlapMaxNodes = 4000000;
 
+// The kernel of the caller-buffer graph that writes y: the far chain's last one, or the
+// scatter where the product has no far part.
+const void *io_output_kernel(const afmpb_t *h, int parts) {
+  return (parts & AFMPB_PART_FAR) ? far_out_kernel(h->order) : scatter_kernel();
+}
+
+// Replaces pointer argument `arg` of a kernel node's `nargs` arguments in a graph.
+Err patch_pointer(cudaGraphExec_t exec, cudaGraphNode_t node, int nargs, int arg, const void *ptr) {
+  cudaKernelNodeParams kp{};
+  AFMPB_CUDA(cudaGraphKernelNodeGetParams(node, &kp));
+  void *args[kFarOutYArg + 1];
+  for (int i = 0; i < nargs; ++i) args[i] = kp.kernelParams[i];
+  args[arg] = (void *)&ptr;
+  kp.kernelParams = args;
+  kp.extra = nullptr;
+  AFMPB_CUDA(cudaGraphExecKernelNodeSetParams(exec, node, &kp));
+  return Err{};
+}
+
+// The product's kernels with a far part: P2P and the near correction folded into its sums
+// on the low-priority side stream beside the far-field chain (up to kOverlapMaxNodes nodes;
+// before the chain above), and the chain, whose last kernel assembles the product into y
+// (caller order) or d_ys (y == nullptr).
+Err enqueue_product_far(afmpb_t *h, cudaStream_t cap, int parts, float *y) {
+  FarOut out;
+  out.diag = (parts & AFMPB_PART_DIAG) != 0;
+  out.y = y;
+  const bool near = (parts & AFMPB_PART_NEAR) != 0, beside = overlap_p2p(h);
+  cudaStream_t s = beside ? h->side : cap;
+  if (beside) {
+    cudaEventRecord(h->ev_fork, cap);
+    cudaStreamWaitEvent(h->side, h->ev_fork, 0);
+    out.join = h->ev_join;
+  }
+  Err e = enqueue_p2p(h, s);
+  if (e.ok() && near) e = enqueue_near_fold(h, s);
+  if (beside) cudaEventRecord(h->ev_join, h->side);
+  if (e.ok()) e = enqueue_far(h, cap, nullptr, kFarAll, &out);
+  else if (beside) cudaStreamWaitEvent(cap, h->ev_join, 0);
+  return e;
+}
+
 Err capture_product(afmpb_t *h, int parts, bool io = false, const float *x = nullptr, float *y = nullptr) {
   // The far-field chain (a long sequence of short, latency-bound launches) is captured
   // from a high-priority stream and P2P from a low-priority one: the kernel nodes keep the
@@ -87,26 +129,12 @@ Err capture_product(afmpb_t *h, int parts, bool io = false, const float *x = nul
   AFMPB_CUDA(cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal));
   Err e;
   if (io) e = enqueue_gather(h, cap, x);
-  int cparts = parts;
-  if (e.ok() && (parts & AFMPB_PART_FAR)) {
-    if (overlap_p2p(h)) {
-      cudaEventRecord(h->ev_fork, cap);
-      cudaStreamWaitEvent(h->side, h->ev_fork, 0);
-      e = enqueue_p2p(h, h->side);
-      if (e.ok() && (parts & AFMPB_PART_NEAR)) {   // the near SpMV beside the rest of the chain
-        e = enqueue_near_fold(h, h->side);
-        cparts |= kNearFolded;
-      }
-      cudaEventRecord(h->ev_join, h->side);
-      if (e.ok()) e = enqueue_far(h, cap);
-      cudaStreamWaitEvent(cap, h->ev_join, 0);
-    } else {
-      e = enqueue_p2p(h, cap);
-      if (e.ok()) e = enqueue_far(h, cap);
-    }
+  if (parts & AFMPB_PART_FAR) {
+    if (e.ok()) e = enqueue_product_far(h, cap, parts, y);
+  } else {
+    if (e.ok()) e = enqueue_combine(h, cap, parts);
+    if (e.ok() && io) e = enqueue_scatter(h, cap, y);
   }
-  if (e.ok()) e = enqueue_combine(h, cap, cparts);
-  if (e.ok() && io) e = enqueue_scatter(h, cap, y);
   cudaGraph_t g = nullptr;
   cudaError_t ce = cudaStreamEndCapture(cap, &g);
   if (!e.ok()) {
@@ -137,9 +165,9 @@ Err capture_product(afmpb_t *h, int parts, bool io = false, const float *x = nul
     cudaKernelNodeParams kp{};
     AFMPB_CUDA(cudaGraphKernelNodeGetParams(nd, &kp));
     if (kp.func == gather_kernel()) h->io_gather[parts] = nd;
-    if (kp.func == scatter_kernel()) h->io_scatter[parts] = nd;
+    if (kp.func == io_output_kernel(h, parts)) h->io_output[parts] = nd;
   }
-  if (!h->io_gather[parts] || !h->io_scatter[parts]) return make_err(AFMPB_ECUDA, "captured product: gather/scatter node missing");
+  if (!h->io_gather[parts] || !h->io_output[parts]) return make_err(AFMPB_ECUDA, "captured product: gather/output node missing");
   h->io_x[parts] = x;
   h->io_y[parts] = y;
   return Err{};
@@ -151,27 +179,13 @@ Err product_io(afmpb_t *h, int parts, const float *x, float *y) {
     AFMPB_TRY(capture_product(h, parts, true, x, y));
   } else {
     if (x != h->io_x[parts]) {
-      cudaKernelNodeParams kp{};
-      AFMPB_CUDA(cudaGraphKernelNodeGetParams(h->io_gather[parts], &kp));
-      int64_t n = h->n;
-      const int32_t *perm = h->d_perm;
-      float2 *xs = h->d_xs;
-      void *args[] = {&n, &perm, (void *)&x, &xs};
-      kp.kernelParams = args;
-      kp.extra = nullptr;
-      AFMPB_CUDA(cudaGraphExecKernelNodeSetParams(h->graph_io[parts], h->io_gather[parts], &kp));
+      AFMPB_TRY(patch_pointer(h->graph_io[parts], h->io_gather[parts], kGatherArgs, kGatherXArg, x));
       h->io_x[parts] = x;
     }
     if (y != h->io_y[parts]) {
-      cudaKernelNodeParams kp{};
-      AFMPB_CUDA(cudaGraphKernelNodeGetParams(h->io_scatter[parts], &kp));
-      int64_t n = h->n;
-      const int32_t *perm = h->d_perm;
-      const float *ys = h->d_ys;
-      void *args[] = {&n, &perm, (void *)&ys, (void *)&y};
-      kp.kernelParams = args;
-      kp.extra = nullptr;
-      AFMPB_CUDA(cudaGraphExecKernelNodeSetParams(h->graph_io[parts], h->io_scatter[parts], &kp));
+      const bool far = parts & AFMPB_PART_FAR;
+      AFMPB_TRY(patch_pointer(h->graph_io[parts], h->io_output[parts], far ? kFarOutYArg + 1 : kScatterArgs,
+                              far ? kFarOutYArg : kScatterYArg, y));
       h->io_y[parts] = y;
     }
   }
@@ -353,29 +367,10 @@ Err product_from64(afmpb_t *h, cudaStream_t s, const double *v) {
   return Err{};
 }
 
-// The product's kernels from d_xs to d_ys, enqueued on a capturing stream: P2P forked onto
-// the low-priority side stream beside the far-field chain (up to kOverlapMaxNodes), then
-// the combine.  Used by the GMRES cycle graph.
+// The product's kernels from d_xs to d_ys, enqueued on a capturing stream.  Used by the
+// GMRES cycle graph.
 Err enqueue_product_kernels(afmpb_t *h, cudaStream_t cap) {
-  Err e;
-  int cparts = AFMPB_PART_ALL;
-  if (overlap_p2p(h)) {
-    cudaEventRecord(h->ev_fork, cap);
-    cudaStreamWaitEvent(h->side, h->ev_fork, 0);
-    e = enqueue_p2p(h, h->side);
-    if (e.ok()) {                                  // the near SpMV beside the rest of the chain
-      e = enqueue_near_fold(h, h->side);
-      cparts |= kNearFolded;
-    }
-    cudaEventRecord(h->ev_join, h->side);
-    if (e.ok()) e = enqueue_far(h, cap);
-    cudaStreamWaitEvent(cap, h->ev_join, 0);
-  } else {
-    e = enqueue_p2p(h, cap);
-    if (e.ok()) e = enqueue_far(h, cap);
-  }
-  if (e.ok()) e = enqueue_combine(h, cap, cparts);
-  return e;
+  return enqueue_product_far(h, cap, AFMPB_PART_ALL, nullptr);
 }
 
 // Launch shapes and work lists live in the captured graphs: after the tile tuner changes
@@ -390,7 +385,7 @@ Err recapture_products(afmpb_t *h) {
     h->graph[p] = nullptr;
     h->graph_io[p] = nullptr;
     h->graph_io_tmpl[p] = nullptr;
-    h->io_gather[p] = h->io_scatter[p] = nullptr;
+    h->io_gather[p] = h->io_output[p] = nullptr;
     h->io_x[p] = nullptr;
     h->io_y[p] = nullptr;
   }
@@ -906,9 +901,9 @@ afmpb_status afmpb_profile_product(afmpb_t *h, int reps, void *flush, size_t flu
       out->launches[i] = launches[i];
       kernels += launches[i];
     }
-    // the captured product (overlapped P2P) runs the near correction as a kernel of its own
-    // on the P2P branch and an elementwise combine, where the stages above run one k_combine
-    out->kernels_per_product = kernels + (overlap_p2p(h) ? 1 : 0);
+    // the captured product runs the near correction as a kernel of its own after P2P and
+    // assembles y in L2P, where the stages above run k_combine and k_scatter
+    out->kernels_per_product = kernels - 1;
     // graph replays (the path afmpb_matvec takes), same flush between repetitions
     cudaEvent_t a = nullptr, b = nullptr;
     cudaEventCreate(&a);

@@ -61,93 +61,161 @@ __device__ __forceinline__ void cheb_basis(float x, float s[N], float ds[N]) {
   }
 }
 
+// 1 / w of a box of `level` (w = w0 2^-level; the power of two is exact).
+__device__ __forceinline__ float inv_width(float inv_w0, int level) { return ldexpf(inv_w0, level); }
+
+__device__ __forceinline__ float2 dup2(float a) { return make_float2(a, a); }
+
 // ------------------------------------------------------------------------------------
 // P2M: leaf sources -> Laplace and Yukawa multipole weights.
+//   A[ijk] += c Sx[i] (Sy[j] Sz[k]),  B[ijk] += dSx[i] (g_x Sy Sz) + Sx[i] (g_y dSy Sz + g_z Sy dSz)
+// A leaf takes 2 N lanes of a warp (so N = 6 puts two leaves in a warp, N = 8 two, N = 4
+// four): lane (half, k) holds the weights (., j, k) of both sums for half of the j, so that
+// a node's factors are read once per N N / 2 weights, and the x direction runs on packed
+// FP32 pairs.  Each weight adds its leaf's nodes in order.  Instruction issue bounds it: a
+// thread per (j, k) with N weights took 3.3 times the instructions and left 28 of 64 lanes
+// idle at N = 6 (35.8 us on the 163,842-node sphere, alone).
 // ------------------------------------------------------------------------------------
+constexpr int kP2MWarps = 4;        // warps per CTA
+
 template <int N>
-__global__ void __launch_bounds__(256) k_p2m(int nleaf, const int32_t *__restrict__ leaves,
-                                            const int32_t *__restrict__ bbeg, const int32_t *__restrict__ bend,
-                                            const dbl4 *__restrict__ center, const float4 *__restrict__ pos,
-                                            const float4 *__restrict__ nrm, const float2 *__restrict__ xs,
-                                            float inv_ebar, float *__restrict__ M) {
-  // Four leaves per CTA, a group of 64 threads each (synchronised by its own named
-  // barrier); thread (j, k) of a group holds the N weights (i, j, k) of both sums, so a
-  // node's y-z factors are formed once and applied along the whole x axis:
-  //   A[ijk] += c Sx[i] (Sy[j] Sz[k]),  B[ijk] += dSx[i] (g_x Sy Sz) + Sx[i] (g_y dSy Sz + g_z Sy dSz)
-  // (one leaf per 64-thread CTA ran P2M faster alone but held up P2P beside it: the
-  // product took 0.565 against 0.532 ms on the 163,842-node sphere)
-  constexpr int N2 = N * N, N3 = N2 * N;
-  constexpr int CH = 64;
-  static_assert(N2 <= 64, "one thread per (j, k)");
-  __shared__ float sxa[4][CH][2 * N];   // Sx, dSx
-  __shared__ float syza[4][CH][4 * N];  // Sy, dSy, Sz, dSz
-  __shared__ float4 swa[4][CH];         // c, g nx / w, g ny / w, g nz / w
-  const int grp = threadIdx.x >> 6, gt = threadIdx.x & 63;
-  const int li = blockIdx.x * 4 + grp;
-  if (li >= nleaf) return;                              // whole groups only (named barriers below)
-  float (*sx)[2 * N] = sxa[grp];
-  float (*syz)[4 * N] = syza[grp];
-  float4 *sw = swa[grp];
-  const int b = leaves[li];
-  const int beg = bbeg[b], end = bend[b];
-  const float invw = (float)(1.0 / center[b].w);
-  const bool act = gt < N2;
-  const int j = act ? gt / N : 0, k = act ? gt % N : 0;
-  float A[N], B[N];
+struct P2MShape {
+  static constexpr int H = (N + 1) / 2;               // packed pairs along x; j of a lane
+  static constexpr int G = 2 * N;                     // lanes of a leaf
+  static constexpr int Leaves = 32 / G;               // leaves of a warp
+  static constexpr int CH = 32 / Leaves;              // nodes of a leaf staged at a time
+  // a node's row: Sx (2 H), dSx (2 H), (Sy, Sy, dSy, dSy) per j, (Sz, dSz) per k, (c, gx, gy, gz)
+  static constexpr int oY = 4 * H, oZ = oY + 4 * N, oW = (oZ + 2 * N + 3) & ~3, Row = oW + 4;
+};
+
+template <int N>
+__global__ void __launch_bounds__(32 * kP2MWarps) k_p2m(int nleaf, const int4 *__restrict__ leaf_rec,
+                                                        float inv_w0, const float4 *__restrict__ pos,
+                                                        const float4 *__restrict__ nrm, const float2 *__restrict__ xs,
+                                                        float inv_ebar, float *__restrict__ M) {
+  using P = P2MShape<N>;
+  constexpr int N3 = N * N * N, H = P::H, CH = P::CH;
+  __shared__ __align__(16) float sm[kP2MWarps][32 * P::Row];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int l0 = (blockIdx.x * kP2MWarps + warp) * P::Leaves;
+  if (l0 >= nleaf) return;                              // whole warps
+  float *buf = sm[warp];
+  const int sub = lane / P::G, half = lane % P::G / N, k = lane % N;   // this lane's weights
+  const int ssub = lane / CH, snode = lane % CH;                       // the node that it stages
+  const int4 none = make_int4(0, 0, 0, 0);
+  const int4 rec = sub < P::Leaves && l0 + sub < nleaf ? leaf_rec[l0 + sub] : none;
+  const int4 srec = ssub < P::Leaves && l0 + ssub < nleaf ? leaf_rec[l0 + ssub] : none;
+  const int nodes = rec.z - rec.y, snodes = srec.z - srec.y;
+  const int most = __reduce_max_sync(0xffffffffu, nodes);
+  const float invw = inv_width(inv_w0, srec.w);
+  float2 A[H][H], B[H][H];
 #pragma unroll
-  for (int i = 0; i < N; ++i) A[i] = B[i] = 0.0f;
-  for (int c0 = beg; c0 < end; c0 += CH) {
-    const int cnt = min(CH, end - c0);
-    if (gt < cnt) {
-      const int t = gt;
-      const float4 p = pos[c0 + t], q = nrm[c0 + t];
-      const float2 fh = xs[c0 + t];
+  for (int j = 0; j < H; ++j)
+#pragma unroll
+    for (int i = 0; i < H; ++i) A[j][i] = B[j][i] = make_float2(0.f, 0.f);
+  float4 pn = make_float4(0.f, 0.f, 0.f, 0.f), qn = pn;  // the next chunk's node, read ahead
+  float2 fn = make_float2(0.f, 0.f);
+  auto fetch = [&](int c0) {
+    if (c0 + snode >= snodes) return;
+    const int t = srec.y + c0 + snode;
+    pn = pos[t];
+    qn = nrm[t];
+    fn = xs[t];
+  };
+  fetch(0);
+  for (int c0 = 0; c0 < most; c0 += CH) {
+    const float4 p = pn, q = qn;
+    const float2 fh = fn;
+    fetch(c0 + CH);
+    if (c0 + snode < snodes) {
+      float *row = buf + (ssub * CH + snode) * P::Row;
       float s[N], ds[N];
       cheb_basis<N>(p.x * invw, s, ds);
 #pragma unroll
-      for (int m = 0; m < N; ++m) { sx[t][m] = s[m]; sx[t][N + m] = ds[m]; }
+      for (int i = 0; i < H; ++i) {
+        const bool two = 2 * i + 1 < N;
+        *reinterpret_cast<float2 *>(row + 2 * i) = make_float2(s[2 * i], two ? s[(2 * i + 1) % N] : 0.f);
+        *reinterpret_cast<float2 *>(row + 2 * H + 2 * i) = make_float2(ds[2 * i], two ? ds[(2 * i + 1) % N] : 0.f);
+      }
       cheb_basis<N>(p.y * invw, s, ds);
 #pragma unroll
-      for (int m = 0; m < N; ++m) { syz[t][m] = s[m]; syz[t][N + m] = ds[m]; }
+      for (int j = 0; j < N; ++j)
+        *reinterpret_cast<float4 *>(row + P::oY + 4 * j) = make_float4(s[j], s[j], ds[j], ds[j]);
       cheb_basis<N>(p.z * invw, s, ds);
 #pragma unroll
-      for (int m = 0; m < N; ++m) { syz[t][2 * N + m] = s[m]; syz[t][3 * N + m] = ds[m]; }
+      for (int m = 0; m < N; ++m) *reinterpret_cast<float2 *>(row + P::oZ + 2 * m) = make_float2(s[m], ds[m]);
       const float g = -p.w * fh.x * invw;
-      sw[t] = make_float4(p.w * fh.y, g * q.x, g * q.y, g * q.z);
+      *reinterpret_cast<float4 *>(row + P::oW) = make_float4(p.w * fh.y, g * q.x, g * q.y, g * q.z);
     }
-    asm volatile("bar.sync %0, 64;" ::"r"(grp + 1) : "memory");
-    if (act) {
-      for (int t = 0; t < cnt; ++t) {
-        const float sy = syz[t][j], dsy = syz[t][N + j], sz = syz[t][2 * N + k], dsz = syz[t][3 * N + k];
-        const float4 w = sw[t];
-        const float yz = sy * sz;
-        const float pa = w.x * yz, pb = w.y * yz, pq = fmaf(w.z, dsy * sz, w.w * (sy * dsz));
+    __syncwarp();
+    const int cnt = min(CH, nodes - c0);
+#pragma unroll 2
+    for (int t = 0; t < cnt; ++t) {
+      const float *row = buf + (sub * CH + t) * P::Row;
+      const float4 w = *reinterpret_cast<const float4 *>(row + P::oW);
+      const float2 z = *reinterpret_cast<const float2 *>(row + P::oZ + 2 * k);
+      float2 x[H], dx[H];
 #pragma unroll
-        for (int i = 0; i < N; ++i) {
-          const float x = sx[t][i], dx = sx[t][N + i];
-          A[i] = fmaf(pa, x, A[i]);
-          B[i] = fmaf(pb, dx, fmaf(pq, x, B[i]));
+      for (int i = 0; i < H; ++i) {
+        x[i] = *reinterpret_cast<const float2 *>(row + 2 * i);
+        dx[i] = *reinterpret_cast<const float2 *>(row + 2 * H + 2 * i);
+      }
+      const float2 sz = dup2(z.x), dsz = dup2(z.y);
+      const float2 wc = dup2(w.x), wx = dup2(w.y), wy = dup2(w.z), wz = dup2(w.w);
+#pragma unroll
+      for (int jj = 0; jj < H; ++jj) {
+        const int j = half * H + jj;                    // the second half of an odd N has one j less
+        if (N % 2 && j >= N) continue;
+        const float4 y = *reinterpret_cast<const float4 *>(row + P::oY + 4 * j);
+        const float2 sy = make_float2(y.x, y.y), dsy = make_float2(y.z, y.w);
+        const float2 yz = __fmul2_rn(sy, sz);
+        const float2 pa = __fmul2_rn(wc, yz), pb = __fmul2_rn(wx, yz);
+        const float2 pq = __ffma2_rn(wy, __fmul2_rn(dsy, sz), __fmul2_rn(wz, __fmul2_rn(sy, dsz)));
+#pragma unroll
+        for (int i = 0; i < H; ++i) {
+          A[jj][i] = __ffma2_rn(pa, x[i], A[jj][i]);
+          B[jj][i] = __ffma2_rn(pb, dx[i], __ffma2_rn(pq, x[i], B[jj][i]));
         }
       }
     }
-    asm volatile("bar.sync %0, 64;" ::"r"(grp + 1) : "memory");
+    __syncwarp();
   }
-  if (act) {
+  if (sub >= P::Leaves || l0 + sub >= nleaf) return;
+  float *out = M + (size_t)rec.x * 2 * N3 + k;
+#pragma unroll
+  for (int jj = 0; jj < H; ++jj) {
+    const int j = half * H + jj;
+    if (N % 2 && j >= N) continue;
 #pragma unroll
     for (int i = 0; i < N; ++i) {
-      const int m = (i * N + j) * N + k;
-      M[(size_t)b * 2 * N3 + m] = fmaf(B[i], inv_ebar, A[i]);
-      M[(size_t)b * 2 * N3 + N3 + m] = A[i] + B[i];
+      const float a = (i & 1) ? A[jj][i / 2].y : A[jj][i / 2].x, v = (i & 1) ? B[jj][i / 2].y : B[jj][i / 2].x;
+      out[(i * N + j) * N] = fmaf(v, inv_ebar, a);
+      out[N3 + (i * N + j) * N] = a + v;
     }
   }
 }
 
-// Apply the separable 1-D operator S2[c] along the three axes of a box of weights.
-// transpose == false: out[i,j,k] = sum S[cx][i][i'] S[cy][j][j'] S[cz][k][k'] in[i',j',k']
-// transpose == true : out[i',j',k'] = sum S[cx][i][i'] ... in[i,j,k]
-// The operators come from shared memory (sS[c][row][q], staged by stage_m2m_ops): a
-// thread's row depends on its output point, and constant-memory reads that differ across
-// a warp are serialised.
+// ------------------------------------------------------------------------------------
+// M2M and L2L: one CTA per (parent, kernel), all of its children together, one tensor axis
+// at a time behind three barriers (six per child when a CTA took one child after the
+// other).  L2L does once what the children of a parent share: two and four applications of
+// the 1-D operators S2[c] along x and y instead of eight.  M2M keeps the children's sums
+// apart until the end and adds them in child order (sharing their sums the same way is
+// faster, 28 against 36 us on the 163,842-node sphere, but its rounding reaches the
+// solution through the BF16 pairs that the weights become).  Latency bounds both on small
+// levels (M2M took 11 us a level, alone), shared-memory reads on large ones.  A thread's
+// rows of S2 along an axis stay in registers (from constant memory, reads that differ
+// across a warp are serialised).
+// ------------------------------------------------------------------------------------
+// Rows of S2[0] and S2[1] (columns with kTranspose) at point `row`, from shared memory.
+template <int N, bool kTranspose>
+__device__ __forceinline__ void axis_rows(const float *sS, int row, float (&S)[2][N]) {
+#pragma unroll
+  for (int c = 0; c < 2; ++c)
+#pragma unroll
+    for (int q = 0; q < N; ++q) S[c][q] = sS[c * N * N + (kTranspose ? q * N + row : row * N + q)];
+}
+
 template <int N>
 __device__ __forceinline__ void stage_m2m_ops(float *sS) {
   for (int e = threadIdx.x; e < 2 * N * N; e += blockDim.x) {
@@ -156,83 +224,129 @@ __device__ __forceinline__ void stage_m2m_ops(float *sS) {
   }
 }
 
+// The children of this CTA's parent by octant.
+__device__ __forceinline__ void load_children(const int32_t *__restrict__ par_child, int (&child)[8]) {
+  const int4 *p = reinterpret_cast<const int4 *>(par_child) + 2 * (size_t)blockIdx.x;
+  const int4 a = p[0], b = p[1];
+  child[0] = a.x; child[1] = a.y; child[2] = a.z; child[3] = a.w;
+  child[4] = b.x; child[5] = b.y; child[6] = b.z; child[7] = b.w;
+}
+
 template <int N>
-__device__ __forceinline__ float apply_axis(const float *in, const float *sS, int m, int axis, int c, bool transpose) {
+constexpr int kAxisThreads = (N * N * N + 31) / 32 * 32;     // a thread to a weight
+
+// Every parent of one level sums its children's translated multipoles.
+template <int N>
+__global__ void __launch_bounds__(kAxisThreads<N>) k_m2m(const int32_t *__restrict__ par,
+                                                         const int32_t *__restrict__ par_child, float *__restrict__ M) {
+  constexpr int N3 = N * N * N;
+  __shared__ float s8[8][N3], t8[8][N3], sS[2 * N * N];
+  const int b = par[blockIdx.x], kt = blockIdx.y;
+  int child[8];
+  load_children(par_child, child);
+  stage_m2m_ops<N>(sS);
+  const int m = threadIdx.x;
+  const bool act = m < N3;
   const int i = m / (N * N), j = (m / N) % N, k = m % N;
-  const float *S = sS + c * N * N;
-  float acc = 0.0f;
+  if (act) {
+    float v[8];
 #pragma unroll
-  for (int q = 0; q < N; ++q) {
-    int src;
-    int row = axis == 0 ? i : (axis == 1 ? j : k);
-    float w = transpose ? S[q * N + row] : S[row * N + q];
-    if (axis == 0) src = q * N * N + j * N + k;
-    else if (axis == 1) src = i * N * N + q * N + k;
-    else src = i * N * N + j * N + q;
-    acc = fmaf(w, in[src], acc);
+    for (int c = 0; c < 8; ++c) v[c] = child[c] >= 0 ? M[((size_t)child[c] * 2 + kt) * N3 + m] : 0.f;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) s8[c][m] = v[c];
   }
-  return acc;
+  __syncthreads();
+  float S[2][N];
+  if (act) {
+    axis_rows<N, false>(sS, k, S);
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {                       // octants 4 cx + 2 cy + cz
+      float t = 0.f;
+#pragma unroll
+      for (int q = 0; q < N; ++q) t = fmaf(S[c & 1][q], s8[c][m - k + q], t);
+      t8[c][m] = t;
+    }
+  }
+  __syncthreads();
+  if (act) {
+    axis_rows<N, false>(sS, j, S);
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      float t = 0.f;
+#pragma unroll
+      for (int q = 0; q < N; ++q) t = fmaf(S[(c >> 1) & 1][q], t8[c][m + (q - j) * N], t);
+      s8[c][m] = t;
+    }
+  }
+  __syncthreads();
+  if (act) {
+    axis_rows<N, false>(sS, i, S);
+    float sum = 0.f;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      float t = 0.f;
+#pragma unroll
+      for (int q = 0; q < N; ++q) t = fmaf(S[c >> 2][q], s8[c][m + (q - i) * N * N], t);
+      sum += t;
+    }
+    M[((size_t)b * 2 + kt) * N3 + m] = sum;
+  }
 }
 
-// M2M: every parent of one level sums its children's translated multipoles.
+// Every box of the level below `ls` adds its parent's local expansion, re-interpolated.
 template <int N>
-__global__ void k_m2m(int ls, const int32_t *__restrict__ child0, const int32_t *__restrict__ nchild,
-                      const int4 *__restrict__ anchor, float *__restrict__ M) {
+__global__ void __launch_bounds__(kAxisThreads<N>) k_l2l(const int32_t *__restrict__ par,
+                                                         const int32_t *__restrict__ par_child, float *__restrict__ L) {
   constexpr int N3 = N * N * N;
-  __shared__ float s0[2 * N3], s1[2 * N3], sS[2 * N * N];
-  const int b = ls + blockIdx.x;
-  const int nc = nchild[b];
-  if (nc == 0) return;
+  __shared__ float s1[N3], s2[2][N3], s4[4][N3], sS[2 * N * N];
+  const int b = par[blockIdx.x], kt = blockIdx.y;
+  int child[8];
+  load_children(par_child, child);
   stage_m2m_ops<N>(sS);
-  const int e = threadIdx.x;               // (kernel, m)
-  const bool act = e < 2 * N3;
-  const int kt = e / N3, m = e % N3;
-  float acc = 0.0f;
-  for (int q = 0; q < nc; ++q) {
-    const int c = child0[b] + q;
-    const int4 a = anchor[c];
-    if (act) s0[e] = M[(size_t)c * 2 * N3 + e];
-    __syncthreads();
-    float v = act ? apply_axis<N>(s0 + kt * N3, sS, m, 2, a.z & 1, false) : 0.0f;
-    __syncthreads();
-    if (act) s1[e] = v;
-    __syncthreads();
-    v = act ? apply_axis<N>(s1 + kt * N3, sS, m, 1, a.y & 1, false) : 0.0f;
-    __syncthreads();
-    if (act) s0[e] = v;
-    __syncthreads();
-    v = act ? apply_axis<N>(s0 + kt * N3, sS, m, 0, a.x & 1, false) : 0.0f;
-    acc += v;
-    __syncthreads();
+  const int m = threadIdx.x;
+  const bool act = m < N3;
+  const int i = m / (N * N), j = (m / N) % N, k = m % N;
+  float v[8];                                           // the children's own expansions
+  if (act) {
+    s1[m] = L[((size_t)b * 2 + kt) * N3 + m];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) v[c] = child[c] >= 0 ? L[((size_t)child[c] * 2 + kt) * N3 + m] : 0.f;
   }
-  if (act) M[(size_t)b * 2 * N3 + e] = acc;
-}
-
-// L2L: every box of one level adds its parent's local expansion, re-interpolated.
-template <int N>
-__global__ void k_l2l(int ls, const int32_t *__restrict__ parent, const int4 *__restrict__ anchor,
-                      float *__restrict__ L) {
-  constexpr int N3 = N * N * N;
-  __shared__ float s0[2 * N3], s1[2 * N3], sS[2 * N * N];
-  const int b = ls + blockIdx.x;
-  const int p = parent[b];
-  stage_m2m_ops<N>(sS);
-  const int4 a = anchor[b];
-  const int e = threadIdx.x;
-  const bool act = e < 2 * N3;
-  const int kt = e / N3, m = e % N3;
-  if (act) s0[e] = L[(size_t)p * 2 * N3 + e];
   __syncthreads();
-  float v = act ? apply_axis<N>(s0 + kt * N3, sS, m, 0, a.x & 1, true) : 0.0f;
+  float S[2][N];
+  if (act) {
+    axis_rows<N, true>(sS, i, S);
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {                       // cx
+      float t = 0.f;
+#pragma unroll
+      for (int q = 0; q < N; ++q) t = fmaf(S[c][q], s1[m + (q - i) * N * N], t);
+      s2[c][m] = t;
+    }
+  }
   __syncthreads();
-  if (act) s1[e] = v;
+  if (act) {
+    axis_rows<N, true>(sS, j, S);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {                       // (cx, cy)
+      float t = 0.f;
+#pragma unroll
+      for (int q = 0; q < N; ++q) t = fmaf(S[c & 1][q], s2[c >> 1][m + (q - j) * N], t);
+      s4[c][m] = t;
+    }
+  }
   __syncthreads();
-  v = act ? apply_axis<N>(s1 + kt * N3, sS, m, 1, a.y & 1, true) : 0.0f;
-  __syncthreads();
-  if (act) s0[e] = v;
-  __syncthreads();
-  v = act ? apply_axis<N>(s0 + kt * N3, sS, m, 2, a.z & 1, true) : 0.0f;
-  if (act) L[(size_t)b * 2 * N3 + e] += v;
+  if (act) {
+    axis_rows<N, true>(sS, k, S);
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      if (child[c] < 0) continue;
+      float t = 0.f;
+#pragma unroll
+      for (int q = 0; q < N; ++q) t = fmaf(S[c & 1][q], s4[c >> 1][m - k + q], t);
+      L[((size_t)child[c] * 2 + kt) * N3 + m] = v[c] + t;
+    }
+  }
 }
 
 // ------------------------------------------------------------------------------------
@@ -394,56 +508,122 @@ __global__ void __launch_bounds__(256) k_p2l(const int32_t *__restrict__ xbox, c
 
 // ------------------------------------------------------------------------------------
 // L2P: evaluate both local expansions and their normal derivatives at leaf targets.
+// One thread per node in Morton order, whatever leaf it is in: every lane has a node (a CTA
+// per leaf left 28 of 64 lanes idle on leaves of 36).  A CTA's nodes span a few leaves,
+// whose weights are staged in shared memory a few leaves at a time.  Each sum runs in
+// ascending order of its points: the gradient of a nearly constant field is a small
+// difference, and a sum in another order moves it by more than the rest of the product's
+// rounding (which rules out packed pairs along z; pairs along y or of value and derivative
+// need the weights twice or transposed, and shared memory bounds them: 0.65 ms on 5.03M
+// nodes).  Instruction issue and the weights' reads bound it on large meshes and the
+// chain of loads (block record, leaf records, weights) on small ones.
+//
+// With kOut the product is assembled here (Eq. 5), where the far sums are in registers:
+//   y1 = alpha f - PhiL + PhiY,   y2 = alpha h - dn PhiL + dn PhiY / eps_bar
+// over far and P2P sums, the near correction being in the P2P sums; y goes to y[perm[t]]
+// (kOut == 2: caller order) or y[t] (kOut == 1).  That takes the combine and the scatter
+// (two launches and their passes over memory) off the end of the product.
 // ------------------------------------------------------------------------------------
-constexpr int kL2PThreads = 64;   // leaves hold ~cap/3 nodes on surfaces
+constexpr int kL2PLeaves = 6;
 
+// (phi, grad phi) of a local expansion at a node, the gradient in box half widths.
 template <int N>
-__global__ void __launch_bounds__(kL2PThreads, 12) k_l2p(const int32_t *__restrict__ leaves, const int32_t *__restrict__ bbeg,
-                                             const int32_t *__restrict__ bend, const dbl4 *__restrict__ center,
-                                             const float4 *__restrict__ pos, const float4 *__restrict__ nrm,
-                                             const float *__restrict__ L, float4 *__restrict__ phi) {
+__device__ __forceinline__ float4 l2p_eval(const float *Lk, const float (&sx)[N], const float (&dsx)[N],
+                                           const float (&sy)[N], const float (&dsy)[N], const float (&sz)[N],
+                                           const float (&dsz)[N]) {
+  float phi0 = 0.f, gx = 0.f, gy = 0.f, gz = 0.f;
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    float a = 0.f, bj = 0.f, cj = 0.f;
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      const float *row = Lk + (i * N + j) * N;
+      float u = 0.f, du = 0.f;
+#pragma unroll
+      for (int k = 0; k < N; ++k) {
+        float l;
+        if (N % 2 == 0) {                        // two weights to an 8-byte load
+          const float2 v = reinterpret_cast<const float2 *>(row)[k / 2];
+          l = (k & 1) ? v.y : v.x;
+        } else {
+          l = row[k];
+        }
+        u = fmaf(l, sz[k], u);
+        du = fmaf(l, dsz[k], du);
+      }
+      a = fmaf(u, sy[j], a);
+      bj = fmaf(u, dsy[j], bj);
+      cj = fmaf(du, sy[j], cj);
+    }
+    phi0 = fmaf(a, sx[i], phi0);
+    gx = fmaf(a, dsx[i], gx);
+    gy = fmaf(bj, sx[i], gy);
+    gz = fmaf(cj, sx[i], gz);
+  }
+  return make_float4(phi0, gx, gy, gz);
+}
+
+template <int N, int kOut>
+__global__ void __launch_bounds__(kL2PNodes) k_l2p(int64_t n, const int2 *__restrict__ blk,
+                                                   const int4 *__restrict__ leaf_rec, float inv_w0,
+                                                   const float4 *__restrict__ pos, const float4 *__restrict__ nrm,
+                                                   const float *__restrict__ L, float4 *__restrict__ phi,
+                                                   const float2 *__restrict__ xs, const float4 *__restrict__ pnear,
+                                                   const int32_t *__restrict__ perm, float alpha, float inv_ebar,
+                                                   int64_t ldy, float *__restrict__ y) {
   constexpr int N3 = N * N * N;
-  __shared__ float sL[2 * N3];
-  const int b = leaves[blockIdx.x];
-  for (int e = threadIdx.x; e < 2 * N3; e += blockDim.x) sL[e] = L[(size_t)b * 2 * N3 + e];
-  __syncthreads();
-  const float invw = (float)(1.0 / center[b].w);
-  for (int t = bbeg[b] + threadIdx.x; t < bend[b]; t += blockDim.x) {
-    const float4 p = pos[t], q = nrm[t];
-    float sx[N], dsx[N], sy[N], dsy[N], sz[N], dsz[N];
+  __shared__ __align__(16) float sL[kL2PLeaves][2 * N3];
+  __shared__ int4 srec[kL2PLeaves];
+  const int64_t t = blockIdx.x * (int64_t)kL2PNodes + threadIdx.x;
+  const int2 lr = blk[blockIdx.x];
+  const bool node = t < n;
+  float4 p = make_float4(0.f, 0.f, 0.f, 0.f), q = p, pn = p;
+  float2 x = make_float2(0.f, 0.f);
+  int64_t o = t;
+  if (node) {
+    p = pos[t];
+    q = nrm[t];
+    if (kOut) {
+      x = xs[t];
+      pn = pnear[t];
+      if (kOut == 2) o = perm[t];
+    }
+  }
+  for (int l0 = lr.x; l0 <= lr.y; l0 += kL2PLeaves) {
+    const int nl = min(kL2PLeaves, lr.y + 1 - l0);
+    if (l0 > lr.x) __syncthreads();
+    if (threadIdx.x < nl) srec[threadIdx.x] = leaf_rec[l0 + threadIdx.x];
+    __syncthreads();
+#pragma unroll 4
+    for (int e = threadIdx.x; e < nl * N3; e += kL2PNodes) {     // two weights at a time
+      const int l = e / N3;
+      reinterpret_cast<float2 *>(&sL[0][0])[e] =
+          reinterpret_cast<const float2 *>(L + (size_t)srec[l].x * 2 * N3)[e - l * N3];
+    }
+    __syncthreads();
+    int l = 0;
+    while (l + 1 < nl && t >= srec[l].z) ++l;
+    if (!node || t < srec[l].y || t >= srec[l].z) continue;
+    const float invw = inv_width(inv_w0, srec[l].w);
+    float sx[N], dsx[N], sy[N], dsy[N];
+    float sz[N], dsz[N];
+    cheb_basis<N>(p.z * invw, sz, dsz);
     cheb_basis<N>(p.x * invw, sx, dsx);
     cheb_basis<N>(p.y * invw, sy, dsy);
-    cheb_basis<N>(p.z * invw, sz, dsz);
-    float out[4];
+    float2 out[2];
 #pragma unroll 1
     for (int kt = 0; kt < 2; ++kt) {
-      const float *Lk = sL + kt * N3;
-      float phi0 = 0.f, gx = 0.f, gy = 0.f, gz = 0.f;
-#pragma unroll
-      for (int i = 0; i < N; ++i) {
-        float a = 0.f, bj = 0.f, cj = 0.f;
-#pragma unroll
-        for (int j = 0; j < N; ++j) {
-          float u = 0.f, du = 0.f;
-#pragma unroll
-          for (int k = 0; k < N; ++k) {
-            const float l = Lk[(i * N + j) * N + k];
-            u = fmaf(l, sz[k], u);
-            du = fmaf(l, dsz[k], du);
-          }
-          a = fmaf(u, sy[j], a);
-          bj = fmaf(u, dsy[j], bj);
-          cj = fmaf(du, sy[j], cj);
-        }
-        phi0 = fmaf(a, sx[i], phi0);
-        gx = fmaf(a, dsx[i], gx);
-        gy = fmaf(bj, sx[i], gy);
-        gz = fmaf(cj, sx[i], gz);
-      }
-      const float dn = (q.x * gx + q.y * gy + q.z * gz) * invw;
-      if (kt == 0) { out[0] = phi0; out[1] = dn; } else { out[2] = phi0; out[3] = dn; }
+      const float4 v = l2p_eval<N>(&sL[l][kt * N3], sx, dsx, sy, dsy, sz, dsz);
+      const float2 u = make_float2(v.x, (q.x * v.y + q.y * v.z + q.z * v.w) * invw);
+      if (kt == 0) out[0] = u;
+      else out[1] = u;
     }
-    phi[t] = make_float4(out[0], out[1], out[2], out[3]);
+    if (kOut) {
+      y[o] = alpha * x.x + (-(out[0].x + pn.x) + (out[1].x + pn.z));
+      y[ldy + o] = alpha * x.y + (-(out[0].y + pn.y) + (out[1].y + pn.w) * inv_ebar);
+    } else {
+      phi[t] = make_float4(out[0].x, out[0].y, out[1].x, out[1].y);
+    }
   }
 }
 
@@ -478,8 +658,6 @@ constexpr int kP2PRegBlocks = kP2PResident;
 // paired with its neighbour's, so no instruction of the loop packs or broadcasts.
 // Every packed operation rounds each lane as its scalar counterpart does, so the
 // distance and skip test below are the scalar p2p_r2 / p2p_evaluates, bit for bit.
-__device__ __forceinline__ float2 dup2(float a) { return make_float2(a, a); }
-
 // 2^x on the special-function unit (PTX ex2.approx); e^-kr = 2^(-kr log2 e).
 __device__ __forceinline__ float ex2_approx(float x) {
   float y;
@@ -896,11 +1074,11 @@ Err init_cheb_tables() {
 }
 
 template <int N>
-Err launch_far(afmpb_t *h, cudaStream_t s, StageTimer *tm, int parts) {
+Err launch_far(afmpb_t *h, cudaStream_t s, StageTimer *tm, int parts, const FarOut *out) {
   constexpr int N3 = N * N * N;
   const auto &T = h->shape;
   const float inv_ebar = (float)(1.0 / h->ebar);
-  const int mthreads = ((2 * N3 + 31) / 32) * 32;
+  const float inv_w0 = (float)(1.0 / T.w0);
   const bool plane_wave = h->opt.m2l_method == AFMPB_M2L_PLANE_WAVE;
   const bool compressed = !h->m2l_groups.empty() && h->m2l_rank > 0 && !plane_wave;
   // P2L adds into L, which the compressed M2L does not touch (it writes Lc; the expansion
@@ -921,13 +1099,14 @@ Err launch_far(afmpb_t *h, cudaStream_t s, StageTimer *tm, int parts) {
     AFMPB_TRY(launch_p2l(h->side2));
     AFMPB_CUDA(cudaEventRecord(h->ev_join2, h->side2));
   }
-  k_p2m<N><<<(T.nleaf + 3) / 4, 256, 0, s>>>(T.nleaf, h->d_leaves, h->d_box_begin, h->d_box_end, h->d_box_center, h->d_pos,
-                                   h->d_nrm, h->d_xs, inv_ebar, h->d_M);
+  k_p2m<N><<<div_up(T.nleaf, kP2MWarps * P2MShape<N>::Leaves), 32 * kP2MWarps, 0, s>>>(T.nleaf, h->d_leaf_rec, inv_w0, h->d_pos,
+                                                                 h->d_nrm, h->d_xs, inv_ebar, h->d_M);
   AFMPB_TRY(check_launch("k_p2m"));
   if (tm) tm->mark("p2m", 1);
   for (int level = T.nlevel - 2; level >= 2; --level) {
-    int ls = T.lvl_start[level], nl = T.lvl_start[level + 1] - ls;
-    k_m2m<N><<<nl, mthreads, 0, s>>>(ls, h->d_box_child0, h->d_box_nchild, h->d_box_anchor, h->d_M);
+    const int p0 = T.par_start[level], np = T.par_start[level + 1] - p0;
+    if (np == 0) continue;
+    k_m2m<N><<<dim3(np, 2), kAxisThreads<N>, 0, s>>>(h->d_par + p0, h->d_par_child + 8 * (size_t)p0, h->d_M);
     AFMPB_TRY(check_launch("k_m2m"));
   }
   if (tm) tm->mark("m2m", std::max(0, T.nlevel - 3));
@@ -956,14 +1135,28 @@ Err launch_far(afmpb_t *h, cudaStream_t s, StageTimer *tm, int parts) {
   if (!(parts & kFarDown)) return Err{};
   if (h->n_xbox > 0 && !p2l_beside) AFMPB_TRY(launch_p2l(s));
   if (tm) tm->mark("p2l", h->n_xbox > 0 ? 1 : 0);
-  for (int level = 3; level < T.nlevel; ++level) {
-    int ls = T.lvl_start[level], nl = T.lvl_start[level + 1] - ls;
-    k_l2l<N><<<nl, mthreads, 0, s>>>(ls, h->d_box_parent, h->d_box_anchor, h->d_L);
+  for (int level = 2; level + 1 < T.nlevel; ++level) {
+    const int p0 = T.par_start[level], np = T.par_start[level + 1] - p0;
+    if (np == 0) continue;
+    k_l2l<N><<<dim3(np, 2), kAxisThreads<N>, 0, s>>>(h->d_par + p0, h->d_par_child + 8 * (size_t)p0, h->d_L);
     AFMPB_TRY(check_launch("k_l2l"));
   }
   if (tm) tm->mark("l2l", std::max(0, T.nlevel - 3));
-  k_l2p<N><<<T.nleaf, kL2PThreads, 0, s>>>(h->d_leaves, h->d_box_begin, h->d_box_end, h->d_box_center, h->d_pos, h->d_nrm,
-                                   h->d_L, h->d_phi_far);
+  const int nblk = div_up(h->n, kL2PNodes);
+  const float alpha = out && out->diag ? (float)h->alpha : 0.f;
+  if (out) {
+    if (out->join) AFMPB_CUDA(cudaStreamWaitEvent(s, out->join, 0));
+    if (out->fold) AFMPB_TRY(enqueue_near_fold(h, s));
+  }
+  if (!out)
+    k_l2p<N, 0><<<nblk, kL2PNodes, 0, s>>>(h->n, h->d_l2p_blk, h->d_leaf_rec, inv_w0, h->d_pos, h->d_nrm, h->d_L,
+                                           h->d_phi_far, nullptr, nullptr, nullptr, 0.f, 0.f, 0, nullptr);
+  else if (out->y)
+    k_l2p<N, 2><<<nblk, kL2PNodes, 0, s>>>(h->n, h->d_l2p_blk, h->d_leaf_rec, inv_w0, h->d_pos, h->d_nrm, h->d_L,
+                                           nullptr, h->d_xs, h->d_phi_near, h->d_perm, alpha, inv_ebar, h->n, out->y);
+  else
+    k_l2p<N, 1><<<nblk, kL2PNodes, 0, s>>>(h->n, h->d_l2p_blk, h->d_leaf_rec, inv_w0, h->d_pos, h->d_nrm, h->d_L,
+                                           nullptr, h->d_xs, h->d_phi_near, nullptr, alpha, inv_ebar, h->n, h->d_ys);
   AFMPB_TRY(check_launch("k_l2p"));
   if (tm) tm->mark("l2p", 1);
   return Err{};
@@ -979,15 +1172,15 @@ Err set_m2l_smem() {
 
 }  // namespace
 
-Err enqueue_far(afmpb_t *h, cudaStream_t s, StageTimer *tm, int parts) {
+Err enqueue_far(afmpb_t *h, cudaStream_t s, StageTimer *tm, int parts, const FarOut *out) {
   switch (h->order) {
-    case 2: return launch_far<2>(h, s, tm, parts);
-    case 3: return launch_far<3>(h, s, tm, parts);
-    case 4: return launch_far<4>(h, s, tm, parts);
-    case 5: return launch_far<5>(h, s, tm, parts);
-    case 6: return launch_far<6>(h, s, tm, parts);
-    case 7: return launch_far<7>(h, s, tm, parts);
-    case 8: return launch_far<8>(h, s, tm, parts);
+    case 2: return launch_far<2>(h, s, tm, parts, out);
+    case 3: return launch_far<3>(h, s, tm, parts, out);
+    case 4: return launch_far<4>(h, s, tm, parts, out);
+    case 5: return launch_far<5>(h, s, tm, parts, out);
+    case 6: return launch_far<6>(h, s, tm, parts, out);
+    case 7: return launch_far<7>(h, s, tm, parts, out);
+    case 8: return launch_far<8>(h, s, tm, parts, out);
     default: return make_err(AFMPB_EINVAL, "fmm_order must be in [2, 8]");
   }
 }
@@ -995,6 +1188,18 @@ Err enqueue_far(afmpb_t *h, cudaStream_t s, StageTimer *tm, int parts) {
 // kappa as the P2P pass takes it: k^2 enters it, so a value whose screening is complete
 // (e^-kr = 0 for every r above 1e-13) is cut to where k^2 and its products stay finite.
 static float p2p_kappa(const afmpb_t *h) { return (float)std::min(h->kappa, 1e15); }
+
+const void *far_out_kernel(int order) {
+  switch (order) {
+    case 2: return (const void *)k_l2p<2, 2>;
+    case 3: return (const void *)k_l2p<3, 2>;
+    case 4: return (const void *)k_l2p<4, 2>;
+    case 5: return (const void *)k_l2p<5, 2>;
+    case 6: return (const void *)k_l2p<6, 2>;
+    case 7: return (const void *)k_l2p<7, 2>;
+    default: return (const void *)k_l2p<8, 2>;
+  }
+}
 
 Err enqueue_p2p(afmpb_t *h, cudaStream_t s) {
   // Beside the far-field chain, six resident blocks per SM walk the units while the
@@ -1049,7 +1254,7 @@ Err enqueue_p2p_batch(const P2PReq *d_reqs, const int4 *d_units, int nunits, int
 // The near-field correction of Eq. 5 folded into the P2P sums, on the P2P branch right
 // after P2P, so that it overlaps the rest of the far-field chain instead of following it:
 //   PhiL <- PhiL - sum_near (dB f - dA h),   dn PhiL <- dn PhiL - sum_near (dD f - dC h)
-// (the combine subtracts PhiL and dn PhiL, so the correction enters with its own sign).
+// (the assembly subtracts PhiL and dn PhiL, so the correction enters with its own sign).
 // Eight lanes per row walk the near-field CSR, as in k_combine.
 __global__ void __launch_bounds__(256) k_near_fold(int64_t n, const float2 *__restrict__ xs,
                                                    const int64_t *__restrict__ nptr, const int32_t *__restrict__ ncol,
@@ -1080,25 +1285,6 @@ __global__ void __launch_bounds__(256) k_near_fold(int64_t n, const float2 *__re
   }
 }
 
-// Eq. 5 assembly when the near correction is already in the P2P sums: one thread per row.
-__global__ void __launch_bounds__(256) k_combine_folded(int64_t n, int parts, float alpha, float inv_ebar,
-                                                        const float2 *__restrict__ xs, const float4 *__restrict__ pfar,
-                                                        const float4 *__restrict__ pnear, float *__restrict__ ys) {
-  const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (p >= n) return;
-  float a1 = 0.f, a2 = 0.f;
-  if (parts & AFMPB_PART_DIAG) {
-    const float2 x = xs[p];
-    a1 = alpha * x.x;
-    a2 = alpha * x.y;
-  }
-  const float4 u = pfar[p], v = pnear[p];
-  a1 += -(u.x + v.x) + (u.z + v.z);
-  a2 += -(u.y + v.y) + (u.w + v.w) * inv_ebar;
-  ys[p] = a1;
-  ys[n + p] = a2;
-}
-
 Err enqueue_near_fold(afmpb_t *h, cudaStream_t s) {
   if (h->n == 0) return Err{};
   k_near_fold<<<div_up(h->n * 8, 256), 256, 0, s>>>(h->n, h->d_xs, h->d_near_ptr, h->d_near_col, h->d_near_coef,
@@ -1107,12 +1293,6 @@ Err enqueue_near_fold(afmpb_t *h, cudaStream_t s) {
 }
 
 Err enqueue_combine(afmpb_t *h, cudaStream_t s, int parts) {
-  if (parts & kNearFolded) {          // near correction already in the P2P sums (with the far part)
-    if (h->n == 0) return Err{};
-    k_combine_folded<<<div_up(h->n, 256), 256, 0, s>>>(h->n, parts, (float)h->alpha, (float)(1.0 / h->ebar), h->d_xs,
-                                                        h->d_phi_far, h->d_phi_near, h->d_ys);
-    return check_launch("k_combine_folded");
-  }
   k_combine<<<div_up(h->n * 8, 256), 256, 0, s>>>(h->n, parts, (float)h->alpha, (float)(1.0 / h->ebar), h->d_xs,
                                                    h->d_phi_far, h->d_phi_near, h->d_near_ptr, h->d_near_col,
                                                    h->d_near_coef, h->d_ys);

@@ -32,6 +32,7 @@ constexpr double kInv4Pi = 0.07957747154594767;  // 1 / (4 pi)
 constexpr int kP2PThreads = 128;   // threads of a P2P block (one work unit of one target leaf at a time)
 constexpr int kP2PResident = 6;    // P2P blocks kept resident per SM (<= 80 registers per thread)
 constexpr int kP2PUnitsPerBlock = 3;   // P2P work units per resident block (sets the unit size; 2-3 best of 1-32)
+constexpr int kL2PNodes = 128;     // nodes of an L2P block, in Morton order
 constexpr double kP2PSkip = 0.9;    // P2P leaves out pairs closer than kP2PSkip * c * (rho_p + rho_t)
 
 // Pair geometry of the P2P pass in FP32.  Positions are relative to the target's leaf
@@ -166,6 +167,7 @@ struct DeviceArena {
 struct TreeShape {
   int nbox = 0, nleaf = 0, nlevel = 0;     // levels 0 .. nlevel-1
   std::vector<int> lvl_start;              // [nlevel + 1] box index ranges per level
+  std::vector<int> par_start;              // [nlevel + 1] the same over the boxes with children
   double c0[3] = {0, 0, 0};                // root centre
   double w0 = 1;                           // root half width (power of two)
   int64_t n_u = 0, n_v = 0, n_w = 0, n_x = 0, n_p2p_pairs = 0;
@@ -286,6 +288,10 @@ struct afmpb_t {
   int32_t *d_leaves = nullptr;     // [nleaf] leaf box ids in Morton order
   int32_t *d_node_leaf = nullptr;  // [n] Morton position -> leaf box
   int32_t *d_leaf_index = nullptr; // [nbox] leaf box -> position in d_leaves, -1 otherwise
+  int4 *d_leaf_rec = nullptr;      // [nleaf] (box, first node, end node, level)
+  int2 *d_l2p_blk = nullptr;       // [n / kL2PNodes] first and last leaf of an L2P block's nodes
+  int32_t *d_par = nullptr;        // boxes with children, ascending
+  int32_t *d_par_child = nullptr;  // [8 per such box] children by octant (4 x + 2 y + z), or -1
   // lists (CSR over boxes; u and w non-empty only for leaves)
   int64_t *d_u_ptr = nullptr, *d_v_ptr = nullptr, *d_w_ptr = nullptr, *d_x_ptr = nullptr;
   int32_t *d_u_idx = nullptr, *d_v_idx = nullptr, *d_w_idx = nullptr, *d_x_idx = nullptr;
@@ -376,7 +382,7 @@ struct afmpb_t {
   cudaGraphExec_t graph[8] = {};   // captured product (Morton-ordered d_xs -> d_ys), per parts mask
   cudaGraphExec_t graph_io[8] = {};          // the same with gather and scatter of caller buffers
   cudaGraph_t graph_io_tmpl[8] = {};         // templates of graph_io (their nodes are updated)
-  cudaGraphNode_t io_gather[8] = {}, io_scatter[8] = {};
+  cudaGraphNode_t io_gather[8] = {}, io_output[8] = {};   // the nodes that read x and write y
   const float *io_x[8] = {};                 // buffers the io graphs currently point at
   float *io_y[8] = {};
   cudaGraphExec_t graph_gm = nullptr;        // solver product: FP64 Krylov vector -> d_ys
@@ -421,7 +427,20 @@ Err build_fmm(afmpb_t *h);
 // Parts of the far-field chain: the upward pass to the compressed expansions, the M2L,
 // and the downward pass from the local expansions to d_phi_far.
 constexpr int kFarUp = 1, kFarM2L = 2, kFarDown = 4, kFarAll = 7;
-Err enqueue_far(afmpb_t *h, cudaStream_t s, StageTimer *tm = nullptr, int parts = kFarAll);   // P2M .. L2P
+// What the last pass of the chain (L2P) does with the far sums.  Without this they go to
+// d_phi_far.  With it L2P waits for `join` (the P2P sums, if given), adds the near
+// correction to those sums first when `fold` is set, and writes the product itself (Eq. 5):
+// y in caller order, or d_ys when y is null.
+struct FarOut {
+  cudaEvent_t join = nullptr;
+  bool fold = false;
+  bool diag = true;          // with alpha x
+  float *y = nullptr;
+};
+Err enqueue_far(afmpb_t *h, cudaStream_t s, StageTimer *tm = nullptr, int parts = kFarAll,
+                const FarOut *out = nullptr);   // P2M .. L2P
+const void *far_out_kernel(int order);                // the L2P kernel that writes caller-order y
+constexpr int kFarOutYArg = 14;                       // its argument y
 Err enqueue_p2p(afmpb_t *h, cudaStream_t s);          // P2P into d_phi_near
 bool overlap_p2p(const afmpb_t *h);                   // P2P runs beside the far-field chain
 // The P2P arguments of a handle, with a stop flag for batched launches.
@@ -429,9 +448,6 @@ P2PReq p2p_req_of(const afmpb_t *h, const int *active);
 // One P2P launch over the units of several problems (unit.w names the problem); every
 // problem's d_phi_near must be zeroed before it.
 Err enqueue_p2p_batch(const P2PReq *d_reqs, const int4 *d_units, int nunits, int resident, cudaStream_t s);
-// Combine flag beside the AFMPB_PART_* bits: the near correction was folded into the P2P
-// sums by enqueue_near_fold (on the P2P branch, after P2P), which requires the far part.
-constexpr int kNearFolded = 8;
 Err enqueue_near_fold(afmpb_t *h, cudaStream_t s);   // near SpMV into phi_near, after P2P
 Err enqueue_combine(afmpb_t *h, cudaStream_t s, int parts);
 Err enqueue_m2l_tc(afmpb_t *h, cudaStream_t s);       // tensor-core M2L (precision 1)
@@ -467,6 +483,7 @@ Err build_rhs(afmpb_t *h);
 Err enqueue_gather(afmpb_t *h, cudaStream_t s, const float *x_caller);
 const void *gather_kernel();                           // k_gather, to find its graph node
 const void *scatter_kernel();
+constexpr int kGatherArgs = 4, kGatherXArg = 2, kScatterArgs = 4, kScatterYArg = 3;
 const void *to_xs_kernel();
 Err enqueue_to_xs(afmpb_t *h, cudaStream_t s, const double *v);   // FP64 Morton vector -> d_xs
 Err product_from64(afmpb_t *h, cudaStream_t s, const double *v);  // d_ys = L v (one graph launch)

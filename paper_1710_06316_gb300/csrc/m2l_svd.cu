@@ -199,9 +199,11 @@ __device__ __forceinline__ void cp_async_wait_1() { asm volatile("cp.async.wait_
 // ncol = n^3), X = Lc, Y = L (accumulated).  The chunk's X vectors (X[k][box]) and slabs
 // of kSlabRows rows of A reach shared memory by cp.async in a kStages-deep pipeline, so
 // the copy of slab s + 2 overlaps the products of slab s (a K of one or two slabs gets
-// one or two buffers: the expand of r = 64 fits three CTAs per SM instead of two).  A thread owns 4 boxes x 4
-// columns per tile (two 16-byte shared loads per 16 FMAs) and up to TILES tiles; ncol is
-// a multiple of 4.
+// one or two buffers).  A thread owns TB boxes x 4 columns on packed FMAs, and adds its rows
+// in ascending order whatever TB is.  Compress takes two boxes to a thread: with four, the
+// 64 threads of r = 64 left 2.5 warps to a scheduler for a chain of 216 rows (17.8 us on 65
+// boxes, 24.6 us on 5,537, alone; row groups whose sums are added at the end are no faster
+// on large meshes and round differently).
 constexpr int kSlabRows = 32;
 constexpr int kStages = 3;
 // buffers the pipeline needs for K rows: slab s + 2 is issued while slab s is used
@@ -209,8 +211,8 @@ __host__ __device__ __forceinline__ int basis_stages(int K) {
   const int nslab = (K + kSlabRows - 1) / kSlabRows;
   return nslab < kStages ? (nslab > 0 ? nslab : 1) : kStages;
 }
-template <int TILES, bool ACCUM>
-__global__ void __launch_bounds__(256) k_box_basis(int K, int ncol, const int4 *__restrict__ chunks,
+template <int TB, bool ACCUM>
+__global__ void __launch_bounds__(512) k_box_basis(int K, int ncol, const int4 *__restrict__ chunks,
                                                    const int *__restrict__ level_table,
                                                    const int *__restrict__ table_rank, int yuk_min,
                                                    const float *__restrict__ A, const float *__restrict__ X,
@@ -229,18 +231,21 @@ __global__ void __launch_bounds__(256) k_box_basis(int K, int ncol, const int4 *
   const int slab_elems = kSlabRows * ncol;
   const int nslab = (Keff + kSlabRows - 1) / kSlabRows;
   const int nst = basis_stages(K);                     // slab buffers (fewer when K has fewer slabs)
+  const int nthr = blockDim.x, tid = threadIdx.x;
   // X: the box index runs fastest so that the shared stores hit distinct banks
-  for (int e = threadIdx.x; e < Keff * kChunkBoxes; e += blockDim.x) {
-    const int j = e % kChunkBoxes, k = e / kChunkBoxes;
+  {
+    const int j = tid % kChunkBoxes;                   // nthr is a multiple of kChunkBoxes
     const bool v = j < ch.y;
-    cp_async4(Xs + e, v ? X + ((size_t)(ch.x + j) * 2 + kt) * K + k : X, v);
+    const float *src = v ? X + ((size_t)(ch.x + j) * 2 + kt) * K : X;
+    for (int k = tid / kChunkBoxes; k < Keff; k += nthr / kChunkBoxes)
+      cp_async4(Xs + k * kChunkBoxes + j, v ? src + k : X, v);
   }
-  // a thread's 16-byte groups of a slab: (row, group) from threadIdx.x, advanced by
-  // blockDim.x groups with a carry (no division in the copy loop)
+  // a thread's 16-byte groups of a slab: (row, group) from its number, advanced by the
+  // CTA's threads with a carry (no division in the copy loop)
   const int c4n = ceff / 4;
   const int c4d = max(c4n, 1);
-  const int r_first = c4n > 0 ? (int)threadIdx.x / c4d : kSlabRows, c_first = (int)threadIdx.x % c4d;
-  const int r_step = (int)blockDim.x / c4d, c_step = (int)blockDim.x % c4d;
+  const int r_first = c4n > 0 ? tid / c4d : kSlabRows, c_first = tid % c4d;
+  const int r_step = nthr / c4d, c_step = nthr % c4d;
   auto issue_slab = [&](int sl) {
     if (sl < nslab) {
       float *dst = As + (size_t)(sl % nst) * slab_elems;
@@ -249,7 +254,7 @@ __global__ void __launch_bounds__(256) k_box_basis(int K, int ncol, const int4 *
       const float *src = At + (size_t)k0 * ncol;
       for (int r = r_first, c = c_first; r < kSlabRows;) {   // 16-byte groups used
         const bool v = r < rows;
-        cp_async16(dst + r * ncol + 4 * c, v ? src + (size_t)r * ncol + 4 * c : At, v);
+        cp_async16(dst + r * ncol + 4 * c, v ? src + r * ncol + 4 * c : At, v);
         r += r_step;
         c += c_step;
         if (c >= c4n) { c -= c4n; ++r; }
@@ -259,64 +264,65 @@ __global__ void __launch_bounds__(256) k_box_basis(int K, int ncol, const int4 *
   };
   issue_slab(0);                                       // commits X together with slab 0
   issue_slab(1);
-  const int ncol4 = ceff / 4;
-  const int ntiles = (kChunkBoxes / 4) * ncol4;
-  float acc[TILES][4][4] = {};
+  const int nct = ceff / 4;
+  const bool own = tid < (kChunkBoxes / TB) * nct;
+  const int c0 = (tid % max(nct, 1)) * 4, b0 = own ? (tid / nct) * TB : 0;
+  float2 acc[TB][2];
+#pragma unroll
+  for (int i = 0; i < TB; ++i) acc[i][0] = acc[i][1] = make_float2(0.f, 0.f);
   for (int sl = 0; sl < nslab; ++sl) {
     cp_async_wait_1();                                 // X and slab sl have landed
     __syncthreads();
     issue_slab(sl + 2);                                // its buffer held slab sl - 1
-    const float *as = As + (size_t)(sl % nst) * slab_elems;
     const int k0 = sl * kSlabRows, rows = min(kSlabRows, Keff - k0);
+    if (own) {
+      const float *pa = As + (size_t)(sl % nst) * slab_elems + c0;
+      const float *px = Xs + k0 * kChunkBoxes + b0;
+#pragma unroll 8
+      for (int kk = 0; kk < rows; ++kk, pa += ncol, px += kChunkBoxes) {
+        const float4 a = *reinterpret_cast<const float4 *>(pa);
+        float xv[TB];
+        if (TB == 4) {
+          const float4 x = *reinterpret_cast<const float4 *>(px);
+          xv[0] = x.x; xv[1] = x.y; xv[2 % TB] = x.z; xv[3 % TB] = x.w;
+        } else {
+          const float2 x = *reinterpret_cast<const float2 *>(px);
+          xv[0] = x.x; xv[1] = x.y;
+        }
 #pragma unroll
-    for (int t = 0; t < TILES; ++t) {
-      const int tile = threadIdx.x + t * blockDim.x;
-      if (tile >= ntiles) continue;
-      const int c0 = (tile % ncol4) * 4, b0 = (tile / ncol4) * 4;
-#pragma unroll 4
-      for (int kk = 0; kk < rows; ++kk) {
-        const float4 a = *reinterpret_cast<const float4 *>(as + (size_t)kk * ncol + c0);
-        const float4 x = *reinterpret_cast<const float4 *>(Xs + (size_t)(k0 + kk) * kChunkBoxes + b0);
-        const float av[4] = {a.x, a.y, a.z, a.w}, xv[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) acc[t][i][j] = fmaf(xv[i], av[j], acc[t][i][j]);
+        for (int i = 0; i < TB; ++i) {
+          acc[i][0] = __ffma2_rn(make_float2(xv[i], xv[i]), make_float2(a.x, a.y), acc[i][0]);
+          acc[i][1] = __ffma2_rn(make_float2(xv[i], xv[i]), make_float2(a.z, a.w), acc[i][1]);
+        }
       }
     }
   }
+  if (!own) return;
 #pragma unroll
-  for (int t = 0; t < TILES; ++t) {
-    const int tile = threadIdx.x + t * blockDim.x;
-    if (tile >= ntiles) continue;
-    const int c4 = tile % ncol4, b0 = (tile / ncol4) * 4;
+  for (int i = 0; i < TB; ++i) {
+    if (b0 + i >= ch.y) continue;
+    float4 *y = reinterpret_cast<float4 *>(Y + ((size_t)(ch.x + b0 + i) * 2 + kt) * ncol + c0);
+    float4 v = make_float4(acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y);
+    if (ACCUM) {
+      const float4 o = *y;
+      v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
+    }
+    *y = v;
+    if (!ACCUM && Y16) {   // the same vector split into BF16 hi / lo for the tensor-core M2L
+      const float w[4] = {v.x, v.y, v.z, v.w};
+      __align__(8) __nv_bfloat16 hi[4], lo[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      if (b0 + i >= ch.y) continue;
-      float4 *y = reinterpret_cast<float4 *>(Y + ((size_t)(ch.x + b0 + i) * 2 + kt) * ncol) + c4;
-      float4 v = make_float4(acc[t][i][0], acc[t][i][1], acc[t][i][2], acc[t][i][3]);
-      if (ACCUM) {
-        const float4 o = *y;
-        v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
+      for (int j = 0; j < 4; ++j) {
+        hi[j] = __float2bfloat16_rn(w[j]);
+        lo[j] = __float2bfloat16_rn(w[j] - __bfloat162float(hi[j]));
       }
-      *y = v;
-      if (!ACCUM && Y16) {   // the same vector split into BF16 hi / lo for the tensor-core M2L
-        const float w[4] = {v.x, v.y, v.z, v.w};
-        __align__(8) __nv_bfloat16 hi[4], lo[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          hi[j] = __float2bfloat16_rn(w[j]);
-          lo[j] = __float2bfloat16_rn(w[j] - __bfloat162float(hi[j]));
-        }
-        __nv_bfloat16 *y16 = Y16 + ((size_t)(ch.x + b0 + i) * 2 + kt) * 2 * ncol + 4 * c4;
-        *reinterpret_cast<uint2 *>(y16) = *reinterpret_cast<const uint2 *>(hi);
-        *reinterpret_cast<uint2 *>(y16 + ncol) = *reinterpret_cast<const uint2 *>(lo);
-      }
+      __nv_bfloat16 *y16 = Y16 + ((size_t)(ch.x + b0 + i) * 2 + kt) * 2 * ncol + c0;
+      *reinterpret_cast<uint2 *>(y16) = *reinterpret_cast<const uint2 *>(hi);
+      *reinterpret_cast<uint2 *>(y16 + ncol) = *reinterpret_cast<const uint2 *>(lo);
     }
   }
 }
 
-int basis_tiles(int ncol) { return ((kChunkBoxes / 4) * (ncol / 4) + 255) / 256; }
 size_t basis_smem(int K, int ncol) {
   return sizeof(float) * ((size_t)K * kChunkBoxes + (size_t)basis_stages(K) * kSlabRows * ncol);
 }
@@ -326,26 +332,16 @@ Err launch_box_basis(cudaStream_t s, dim3 grid, int K, int ncol, const int4 *chu
                      const int *table_rank, int yuk_min, const float *A, const float *X, float *Y,
                      __nv_bfloat16 *Y16 = nullptr) {
   const size_t smem = basis_smem(K, ncol);
-  const int nthr = std::min(256, (((kChunkBoxes / 4) * (ncol / 4) + 31) / 32) * 32);   // threads with a tile
-  switch (basis_tiles(ncol)) {
-    case 1: k_box_basis<1, ACCUM><<<grid, nthr, smem, s>>>(K, ncol, chunks, level_table, table_rank, yuk_min, A, X, Y, Y16); break;
-    case 2: k_box_basis<2, ACCUM><<<grid, 256, smem, s>>>(K, ncol, chunks, level_table, table_rank, yuk_min, A, X, Y, Y16); break;
-    case 3: k_box_basis<3, ACCUM><<<grid, 256, smem, s>>>(K, ncol, chunks, level_table, table_rank, yuk_min, A, X, Y, Y16); break;
-    default: k_box_basis<4, ACCUM><<<grid, 256, smem, s>>>(K, ncol, chunks, level_table, table_rank, yuk_min, A, X, Y, Y16); break;
-  }
+  // a thread to each tile: at most 512 (compress: rank <= kMaxRank; expand: n^3 <= 512)
+  constexpr int TB = ACCUM ? 4 : 2;
+  const int nthr = ((kChunkBoxes / TB) * (ncol / 4) + 31) / 32 * 32;
+  k_box_basis<TB, ACCUM><<<grid, nthr, smem, s>>>(K, ncol, chunks, level_table, table_rank, yuk_min, A, X, Y, Y16);
   return check_launch(ACCUM ? "k_box_basis expand" : "k_box_basis compress");
 }
 
 template <bool ACCUM>
 Err set_box_basis_smem(int K, int ncol) {
-  const int smem = (int)basis_smem(K, ncol);
-  switch (basis_tiles(ncol)) {
-    case 1: AFMPB_TRY(raise_smem_limit((const void *)k_box_basis<1, ACCUM>, smem)); break;
-    case 2: AFMPB_TRY(raise_smem_limit((const void *)k_box_basis<2, ACCUM>, smem)); break;
-    case 3: AFMPB_TRY(raise_smem_limit((const void *)k_box_basis<3, ACCUM>, smem)); break;
-    default: AFMPB_TRY(raise_smem_limit((const void *)k_box_basis<4, ACCUM>, smem)); break;
-  }
-  return Err{};
+  return raise_smem_limit((const void *)k_box_basis<ACCUM ? 4 : 2, ACCUM>, (int)basis_smem(K, ncol));
 }
 
 // Compressed M2L on the CUDA cores: one CTA per ((level, offset) group, kernel); the

@@ -1024,9 +1024,10 @@ Err build_batch_graph(afmpb_t *const *hs, int k, const int *ms, bool fuse_m2l, c
       afmpb_t *h = hs[i];
       const int *act = h->d_gm_int + 4;
       if (fuse_m2l) AFMPB_CUDA(cudaStreamWaitEvent(si[i], ev_m, 0));
-      AFMPB_TRY(enqueue_far(h, si[i], nullptr, kFarDown));
-      AFMPB_CUDA(cudaStreamWaitEvent(si[i], ev_p, 0));
-      AFMPB_TRY(enqueue_combine(h, si[i], AFMPB_PART_ALL));
+      FarOut out;                              // L2P after P2P and the near correction
+      out.join = ev_p;
+      out.fold = true;
+      AFMPB_TRY(enqueue_far(h, si[i], nullptr, kFarDown, &out));
       AFMPB_TRY(enqueue_step_tail(h, ms[i], si[i], act, true, loop));
       AFMPB_CUDA(cudaEventRecord(ev_e[i], si[i]));
       AFMPB_CUDA(cudaStreamWaitEvent(cap, ev_e[i], 0));

@@ -511,6 +511,47 @@ __global__ void k_p2p_units(int nleaf, const int32_t *__restrict__ leaves, const
   if (!fill) cnt[i] = nu;
 }
 
+// Work records of the far-field passes: (box, first node, end node, level) of every leaf,
+// the first and last leaf of every kL2PNodes nodes, and for every box with children its
+// eight children by octant (4 x + 2 y + z, -1 where there is none).  One load gives a CTA
+// what a chain of dependent ones over the box arrays did.
+__global__ void k_leaf_recs(int nleaf, const int32_t *__restrict__ leaves, const int32_t *__restrict__ bbeg,
+                            const int32_t *__restrict__ bend, const int32_t *__restrict__ level,
+                            int4 *__restrict__ rec) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= nleaf) return;
+  const int b = leaves[i];
+  rec[i] = make_int4(b, bbeg[b], bend[b], level[b]);
+}
+
+__global__ void k_l2p_blocks(int64_t n, const int32_t *__restrict__ node_leaf, const int32_t *__restrict__ leaf_index,
+                             int2 *__restrict__ blk) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t t0 = i * kL2PNodes;
+  if (t0 >= n) return;
+  const int64_t t1 = min(n, t0 + kL2PNodes) - 1;
+  blk[i] = make_int2(leaf_index[node_leaf[t0]], leaf_index[node_leaf[t1]]);
+}
+
+__global__ void k_parent_flag(int nbox, const int32_t *__restrict__ nchild, uint8_t *__restrict__ flag) {
+  const int b = blockIdx.x * blockDim.x + threadIdx.x;
+  if (b < nbox) flag[b] = nchild[b] > 0 ? 1 : 0;
+}
+
+__global__ void k_parent_recs(int npar, const int32_t *__restrict__ par, const int32_t *__restrict__ child0,
+                              const int32_t *__restrict__ nchild, const int4 *__restrict__ anchor,
+                              int32_t *__restrict__ child) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= npar) return;
+  const int b = par[i];
+  int c8[8] = {-1, -1, -1, -1, -1, -1, -1, -1};
+  for (int q = 0; q < nchild[b]; ++q) {
+    const int4 a = anchor[child0[b] + q];
+    c8[4 * (a.x & 1) + 2 * (a.y & 1) + (a.z & 1)] = child0[b] + q;
+  }
+  for (int c = 0; c < 8; ++c) child[8 * (size_t)i + c] = c8[c];
+}
+
 // Extent of each leaf's nodes about its centre (as P2P sees them, FP32): one warp a leaf.
 // An empty leaf gets an extent that is far from everything.
 __global__ void k_leaf_extent(int nleaf, const int32_t *__restrict__ leaves, const int32_t *__restrict__ bbeg,
@@ -1125,6 +1166,40 @@ Err build_tree(afmpb_t *h) {
     int ls = T.lvl_start[level], nl = T.lvl_start[level + 1] - ls;
     k_box_rho_up<<<div_up(nl, 128), 128, 0, s>>>(ls, nl, bchild0, bnchild, h->d_box_rho);
     AFMPB_TRY(check_launch("k_box_rho_up"));
+  }
+  // work records of the far-field passes
+  AFMPB_TRY(A.alloc(&h->d_leaf_rec, T.nleaf, "leaf records"));
+  k_leaf_recs<<<div_up(T.nleaf, 128), 128, 0, s>>>(T.nleaf, h->d_leaves, bbeg, bend, h->d_box_level, h->d_leaf_rec);
+  AFMPB_TRY(A.alloc(&h->d_l2p_blk, div_up(n, kL2PNodes), "l2p blocks"));
+  k_l2p_blocks<<<div_up(div_up(n, kL2PNodes), 128), 128, 0, s>>>(n, h->d_node_leaf, h->d_leaf_index, h->d_l2p_blk);
+  AFMPB_TRY(check_launch("k_l2p_blocks"));
+  {
+    uint8_t *flag = nullptr;
+    int32_t *iota = nullptr, *d_npar = nullptr;
+    int npar = 0;
+    AFMPB_TRY(A.alloc(&flag, nbox, "parent flags"));
+    AFMPB_TRY(A.alloc(&iota, nbox, "parent iota"));
+    AFMPB_TRY(A.alloc(&d_npar, 1, "parent count"));
+    AFMPB_TRY(A.alloc(&h->d_par, nbox, "parents"));
+    k_parent_flag<<<div_up(nbox, 256), 256, 0, s>>>(nbox, bnchild, flag);
+    k_iota<<<div_up(nbox, 256), 256, 0, s>>>(nbox, iota);
+    AFMPB_TRY(check_launch("k_parent_flag"));
+    AFMPB_TRY(cub_call(h, "parent select", [&](void *t, size_t &bytes) {
+      return cub::DeviceSelect::Flagged(t, bytes, iota, flag, h->d_par, d_npar, nbox, s);
+    }));
+    AFMPB_TRY(read_one(&npar, d_npar, s));
+    A.release(flag);
+    A.release(iota);
+    A.release(d_npar);
+    AFMPB_TRY(A.alloc(&h->d_par_child, 8 * (size_t)npar, "parent records"));
+    k_parent_recs<<<div_up(std::max(npar, 1), 128), 128, 0, s>>>(npar, h->d_par, bchild0, bnchild, banchor,
+                                                                h->d_par_child);
+    AFMPB_TRY(check_launch("k_parent_recs"));
+    std::vector<int32_t> par(npar);
+    if (npar > 0) AFMPB_TRY(to_host(par, h->d_par, npar, s));
+    T.par_start.assign(T.nlevel + 1, npar);
+    for (int l = 0; l <= T.nlevel; ++l)
+      T.par_start[l] = (int)(std::lower_bound(par.begin(), par.end(), T.lvl_start[l]) - par.begin());
   }
   // which P2P source boxes can hold a pair inside the skip radius
   float *d_ext = nullptr;
