@@ -73,7 +73,9 @@ Err build_batch_lists(afmpb_t *const *hs, int k, bool fuse_m2l, BatchLists &L) {
     nunits += h->p2p_nunits;
     if (fuse_m2l) {
       ts[i].runs = h->d_ts_runs;
+      ts[i].masks = h->d_ts_masks;
       ts[i].ent = h->d_ts_ent;
+      ts[i].box = h->d_ts_box;
       ts[i].Mc16 = h->d_Mc16;
       ts[i].tiles = h->d_ts_tiles;
       ts[i].Lc = h->d_Lc;

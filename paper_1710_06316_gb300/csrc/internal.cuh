@@ -202,8 +202,13 @@ struct TCItem {
   int group, start, count;
 };
 
+// Target boxes of the target-stationary M2L: slots [begin, end) of d_ts_box, all of one level.
+struct TSBlock {
+  int begin, end, level;
+};
+
 // One item of the target-stationary tensor-core M2L: a block of up to 128 target boxes
-// [base, end) of one level, the runs [run0, run1) of its (offset, pairs) work and their
+// (slots [base, end) of d_ts_box) of one level, the runs [run0, run1) of its (offset, pairs) work and their
 // entries [ent0, ent1), the kernel (0 Laplace, 1 Yukawa), its compressed table and rank,
 // and the output scale.
 struct __align__(16) TSItem {
@@ -234,7 +239,9 @@ struct P2PReq {
 // multipoles, tables and local expansions, and its stop flag.
 struct TSReq {
   const int4 *runs;
+  const uint4 *masks;
   const uint64_t *ent;
+  const int32_t *box;
   const void *Mc16, *tiles;
   float *Lc;
   const int *active;
@@ -366,7 +373,10 @@ struct afmpb_t {
   float *d_pw_exs = nullptr, *d_pw_ext = nullptr, *d_pw_om = nullptr;
   float2 *d_pw_phx = nullptr, *d_pw_phy = nullptr, *d_pw_shift = nullptr, *d_pw_X = nullptr;
   int *d_pw_tbox = nullptr, *d_pw_dptr = nullptr, *d_pw_esrc = nullptr, *d_pw_eslot = nullptr;
+  std::vector<afmpb::TSBlock> ts_blocks;
+  int32_t *d_ts_box = nullptr;     // [nbox] target box of each slot: by level, and by octant on large levels
   int4 *d_ts_runs = nullptr;       // (offset slot, first entry, end entry, -)
+  uint4 *d_ts_masks = nullptr;     // the block rows present in each run
   uint64_t *d_ts_ent = nullptr;    // row in the block << 32 | source box
   uint16_t *d_ts_tiles = nullptr;  // C_o as BF16 hi/lo B-operand tiles [table][slot][2][R x R]
 

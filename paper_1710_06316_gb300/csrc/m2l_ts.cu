@@ -3,7 +3,7 @@
 //
 // The M2L of a level sums, for every target box b,   Lc[b] += sum_o C_o Mc[src(b, o)]
 // over the offsets o of its list 2 (paper Sec. 3: the V-list translations of the FMM).
-// Here a work item is a block of 128 consecutive target boxes of one level and one kernel
+// Here a work item is a block of up to 128 target boxes of one level and one kernel
 // (Laplace or Yukawa) with a range of its offsets (each offset's pairs form one run).  For each offset the source vectors of
 // the targets that have a source there are gathered into the rows of the A operand (absent
 // targets get zero rows), the translation C_o is the B operand, and
@@ -13,13 +13,22 @@
 // read once per item and added into the targets' compressed local vectors: one write per
 // target and item instead of one per translated pair.
 //
-// Warp roles (288 threads): warps 0-3 gather the A operand of the next offset (16-byte
-// cp.async, zero fill for absent rows) while one thread brings C_o by bulk asynchronous
+// Blocks: a list-2 source of a child in octant (cx, cy, cz) of its parent lies at -3 .. 2 or
+// -2 .. 3 along each axis, by the octant, so boxes of one octant share 189 of the 316
+// offsets.  On levels of many boxes a block therefore takes boxes of one octant (in box
+// order), which leaves fewer runs with more pairs each.
+//
+// Warp roles (288 threads): warps 0-3 gather the A operand of the next runs (16-byte
+// cp.async) while one thread brings C_o by bulk asynchronous
 // copy; warp 8 issues the MMAs; warps 4-7 read the accumulator (tcgen05.ld, one target
 // per lane) and add it into Lc.  Two operand stages and two accumulators let the gather of
-// offset k + 1, the MMAs of offset k and the epilogue of the previous item overlap.  Every
-// mbarrier wait is bounded: on expiry the CTA records the handle's error flag, lets its
-// own MMAs drain (bounded), frees its tensor memory and returns.
+// offset k + 1, the MMAs of offset k and the epilogue of the previous item overlap.  A stage
+// belongs to two of the gather warps, so that one run's copies are in flight while the other
+// two warps issue the next run's (with all four on every run and a barrier of theirs before
+// and after it, the kernel's time was that of its ~1.3 us chain of issue, latency and MMAs
+// per run: 122 us on the 163,842-node sphere, 94 now; 4.90 -> 2.76 ms on 5.03M nodes).  Every mbarrier wait is bounded: on expiry the
+// warp records the handle's error flag, the CTA's MMAs drain (bounded), its tensor memory is
+// freed and it returns.
 #include <cuda_bf16.h>
 
 #include <cub/cub.cuh>
@@ -35,7 +44,10 @@ constexpr int kTsRows = 128;                   // target boxes per block (MMA M,
 constexpr int kTsThreads = 288;                // 4 gather warps, 4 epilogue warps, 1 MMA warp
 constexpr int kTsMaxR = 112;                   // largest compressed rank this kernel takes
 constexpr int kTsItemRuns = 32;                // most runs (offsets) in one item
-constexpr int kTsItemEnt = 512;                // most entries (translated pairs) in one item
+constexpr int kTsItemEnt = 768;                // most entries (translated pairs) in one item
+// Levels with at least this many boxes are blocked by octant: eight part-filled blocks of
+// 189 offsets replace six full ones of 316.
+constexpr int kTsOctantBoxes = 6 * kTsRows;
 
 // B operand tiles: C_o split into BF16 hi / lo in the canonical K-major layout with R rows.
 // out: [table][slot][hi, lo][R x R]
@@ -54,32 +66,66 @@ __global__ void k_ts_tables(int R, int ntables, const float *__restrict__ C, __n
   }
 }
 
+// Block group of every box: level * 8 + octant on levels blocked by octant, level * 8 else.
+__global__ void k_ts_groups(int nbox, const int4 *__restrict__ anchor, const int *__restrict__ lvl_start,
+                            uint32_t *__restrict__ group, int32_t *__restrict__ box) {
+  const int b = blockIdx.x * blockDim.x + threadIdx.x;
+  if (b >= nbox) return;
+  const int4 a = anchor[b];
+  const bool split = lvl_start[a.w + 1] - lvl_start[a.w] >= kTsOctantBoxes;
+  group[b] = (uint32_t)(8 * a.w + (split ? 4 * (a.x & 1) + 2 * (a.y & 1) + (a.z & 1) : 0));
+  box[b] = b;
+}
+
+// start[g] = first slot (position in the order by group) of group g, start[ngroup] = nbox;
+// slot_of[box] = its slot
+__global__ void k_ts_slots(int nbox, int ngroup, const uint32_t *__restrict__ group, const int32_t *__restrict__ box,
+                           int *__restrict__ start, int32_t *__restrict__ slot_of) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < nbox) slot_of[box[i]] = i;
+  if (i <= ngroup) {
+    int lo = 0, hi = nbox;
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if (group[mid] < (uint32_t)i) lo = mid + 1;
+      else hi = mid;
+    }
+    start[i] = lo;
+  }
+}
+
 // (block, offset) key and (row, source) entry of every list-2 pair: key = global block *
 // kNumOffsets + offset slot, entry = row << 32 | source box.
 __global__ void k_ts_keys(const M2LGroup *__restrict__ groups, const int2 *__restrict__ pairs,
-                          const int *__restrict__ lvl_start, const int *__restrict__ blk_start,
+                          const uint32_t *__restrict__ group, const int32_t *__restrict__ slot_of,
+                          const int *__restrict__ grp_start, const int *__restrict__ grp_block,
                           uint32_t *__restrict__ key, uint64_t *__restrict__ ent) {
   const M2LGroup g = groups[blockIdx.x];
   for (int j = threadIdx.x; j < g.count; j += blockDim.x) {
     const int2 pr = pairs[g.start + j];
-    const int rel = pr.x - lvl_start[g.level];
-    const int blk = blk_start[g.level] + rel / kTsRows;
+    const int slot = slot_of[pr.x];
+    const int q = (int)group[slot], rel = slot - grp_start[q];
+    const int blk = grp_block[q] + rel / kTsRows;
     key[g.start + j] = (uint32_t)blk * kNumOffsets + (uint32_t)g.offset;
     ent[g.start + j] = ((uint64_t)(uint32_t)(rel % kTsRows) << 32) | (uint32_t)pr.y;
   }
 }
 
-__device__ __forceinline__ void ts_producer_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
-__device__ __forceinline__ bool ts_producer_all(bool v) {
-  uint32_t r;
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 q, %1, 0;\n\tbar.red.and.pred p, 1, 128, q;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(r)
-      : "r"((uint32_t)v)
-      : "memory");
-  return r != 0;
+// The rows present in each run, as a 128-bit mask.
+__global__ void k_ts_masks(int nruns, const int4 *__restrict__ runs, const uint64_t *__restrict__ ent,
+                           uint4 *__restrict__ mask) {
+  const int r = blockIdx.x * blockDim.x + threadIdx.x;
+  if (r >= nruns) return;
+  uint32_t m[4] = {0, 0, 0, 0};
+  for (int e = runs[r].y; e < runs[r].z; ++e) {
+    const int row = (int)(ent[e] >> 32);
+#pragma unroll
+    for (int w = 0; w < 4; ++w) m[w] |= row >> 5 == w ? 1u << (row & 31) : 0u;
+  }
+  mask[r] = make_uint4(m[0], m[1], m[2], m[3]);
 }
+
+__device__ __forceinline__ void ts_producer_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
 __device__ __forceinline__ void red_add_v4(float *addr, float a, float b, float c, float d) {
   asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(addr), "f"(a), "f"(b), "f"(c), "f"(d)
                : "memory");
@@ -91,7 +137,9 @@ __device__ __forceinline__ void red_add_v4(float *addr, float a, float b, float 
 template <int NS, bool kBatch>
 __global__ void __launch_bounds__(kTsThreads) k_m2l_ts(int R, int nitems_arg, const TSItem *__restrict__ items,
                                                       const int4 *__restrict__ runs_1,
+                                                      const uint4 *__restrict__ masks_1,
                                                       const uint64_t *__restrict__ ent_1,
+                                                      const int32_t *__restrict__ box_1,
                                                       const __nv_bfloat16 *__restrict__ Mc16_1,
                                                       const __nv_bfloat16 *__restrict__ tiles_1,
                                                       float *__restrict__ Lc_1, int *__restrict__ err_flag,
@@ -100,6 +148,8 @@ __global__ void __launch_bounds__(kTsThreads) k_m2l_ts(int R, int nitems_arg, co
   extern __shared__ __align__(128) uint8_t smem[];
   const int nitems = kBatch ? *d_nitems : nitems_arg;
   auto runs_of = [&](const TSItem &it) -> const int4 * { return kBatch ? reqs[it.req].runs : runs_1; };
+  auto masks_of = [&](const TSItem &it) -> const uint4 * { return kBatch ? reqs[it.req].masks : masks_1; };
+  auto box_of = [&](const TSItem &it) -> const int32_t * { return kBatch ? reqs[it.req].box : box_1; };
   auto ent_of = [&](const TSItem &it) -> const uint64_t * { return kBatch ? reqs[it.req].ent : ent_1; };
   auto mc_of = [&](const TSItem &it) -> const __nv_bfloat16 * {
     return kBatch ? reinterpret_cast<const __nv_bfloat16 *>(reqs[it.req].Mc16) : Mc16_1;
@@ -114,15 +164,19 @@ __global__ void __launch_bounds__(kTsThreads) k_m2l_ts(int R, int nitems_arg, co
   const uint32_t s_base = cvta_smem(smem);
   __shared__ __align__(8) uint64_t bar_full[NS], bar_empty[NS], bar_accf[2], bar_acce[2];
   __shared__ uint32_t tmem_base;
-  __shared__ uint32_t s_old[NS][4], s_new[NS][4];        // rows present in each stage: last run, run being staged
-  __shared__ __align__(16) int4 s_runs[2][kTsItemRuns];   // the runs and entries of two items, brought
-  __shared__ __align__(16) uint64_t s_ent[2][kTsItemEnt + 2];   // in by bulk copy one item ahead
-  __shared__ __align__(8) uint64_t bar_item[2];
+  __shared__ __align__(16) int4 s_runs[2][kTsItemRuns];   // the runs, their row masks and the entries of
+  __shared__ __align__(16) uint4 s_mask[2][kTsItemRuns];  // two items, brought in by bulk copy one item
+  __shared__ __align__(16) uint64_t s_ent[2][kTsItemEnt + 2];   // ahead
+  __shared__ __align__(8) uint64_t bar_item[2], bar_ifree[2];
   __shared__ int s_last;                                 // runs whose MMAs were committed (failure drain)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int per = (nitems + (int)gridDim.x - 1) / (int)gridDim.x;
-  const int i0 = (int)blockIdx.x * per, i1 = min(nitems, i0 + per);
-  if (i0 >= i1) return;                                  // uniform per CTA
+  // The items are ordered by cost (few to a CTA) or by block (many): round k of the CTAs
+  // takes the next gridDim.x items, in alternating direction.
+  const int G = (int)gridDim.x;
+  auto item_at = [&](int k) { return k * G + ((k & 1) ? G - 1 - (int)blockIdx.x : (int)blockIdx.x); };
+  int nk = 0;                                            // this CTA's items: item_at(0 .. nk - 1)
+  while (nk * G < nitems && item_at(nk) < nitems) ++nk;
+  if (nk == 0) return;                                   // uniform per CTA
   uint32_t mb_full[NS], mb_empty[NS], mb_accf[2], mb_acce[2];
   for (int b = 0; b < NS; ++b) {
     mb_full[b] = cvta_smem(&bar_full[b]);
@@ -142,13 +196,14 @@ __global__ void __launch_bounds__(kTsThreads) k_m2l_ts(int R, int nitems_arg, co
   }
   if (threadIdx.x == 0) {
     for (int b = 0; b < NS; ++b) {
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mb_full[b]));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(mb_full[b]), "r"(4 / NS + 1));   // its warps, and C_o
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mb_empty[b]));
     }
     for (int b = 0; b < 2; ++b) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mb_accf[b]));
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 4;" ::"r"(mb_acce[b]));   // one arrival per epilogue warp
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(cvta_smem(&bar_item[b])));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 4;" ::"r"(cvta_smem(&bar_ifree[b])));
     }
     asm volatile("fence.mbarrier_init.release.cluster;");
     s_last = 0;
@@ -160,148 +215,119 @@ __global__ void __launch_bounds__(kTsThreads) k_m2l_ts(int R, int nitems_arg, co
   bool failed = false;
 
   if (warp < 4) {
-    // ---- gather: the A operand of run k + 1 is staged while run k's MMAs are issued -----
-    // Each run has at most one entry per target row (a target has one source per offset),
-    // so producer thread t copies the row of the run's t-th entry.  A stage keeps the rows
-    // of its last run: a 128-bit mask per stage records them, and a row that was present
-    // and is not now is cleared, so rows that stay absent cost nothing.  The runs and
-    // entries of an item are brought into shared memory by bulk copy one item ahead.
+    // ---- gather -------------------------------------------------------------------------
+    // Each run has at most one entry per target row (a target has one source per offset).  A
+    // stage keeps the rows of its last run: a row that was present and is not now is
+    // cleared by the row's thread, so rows that stay absent cost nothing.
     const uint32_t mb_item[2] = {cvta_smem(&bar_item[0]), cvta_smem(&bar_item[1])};
-    auto load_item = [&](int k, int b) {                 // thread 0: item k's runs and entries -> buffer b
-      const TSItem it = items[k];
+    const uint32_t mb_ifree[2] = {cvta_smem(&bar_ifree[0]), cvta_smem(&bar_ifree[1])};
+    auto load_item = [&](int k) {                        // thread 0: item k's runs and entries -> buffer k & 1
+      const TSItem it = items[item_at(k)];
+      const int b = k & 1;
       const uint32_t rb = (uint32_t)(it.run1 - it.run0) * 16;
       const int a0 = it.ent0 & ~1;                       // 16-byte aligned start (entries are 8 bytes)
       const uint32_t eb = (uint32_t)(((it.ent1 - a0) + 1) & ~1) * 8;
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // earlier reads of the buffer done
-      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mb_item[b]), "r"(rb + eb) : "memory");
-      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                       cvta_smem(&s_runs[b][0])),
-                   "l"(runs_of(it) + it.run0), "r"(rb), "r"(mb_item[b])
-                   : "memory");
-      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                       cvta_smem(&s_ent[b][0])),
-                   "l"(ent_of(it) + a0), "r"(eb), "r"(mb_item[b])
-                   : "memory");
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mb_item[b]), "r"(2 * rb + eb) : "memory");
+      auto copy = [&](const void *dst, const void *src, uint32_t bytes) {
+        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                         cvta_smem(dst)),
+                     "l"(src), "r"(bytes), "r"(mb_item[b])
+                     : "memory");
+      };
+      copy(&s_runs[b][0], runs_of(it) + it.run0, rb);
+      copy(&s_mask[b][0], masks_of(it) + it.run0, rb);
+      copy(&s_ent[b][0], ent_of(it) + a0, eb);
     };
     int issued = -1, waited = -1;                        // item positions loaded / waited for (thread 0 issues)
-    if (threadIdx.x == 0) {
-      load_item(i0, 0);
-      issued = 0;
-      if (i0 + 1 < i1) {
-        load_item(i0 + 1, 1);
-        issued = 1;
-      }
-    }
-    // cursor over this CTA's runs
-    int c_it = i0, c_k = 0;                              // item, its position among this CTA's items
-    TSItem c_item = items[i0];
-    int c_r = c_item.run0;
-    if (!ts_producer_all(mbar_wait(mb_item[0], 0))) failed = true;
-    waited = 0;
-    auto stage_run = [&](int s) {                        // stage run (c_item, c_r) into stage s
-      const int b = c_k & 1;
-      const int4 run = s_runs[b][c_r - c_item.run0];     // (offset slot, first entry, end entry, -)
-      const uint32_t st = s_base + (uint32_t)s * stage_bytes;
-      if (threadIdx.x == 0) {
-        // C_o of the item's table: hi and lo tiles, counted on the stage's full barrier
-        const __nv_bfloat16 *src = tiles_of(c_item) + ((size_t)c_item.table * kNumOffsets + run.x) * 2 * R * R;
-        asm volatile("mbarrier.expect_tx.shared::cta.b64 [%0], %1;" ::"r"(mb_full[s]), "r"(2 * b_bytes) : "memory");
-        asm volatile(
-            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                st + 2 * a_bytes),
-            "l"(src), "r"(b_bytes), "r"(mb_full[s])
-            : "memory");
-        asm volatile(
-            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                st + 2 * a_bytes + b_bytes),
-            "l"(src + R * R), "r"(b_bytes), "r"(mb_full[s])
-            : "memory");
-      }
-      const int e = run.y + (int)threadIdx.x;
-      const bool have = e < run.z;
-      const uint64_t v = have ? s_ent[b][(c_item.ent0 & 1) + (e - c_item.ent0)] : 0ull;
-      const int prow = (int)(v >> 32), psrc = (int)(uint32_t)v;
-      if (have) atomicOr(&s_new[s][prow >> 5], 1u << (prow & 31));
-      ts_producer_sync();
-      const int row = threadIdx.x;
-      const bool was = (s_old[s][row >> 5] >> (row & 31)) & 1u;
-      const bool now = (s_new[s][row >> 5] >> (row & 31)) & 1u;
-      if (have) {
-        const int kg = c_item.rank / 8;                  // 16-byte groups along K that the MMAs read
-        const __nv_bfloat16 *g = mc_of(c_item) + ((size_t)psrc * 2 + c_item.kt) * 2 * R;
-        for (int k8 = 0; k8 < kg; ++k8) {
-          const uint32_t off = canon_off(prow, k8 * 8, kTsRows);
-          cp_async16_zfill(st + off, g + k8 * 8, true);
-          cp_async16_zfill(st + a_bytes + off, g + R + k8 * 8, true);
-        }
-      }
-      if (was && !now) {
-        for (int k8 = 0; k8 < R / 8; ++k8) {
-          const uint32_t off = canon_off(row, k8 * 8, kTsRows);
-          asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(st + off), "r"(0u) : "memory");
-          asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(st + a_bytes + off), "r"(0u) : "memory");
-        }
-      }
-      asm volatile("cp.async.commit_group;" ::: "memory");
-      ts_producer_sync();                                // every thread has read the masks and its entry
-      if (threadIdx.x < 4) {
-        s_old[s][threadIdx.x] = s_new[s][threadIdx.x];
-        s_new[s][threadIdx.x] = 0u;
-      }
-    };
-    auto advance = [&]() -> bool {                       // next run of this CTA; false at the end
-      if (++c_r < c_item.run1) return true;
-      // item c_k is fully staged: its buffer takes item c_k + 2
-      if (threadIdx.x == 0 && c_it + 2 < i1) {
-        load_item(c_it + 2, c_k & 1);
-        issued = c_k + 2;
-      }
-      if (++c_it >= i1) return false;
-      ++c_k;
-      c_item = items[c_it];
-      c_r = c_item.run0;
-      if (!ts_producer_all(mbar_wait(mb_item[c_k & 1], (uint32_t)((c_k >> 1) & 1)))) failed = true;
-      waited = c_k;
-      return !failed;
-    };
+    if (threadIdx.x == 0)
+      for (; issued < 1 && issued + 1 < nk; ++issued) load_item(issued + 1);
     // the stages start all zero (no row present)
-    if (threadIdx.x < 4 * NS) {
-      (&s_old[0][0])[threadIdx.x] = 0u;
-      (&s_new[0][0])[threadIdx.x] = 0u;
-    }
     for (uint32_t o = threadIdx.x * 16; o < NS * stage_bytes; o += 128 * 16)
       asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(s_base + o), "r"(0u) : "memory");
     ts_producer_sync();
-    if (!failed) {
-      // runs are staged up to NS - 1 ahead of the MMAs: run `use` is announced as soon as
-      // its copies have landed, then run use + NS - 1 is staged into the stage that run
-      // use - 1 read
-      int staged = 0;
-      bool more = true;
-      for (; staged < NS - 1 && more; ++staged) {
-        stage_run(staged % NS);
-        more = advance();
+    // a stage belongs to 4 / NS of the warps, which gather every NS-th run: the copies of
+    // one run are in flight while the next run's are issued and the previous one's MMAs run
+    constexpr int kStageThreads = 128 / NS;
+    const int s = threadIdx.x / kStageThreads, ts = threadIdx.x % kStageThreads;
+    const uint32_t st = s_base + (uint32_t)s * stage_bytes;
+    uint32_t was = 0;                                    // bit i: row ts + i kStageThreads is present
+    int use = 0;
+    for (int k = 0; k < nk && !failed; ++k) {
+      const TSItem item = items[item_at(k)];
+      const int b = k & 1;
+      if (!__all_sync(0xffffffffu, mbar_wait(mb_item[b], (uint32_t)((k >> 1) & 1)))) {
+        failed = true;
+        break;
       }
-      for (int use = 0; !failed; ++use) {
-        const int s = use % NS;
-        if (more) asm volatile("cp.async.wait_group %0;" ::"n"(NS - 2) : "memory");   // run `use` has landed
-        else asm volatile("cp.async.wait_group 0;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        ts_producer_sync();
-        if (threadIdx.x == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(mb_full[s]) : "memory");
-        if (more) {
-          const int s1 = staged % NS;
-          bool ok = true;
-          if (staged >= NS) ok = mbar_wait(mb_empty[s1], (uint32_t)(((staged / NS) - 1) & 1));   // its last MMAs done
-          if (!ts_producer_all(ok)) {
-            failed = true;
-            break;
-          }
-          stage_run(s1);
-          ++staged;
-          more = advance();
+      waited = k;
+      const __nv_bfloat16 *mc = mc_of(item) + (size_t)item.kt * 2 * R;
+      const __nv_bfloat16 *tl = tiles_of(item) + (size_t)item.table * kNumOffsets * 2 * R * R;
+      const int kg = item.rank / 8;                      // 16-byte groups along K that the MMAs read
+      for (int r = 0; r < item.run1 - item.run0; ++r, ++use) {
+        if (use % NS != s) continue;
+        // the MMAs of the run that this stage held are done
+        if (use >= NS && !__all_sync(0xffffffffu, mbar_wait(mb_empty[s], (uint32_t)((use / NS - 1) & 1)))) {
+          failed = true;
+          break;
         }
-        if (use + 1 >= staged) break;                    // every staged run is announced, none is left
+        const int4 run = s_runs[b][r];                   // (offset slot, first entry, end entry, -)
+        if (ts == 0) {
+          // C_o of the item's table: hi and lo tiles (consecutive), counted on the full barrier
+          asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mb_full[s]), "r"(2 * b_bytes)
+                       : "memory");
+          asm volatile(
+              "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                  st + 2 * a_bytes),
+              "l"(tl + (size_t)run.x * 2 * R * R), "r"(2 * b_bytes), "r"(mb_full[s])
+              : "memory");
+        }
+        // eight entries to a warp at a time, four lanes to an entry
+        const uint64_t *ent = &s_ent[b][(item.ent0 & 1) + (run.y - item.ent0)];
+        for (int e = ts >> 2; e < run.z - run.y; e += kStageThreads / 4) {
+          const uint64_t v = ent[e];
+          const int prow = (int)(v >> 32);
+          const __nv_bfloat16 *g = mc + (size_t)(uint32_t)v * 4 * R;
+          for (int k8 = ts & 3; k8 < kg; k8 += 4) {
+            const uint32_t off = canon_off(prow, k8 * 8, kTsRows);
+            cp_async16_zfill(st + off, g + k8 * 8, true);
+            cp_async16_zfill(st + a_bytes + off, g + R + k8 * 8, true);
+          }
+        }
+        const uint32_t *mask = reinterpret_cast<const uint32_t *>(&s_mask[b][r]);
+#pragma unroll
+        for (int i = 0; i < NS; ++i) {
+          const int row = ts + i * kStageThreads;
+          const bool now = (mask[row >> 5] >> (row & 31)) & 1u;
+          if (((was >> i) & 1u) && !now) {
+            for (int k8 = 0; k8 < R / 8; ++k8) {
+              const uint32_t off = canon_off(row, k8 * 8, kTsRows);
+              asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(st + off), "r"(0u) : "memory");
+              asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(st + a_bytes + off), "r"(0u) : "memory");
+            }
+          }
+          was = (was & ~(1u << i)) | ((now ? 1u : 0u) << i);
+        }
+        // this warp's rows have landed: make them visible to the tensor core
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(mb_full[s]) : "memory");
+      }
+      if (failed) break;
+      // this warp has read item k's buffer; when all four have, it takes item k + 2
+      __syncwarp();
+      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(mb_ifree[b]) : "memory");
+      if (warp == 0 && k + 2 < nk) {
+        if (!__all_sync(0xffffffffu, mbar_wait(mb_ifree[b], (uint32_t)((k >> 1) & 1)))) {
+          failed = true;
+          break;
+        }
+        if (lane == 0) {
+          load_item(k + 2);
+          issued = k + 2;
+        }
       }
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
@@ -312,8 +338,8 @@ __global__ void __launch_bounds__(kTsThreads) k_m2l_ts(int R, int nitems_arg, co
     if (lane == 0) {
       int use = 0, committed = 0;
       const uint32_t lbo_a = (kTsRows / 8) * 128, lbo_b = (uint32_t)(R / 8) * 128, sbo = 128;
-      for (int it = i0, k = 0; it < i1 && !failed; ++it, ++k) {
-        const TSItem item = items[it];
+      for (int k = 0; k < nk && !failed; ++k) {
+        const TSItem item = items[item_at(k)];
         const int a = k & 1;
         if (k >= 2 && !mbar_wait(mb_acce[a], (uint32_t)(((k >> 1) - 1) & 1))) {   // epilogue of item k - 2 read it
           failed = true;
@@ -365,18 +391,18 @@ __global__ void __launch_bounds__(kTsThreads) k_m2l_ts(int R, int nitems_arg, co
     // ---- epilogue: one target box per lane ------------------------------------------------
     const int ew = warp - 4;
     const int row = 32 * ew + lane;
-    for (int it = i0, k = 0; it < i1; ++it, ++k) {
-      const TSItem item = items[it];
+    for (int k = 0; k < nk; ++k) {
+      const TSItem item = items[item_at(k)];
       const int a = k & 1;
+      const bool valid = item.base + row < item.end;
+      const int box = valid ? box_of(item)[item.base + row] : 0;
       const bool ok = __all_sync(0xffffffffu, mbar_wait(mb_accf[a], (uint32_t)((k >> 1) & 1)));
       if (!ok) {
         failed = true;
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;");
-      const int box = item.base + row;
-      const bool valid = box < item.end;
-      float *out = lc_of(item) + ((size_t)(valid ? box : 0) * 2 + item.kt) * R;
+      float *out = lc_of(item) + ((size_t)box * 2 + item.kt) * R;
       for (int c0 = 0; c0 < item.rank; c0 += 16) {
         uint32_t v[16];
         const uint32_t taddr = tmem + ((uint32_t)(32 * ew) << 16) + (uint32_t)(a * R + c0);
@@ -415,7 +441,7 @@ __global__ void __launch_bounds__(kTsThreads) k_m2l_ts(int R, int nitems_arg, co
 namespace {
 int ts_stage_bytes(int R) { return 2 * kTsRows * R * 2 + 2 * R * R * 2; }   // A hi, lo + B hi, lo
 // Two operand stages, two CTAs per SM (R <= 64): measured on the 163,842-node sphere,
-// 120 us against 188 us with four stages on one CTA per SM
+// 94 us against 122 us with four stages (a warp to each) on one CTA per SM
 int ts_stages(int) { return 2; }
 int ts_smem_bytes(int R) { return ts_stages(R) * ts_stage_bytes(R); }
 }  // namespace
@@ -433,16 +459,49 @@ Err build_m2l_ts(afmpb_t *h) {
   const int64_t np = h->n_m2l_pairs;
   h->ts_nitems = 0;
   if (np == 0 || h->m2l_groups.empty()) return Err{};
-  // global block index of each level's first block of kTsRows boxes
-  std::vector<int> blk_start(T.nlevel + 1, 0);
-  for (int l = 0; l < T.nlevel; ++l)
-    blk_start[l + 1] = blk_start[l] + (T.lvl_start[l + 1] - T.lvl_start[l] + kTsRows - 1) / kTsRows;
-  int *d_lvl = nullptr, *d_blk = nullptr;
+  // target boxes by block group (level, octant); blocks of kTsRows within each group
+  const int ngroup = 8 * T.nlevel;
+  int *d_lvl = nullptr, *d_gstart = nullptr, *d_gblk = nullptr;
+  uint32_t *grp = nullptr, *grp_sorted = nullptr;
+  int32_t *ids = nullptr, *slot_of = nullptr;
+  AFMPB_TRY(A.alloc(&d_lvl, T.lvl_start.size(), "ts level start"));
+  AFMPB_TRY(A.alloc(&d_gstart, ngroup + 1, "ts group start"));
+  AFMPB_TRY(A.alloc(&d_gblk, ngroup + 1, "ts group block"));
+  AFMPB_TRY(A.alloc(&grp, T.nbox, "ts groups"));
+  AFMPB_TRY(A.alloc(&grp_sorted, T.nbox, "ts groups sorted"));
+  AFMPB_TRY(A.alloc(&ids, T.nbox, "ts box ids"));
+  AFMPB_TRY(A.alloc(&slot_of, T.nbox, "ts slots"));
+  AFMPB_TRY(A.alloc(&h->d_ts_box, T.nbox, "ts boxes by slot"));
+  AFMPB_CUDA(cudaMemcpyAsync(d_lvl, T.lvl_start.data(), sizeof(int) * T.lvl_start.size(), cudaMemcpyHostToDevice, s));
+  k_ts_groups<<<div_up(T.nbox, 256), 256, 0, s>>>(T.nbox, h->d_box_anchor, d_lvl, grp, ids);
+  AFMPB_TRY(check_launch("k_ts_groups"));
+  {
+    int bits = 1;
+    while ((1 << bits) < ngroup) ++bits;
+    size_t bytes = 0;
+    AFMPB_CUDA(cub::DeviceRadixSort::SortPairs(nullptr, bytes, grp, grp_sorted, ids, h->d_ts_box, T.nbox, 0, bits, s));
+    uint8_t *tmp = nullptr;
+    AFMPB_TRY(A.alloc(&tmp, std::max<size_t>(bytes, 16), "ts group sort scratch"));
+    AFMPB_CUDA(cub::DeviceRadixSort::SortPairs(tmp, bytes, grp, grp_sorted, ids, h->d_ts_box, T.nbox, 0, bits, s));
+    A.release(tmp);
+  }
+  k_ts_slots<<<div_up(std::max(T.nbox, ngroup + 1), 256), 256, 0, s>>>(T.nbox, ngroup, grp_sorted, h->d_ts_box,
+                                                                       d_gstart, slot_of);
+  AFMPB_TRY(check_launch("k_ts_slots"));
+  std::vector<int> gstart(ngroup + 1), gblk(ngroup + 1, 0);
+  AFMPB_CUDA(cudaMemcpyAsync(gstart.data(), d_gstart, sizeof(int) * (ngroup + 1), cudaMemcpyDeviceToHost, s));
+  AFMPB_CUDA(cudaStreamSynchronize(s));
+  h->ts_blocks.clear();
+  for (int g = 0; g < ngroup; ++g) {
+    for (int i = gstart[g]; i < gstart[g + 1]; i += kTsRows)
+      h->ts_blocks.push_back({i, std::min(i + kTsRows, gstart[g + 1]), g / 8});
+    gblk[g + 1] = (int)h->ts_blocks.size();
+  }
+  const int nblocks = (int)h->ts_blocks.size();
+  AFMPB_CUDA(cudaMemcpyAsync(d_gblk, gblk.data(), sizeof(int) * (ngroup + 1), cudaMemcpyHostToDevice, s));
   uint32_t *key = nullptr, *key_sorted = nullptr, *uniq = nullptr;
   uint64_t *ent = nullptr;
   int32_t *cnt = nullptr, *d_nruns = nullptr;
-  AFMPB_TRY(A.alloc(&d_lvl, T.lvl_start.size(), "ts level start"));
-  AFMPB_TRY(A.alloc(&d_blk, blk_start.size(), "ts block start"));
   AFMPB_TRY(A.alloc(&key, np, "ts keys"));
   AFMPB_TRY(A.alloc(&key_sorted, np, "ts keys sorted"));
   AFMPB_TRY(A.alloc(&ent, np, "ts entries unsorted"));
@@ -450,12 +509,11 @@ Err build_m2l_ts(afmpb_t *h) {
   AFMPB_TRY(A.alloc(&uniq, np, "ts run keys"));
   AFMPB_TRY(A.alloc(&cnt, np, "ts run sizes"));
   AFMPB_TRY(A.alloc(&d_nruns, 1, "ts run count"));
-  AFMPB_CUDA(cudaMemcpyAsync(d_lvl, T.lvl_start.data(), sizeof(int) * T.lvl_start.size(), cudaMemcpyHostToDevice, s));
-  AFMPB_CUDA(cudaMemcpyAsync(d_blk, blk_start.data(), sizeof(int) * blk_start.size(), cudaMemcpyHostToDevice, s));
-  k_ts_keys<<<(unsigned)h->m2l_groups.size(), 256, 0, s>>>(h->d_m2l_groups, h->d_m2l_pairs, d_lvl, d_blk, key, ent);
+  k_ts_keys<<<(unsigned)h->m2l_groups.size(), 256, 0, s>>>(h->d_m2l_groups, h->d_m2l_pairs, grp_sorted, slot_of,
+                                                          d_gstart, d_gblk, key, ent);
   AFMPB_TRY(check_launch("k_ts_keys"));
   int bits = 1;
-  while (((uint64_t)1 << bits) < (uint64_t)blk_start.back() * kNumOffsets) ++bits;
+  while (((uint64_t)1 << bits) < (uint64_t)nblocks * kNumOffsets) ++bits;
   {
     size_t bytes = 0;
     AFMPB_CUDA(cub::DeviceRadixSort::SortPairs(nullptr, bytes, key, key_sorted, ent, h->d_ts_ent, np, 0, bits, s));
@@ -479,7 +537,8 @@ Err build_m2l_ts(afmpb_t *h) {
   AFMPB_CUDA(cudaMemcpyAsync(rkey.data(), uniq, sizeof(uint32_t) * nruns, cudaMemcpyDeviceToHost, s));
   AFMPB_CUDA(cudaMemcpyAsync(rcnt.data(), cnt, sizeof(int32_t) * nruns, cudaMemcpyDeviceToHost, s));
   AFMPB_CUDA(cudaStreamSynchronize(s));
-  for (void *q : {(void *)d_lvl, (void *)d_blk, (void *)key, (void *)key_sorted, (void *)ent, (void *)uniq,
+  for (void *q : {(void *)d_lvl, (void *)d_gstart, (void *)d_gblk, (void *)grp, (void *)grp_sorted, (void *)ids,
+                  (void *)slot_of, (void *)key, (void *)key_sorted, (void *)ent, (void *)uniq,
                   (void *)cnt, (void *)d_nruns})
     A.release(q);
   h->ts_rkey = std::move(rkey);
@@ -494,6 +553,9 @@ Err build_m2l_ts(afmpb_t *h) {
     }
     AFMPB_TRY(A.alloc(&h->d_ts_runs, std::max<size_t>(1, runs.size()), "ts runs"));
     AFMPB_CUDA(cudaMemcpyAsync(h->d_ts_runs, runs.data(), sizeof(int4) * runs.size(), cudaMemcpyHostToDevice, s));
+    AFMPB_TRY(A.alloc(&h->d_ts_masks, std::max<size_t>(1, runs.size()), "ts row masks"));
+    k_ts_masks<<<div_up(std::max(nruns, 1), 128), 128, 0, s>>>(nruns, h->d_ts_runs, h->d_ts_ent, h->d_ts_masks);
+    AFMPB_TRY(check_launch("k_ts_masks"));
     AFMPB_CUDA(cudaStreamSynchronize(s));
   }
   AFMPB_TRY(cut_m2l_ts_items(h));
@@ -525,9 +587,6 @@ Err cut_m2l_ts_items(afmpb_t *h) {
   const std::vector<int32_t> &rcnt = h->ts_rcnt;
   const int nruns = (int)rkey.size();
   const std::vector<int> &level_table = h->h_level_table;
-  std::vector<int> blk_start(T.nlevel + 1, 0);
-  for (int l = 0; l < T.nlevel; ++l)
-    blk_start[l + 1] = blk_start[l] + (T.lvl_start[l + 1] - T.lvl_start[l] + kTsRows - 1) / kTsRows;
   std::vector<int64_t> rstart(nruns + 1, 0);
   for (int r = 0; r < nruns; ++r) rstart[r + 1] = rstart[r] + rcnt[r];
   int dev = 0, sms = 0;
@@ -536,29 +595,23 @@ Err cut_m2l_ts_items(afmpb_t *h) {
   const int per_item = h->ts_runs_per_item > 0 ? std::min(kTsItemRuns, h->ts_runs_per_item)
                                                 : std::min(kTsItemRuns, std::max(8, nruns / std::max(1, 4 * sms)));
   std::vector<TSItem> items;
-  auto level_of_block = [&](int blk) {
-    int l = 0;
-    while (l + 1 < (int)blk_start.size() && blk_start[l + 1] <= blk) ++l;
-    return l;
-  };
   for (int kt = 0; kt < 2; ++kt) {
     for (int r = 0; r < nruns;) {
       const int blk = (int)(rkey[r] / kNumOffsets);
       int rend = r;
       while (rend < nruns && (int)(rkey[rend] / kNumOffsets) == blk) ++rend;
-      const int l = level_of_block(blk);
+      const TSBlock &B = h->ts_blocks[blk];
+      const int l = B.level;
       const bool use = kt == 0 || (l >= h->m2l_yuk_levels && !h->laplace_only);
       if (use) {
         const int table = kt == 0 ? 0 : level_table[l];
-        const int base = T.lvl_start[l] + (blk - blk_start[l]) * kTsRows;
-        const int end = std::min(base + kTsRows, T.lvl_start[l + 1]);
         // consecutive runs of the block, at most per_item runs and kTsItemEnt entries each
         for (int q0 = r; q0 < rend;) {
           int q1 = q0, ne = 0;
           while (q1 < rend && q1 - q0 < per_item && ne + rcnt[q1] <= kTsItemEnt) ne += rcnt[q1++];
           TSItem it{};
-          it.base = base;
-          it.end = end;
+          it.base = B.begin;
+          it.end = B.end;
           it.run0 = q0;
           it.run1 = q1;
           it.ent0 = (int)rstart[q0];
@@ -575,6 +628,11 @@ Err cut_m2l_ts_items(afmpb_t *h) {
       r = rend;
     }
   }
+  // few items to a CTA: by cost, so that the CTAs' shares differ by less than one small item
+  if ((int64_t)items.size() <= 32 * (int64_t)sms)
+    std::stable_sort(items.begin(), items.end(), [](const TSItem &x, const TSItem &y) {
+      return (x.run1 - x.run0) * x.rank > (y.run1 - y.run0) * y.rank;
+    });
   h->ts_nitems = (int)items.size();
   if (h->d_ts_items) A.release(h->d_ts_items);
   AFMPB_TRY(A.alloc(&h->d_ts_items, std::max<size_t>(1, items.size()), "ts items"));
@@ -590,17 +648,17 @@ Err enqueue_m2l_ts(afmpb_t *h, cudaStream_t s) {
   AFMPB_CUDA(cudaGetDevice(&dev));
   AFMPB_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const int R = h->m2l_rank;
-  const int per_sm = std::max(1, std::min(2, (227 * 1024) / (ts_smem_bytes(R) + 12 * 1024)));
+  const int per_sm = std::max(1, std::min(2, (227 * 1024) / (ts_smem_bytes(R) + 16 * 1024)));
   const unsigned grid = (unsigned)std::min(h->ts_nitems, per_sm * sms);
   const auto *mc = reinterpret_cast<const __nv_bfloat16 *>(h->d_Mc16);
   const auto *tl = reinterpret_cast<const __nv_bfloat16 *>(h->d_ts_tiles);
   if (ts_stages(R) == 4)
     k_m2l_ts<4, false><<<grid, kTsThreads, ts_smem_bytes(R), s>>>(R, h->ts_nitems, h->d_ts_items, h->d_ts_runs,
-                                                                  h->d_ts_ent, mc, tl, h->d_Lc, h->d_tc_flag,
+                                                                  h->d_ts_masks, h->d_ts_ent, h->d_ts_box, mc, tl, h->d_Lc, h->d_tc_flag,
                                                                   nullptr, nullptr);
   else
     k_m2l_ts<2, false><<<grid, kTsThreads, ts_smem_bytes(R), s>>>(R, h->ts_nitems, h->d_ts_items, h->d_ts_runs,
-                                                                  h->d_ts_ent, mc, tl, h->d_Lc, h->d_tc_flag,
+                                                                  h->d_ts_masks, h->d_ts_ent, h->d_ts_box, mc, tl, h->d_Lc, h->d_tc_flag,
                                                                   nullptr, nullptr);
   return check_launch("k_m2l_ts");
 }
@@ -658,14 +716,14 @@ Err enqueue_m2l_ts_batch(const TSReq *d_reqs, const TSItem *d_items, int nitems,
   AFMPB_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   k_ts_compact<<<1, 1024, 0, s>>>(nitems, d_items, d_reqs, d_items_run, d_count);
   AFMPB_TRY(check_launch("k_ts_compact"));
-  const int per_sm = std::max(1, std::min(2, (227 * 1024) / (ts_smem_bytes(R) + 12 * 1024)));
+  const int per_sm = std::max(1, std::min(2, (227 * 1024) / (ts_smem_bytes(R) + 16 * 1024)));
   const unsigned grid = (unsigned)std::min(nitems, per_sm * sms);
   if (ts_stages(R) == 4)
-    k_m2l_ts<4, true><<<grid, kTsThreads, ts_smem_bytes(R), s>>>(R, 0, d_items_run, nullptr, nullptr, nullptr,
-                                                                 nullptr, nullptr, err_flag, d_count, d_reqs);
+    k_m2l_ts<4, true><<<grid, kTsThreads, ts_smem_bytes(R), s>>>(R, 0, d_items_run, nullptr, nullptr, nullptr, nullptr,
+                                                                 nullptr, nullptr, nullptr, err_flag, d_count, d_reqs);
   else
-    k_m2l_ts<2, true><<<grid, kTsThreads, ts_smem_bytes(R), s>>>(R, 0, d_items_run, nullptr, nullptr, nullptr,
-                                                                 nullptr, nullptr, err_flag, d_count, d_reqs);
+    k_m2l_ts<2, true><<<grid, kTsThreads, ts_smem_bytes(R), s>>>(R, 0, d_items_run, nullptr, nullptr, nullptr, nullptr,
+                                                                 nullptr, nullptr, nullptr, err_flag, d_count, d_reqs);
   return check_launch("k_m2l_ts batch");
 }
 
