@@ -194,7 +194,7 @@ typedef struct {
     double ms_per_m2l_pair, ms_per_box, ms_rest;
     double ms_tuning;          /* host time of the calibration and the candidate trees   */
     /* Tile shapes, chosen on the handle built at best_cap by timing the kernels themselves:
-     * P2P blocks kept resident per SM (4-6) x work units per block (1-6), and the number of
+     * P2P work units cut for blocks per SM (4-6) x units per block (1-6), and the number of
      * offsets per work item of the tensor-core M2L (8-32; 0 when that kernel is not used). */
     int p2p_resident, p2p_units_per_block, m2l_runs_per_item;
     double p2p_ms_default, p2p_ms_tuned;   /* P2P at the library defaults and at the choice  */

@@ -12,8 +12,8 @@
 //   3. predicts the product time  t(s) = t_P2P(s) + b * pairs_V(s) + c * boxes(s) + t_rest
 //      and keeps the smallest.
 // Then, on the handle at the chosen capacity, the tile shapes of the two heaviest kernels
-// are picked by timing them: the P2P blocks kept resident per SM and the size of its work
-// units, and the number of offsets per work item of the tensor-core M2L.
+// are picked by timing them: the size of the P2P work units (by the blocks per SM and the
+// units per block that it is cut for), and the number of offsets per work item of the tensor-core M2L.
 // The choices are cached per (precision, order, screened or not, log2 of the node count),
 // so later handles of the same size class skip the tuning.
 #include <chrono>
@@ -118,7 +118,8 @@ std::tuple<int, int, int, int, int> cache_key(int precision, int order, double k
 
 }  // namespace
 
-// Tile shapes on the finished handle: P2P resident blocks per SM x work units per block,
+// Tile shapes on the finished handle: the P2P work units (cut for resident blocks per SM x
+// units per block),
 // then the M2L offsets per item, each by timing the kernel itself.  The product graphs are
 // captured again afterwards (they hold the launch shapes).
 Err autotune_tiles(afmpb_t *h, afmpb_autotune_report *rep) {
@@ -130,9 +131,9 @@ Err autotune_tiles(afmpb_t *h, afmpb_autotune_report *rep) {
   int best_r = h->p2p_resident, best_u = h->p2p_units_per_block;
   for (int u : {1, 2, 3, 4, 6}) {
     h->p2p_units_per_block = u;
-    AFMPB_TRY(build_p2p_units(h));
     for (int r : {4, 5, 6}) {
       h->p2p_resident = r;
+      AFMPB_TRY(build_p2p_units(h));
       AFMPB_TRY(time_stage(h, kReps, p2p, &ms));
       if (ms < best_ms) {
         best_ms = ms;

@@ -3,7 +3,7 @@
 // Each problem keeps its own handle: tree, operators, expansions and Krylov state.  What a
 // batch adds is one P2P launch and one tensor-core M2L launch per Arnoldi step for all of
 // them.  The P2P units of every problem are merged into one list, ordered by cost across
-// problems (unit.w = problem), so the resident blocks deal out the union longest-first;
+// problems (unit.req = problem), so the resident blocks deal out the union longest-first;
 // the target-stationary M2L items are concatenated (TSItem.req = problem).  Per-problem
 // descriptors give the kernels each problem's arrays and its stop flag (gm[4] of its
 // step state), so a problem that has converged stops costing P2P and M2L work.
@@ -15,21 +15,16 @@ namespace afmpb {
 
 namespace {
 
-// Unit of problem `req` with its cost (targets x sources, the measure the units were cut by).
-__global__ void k_batch_units(int n, const int4 *__restrict__ in, int req, P2PReq q, int4 *__restrict__ out,
+// Unit of problem `req` with its cost (targets x staged sources).
+__global__ void k_batch_units(int n, const P2PUnit *__restrict__ in, int req, P2PReq q, P2PUnit *__restrict__ out,
                               uint64_t *__restrict__ cost) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const int4 u = in[i];
-  const int b = q.leaves[u.x];
-  const int64_t nt = q.bend[b] - q.bbeg[b];
-  int64_t ns = 0;
-  for (int j = u.y; j < u.z; ++j) {
-    const int c = q.pidx[j];
-    ns += q.bend[c] - q.bbeg[c];
-  }
-  out[i] = make_int4(u.x, u.y, u.z, req);
-  cost[i] = (uint64_t)(nt * ns);
+  P2PUnit u = in[i];
+  const int4 rec = q.leaf_rec[u.leaf];
+  u.req = req;
+  out[i] = u;
+  cost[i] = (uint64_t)(rec.z - rec.y) * (uint64_t)u.total;
 }
 
 __global__ void k_batch_items(int n, const TSItem *__restrict__ in, int req, TSItem *__restrict__ out) {
@@ -91,7 +86,7 @@ Err build_batch_lists(afmpb_t *const *hs, int k, bool fuse_m2l, BatchLists &L) {
 
   // P2P: every problem's units with their costs, sorted by cost (descending) across problems
   L.nunits = (int)nunits;
-  int4 *units = nullptr;
+  P2PUnit *units = nullptr;
   uint64_t *cost = nullptr, *cost_sorted = nullptr;
   AFMPB_TRY(L.alloc(&units, nunits, "batch p2p units unsorted"));
   AFMPB_TRY(L.alloc(&cost, nunits, "batch p2p unit costs"));

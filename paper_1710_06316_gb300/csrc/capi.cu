@@ -143,7 +143,7 @@ Err capture_product(afmpb_t *h, int parts, bool io = false, const float *x = nul
   }
   if (ce != cudaSuccess) return make_err(AFMPB_ECUDA, std::string("cudaStreamEndCapture: ") + cudaGetErrorString(ce));
   cudaGraphExec_t *exec = io ? &h->graph_io[parts] : &h->graph[parts];
-  ce = cudaGraphInstantiate(exec, g, 0);
+  ce = cudaGraphInstantiate(exec, g, cudaGraphInstantiateFlagUseNodePriority);
   if (ce != cudaSuccess) {
     cudaGraphDestroy(g);
     return make_err(AFMPB_ECUDA, std::string("cudaGraphInstantiate: ") + cudaGetErrorString(ce));
@@ -332,7 +332,7 @@ Err product_from64(afmpb_t *h, cudaStream_t s, const double *v) {
       if (g) cudaGraphDestroy(g);
       return e.ok() ? make_err(AFMPB_ECUDA, std::string("cudaStreamEndCapture: ") + cudaGetErrorString(ce)) : e;
     }
-    ce = cudaGraphInstantiate(&h->graph_gm, g, 0);
+    ce = cudaGraphInstantiate(&h->graph_gm, g, cudaGraphInstantiateFlagUseNodePriority);
     if (ce != cudaSuccess) {
       cudaGraphDestroy(g);
       return make_err(AFMPB_ECUDA, std::string("cudaGraphInstantiate: ") + cudaGetErrorString(ce));

@@ -632,7 +632,6 @@ __global__ void __launch_bounds__(kL2PNodes) k_l2p(int64_t n, const int2 *__rest
 // ------------------------------------------------------------------------------------
 constexpr int kP2PChunk = 768;      // sources staged in shared memory at a time (8 CTAs/SM)
 constexpr int kP2PPairs = kP2PChunk / 2;
-constexpr int kP2PBoxes = 64;       // source boxes described in shared memory at a time
 constexpr int kP2PRegBlocks = kP2PResident;
 
 // Far-rule sums of one source at one target, without the 1/(4 pi):
@@ -647,9 +646,9 @@ constexpr int kP2PRegBlocks = kP2PResident;
 //   PhiY += e (k1 p2 + c)/r,                 dn PhiY += e (k1 m - k^2 P Q)/r^3.
 // The FP32 pipe bounds the kernel, so the count of its operations per pair is what this
 // form is for: 35 (43 in the order the formulas are printed in), 38 where the pair's
-// distance has to be tested, 27 and 30 without salt (k = 0: e = k1 = 1 and no exp2).
-// Measured, P2P alone: 0.255 -> 0.235 ms (163,842-node sphere, leaves of 80), 0.582 ->
-// 0.519 ms (leaves of 192), 1.032 -> 0.765 ms (655,362 nodes without salt).
+// distance has to be tested, 25 and 27 without salt (k = 0: e = k1 = 1 and no exp2).
+// Measured, P2P alone, at the same deal of work: 0.255 -> 0.235 ms (163,842-node sphere,
+// leaves of 80), 0.582 -> 0.519 ms (leaves of 192).
 //
 // The sums run on packed FP32 pairs (sm_100 FFMA2 / FADD2 / FMUL2): each thread takes
 // its target against two sources per instruction, lane 0 an even and lane 1 an odd
@@ -694,7 +693,9 @@ struct P2PConst {
 // d = (gnz0, gnz1, w0, w1); positions in the target leaf's frame.  kTest: w = skip radius,
 // and pairs inside it contribute nothing here (the near CSR carries their whole near-rule
 // value; t == p is among them).  Otherwise no pair can be inside it and w = (1 - eps_bar) c.
-// Sums: sL, sY as above; nD = eps_bar dn PhiL; dY.
+// Sums: sL, sY as above; nD = eps_bar dn PhiL; dY.  Without salt the two kernels differ in
+// eps_bar alone and the product takes their difference: the parts with and without it are
+// summed apart, sL = sum p2/r, sY = sum c/r, nD = sum (S - 3 p2 Q)/r^3, dY = sum c Q/r^3.
 template <bool kTest, bool kSalt>
 __device__ __forceinline__ void p2p_pair2(const P2PTarget &t, const float4 &a, const float4 &b, const float4 &c,
                                           const float4 &d, const P2PConst &k, float2 &sL, float2 &nD, float2 &sY,
@@ -719,24 +720,34 @@ __device__ __forceinline__ void p2p_pair2(const P2PTarget &t, const float4 &a, c
   const float2 S = __ffma2_rn(t.nx, gx, __ffma2_rn(t.ny, gy, __fmul2_rn(t.nz, gz)));
   const float2 p2 = __fmul2_rn(P, ri2);
   const float2 G3 = __fmul2_rn(ri, ri2);
+  if (!kSalt) {
+    sL = __ffma2_rn(ri, p2, sL);
+    sY = __ffma2_rn(ri, cc, sY);
+    nD = __ffma2_rn(G3, __ffma2_rn(__fmul2_rn(p2, Q), dup2(-3.0f), S), nD);
+    dY = __ffma2_rn(G3, __fmul2_rn(cc, Q), dY);
+    return;
+  }
   const float2 h = __ffma2_rn(p2, dup2(3.0f), cc);
   const float2 m = __ffma2_rn(make_float2(-h.x, -h.y), Q, S);
   const float2 dc = kTest ? __fmul2_rn(cc, k.omce) : make_float2(d.z, d.w);
   nD = __ffma2_rn(G3, __ffma2_rn(dc, Q, m), nD);
   sL = __ffma2_rn(ri, __ffma2_rn(k.inv_e, p2, cc), sL);
-  if (kSalt) {
-    const float2 rr = __fmul2_rn(r2, ri);
-    const float2 arg = __fmul2_rn(rr, k.nkl2e);
-    const float2 ex = make_float2(ex2_approx(arg.x), ex2_approx(arg.y));
-    const float2 k1 = __ffma2_rn(rr, k.kappa, dup2(1.0f));
-    const float2 ei = __fmul2_rn(ex, ri);
-    sY = __ffma2_rn(ei, __ffma2_rn(k1, p2, cc), sY);
-    const float2 V = __fmul2_rn(__fmul2_rn(P, Q), k.kappa2);
-    dY = __ffma2_rn(__fmul2_rn(ei, ri2), __ffma2_rn(k1, m, make_float2(-V.x, -V.y)), dY);
-  } else {
-    sY = __ffma2_rn(ri, __fadd2_rn(p2, cc), sY);
-    dY = __ffma2_rn(G3, m, dY);
-  }
+  const float2 rr = __fmul2_rn(r2, ri);
+  const float2 arg = __fmul2_rn(rr, k.nkl2e);
+  const float2 ex = make_float2(ex2_approx(arg.x), ex2_approx(arg.y));
+  const float2 k1 = __ffma2_rn(rr, k.kappa, dup2(1.0f));
+  const float2 ei = __fmul2_rn(ex, ri);
+  sY = __ffma2_rn(ei, __ffma2_rn(k1, p2, cc), sY);
+  const float2 V = __fmul2_rn(__fmul2_rn(P, Q), k.kappa2);
+  dY = __ffma2_rn(__fmul2_rn(ei, ri2), __ffma2_rn(k1, m, make_float2(-V.x, -V.y)), dY);
+}
+
+// The sums of one target, (PhiL, dn PhiL, PhiY, dn PhiY) without the 1/(4 pi), from its
+// accumulators.
+__device__ __forceinline__ float4 p2p_sums(bool salt, float inv_e, float2 sL, float2 nD, float2 sY, float2 dY) {
+  const float a = sL.x + sL.y, b = nD.x + nD.y, c = sY.x + sY.y, d = dY.x + dY.y;
+  if (salt) return make_float4(a, inv_e * b, c, d);
+  return make_float4(fmaf(inv_e, a, c), fmaf(inv_e, b, -d), a + c, b - d);
 }
 
 // A unit that covers its leaf's whole source list stores; a part of a split leaf adds.
@@ -750,40 +761,33 @@ __device__ __forceinline__ void store_or_add(float4 *p, float4 v, bool whole) {
 #define P2P_ARG(name) (kBatch ? s_req.name : name##_1)
 
 // The body of the P2P kernels: with kBatch the work units of several problems share one
-// launch, unit.w naming the problem whose arrays (reqs[unit.w], copied to shared memory
+// launch, unit.req naming the problem whose arrays (reqs[unit.req], copied to shared memory
 // per unit) it reads, and units of a problem whose *active flag is 0 are skipped.
 template <bool kBatch>
-__device__ __forceinline__ void p2p_body(int nunits, const int4 *__restrict__ units, const int32_t *__restrict__ leaves_1,
-                                         const int64_t *__restrict__ pptr_1, const int32_t *__restrict__ pidx_1,
-                                         const uint8_t *__restrict__ ptest_1,
-                                         const int32_t *__restrict__ bbeg_1, const int32_t *__restrict__ bend_1,
-                                         const dbl4 *__restrict__ center_1, const float4 *__restrict__ pos_1,
+__device__ __forceinline__ void p2p_body(const P2PUnit *__restrict__ units,
+                                         const int4 *__restrict__ leaf_rec_1, const float4 *__restrict__ src_1,
+                                         const int2 *__restrict__ slot_1, const float4 *__restrict__ pos_1,
                                          const float4 *__restrict__ nrm_1, const float2 *__restrict__ xs_1,
                                          float inv_ebar_1, float kappa_1, float skip_scale_1, float4 *__restrict__ phi_1,
                                          const P2PReq *__restrict__ reqs) {
-  static_assert(2 * kP2PThreads <= kP2PPairs, "the reduction reuses the staging buffer");
   __shared__ float4 sa[kP2PPairs], sb[kP2PPairs], sc[kP2PPairs], sd[kP2PPairs];
-  __shared__ int s_beg[kP2PBoxes], s_pos[kP2PBoxes], s_cnt[kP2PBoxes], s_tot[4];
-  __shared__ float s_off[kP2PBoxes][3];
+  __shared__ float4 red[2 * kP2PThreads];
   __shared__ __align__(8) P2PReq s_req;
-  float4 *red = sa;
-  // The resident blocks walk the cost-ordered work units in boustrophedon order: in round
-  // k block b takes unit k G + b for even k and k G + G - 1 - b for odd k (G blocks), so
-  // the block that drew the costliest unit of one round draws the cheapest of the next.  A
-  // unit is one leaf's targets against a range of its source boxes; leaves with more pairs
-  // than the unit budget are split, and their units add into the (zeroed) output.
-  const int G = gridDim.x;
-  for (int k = 0; k * G < nunits; ++k) {
-  const int li = k * G + ((k & 1) ? (G - 1 - (int)blockIdx.x) : (int)blockIdx.x);
-  if (li >= nunits) continue;
-  if (k > 0) __syncthreads();                           // the previous unit's reduction read red
-  const int4 unit = units[li];
+  // One block per work unit, the costliest first: the block scheduler deals them out as
+  // blocks finish (a static deal to resident blocks left the slowest 15% behind: 0.234
+  // against 0.201 ms on the 163,842-node sphere).  A unit is one leaf's targets against a
+  // range of its source boxes; leaves with more pairs than the unit budget are split, and
+  // their units add into the (zeroed) output.  All that a block has to know of its unit
+  // before it can fetch sources is laid out at setup (unit, leaf record, source records and
+  // slots: two dependent loads, no scan of the boxes).
+  const int4 unit = reinterpret_cast<const int4 *>(units + blockIdx.x)[0];
+  const int4 share = reinterpret_cast<const int4 *>(units + blockIdx.x)[1];    // tested, total, whole, -
   if constexpr (kBatch) {
     static_assert(sizeof(P2PReq) % 8 == 0, "copied as 8-byte words");
     if (threadIdx.x < sizeof(P2PReq) / 8)
       reinterpret_cast<uint64_t *>(&s_req)[threadIdx.x] = reinterpret_cast<const uint64_t *>(reqs + unit.w)[threadIdx.x];
     __syncthreads();
-    if (s_req.active && *s_req.active == 0) continue;  // uniform: the problem has stopped
+    if (s_req.active && *s_req.active == 0) return;    // uniform: the problem has stopped
   }
   P2PConst kc;
   {
@@ -795,17 +799,13 @@ __device__ __forceinline__ void p2p_body(int nunits, const int4 *__restrict__ un
     kc.omce = dup2(1.0f - 1.0f / inv_e);
   }
   const bool salt = kc.kappa.x > 0.0f;
-  const int leaf = unit.x;
-  const int b = P2P_ARG(leaves)[leaf];
-  const dbl4 cb = P2P_ARG(center)[b];
-  const int tb = P2P_ARG(bbeg)[b], te = P2P_ARG(bend)[b];
+  const int4 rec = P2P_ARG(leaf_rec)[unit.x];
+  const int tb = rec.y, te = rec.z;
   // each thread takes two targets, t and t + tile, against the same sources
   const int tile = min((te - tb + 1) / 2, kP2PThreads);
   const int slices = kP2PThreads / tile;
   const int ti = threadIdx.x % tile, si = threadIdx.x / tile;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t l0 = unit.y, l1 = unit.z;               // this unit's source boxes
-  const bool whole = l0 == P2P_ARG(pptr)[leaf] && l1 == P2P_ARG(pptr)[leaf + 1];
+  const int nf = share.x, nfe = (nf + 1) & ~1, total = share.y;
   for (int t0 = tb; t0 < te; t0 += 2 * tile) {
     const int t = t0 + ti, t2 = t + tile;
     const bool act = si < slices && t < te;
@@ -826,120 +826,83 @@ __device__ __forceinline__ void p2p_body(int nunits, const int4 *__restrict__ un
     }
     float2 sL = dup2(0.f), nD = dup2(0.f), sY = dup2(0.f), dY = dup2(0.f);
     float2 sL2 = dup2(0.f), nD2 = dup2(0.f), sY2 = dup2(0.f), dY2 = dup2(0.f);
-    for (int64_t g0 = l0; g0 < l1; g0 += kP2PBoxes) {
-      const int nb = (int)min((int64_t)kP2PBoxes, l1 - g0);
-      __syncthreads();
-      // The boxes whose pairs may be inside the skip radius come first in the staged order
-      // (slots [0, nf)), the others after them from the next even slot on.
-      int cf = 0, cu = 0;
-      bool test = false;
-      if (threadIdx.x < nb) {
-        const int c = P2P_ARG(pidx)[g0 + threadIdx.x];
-        const dbl4 cc = P2P_ARG(center)[c];
-        const int beg = P2P_ARG(bbeg)[c], cnt = P2P_ARG(bend)[c] - beg;
-        test = P2P_ARG(ptest)[g0 + threadIdx.x] != 0;
-        cf = test ? cnt : 0;
-        cu = test ? 0 : cnt;
-        s_beg[threadIdx.x] = beg;
-        s_cnt[threadIdx.x] = cnt;
-        s_off[threadIdx.x][0] = (float)(cc.x - cb.x);
-        s_off[threadIdx.x][1] = (float)(cc.y - cb.y);
-        s_off[threadIdx.x][2] = (float)(cc.z - cb.z);
+    for (int c0 = 0; c0 < total; c0 += kP2PChunk) {
+      const int cnt = min(kP2PChunk, total - c0);
+      const int npairs = (cnt + 1) >> 1;
+      const int ntest = min(max(nfe - c0, 0), cnt) >> 1;       // pairs of the tested part
+      int first = unit.y;
+      if (c0 > 0) {
+        for (int last = unit.z - 1; first < last;) {           // the first entry that reaches beyond c0
+          const int mid = (first + last) >> 1;
+          const int2 sl = P2P_ARG(slot)[mid];
+          if (sl.x + sl.y > c0) last = mid;
+          else first = mid + 1;
+        }
+        __syncthreads();                                       // the last chunk has been read
       }
-      int vf = cf, vu = cu;
-      if (warp < 2) {                       // inclusive scans of the (<= 64) box sizes
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int f = __shfl_up_sync(0xffffffffu, vf, o), u = __shfl_up_sync(0xffffffffu, vu, o);
-          if (lane >= o) {
-            vf += f;
-            vu += u;
+      // sixteen threads to a source box
+      for (int en = first + (threadIdx.x >> 4); en < unit.z; en += kP2PThreads / 16) {
+        const int2 sl = P2P_ARG(slot)[en];                     // first slot, nodes
+        if (sl.x >= c0 + kP2PChunk) break;
+        const float4 box = P2P_ARG(src)[en];                   // centre difference, first node
+        const int hi = min(sl.x + sl.y, c0 + kP2PChunk);
+        const bool tested = sl.x < nf;
+        const int beg = __float_as_int(box.w) - sl.x;
+        for (int j = max(sl.x, c0) + (threadIdx.x & 15); j < hi; j += 16) {
+          const float4 p = P2P_ARG(pos)[beg + j], q = P2P_ARG(nrm)[beg + j];
+          const float2 fh = P2P_ARG(xs)[beg + j];
+          const float px = __fadd_rn(p.x, box.x), py = __fadd_rn(p.y, box.y), pz = __fadd_rn(p.z, box.z);
+          const float cw = p.w * fh.y, g = -p.w * fh.x;
+          const int e = j - c0, pr = e >> 1, ln = e & 1;
+          float *fa = reinterpret_cast<float *>(sa + pr), *fb = reinterpret_cast<float *>(sb + pr);
+          float *fc = reinterpret_cast<float *>(sc + pr), *fd = reinterpret_cast<float *>(sd + pr);
+          fa[ln] = -px; fa[2 + ln] = -py;
+          fb[ln] = -pz; fb[2 + ln] = cw;
+          fc[ln] = g * q.x; fc[2 + ln] = g * q.y;
+          fd[ln] = g * q.z;
+          fd[2 + ln] = tested ? p2p_skip_radius(P2P_ARG(skip_scale), q.w) : cw * kc.omce.x;
+          // the odd slot after the last source of either part: its neighbour's place, no
+          // weight, and in the tested part a radius that leaves it out
+          if (ln == 0 && (j + 1 == nf || j + 1 == total)) {
+            fa[1] = -px; fa[3] = -py;
+            fb[1] = -pz; fb[3] = 0.f;
+            fc[1] = 0.f; fc[3] = 0.f;
+            fd[1] = 0.f;
+            fd[3] = tested ? 3.0e18f : 0.f;
           }
         }
-        if (lane == 31) {
-          s_tot[warp] = vf;
-          s_tot[2 + warp] = vu;
-        }
       }
       __syncthreads();
-      const int nf = s_tot[0] + s_tot[1], nfe = (nf + 1) & ~1, total = nfe + s_tot[2] + s_tot[3];
-      if (threadIdx.x < nb) {
-        if (warp == 1) {
-          vf += s_tot[0];
-          vu += s_tot[2];
-        }
-        s_pos[threadIdx.x] = test ? vf - cf : nfe + vu - cu;
-      }
-      __syncthreads();
-      for (int c0 = 0; c0 < total; c0 += kP2PChunk) {
-        const int cnt = min(kP2PChunk, total - c0);
-        const int npairs = (cnt + 1) >> 1;
-        const int ntest = min(max(nfe - c0, 0), cnt) >> 1;       // pairs of the tested part
-        if (c0 > 0) __syncthreads();
-        // sixteen threads to a box
-        for (int bi = threadIdx.x >> 4; bi < nb; bi += kP2PThreads / 16) {
-          const int p0 = s_pos[bi], hi = min(p0 + s_cnt[bi], c0 + kP2PChunk);
-          const float ox = s_off[bi][0], oy = s_off[bi][1], oz = s_off[bi][2];
-          const bool tested = p0 < nf;
-          const int beg = s_beg[bi] - p0;
-          for (int j = max(p0, c0) + (threadIdx.x & 15); j < hi; j += 16) {
-            const float4 p = P2P_ARG(pos)[beg + j], q = P2P_ARG(nrm)[beg + j];
-            const float2 fh = P2P_ARG(xs)[beg + j];
-            const float px = __fadd_rn(p.x, ox), py = __fadd_rn(p.y, oy), pz = __fadd_rn(p.z, oz);
-            const float cw = p.w * fh.y, g = -p.w * fh.x;
-            const int e = j - c0, pr = e >> 1, ln = e & 1;
-            float *fa = reinterpret_cast<float *>(sa + pr), *fb = reinterpret_cast<float *>(sb + pr);
-            float *fc = reinterpret_cast<float *>(sc + pr), *fd = reinterpret_cast<float *>(sd + pr);
-            fa[ln] = -px; fa[2 + ln] = -py;
-            fb[ln] = -pz; fb[2 + ln] = cw;
-            fc[ln] = g * q.x; fc[2 + ln] = g * q.y;
-            fd[ln] = g * q.z;
-            fd[2 + ln] = tested ? p2p_skip_radius(P2P_ARG(skip_scale), q.w) : cw * kc.omce.x;
-            // the odd slot after the last source of either part: its neighbour's place, no
-            // weight, and in the tested part a radius that leaves it out
-            if (ln == 0 && (j + 1 == nf || j + 1 == total)) {
-              fa[1] = -px; fa[3] = -py;
-              fb[1] = -pz; fb[3] = 0.f;
-              fc[1] = 0.f; fc[3] = 0.f;
-              fd[1] = 0.f;
-              fd[3] = tested ? 3.0e18f : 0.f;
-            }
+      if (act) {
+        int e = si;
+        if (salt) {
+          for (; e < ntest; e += slices) {
+            const float4 qa = sa[e], qb = sb[e], qc = sc[e], qd = sd[e];
+            p2p_pair2<true, true>(tg, qa, qb, qc, qd, kc, sL, nD, sY, dY);
+            p2p_pair2<true, true>(tg2, qa, qb, qc, qd, kc, sL2, nD2, sY2, dY2);
           }
-        }
-        __syncthreads();
-        if (act) {
-          int e = si;
-          if (salt) {
-            for (; e < ntest; e += slices) {
-              const float4 qa = sa[e], qb = sb[e], qc = sc[e], qd = sd[e];
-              p2p_pair2<true, true>(tg, qa, qb, qc, qd, kc, sL, nD, sY, dY);
-              p2p_pair2<true, true>(tg2, qa, qb, qc, qd, kc, sL2, nD2, sY2, dY2);
-            }
-            for (; e < npairs; e += slices) {
-              const float4 qa = sa[e], qb = sb[e], qc = sc[e], qd = sd[e];
-              p2p_pair2<false, true>(tg, qa, qb, qc, qd, kc, sL, nD, sY, dY);
-              p2p_pair2<false, true>(tg2, qa, qb, qc, qd, kc, sL2, nD2, sY2, dY2);
-            }
-          } else {
-            for (; e < ntest; e += slices) {
-              const float4 qa = sa[e], qb = sb[e], qc = sc[e], qd = sd[e];
-              p2p_pair2<true, false>(tg, qa, qb, qc, qd, kc, sL, nD, sY, dY);
-              p2p_pair2<true, false>(tg2, qa, qb, qc, qd, kc, sL2, nD2, sY2, dY2);
-            }
-            for (; e < npairs; e += slices) {
-              const float4 qa = sa[e], qb = sb[e], qc = sc[e], qd = sd[e];
-              p2p_pair2<false, false>(tg, qa, qb, qc, qd, kc, sL, nD, sY, dY);
-              p2p_pair2<false, false>(tg2, qa, qb, qc, qd, kc, sL2, nD2, sY2, dY2);
-            }
+          for (; e < npairs; e += slices) {
+            const float4 qa = sa[e], qb = sb[e], qc = sc[e], qd = sd[e];
+            p2p_pair2<false, true>(tg, qa, qb, qc, qd, kc, sL, nD, sY, dY);
+            p2p_pair2<false, true>(tg2, qa, qb, qc, qd, kc, sL2, nD2, sY2, dY2);
+          }
+        } else {
+          for (; e < ntest; e += slices) {
+            const float4 qa = sa[e], qb = sb[e], qc = sc[e], qd = sd[e];
+            p2p_pair2<true, false>(tg, qa, qb, qc, qd, kc, sL, nD, sY, dY);
+            p2p_pair2<true, false>(tg2, qa, qb, qc, qd, kc, sL2, nD2, sY2, dY2);
+          }
+          for (; e < npairs; e += slices) {
+            const float4 qa = sa[e], qb = sb[e], qc = sc[e], qd = sd[e];
+            p2p_pair2<false, false>(tg, qa, qb, qc, qd, kc, sL, nD, sY, dY);
+            p2p_pair2<false, false>(tg2, qa, qb, qc, qd, kc, sL2, nD2, sY2, dY2);
           }
         }
       }
     }
-    __syncthreads();
-    const float ie = kc.inv_e.x;
-    red[threadIdx.x] = make_float4(sL.x + sL.y, ie * (nD.x + nD.y), sY.x + sY.y, dY.x + dY.y);
-    red[kP2PThreads + threadIdx.x] = make_float4(sL2.x + sL2.y, ie * (nD2.x + nD2.y), sY2.x + sY2.y, dY2.x + dY2.y);
-    __syncthreads();
+    red[threadIdx.x] = p2p_sums(salt, kc.inv_e.x, sL, nD, sY, dY);
+    red[kP2PThreads + threadIdx.x] = p2p_sums(salt, kc.inv_e.x, sL2, nD2, sY2, dY2);
+    __syncthreads();                                           // the sums are there, the last chunk is free
     if (si == 0 && t < te) {
       const float s = (float)kInv4Pi;
       float4 a = red[ti];
@@ -947,42 +910,36 @@ __device__ __forceinline__ void p2p_body(int nunits, const int4 *__restrict__ un
         const float4 v = red[k * tile + ti];
         a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
       }
-      store_or_add(P2P_ARG(phi) + t, make_float4(s * a.x, s * a.y, s * a.z, s * a.w), whole);
+      store_or_add(P2P_ARG(phi) + t, make_float4(s * a.x, s * a.y, s * a.z, s * a.w), share.z != 0);
       if (t2 < te) {
         float4 c = red[kP2PThreads + ti];
         for (int k = 1; k < slices; ++k) {
           const float4 v = red[kP2PThreads + k * tile + ti];
           c.x += v.x; c.y += v.y; c.z += v.z; c.w += v.w;
         }
-        store_or_add(P2P_ARG(phi) + t2, make_float4(s * c.x, s * c.y, s * c.z, s * c.w), whole);
+        store_or_add(P2P_ARG(phi) + t2, make_float4(s * c.x, s * c.y, s * c.z, s * c.w), share.z != 0);
       }
     }
-  }
+    if (total == 0) __syncthreads();                           // no staging barrier before the sums' next use
   }
 }
 
-__global__ void __launch_bounds__(kP2PThreads, kP2PRegBlocks) k_p2p(int nunits, const int4 *__restrict__ units,
-                                                      const int32_t *__restrict__ leaves,
-                                                      const int64_t *__restrict__ pptr,
-                                                      const int32_t *__restrict__ pidx,
-                                                      const uint8_t *__restrict__ ptest,
-                                                      const int32_t *__restrict__ bbeg,
-                                                      const int32_t *__restrict__ bend,
-                                                      const dbl4 *__restrict__ center,
-                                                      const float4 *__restrict__ pos,
-                                                      const float4 *__restrict__ nrm,
-                                                      const float2 *__restrict__ xs, float inv_ebar,
-                                                      float kappa, float skip_scale,
-                                                      float4 *__restrict__ phi) {
-  p2p_body<false>(nunits, units, leaves, pptr, pidx, ptest, bbeg, bend, center, pos, nrm, xs, inv_ebar, kappa, skip_scale,
-                  phi, nullptr);
+__global__ void __launch_bounds__(kP2PThreads, kP2PRegBlocks) k_p2p(const P2PUnit *__restrict__ units,
+                                                                    const int4 *__restrict__ leaf_rec,
+                                                                    const float4 *__restrict__ src,
+                                                                    const int2 *__restrict__ slot,
+                                                                    const float4 *__restrict__ pos,
+                                                                    const float4 *__restrict__ nrm,
+                                                                    const float2 *__restrict__ xs, float inv_ebar,
+                                                                    float kappa, float skip_scale,
+                                                                    float4 *__restrict__ phi) {
+  p2p_body<false>(units, leaf_rec, src, slot, pos, nrm, xs, inv_ebar, kappa, skip_scale, phi, nullptr);
 }
 
 // P2P of several problems in one launch: the units of all of them, cost-ordered together.
-__global__ void __launch_bounds__(kP2PThreads, kP2PRegBlocks) k_p2p_batch(int nunits, const int4 *__restrict__ units,
+__global__ void __launch_bounds__(kP2PThreads, kP2PRegBlocks) k_p2p_batch(const P2PUnit *__restrict__ units,
                                                                           const P2PReq *__restrict__ reqs) {
-  p2p_body<true>(nunits, units, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr,
-                 nullptr, 0.f, 0.f, 0.f, nullptr, reqs);
+  p2p_body<true>(units, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 0.f, 0.f, 0.f, nullptr, reqs);
 }
 
 // ------------------------------------------------------------------------------------
@@ -1202,34 +1159,22 @@ const void *far_out_kernel(int order) {
 }
 
 Err enqueue_p2p(afmpb_t *h, cudaStream_t s) {
-  // Beside the far-field chain, six resident blocks per SM walk the units while the
-  // chain's kernels run at a higher stream priority (measured best among four to six, and
-  // against one block per unit: 0.565 against 0.595 ms for the 163,842-node product).
-  // Alone (meshes above the overlap limit) one block per unit lets the block scheduler
-  // hand the cost-ordered units out as blocks finish, which balances better than the
-  // static deal (0.226 against 0.256 ms for the same sphere's P2P timed alone).
-  int dev = 0, sms = 0;
-  AFMPB_CUDA(cudaGetDevice(&dev));
-  AFMPB_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const int grid = overlap_p2p(h) ? std::max(1, std::min(h->p2p_nunits, std::min(h->p2p_resident, kP2PRegBlocks) * sms))
-                                  : std::max(1, h->p2p_nunits);
+  // Beside the far-field chain the graph's node priorities let the chain's blocks in first
+  // as P2P blocks finish.  Against a static deal to six resident blocks per SM, products of
+  // 163,842 nodes 0.429 / 0.426 ms, 191,944 0.572 / 0.592, 655,362 1.306 / 1.399.
   AFMPB_CUDA(cudaMemsetAsync(h->d_phi_near, 0, sizeof(float4) * h->n, s));   // split leaves add into it
-  k_p2p<<<grid, kP2PThreads, 0, s>>>(h->p2p_nunits, h->d_p2p_units, h->d_leaves, h->d_p2p_ptr, h->d_p2p_idx, h->d_p2p_test, h->d_box_begin,
-                                                  h->d_box_end, h->d_box_center, h->d_pos, h->d_nrm, h->d_xs,
-                                                  (float)(1.0 / h->ebar), p2p_kappa(h),
-                                                  (float)(kP2PSkip * h->opt.near_c), h->d_phi_near);
+  if (h->p2p_nunits == 0) return Err{};
+  k_p2p<<<h->p2p_nunits, kP2PThreads, 0, s>>>(h->d_p2p_units, h->d_leaf_rec, h->d_p2p_src, h->d_p2p_slot, h->d_pos,
+                                     h->d_nrm, h->d_xs, (float)(1.0 / h->ebar), p2p_kappa(h),
+                                     (float)(kP2PSkip * h->opt.near_c), h->d_phi_near);
   return check_launch("k_p2p");
 }
 
 P2PReq p2p_req_of(const afmpb_t *h, const int *active) {
   P2PReq q{};
-  q.leaves = h->d_leaves;
-  q.pptr = h->d_p2p_ptr;
-  q.pidx = h->d_p2p_idx;
-  q.ptest = h->d_p2p_test;
-  q.bbeg = h->d_box_begin;
-  q.bend = h->d_box_end;
-  q.center = h->d_box_center;
+  q.leaf_rec = h->d_leaf_rec;
+  q.src = h->d_p2p_src;
+  q.slot = h->d_p2p_slot;
   q.pos = h->d_pos;
   q.nrm = h->d_nrm;
   q.xs = h->d_xs;
@@ -1241,13 +1186,9 @@ P2PReq p2p_req_of(const afmpb_t *h, const int *active) {
   return q;
 }
 
-Err enqueue_p2p_batch(const P2PReq *d_reqs, const int4 *d_units, int nunits, int resident, cudaStream_t s) {
+Err enqueue_p2p_batch(const P2PReq *d_reqs, const P2PUnit *d_units, int nunits, cudaStream_t s) {
   if (nunits == 0) return Err{};
-  int dev = 0, sms = 0;
-  AFMPB_CUDA(cudaGetDevice(&dev));
-  AFMPB_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const int grid = std::max(1, std::min(nunits, std::min(resident, kP2PRegBlocks) * sms));
-  k_p2p_batch<<<grid, kP2PThreads, 0, s>>>(nunits, d_units, d_reqs);
+  k_p2p_batch<<<nunits, kP2PThreads, 0, s>>>(d_units, d_reqs);
   return check_launch("k_p2p_batch");
 }
 

@@ -30,7 +30,7 @@ constexpr int kNumOffsets = 316;    // M2L offsets: [-3,3]^3 minus [-1,1]^3
 constexpr double kPi = 3.14159265358979323846;
 constexpr double kInv4Pi = 0.07957747154594767;  // 1 / (4 pi)
 constexpr int kP2PThreads = 128;   // threads of a P2P block (one work unit of one target leaf at a time)
-constexpr int kP2PResident = 6;    // P2P blocks kept resident per SM (<= 80 registers per thread)
+constexpr int kP2PResident = 6;    // P2P blocks resident per SM (<= 80 registers per thread)
 constexpr int kP2PUnitsPerBlock = 3;   // P2P work units per resident block (sets the unit size; 2-3 best of 1-32)
 constexpr int kL2PNodes = 128;     // nodes of an L2P block, in Morton order
 constexpr double kP2PSkip = 0.9;    // P2P leaves out pairs closer than kP2PSkip * c * (rho_p + rho_t)
@@ -219,15 +219,20 @@ struct __align__(16) TSItem {
                                 // req: the problem of a batched launch (0 otherwise)
 };
 
+// One P2P work unit: a leaf's targets against the entries [e0, e1) of its source boxes.  The
+// sources are staged in `total` slots, those of boxes whose pairs need the distance test in
+// the first `tested`; whole: the unit holds all of its leaf's entries.
+struct __align__(32) P2PUnit {
+  int leaf, e0, e1, req;        // req: the problem of a batched launch (0 otherwise)
+  int tested, total, whole, pad;
+};
+
 // One problem of a batched P2P launch: the arrays and constants k_p2p takes, and a device
 // flag (nullable) that stops its units when 0.
 struct P2PReq {
-  const int32_t *leaves;
-  const int64_t *pptr;
-  const int32_t *pidx;
-  const uint8_t *ptest;
-  const int32_t *bbeg, *bend;
-  const dbl4 *center;
+  const int4 *leaf_rec;
+  const float4 *src;
+  const int2 *slot;
   const float4 *pos, *nrm;
   const float2 *xs;
   float4 *phi;
@@ -305,9 +310,12 @@ struct afmpb_t {
   int64_t *d_p2p_ptr = nullptr;    // [nleaf+1] lists 1 + 3 per leaf (leaf order)
   int32_t *d_p2p_idx = nullptr;
   uint8_t *d_p2p_test = nullptr;   // [entries of p2p_idx] 1 where a pair may be inside the skip radius
-  int4 *d_p2p_units = nullptr;     // [p2p_nunits] P2P work units (leaf, first and end entry of its
-  int p2p_nunits = 0;              // source boxes in p2p_idx, -), most pairs first
-  int p2p_resident = afmpb::kP2PResident;            // P2P blocks per SM (tile tuner)
+  int64_t n_p2p_src = 0;           // entries of p2p_idx
+  float4 *d_p2p_src = nullptr;     // [n_p2p_src] by unit, then slot: source minus target box centre, first node
+  int2 *d_p2p_slot = nullptr;      // [n_p2p_src] the same: first slot in the unit, nodes
+  afmpb::P2PUnit *d_p2p_units = nullptr;   // [p2p_nunits] P2P work units, most pairs first
+  int p2p_nunits = 0;
+  int p2p_resident = afmpb::kP2PResident;            // P2P blocks per SM that the unit size is cut for (tile tuner)
   int p2p_units_per_block = afmpb::kP2PUnitsPerBlock;   // P2P unit size (tile tuner)
   int n_xbox = 0;                  // boxes whose list 4 goes to their local expansion (P2L)
   int32_t *d_xbox = nullptr;       // those boxes
@@ -455,9 +463,9 @@ Err enqueue_p2p(afmpb_t *h, cudaStream_t s);          // P2P into d_phi_near
 bool overlap_p2p(const afmpb_t *h);                   // P2P runs beside the far-field chain
 // The P2P arguments of a handle, with a stop flag for batched launches.
 P2PReq p2p_req_of(const afmpb_t *h, const int *active);
-// One P2P launch over the units of several problems (unit.w names the problem); every
+// One P2P launch over the units of several problems (unit.req names the problem); every
 // problem's d_phi_near must be zeroed before it.
-Err enqueue_p2p_batch(const P2PReq *d_reqs, const int4 *d_units, int nunits, int resident, cudaStream_t s);
+Err enqueue_p2p_batch(const P2PReq *d_reqs, const P2PUnit *d_units, int nunits, cudaStream_t s);
 Err enqueue_near_fold(afmpb_t *h, cudaStream_t s);   // near SpMV into phi_near, after P2P
 Err enqueue_combine(afmpb_t *h, cudaStream_t s, int parts);
 Err enqueue_m2l_tc(afmpb_t *h, cudaStream_t s);       // tensor-core M2L (precision 1)
@@ -513,7 +521,7 @@ struct BatchLists {
   std::vector<void *> bufs;
   P2PReq *d_p2p = nullptr;
   int **d_gms = nullptr;              // each problem's step state (gm[4]: running)
-  int4 *d_units = nullptr;            // P2P units of all problems, by cost (unit.w = problem)
+  P2PUnit *d_units = nullptr;         // P2P units of all problems, by cost
   int nunits = 0;
   TSReq *d_ts = nullptr;
   TSItem *d_items = nullptr, *d_items_run = nullptr;   // M2L items of all problems; the running ones

@@ -747,7 +747,7 @@ Err build_cycle_graph(afmpb_t *h, int m) {
   cudaError_t ce = cudaStreamEndCapture(cap, &out);
   if (!e.ok()) return e;
   if (ce != cudaSuccess) return make_err(AFMPB_ECUDA, std::string("cudaStreamEndCapture (cycle): ") + cudaGetErrorString(ce));
-  ce = cudaGraphInstantiate(&h->graph_cycle, g, 0);
+  ce = cudaGraphInstantiate(&h->graph_cycle, g, cudaGraphInstantiateFlagUseNodePriority);
   if (ce != cudaSuccess) return make_err(AFMPB_ECUDA, std::string("cudaGraphInstantiate (cycle): ") + cudaGetErrorString(ce));
   h->cycle_m = m;
   h->cycle_orth = orth;
@@ -1012,7 +1012,7 @@ Err build_batch_graph(afmpb_t *const *hs, int k, const int *ms, bool fuse_m2l, c
       AFMPB_CUDA(cudaEventRecord(ev_b[i], si[i]));
     }
     for (int i = 0; i < k; ++i) AFMPB_CUDA(cudaStreamWaitEvent(sp, ev_a[i], 0));
-    AFMPB_TRY(enqueue_p2p_batch(L.d_p2p, L.d_units, L.nunits, kP2PResident, sp));
+    AFMPB_TRY(enqueue_p2p_batch(L.d_p2p, L.d_units, L.nunits, sp));
     AFMPB_CUDA(cudaEventRecord(ev_p, sp));
     if (fuse_m2l) {
       for (int i = 0; i < k; ++i) AFMPB_CUDA(cudaStreamWaitEvent(sm, ev_b[i], 0));
@@ -1040,7 +1040,7 @@ Err build_batch_graph(afmpb_t *const *hs, int k, const int *ms, bool fuse_m2l, c
   cudaError_t ce = cudaStreamEndCapture(cap, &out);
   if (!e.ok()) return e;
   if (ce != cudaSuccess) return make_err(AFMPB_ECUDA, std::string("cudaStreamEndCapture (batch): ") + cudaGetErrorString(ce));
-  ce = cudaGraphInstantiate(&G.exec, g, 0);
+  ce = cudaGraphInstantiate(&G.exec, g, cudaGraphInstantiateFlagUseNodePriority);
   if (ce != cudaSuccess) return make_err(AFMPB_ECUDA, std::string("cudaGraphInstantiate (batch): ") + cudaGetErrorString(ce));
   return Err{};
 }

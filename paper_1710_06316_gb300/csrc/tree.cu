@@ -474,41 +474,94 @@ __global__ void k_p2p_lists(int nleaf, const int32_t *__restrict__ leaves, const
   cost[i] = (uint64_t)(ntiles * (4 * ((src + slices - 1) / slices) + src + 256));
 }
 
+// Blocks' time of a unit of nt targets and `total` staged sources, in cycles of a scheduler
+// with a block of its own: 146 for an iteration (two targets, two sources, 36 packed
+// operations each), 3 for a staged source, 3,000 for the unit's loads and sums.
+__device__ __forceinline__ uint64_t p2p_unit_cost(int64_t nt, int64_t total) {
+  const int64_t tile = max((int64_t)1, min((nt + 1) / 2, (int64_t)kP2PThreads));
+  const int64_t slices = kP2PThreads / tile, ntiles = (nt + 2 * tile - 1) / (2 * tile);
+  return (uint64_t)(ntiles * (146 * (((total + 1) / 2 + slices - 1) / slices) + 3 * total) + 3000);
+}
+
 // P2P work units: a leaf's source boxes cut into consecutive ranges of at most `budget`
 // target-source pairs (a range holds at least one box), so that blocks of comparable cost
-// can be dealt out statically.  fill == false counts the units of each leaf.
-// unit = (leaf, first box entry, end box entry, pairs)
-__global__ void k_p2p_units(int nleaf, const int32_t *__restrict__ leaves, const int32_t *__restrict__ bbeg,
+// can be dealt out.  fill == false counts the units of each leaf.  With it the entries of a
+// unit are put in the order of their slots (ord: the box that an entry now stands for): the
+// boxes whose pairs need the distance test first, the others from the next even slot on.
+__global__ void k_p2p_units(int nleaf, const int4 *__restrict__ leaf_rec, const int32_t *__restrict__ bbeg,
                             const int32_t *__restrict__ bend, const int64_t *__restrict__ pptr,
-                            const int32_t *__restrict__ pidx, int64_t budget, int64_t *__restrict__ cnt,
-                            const int64_t *__restrict__ uptr, int4 *__restrict__ units, uint64_t *__restrict__ ucost,
+                            const int32_t *__restrict__ pidx, const uint8_t *__restrict__ test, int64_t budget,
+                            int64_t *__restrict__ cnt, const int64_t *__restrict__ uptr, P2PUnit *__restrict__ units,
+                            uint64_t *__restrict__ ucost, int2 *__restrict__ slot, int32_t *__restrict__ ord,
                             bool fill) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nleaf) return;
-  const int b = leaves[i];
-  const int64_t nt = bend[b] - bbeg[b];
+  const int4 rec = leaf_rec[i];
+  const int64_t nt = rec.z - rec.y;
   int64_t k = fill ? uptr[i] : 0, nu = 0, acc = 0;
   int64_t start = pptr[i];
+  auto close = [&](int64_t end) {
+    if (fill) {
+      int64_t o = start;
+      int at = 0, nf = 0;
+      for (int pass = 1; pass >= 0; --pass) {           // tested boxes, then the others
+        for (int64_t j = start; j < end; ++j)
+          if ((test[j] != 0) == (pass == 1)) {
+            const int c = pidx[j], n = bend[c] - bbeg[c];
+            ord[o] = c;
+            slot[o++] = make_int2(at, n);
+            at += n;
+          }
+        if (pass == 1) {
+          nf = at;
+          at = (nf + 1) & ~1;
+        }
+      }
+      P2PUnit u{};
+      u.leaf = i;
+      u.e0 = (int)start;
+      u.e1 = (int)end;
+      u.tested = nf;
+      u.total = at;
+      u.whole = start == pptr[i] && end == pptr[i + 1];
+      units[k + nu] = u;
+      ucost[k + nu] = p2p_unit_cost(nt, at);
+    }
+    ++nu;
+  };
   for (int64_t j = pptr[i]; j < pptr[i + 1]; ++j) {
     const int c = pidx[j];
     const int64_t add = nt * (bend[c] - bbeg[c]);
     if (j > start && acc + add > budget) {
-      if (fill) {
-        units[k + nu] = make_int4(i, (int)start, (int)j, 0);
-        ucost[k + nu] = (uint64_t)acc;
-      }
-      ++nu;
+      close(j);
       start = j;
       acc = 0;
     }
     acc += add;
   }
-  if (fill) {
-    units[k + nu] = make_int4(i, (int)start, (int)pptr[i + 1], 0);
-    ucost[k + nu] = (uint64_t)acc;
-  }
-  ++nu;
+  close(pptr[i + 1]);
   if (!fill) cnt[i] = nu;
+}
+
+// What P2P needs of a unit's source box: the difference of the centres of the box and the
+// target leaf (formed in FP64) and the box's first node.  One warp a leaf.
+__global__ void k_p2p_src(int nleaf, const int4 *__restrict__ leaf_rec, const int64_t *__restrict__ pptr,
+                          const int32_t *__restrict__ ord, const int32_t *__restrict__ bbeg,
+                          const dbl4 *__restrict__ center, float4 *__restrict__ src) {
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (i >= nleaf) return;
+  const dbl4 ct = center[leaf_rec[i].x];
+  for (int64_t j = pptr[i] + lane; j < pptr[i + 1]; j += 32) {
+    const int c = ord[j];
+    const dbl4 cs = center[c];
+    src[j] = make_float4((float)(cs.x - ct.x), (float)(cs.y - ct.y), (float)(cs.z - ct.z), __int_as_float(bbeg[c]));
+  }
+}
+
+__global__ void k_gather_units(int64_t n, const int32_t *__restrict__ idx, const P2PUnit *__restrict__ src,
+                               P2PUnit *__restrict__ dst) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i < n) dst[i] = src[idx[i]];
 }
 
 // Work records of the far-field passes: (box, first node, end node, level) of every leaf,
@@ -605,12 +658,6 @@ __global__ void k_p2p_test(int nleaf, const int32_t *__restrict__ leaves, const 
     const double R = skip * (brho[b] + brho[c]) * (1.0 + 1e-5) + 1e-6 * size;
     test[j] = gap2 <= R * R ? 1 : 0;
   }
-}
-
-__global__ void k_gather_int4(int64_t n, const int32_t *__restrict__ idx, const int4 *__restrict__ src,
-                              int4 *__restrict__ dst) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i < n) dst[i] = src[idx[i]];
 }
 
 // (level, offset) key and (target, source) pair of every list-2 entry, in box order
@@ -748,22 +795,28 @@ Err build_p2p_units(afmpb_t *h) {
   int64_t *cnt = nullptr;
   AFMPB_TRY(A.alloc(&cnt, nl + 1, "p2p unit counts"));
   AFMPB_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int64_t) * (nl + 1), s));
-  k_p2p_units<<<div_up(nl, 128), 128, 0, s>>>(nl, h->d_leaves, h->d_box_begin, h->d_box_end, h->d_p2p_ptr,
-                                              h->d_p2p_idx, budget, cnt, nullptr, nullptr, nullptr, false);
+  k_p2p_units<<<div_up(nl, 128), 128, 0, s>>>(nl, h->d_leaf_rec, h->d_box_begin, h->d_box_end, h->d_p2p_ptr,
+                                              h->d_p2p_idx, h->d_p2p_test, budget, cnt, nullptr, nullptr, nullptr,
+                                              nullptr, nullptr, false);
   AFMPB_TRY(check_launch("k_p2p_units count"));
   int64_t *d_uptr = nullptr, nunits = 0;
   AFMPB_TRY(csr_ptr(h, cnt, nl, &d_uptr, &nunits, "p2p unit ptr"));
-  int4 *units = nullptr;
+  P2PUnit *units = nullptr;
   uint64_t *ucost = nullptr, *ucost_sorted = nullptr;
-  int32_t *uiota = nullptr, *uorder = nullptr;
+  int32_t *uiota = nullptr, *uorder = nullptr, *ord = nullptr;
+  AFMPB_TRY(A.alloc(&ord, h->n_p2p_src, "p2p source order"));
   AFMPB_TRY(A.alloc(&units, nunits, "p2p units unsorted"));
   AFMPB_TRY(A.alloc(&ucost, nunits, "p2p unit cost"));
   AFMPB_TRY(A.alloc(&ucost_sorted, nunits, "p2p unit cost sorted"));
   AFMPB_TRY(A.alloc(&uiota, nunits, "p2p unit iota"));
   AFMPB_TRY(A.alloc(&uorder, nunits, "p2p unit order"));
-  k_p2p_units<<<div_up(nl, 128), 128, 0, s>>>(nl, h->d_leaves, h->d_box_begin, h->d_box_end, h->d_p2p_ptr,
-                                              h->d_p2p_idx, budget, nullptr, d_uptr, units, ucost, true);
+  k_p2p_units<<<div_up(nl, 128), 128, 0, s>>>(nl, h->d_leaf_rec, h->d_box_begin, h->d_box_end, h->d_p2p_ptr,
+                                              h->d_p2p_idx, h->d_p2p_test, budget, nullptr, d_uptr, units, ucost,
+                                              h->d_p2p_slot, ord, true);
   AFMPB_TRY(check_launch("k_p2p_units fill"));
+  k_p2p_src<<<div_up((int64_t)nl * 32, 128), 128, 0, s>>>(nl, h->d_leaf_rec, h->d_p2p_ptr, ord, h->d_box_begin,
+                                                          h->d_box_center, h->d_p2p_src);
+  AFMPB_TRY(check_launch("k_p2p_src"));
   k_iota<<<div_up(nunits, 256), 256, 0, s>>>((int)nunits, uiota);
   AFMPB_TRY(check_launch("k_iota"));
   AFMPB_TRY(cub_call(h, "p2p unit order", [&](void *t, size_t &bytes) {
@@ -771,12 +824,12 @@ Err build_p2p_units(afmpb_t *h) {
   }));
   if (h->d_p2p_units) A.release(h->d_p2p_units);
   AFMPB_TRY(A.alloc(&h->d_p2p_units, nunits, "p2p units"));
-  k_gather_int4<<<div_up(nunits, 256), 256, 0, s>>>(nunits, uorder, units, h->d_p2p_units);
-  AFMPB_TRY(check_launch("k_gather_int4"));
+  k_gather_units<<<div_up(nunits, 256), 256, 0, s>>>(nunits, uorder, units, h->d_p2p_units);
+  AFMPB_TRY(check_launch("k_gather_units"));
   h->p2p_nunits = (int)nunits;
   AFMPB_CUDA(cudaStreamSynchronize(s));
   for (void *q : {(void *)cnt, (void *)d_uptr, (void *)units, (void *)ucost, (void *)ucost_sorted, (void *)uiota,
-                  (void *)uorder})
+                  (void *)uorder, (void *)ord})
     A.release(q);
   return Err{};
 }
@@ -1071,6 +1124,9 @@ Err build_tree(afmpb_t *h) {
     AFMPB_TRY(csr_ptr(h, cnt, nl, &h->d_p2p_ptr, &n_p, "p2p_ptr"));
     AFMPB_TRY(A.alloc(&h->d_p2p_idx, n_p, "p2p_idx"));
     AFMPB_TRY(A.alloc(&h->d_p2p_test, n_p, "p2p test flags"));
+    AFMPB_TRY(A.alloc(&h->d_p2p_src, n_p, "p2p sources"));
+    AFMPB_TRY(A.alloc(&h->d_p2p_slot, n_p, "p2p slots"));
+    h->n_p2p_src = n_p;
     k_p2p_lists<<<div_up(nl, 64), 64, 0, s>>>(nl, h->d_leaves, bbeg, bend, bparent, bchild0, bnchild, d_uptr,
                                               h->d_u_idx, d_xptr, h->d_x_idx, d_xdirect, d_wptr, h->d_w_idx, nullptr,
                                               nullptr, nullptr, h->d_p2p_ptr, h->d_p2p_idx, true);
@@ -1082,7 +1138,6 @@ Err build_tree(afmpb_t *h) {
     int64_t pairs = 0;
     AFMPB_TRY(read_one(&pairs, d_pairs, s));
     T.n_p2p_pairs = pairs - h->n;     // the diagonal t == p is skipped
-    AFMPB_TRY(build_p2p_units(h));
     for (void *q : {(void *)cnt, (void *)pairs_l, (void *)d_pairs, (void *)cost, (void *)cost_sorted, (void *)iota})
       A.release(q);
   }
@@ -1210,6 +1265,7 @@ Err build_tree(afmpb_t *h) {
                                                                 kP2PSkip * h->opt.near_c, h->d_p2p_test);
   AFMPB_TRY(check_launch("k_p2p_test"));
   A.release(d_ext);
+  AFMPB_TRY(build_p2p_units(h));
   A.release(d_cnt1);
   A.release(d_cnt2);
   A.release(d_lvl_start);
