@@ -443,14 +443,30 @@ __global__ void k_step_end(int *__restrict__ gm, int m, const double *__restrict
   cudaGraphSetConditional(loop, go ? 1u : 0u);
 }
 
-// back substitution H(0:k,0:k) y = g(0:k), k = gm[0] steps of the cycle, y over g
-__global__ void k_backsolve_j(const int *__restrict__ gm, int m, const double *__restrict__ H, double *__restrict__ g) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// back substitution H(0:k,0:k) y = g(0:k), k = gm[0] steps of the cycle, y over g: one block,
+// a column of H at a time, from shared memory where the triangle fits (a thread on global
+// memory took 60 us for 25 steps)
+constexpr int kBackShared = 72;
+__global__ void __launch_bounds__(256) k_backsolve_j(const int *__restrict__ gm, int m, const double *__restrict__ H,
+                                                     double *__restrict__ g) {
+  __shared__ double h[kBackShared * (kBackShared + 1) / 2];
+  __shared__ double y;
   const int k = gm[0];
-  for (int i = k - 1; i >= 0; --i) {
-    double s = g[i];
-    for (int c = i + 1; c < k; ++c) s -= H[(int64_t)c * (m + 1) + i] * g[c];
-    g[i] = s / H[(int64_t)i * (m + 1) + i];
+  const bool staged = k <= kBackShared;
+  if (staged)
+    for (int c = threadIdx.x >> 5; c < k; c += blockDim.x >> 5)
+      for (int i = threadIdx.x & 31; i <= c; i += 32) h[c * (c + 1) / 2 + i] = H[(int64_t)c * (m + 1) + i];
+  __syncthreads();
+  for (int c = k - 1; c >= 0; --c) {
+    const double *col = staged ? h + c * (c + 1) / 2 : H + (int64_t)c * (m + 1);
+    if (threadIdx.x == 0) {
+      y = g[c] / col[c];
+      g[c] = y;
+    }
+    __syncthreads();
+    const double yc = y;
+    for (int i = threadIdx.x; i < c; i += blockDim.x) g[i] -= col[i] * yc;
+    __syncthreads();
   }
 }
 
@@ -500,23 +516,67 @@ __device__ __forceinline__ void fold_parts(int nb, int cnt, const double *part, 
   }
 }
 
+// A block's chunk of w passes through shared memory kGsTile elements at a time: the threads
+// form w for it (an element each, the basis vectors' loads independent), then each warp
+// takes every eighth basis vector for its dot with the tile, so that a warp has a tile's
+// worth of loads in flight and one shuffle tree per vector.  With a vector after the other
+// on the whole block (a barrier pair each) and 2,048 elements to a block, the step's kernels
+// took 88 us of a 225 us step on 20,838 nodes; latency and the FP64 pipe (2 FMA per clock
+// and SM) bound them, so small problems spread over as many SMs as they have tiles.
+constexpr int kGsTile = 256;
+
+// The dots of the tile `t` (cnt elements of w from `k0` on) with V_0 .. V_{nv-1}, into the
+// block's partial sums (set by its first tile, added to by the others).
+__device__ __forceinline__ void gs_tile_dots(const double *t, int64_t k0, int cnt, int nv, const double *__restrict__ V,
+                                             int64_t ldv, double *part, bool first) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int i = warp; i < nv; i += kRedThreads / 32) {
+    const double *v = V + (int64_t)i * ldv + k0;
+    double a[2] = {0.0, 0.0};
+#pragma unroll
+    for (int q = 0; q < kGsTile / 32; ++q) {
+      const int e = lane + 32 * q;
+      if (e < cnt) a[q & 1] = fma(v[e], t[e], a[q & 1]);
+    }
+    double s = a[0] + a[1];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) part[i] = first ? s : part[i] + s;
+  }
+}
+
+// sum_i c_i V_i at element k
+__device__ __forceinline__ double gs_combo(int64_t k, int nv, const double *__restrict__ V, int64_t ldv,
+                                           const double *c) {
+  double a[4] = {0.0, 0.0, 0.0, 0.0};
+  int i = 0;
+  for (; i + 8 <= nv; i += 8)
+#pragma unroll
+    for (int q = 0; q < 8; ++q) a[q & 3] = fma(c[i + q], V[(int64_t)(i + q) * ldv + k], a[q & 3]);
+  for (; i < nv; ++i) a[0] = fma(c[i], V[(int64_t)i * ldv + k], a[0]);
+  return (a[0] + a[1]) + (a[2] + a[3]);
+}
+
 // w = ys (FP32 -> FP64); h1 = V_{0..j}^T w
-__global__ void __launch_bounds__(kRedThreads) k_gs_first(int64_t len, int *__restrict__ gm, const double *__restrict__ V,
-                                                          int64_t ldv, const float *__restrict__ ys,
-                                                          double *__restrict__ w, double *__restrict__ part, int stride,
-                                                          double *__restrict__ hcol, const int *__restrict__ guard) {
+__global__ void __launch_bounds__(kRedThreads) k_gs_first(int64_t len, int64_t chunk, int *__restrict__ gm,
+                                                          const double *__restrict__ V, int64_t ldv,
+                                                          const float *__restrict__ ys, double *__restrict__ w,
+                                                          double *part, int stride, double *__restrict__ hcol,
+                                                          const int *__restrict__ guard) {
   if (guard && *guard == 0) return;
-  __shared__ double sh[32];
+  __shared__ double tile[kGsTile];
   const int nv = gm[0] + 1;
-  const int64_t chunk = (len + gridDim.x - 1) / gridDim.x;
   const int64_t lo = blockIdx.x * chunk, hi = min(len, lo + chunk);
-  for (int64_t k = lo + threadIdx.x; k < hi; k += blockDim.x) w[k] = (double)ys[k];
-  for (int i = 0; i < nv; ++i) {
-    const double *v = V + (int64_t)i * ldv;
-    double a = 0.0;
-    for (int64_t k = lo + threadIdx.x; k < hi; k += blockDim.x) a = fma(v[k], w[k], a);
-    a = block_sum(a, sh);
-    if (threadIdx.x == 0) part[(int64_t)blockIdx.x * stride + i] = a;
+  for (int64_t k0 = lo; k0 < hi; k0 += kGsTile) {
+    const int64_t k = k0 + threadIdx.x;
+    __syncthreads();
+    if (k < hi) {
+      const double x = (double)ys[k];
+      tile[threadIdx.x] = x;
+      w[k] = x;
+    }
+    __syncthreads();
+    gs_tile_dots(tile, k0, (int)min((int64_t)kGsTile, hi - k0), nv, V, ldv, part + (int64_t)blockIdx.x * stride, k0 == lo);
   }
   if (last_block_of(gm + 5)) {
     fold_parts(gridDim.x, nv, part, stride, hcol);
@@ -525,26 +585,25 @@ __global__ void __launch_bounds__(kRedThreads) k_gs_first(int64_t len, int *__re
 }
 
 // w -= V h1; h2 = V^T w; h1 += h2
-__global__ void __launch_bounds__(kRedThreads) k_gs_second(int64_t len, int *__restrict__ gm, const double *__restrict__ V,
-                                                           int64_t ldv, double *__restrict__ w, double *__restrict__ part,
-                                                           int stride, double *__restrict__ hcol, double *__restrict__ hcol2,
+__global__ void __launch_bounds__(kRedThreads) k_gs_second(int64_t len, int64_t chunk, int *__restrict__ gm,
+                                                           const double *__restrict__ V, int64_t ldv,
+                                                           double *__restrict__ w, double *part, int stride,
+                                                           double *__restrict__ hcol, double *__restrict__ hcol2,
                                                            const int *__restrict__ guard) {
   if (guard && *guard == 0) return;
-  __shared__ double sh[32];
+  __shared__ double tile[kGsTile];
   const int nv = gm[0] + 1;
-  const int64_t chunk = (len + gridDim.x - 1) / gridDim.x;
   const int64_t lo = blockIdx.x * chunk, hi = min(len, lo + chunk);
-  for (int64_t k = lo + threadIdx.x; k < hi; k += blockDim.x) {
-    double a = 0.0;
-    for (int i = 0; i < nv; ++i) a = fma(hcol[i], V[(int64_t)i * ldv + k], a);
-    w[k] -= a;
-  }
-  for (int i = 0; i < nv; ++i) {
-    const double *v = V + (int64_t)i * ldv;
-    double a = 0.0;
-    for (int64_t k = lo + threadIdx.x; k < hi; k += blockDim.x) a = fma(v[k], w[k], a);
-    a = block_sum(a, sh);
-    if (threadIdx.x == 0) part[(int64_t)blockIdx.x * stride + i] = a;
+  for (int64_t k0 = lo; k0 < hi; k0 += kGsTile) {
+    const int64_t k = k0 + threadIdx.x;
+    __syncthreads();
+    if (k < hi) {
+      const double x = w[k] - gs_combo(k, nv, V, ldv, hcol);
+      tile[threadIdx.x] = x;
+      w[k] = x;
+    }
+    __syncthreads();
+    gs_tile_dots(tile, k0, (int)min((int64_t)kGsTile, hi - k0), nv, V, ldv, part + (int64_t)blockIdx.x * stride, k0 == lo);
   }
   if (last_block_of(gm + 6)) {
     fold_parts(gridDim.x, nv, part, stride, hcol2);
@@ -554,11 +613,53 @@ __global__ void __launch_bounds__(kRedThreads) k_gs_second(int64_t len, int *__r
   }
 }
 
+// givens_update by a block: column, rotations and the new entry pass through shared memory
+// (a thread on global memory waits for each of the column's j dependent updates).
+constexpr int kGivensShared = 256;
+__device__ __forceinline__ void givens_update_block(int j, int m, double nrm, double *__restrict__ hcol,
+                                                    double *__restrict__ H, double *__restrict__ cs,
+                                                    double *__restrict__ sn, double *__restrict__ g,
+                                                    double *__restrict__ res) {
+  __shared__ double col[kGivensShared + 1], c[kGivensShared], z[kGivensShared];
+  if (threadIdx.x == 0) hcol[j + 1] = nrm;
+  if (j >= kGivensShared) {
+    __syncthreads();
+    if (threadIdx.x == 0) givens_update(j, m, hcol, H, cs, sn, g, res);
+    __syncthreads();
+    return;
+  }
+  for (int i = threadIdx.x; i < j; i += blockDim.x) {
+    c[i] = cs[i];
+    z[i] = sn[i];
+  }
+  for (int i = threadIdx.x; i <= j; i += blockDim.x) col[i] = hcol[i];
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double a = col[0];
+    for (int i = 0; i < j; ++i) {                       // a: the rotated entry i so far
+      const double b = col[i + 1];
+      col[i] = c[i] * a + z[i] * b;
+      a = -z[i] * a + c[i] * b;
+    }
+    const double den = hypot(a, nrm), gj = g[j];
+    const double cj = den > 0 ? a / den : 1.0, sj = den > 0 ? nrm / den : 0.0;
+    col[j] = den;
+    cs[j] = cj;
+    sn[j] = sj;
+    g[j + 1] = -sj * gj;
+    g[j] = cj * gj;
+    res[0] = fabs(sj * gj);
+  }
+  __syncthreads();
+  double *out = H + (int64_t)j * (m + 1);
+  for (int i = threadIdx.x; i <= j + 1; i += blockDim.x) out[i] = i <= j ? col[i] : 0.0;
+}
+
 // w -= V h2; ||w||; Givens update; j += 1 and the stop test (batch: the problem's running
 // flag, else the condition of the graph's WHILE loop)
-__global__ void __launch_bounds__(kRedThreads) k_gs_norm(int64_t len, int *__restrict__ gm, int m,
+__global__ void __launch_bounds__(kRedThreads) k_gs_norm(int64_t len, int64_t chunk, int *__restrict__ gm, int m,
                                                          const double *__restrict__ V, int64_t ldv, double *__restrict__ w,
-                                                         double *__restrict__ part, int stride, double *__restrict__ hcol,
+                                                         double *part, int stride, double *__restrict__ hcol,
                                                          const double *__restrict__ hcol2, double *__restrict__ H,
                                                          double *__restrict__ cs, double *__restrict__ sn,
                                                          double *__restrict__ g, double *__restrict__ res,
@@ -567,13 +668,10 @@ __global__ void __launch_bounds__(kRedThreads) k_gs_norm(int64_t len, int *__res
   if (guard && *guard == 0) return;
   __shared__ double sh[32];
   const int j = gm[0], nv = j + 1;
-  const int64_t chunk = (len + gridDim.x - 1) / gridDim.x;
   const int64_t lo = blockIdx.x * chunk, hi = min(len, lo + chunk);
   double q = 0.0;
   for (int64_t k = lo + threadIdx.x; k < hi; k += blockDim.x) {
-    double a = 0.0;
-    for (int i = 0; i < nv; ++i) a = fma(hcol2[i], V[(int64_t)i * ldv + k], a);
-    const double x = w[k] - a;
+    const double x = w[k] - gs_combo(k, nv, V, ldv, hcol2);
     w[k] = x;
     q = fma(x, x, q);
   }
@@ -583,10 +681,9 @@ __global__ void __launch_bounds__(kRedThreads) k_gs_norm(int64_t len, int *__res
     __shared__ double s_nrm;
     fold_parts(gridDim.x, 1, part, stride, &s_nrm);
     __syncthreads();
+    givens_update_block(j, m, sqrt(s_nrm), hcol, H, cs, sn, g, res);
     if (threadIdx.x == 0) {
       gm[7] = 0;
-      hcol[j + 1] = sqrt(s_nrm);
-      givens_update(j, m, hcol, H, cs, sn, g, res);
       gm[0] = j + 1;
       gm[1] += 1;
       const bool go = j + 1 < m && res[0] > tol[0];      // a NaN residual stops as well
@@ -665,11 +762,14 @@ Err enqueue_step_tail(afmpb_t *h, int m, cudaStream_t cap, const int *act, bool 
   const int64_t n = h->n, n2 = 2 * n;
   const int orth = h->opt.orth;
   if (orth == 0) {
-    const int nb = red_blocks(n2), stride = m + 2;
+    // a tile to a block, more of them above the partial sums' 1,184 blocks
+    const int64_t chunk = ((n2 + 1183) / 1184 + kGsTile - 1) / kGsTile * kGsTile;
+    const int nb = div_up(n2, chunk), stride = m + 2;
     int *gm = h->d_gm_int;
-    k_gs_first<<<nb, kRedThreads, 0, cap>>>(n2, gm, h->d_V, n2, h->d_ys, h->d_w, h->d_part, stride, h->d_hcol, act);
-    k_gs_second<<<nb, kRedThreads, 0, cap>>>(n2, gm, h->d_V, n2, h->d_w, h->d_part, stride, h->d_hcol, h->d_hcol2, act);
-    k_gs_norm<<<nb, kRedThreads, 0, cap>>>(n2, gm, m, h->d_V, n2, h->d_w, h->d_part, stride, h->d_hcol, h->d_hcol2,
+    k_gs_first<<<nb, kRedThreads, 0, cap>>>(n2, chunk, gm, h->d_V, n2, h->d_ys, h->d_w, h->d_part, stride, h->d_hcol, act);
+    k_gs_second<<<nb, kRedThreads, 0, cap>>>(n2, chunk, gm, h->d_V, n2, h->d_w, h->d_part, stride, h->d_hcol, h->d_hcol2,
+                                             act);
+    k_gs_norm<<<nb, kRedThreads, 0, cap>>>(n2, chunk, gm, m, h->d_V, n2, h->d_w, h->d_part, stride, h->d_hcol, h->d_hcol2,
                                            h->d_H, h->d_cs, h->d_sn, h->d_g, h->d_scal + 2, h->d_scal + 4,
                                            batch ? 1 : 0, loop, act);
     k_gs_normalize<<<div_up(n, 256), 256, 0, cap>>>(n, gm, h->d_w, h->d_hcol, h->d_V, n2, h->d_xs, act);
@@ -846,7 +946,7 @@ Err run_solve(afmpb_t *h, afmpb_solve_info *info) {
     // the Arnoldi steps of the cycle: one graph launch, no host synchronisation inside
     AFMPB_CUDA(cudaGraphLaunch(h->graph_cycle, s));
     // x += V y, H y = g
-    k_backsolve_j<<<1, 1, 0, s>>>(h->d_gm_int, m, h->d_H, h->d_g);
+    k_backsolve_j<<<1, 256, 0, s>>>(h->d_gm_int, m, h->d_H, h->d_g);
     k_update_x<<<nb_comb, 256, 0, s>>>(n2, h->d_gm_int, h->d_V, n2, h->d_g, x);
     AFMPB_TRY(check_launch("gmres update"));
     AFMPB_CUDA(cudaMemcpyAsync(h_gm, h->d_gm_int, sizeof(h_gm), cudaMemcpyDeviceToHost, s));
@@ -1145,7 +1245,7 @@ Err run_solve_batch(afmpb_t *const *hs, int k, afmpb_solve_info *infos, afmpb_st
       State &S = st[i];
       if (!S.running) continue;
       const int64_t n2 = 2 * h->n;
-      k_backsolve_j<<<1, 1, 0, h->stream>>>(h->d_gm_int, ms[i], h->d_H, h->d_g);
+      k_backsolve_j<<<1, 256, 0, h->stream>>>(h->d_gm_int, ms[i], h->d_H, h->d_g);
       k_update_x<<<std::min(div_up(n2, 256), 4 * 1184), 256, 0, h->stream>>>(n2, h->d_gm_int, h->d_V, n2, h->d_g,
                                                                               h->d_sol);
       AFMPB_TRY(check_launch("batch gmres update"));
