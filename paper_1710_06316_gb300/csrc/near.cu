@@ -15,10 +15,8 @@
 // integrands vanish and A, D are weakly singular; polar (Duffy) map about x_p with a
 // 16 x 16 Gauss-Legendre rule.
 //
-// Scheduling: self entries take one thread per node.  Off-diagonal entries are handed to
-// lanes by a global counter, and each lane's adaptive walk is split into a cheap
-// advance-to-next-leaf phase and a leaf-evaluation phase that the whole warp runs
-// together (a lane per row with each lane walking its own tree left ~3 of 32 lanes busy).
+// Scheduling: lanes share a node's self rule and its search, and a warp shares the leaves of
+// a batch of off-diagonal entries (see the kernels).
 //
 // Precision: all geometry is first taken relative to the target x_p in FP64 (so no
 // large-coordinate cancellation reaches the quadrature), then the quadrature runs in
@@ -165,8 +163,9 @@ __device__ __forceinline__ void tri_rel_f32(const GeomF32 &g, const int32_t *tri
 }
 
 template <class Real>
-__device__ void self_rule(Real kappa, Real inv_ebar, const GeomF32 &gf, const int32_t *tri, const int64_t *inc_ptr,
-                          const int32_t *inc_tri, int64_t op, const V3<Real> &np, Real o[4]) {
+__device__ void self_rule(Real kappa, const GeomF32 &gf, const int32_t *tri, const int64_t *inc_ptr,
+                          const int32_t *inc_tri, int64_t op, const V3<Real> &np, int first, int step, Real &Asum,
+                          Real &Dsum) {
   Real As = 0, Ds = 0;
   for (int64_t j = inc_ptr[op]; j < inc_ptr[op + 1]; ++j) {
     V3<Real> P[3];
@@ -185,7 +184,7 @@ __device__ void self_rule(Real kappa, Real inv_ebar, const GeomF32 &gf, const in
       const V3<Real> cr{e[0].y * e[1].z - e[0].z * e[1].y, e[0].z * e[1].x - e[0].x * e[1].z,
                         e[0].x * e[1].y - e[0].y * e[1].x};
       const Real J = sqrt(dot(cr, cr));
-      for (int it = 0; it < 16; ++it) {
+      for (int it = first; it < 16; it += step) {
         const Real tt = c_gl_xf[it], wt = c_gl_wf[it];
         const V3<Real> w{e[0].x + tt * (e[1].x - e[0].x), e[0].y + tt * (e[1].y - e[0].y),
                          e[0].z + tt * (e[1].z - e[0].z)};
@@ -206,48 +205,75 @@ __device__ void self_rule(Real kappa, Real inv_ebar, const GeomF32 &gf, const in
       }
     }
   }
-  o[0] = As;
-  o[1] = 0;
-  o[2] = 0;
-  o[3] = Ds * inv_ebar;
+  Asum = As;
+  Dsum = Ds;
 }
 
 // Near-set walk.  fill == false: count per row; else write the columns.
-__global__ void k_near_search(int64_t n, double cnear, const int32_t *__restrict__ perm,
-                              const double *__restrict__ xyz, const double *__restrict__ rho,
-                              const float4 *__restrict__ pos, const float4 *__restrict__ nrm,
-                              const dbl4 *__restrict__ center, const double *__restrict__ brho,
-                              const int32_t *__restrict__ child0, const int32_t *__restrict__ nchild,
-                              const int32_t *__restrict__ bbeg, const int32_t *__restrict__ bend,
-                              int64_t *__restrict__ cnt, const int64_t *__restrict__ ptr,
-                              int32_t *__restrict__ col, bool fill) {
-  int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (p >= n) return;
+//
+// Bound by the latency of its dependent loads, so kNearLanes lanes share a node: they test
+// the children of a box together and a leaf's nodes kNearLanes at a time, in the order of a
+// walk by one thread (20,838 nodes, both passes: 0.89 ms with a thread to a node, 0.36 so).
+constexpr int kNearLanes = 8;
+constexpr int kNearSearchBlock = 128;
+
+__global__ void __launch_bounds__(kNearSearchBlock)
+    k_near_search(int64_t n, double cnear, const int32_t *__restrict__ perm, const double *__restrict__ xyz,
+                  const double *__restrict__ rho, const float4 *__restrict__ pos, const float4 *__restrict__ nrm,
+                  const dbl4 *__restrict__ center, const double *__restrict__ brho, const int32_t *__restrict__ child0,
+                  const int32_t *__restrict__ nchild, const int32_t *__restrict__ bbeg,
+                  const int32_t *__restrict__ bend, int64_t *__restrict__ cnt, const int64_t *__restrict__ ptr,
+                  int32_t *__restrict__ col, bool fill) {
+  __shared__ int stacks[kNearSearchBlock / kNearLanes][kNearStack];
+  const int64_t p = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / kNearLanes;
+  if (p >= n) return;                          // a whole group of lanes
+  const int lane = threadIdx.x % kNearLanes, shift = threadIdx.x % 32 / kNearLanes * kNearLanes;
+  const unsigned group = ((1u << kNearLanes) - 1u) << shift, below = (1u << lane) - 1u;
+  int *stack = stacks[threadIdx.x / kNearLanes];
   int64_t op = perm[p];
   const double x0 = xyz[3 * op], x1 = xyz[3 * op + 1], x2 = xyz[3 * op + 2];
   const double rp = rho[op];
-  int64_t k = 0, base = fill ? ptr[p] : 0;
-  int stack[kNearStack];
-  int sp = 0;
-  stack[sp++] = 0;
-  while (sp > 0) {
-    int b = stack[--sp];
-    dbl4 c = center[b];
-    double dx = fmax(fabs(x0 - c.x) - c.w, 0.0), dy = fmax(fabs(x1 - c.y) - c.w, 0.0),
-           dz = fmax(fabs(x2 - c.z) - c.w, 0.0);
-    // box pruning: compared squared (a box at the boundary is kept, never wrongly dropped:
-    // the squared test errs by a few ulps and a kept box is only searched)
+  // box pruning: compared squared (a box at the boundary is kept, never wrongly dropped:
+  // the squared test errs by a few ulps and a kept box is only searched)
+  const auto within = [&](int b) {
+    const dbl4 c = center[b];
+    const double dx = fmax(fabs(x0 - c.x) - c.w, 0.0), dy = fmax(fabs(x1 - c.y) - c.w, 0.0),
+                 dz = fmax(fabs(x2 - c.z) - c.w, 0.0);
     const double bR = cnear * (rp + brho[b]);
-    if (dx * dx + dy * dy + dz * dz >= bR * bR * (1.0 + 1e-12)) continue;
-    if (nchild[b] == 0) {
-      // FP32 pre-test on the leaf-relative positions.  The FP32 distance carries an
-      // absolute error below 2^-22 (|o| + |q|) per component (|o|, |q|: the offsets it is
-      // formed from), so d^2 is off by less than 5e-7 R S + 1e-6 R^2 near the boundary
-      // (S = sum of the |o| and |q| components); the FP64 test decides inside twice that.
-      const float ox = (float)(x0 - c.x), oy = (float)(x1 - c.y), oz = (float)(x2 - c.z);
-      const float so = fabsf(ox) + fabsf(oy) + fabsf(oz);
-      const float frp = (float)(cnear * rp), fc = (float)cnear;
-      for (int t = bbeg[b]; t < bend[b]; ++t) {
+    return !(dx * dx + dy * dy + dz * dz >= bR * bR * (1.0 + 1e-12));
+  };
+  int64_t k = 0;
+  const int64_t base = fill ? ptr[p] : 0;
+  int sp = 0;
+  if (within(0)) {
+    if (lane == 0) stack[0] = 0;
+    sp = 1;
+  }
+  __syncwarp(group);
+  while (sp > 0) {
+    const int b = stack[--sp];
+    const int nc = nchild[b];
+    if (nc > 0) {
+      const bool keep = lane < nc && within(child0[b] + lane);
+      const unsigned m = (__ballot_sync(group, keep) >> shift) & ((1u << kNearLanes) - 1u);
+      if (keep) stack[sp + __popc(m) - 1 - __popc(m & below)] = child0[b] + lane;   // the first on top
+      sp += __popc(m);
+      __syncwarp(group);
+      continue;
+    }
+    // FP32 pre-test on the leaf-relative positions.  The FP32 distance carries an
+    // absolute error below 2^-22 (|o| + |q|) per component (|o|, |q|: the offsets it is
+    // formed from), so d^2 is off by less than 5e-7 R S + 1e-6 R^2 near the boundary
+    // (S = sum of the |o| and |q| components); the FP64 test decides inside twice that.
+    const dbl4 c = center[b];
+    const float ox = (float)(x0 - c.x), oy = (float)(x1 - c.y), oz = (float)(x2 - c.z);
+    const float so = fabsf(ox) + fabsf(oy) + fabsf(oz);
+    const float frp = (float)(cnear * rp), fc = (float)cnear;
+    const int end = bend[b];
+    for (int t0 = bbeg[b]; t0 < end; t0 += kNearLanes) {
+      const int t = t0 + lane;
+      bool in = false;
+      if (t < end) {
         const float4 q = pos[t];
         const float fx = ox - q.x, fy = oy - q.y, fz = oz - q.z;
         const float fd2 = fx * fx + fy * fy + fz * fz;
@@ -255,7 +281,6 @@ __global__ void k_near_search(int64_t n, double cnear, const int32_t *__restrict
         const float fR2 = fR * fR;
         const float S = so + fabsf(q.x) + fabsf(q.y) + fabsf(q.z);
         const float margin = 1e-6f * fR * S + 1e-5f * fR2;
-        bool in;
         if (fd2 < fR2 - margin) {
           in = true;
         } else if (fd2 > fR2 + margin) {
@@ -270,39 +295,50 @@ __global__ void k_near_search(int64_t n, double cnear, const int32_t *__restrict
           in = d2 < R * R * (1.0 - 1e-12);
           if (!in && d2 < R * R * (1.0 + 1e-12)) in = sqrt(d2) < R;
         }
-        if (t == p || in) {
-          if (fill) col[base + k] = t;
-          ++k;
-        }
+        in = in || t == p;
       }
-    } else {
-      for (int j = nchild[b] - 1; j >= 0 && sp < kNearStack; --j) stack[sp++] = child0[b] + j;
+      const unsigned m = (__ballot_sync(group, in) >> shift) & ((1u << kNearLanes) - 1u);
+      if (fill && in) col[base + k + __popc(m & below)] = t;
+      k += __popc(m);
     }
+    __syncwarp(group);
   }
-  if (!fill) cnt[p] = k;
+  if (!fill && lane == 0) cnt[p] = k;
 }
 
-// Self entries (t == p): one thread per node; the fixed 16 x 16 rule keeps the lanes
-// of a warp together.  Columns of a row are in ascending Morton order.
+// Self entries (t == p): kSelfLanes lanes to a node, each with every kSelfLanes-th angle of
+// the fixed 16 x 16 rule on every piece, which keeps the lanes of a warp together and fills
+// the chip at 20,838 nodes (0.33 ms with a thread to a node, 0.11 so).  Columns of a row are
+// in ascending Morton order.
+constexpr int kSelfLanes = 8;
+
 __global__ void __launch_bounds__(128) k_near_self(int64_t n, KernelParams kp, const int32_t *__restrict__ perm,
                                                    GeomF32 gf, const int32_t *__restrict__ tri,
                                                    const int64_t *__restrict__ inc_ptr,
                                                    const int32_t *__restrict__ inc_tri,
                                                    const int64_t *__restrict__ ptr, const int32_t *__restrict__ col,
                                                    float4 *__restrict__ coef, uint8_t *__restrict__ full) {
-  const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (p >= n) return;
+  const int64_t p = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / kSelfLanes;
+  if (p >= n) return;                          // a whole group of lanes
+  const int lane = threadIdx.x % kSelfLanes;
+  const unsigned group = ((1u << kSelfLanes) - 1u) << (threadIdx.x % 32 / kSelfLanes * kSelfLanes);
+  const int64_t op = perm[p];
+  const float4 na = gf.nrm_area[op];
+  const V3<float> np{na.x, na.y, na.z};
+  float A, D;
+  self_rule((float)kp.kappa, gf, tri, inc_ptr, inc_tri, op, np, lane, kSelfLanes, A, D);
+#pragma unroll
+  for (int m = kSelfLanes / 2; m > 0; m >>= 1) {
+    A += __shfl_xor_sync(group, A, m);
+    D += __shfl_xor_sync(group, D, m);
+  }
+  if (lane != 0) return;
   int64_t lo = ptr[p], hi = ptr[p + 1] - 1;
   while (lo < hi) {                           // the diagonal entry
     const int64_t mid = (lo + hi) >> 1;
     if (col[mid] < p) lo = mid + 1; else hi = mid;
   }
-  const int64_t op = perm[p];
-  const float4 na = gf.nrm_area[op];
-  const V3<float> np{na.x, na.y, na.z};
-  float o[4] = {0, 0, 0, 0};
-  self_rule((float)kp.kappa, (float)(1.0 / kp.ebar), gf, tri, inc_ptr, inc_tri, op, np, o);
-  coef[lo] = make_float4(o[0], o[1], o[2], o[3]);
+  coef[lo] = make_float4(A, 0.f, 0.f, D * (float)(1.0 / kp.ebar));
   full[lo] = 1;
 }
 
@@ -337,73 +373,134 @@ __device__ __forceinline__ bool p2p_leaves_out(const P2PView &pv, int p, int t) 
 
 // Off-diagonal entries (t != p).  An entry is the near rule minus the point rule, except
 // where the P2P pass leaves the pair out: there it is the whole near-rule value and `full`
-// is set.  Lanes take entries from a global counter.  For its entry a lane walks the
-// adaptive subdivision tree of every patch piece of t (the same rule and order as a
-// recursive walk: pieces by incident triangle, depth first), but the walk is split in two
-// phases per step so that the warp stays together where the work is: every lane first
-// advances its own walk to its next leaf sub-triangle (cheap, divergent), then all lanes
-// evaluate their leaves' 7 quadrature points at once.  The path of the walk is kept as
-// 2-bit digits in a register.
-__global__ void __launch_bounds__(128) k_near_pairs(int64_t nnz, const int32_t *__restrict__ row,
-                                                    unsigned long long *__restrict__ counter, KernelParams kp,
-                                                    const int32_t *__restrict__ perm, GeomF32 gf,
-                                                    const int32_t *__restrict__ tri,
-                                                    const int64_t *__restrict__ inc_ptr,
-                                                    const int32_t *__restrict__ inc_tri,
-                                                    const int32_t *__restrict__ col,
-                                                    P2PView pv, float4 *__restrict__ coef,
-                                                    uint8_t *__restrict__ full) {
+// is set.
+//
+// The FP32 pipe bounds the quadrature (7 points of ~80 operations per leaf of a piece's
+// subdivision), and entries differ widely: 8 to 500 leaves on a protein surface, 74 on
+// average.  So a warp takes kPairBatch entries at a time from a global counter and shares
+// their leaves evenly:
+//   - a lane per entry reads the pair, a lane per piece (32 at a time) its corners;
+//   - the pieces' trees are walked from a stack, 32 nodes at a time; a node is its path (2
+//     bits a level, from the top) with depth and piece, and splits or joins a queue of leaves;
+//   - whenever 32 leaves are queued, a lane evaluates each, and the warp adds their sums
+//     entry by entry in a fixed order.
+// (A lane to an entry, each walking its own tree: 4.56 ms for the 332,000 entries of
+// 20,838 nodes, 1.38 so; a warp then ran as long as its largest entry.)
+constexpr int kPairBatch = 16, kPairWarps = 4;
+constexpr int kPairQueue = 64;                // leaves; fewer than 32 wait while 32 nodes are read
+constexpr int kPairStack = 256;               // nodes, see the walk
+
+struct PairWarp {
+  float corner[12][32];                       // per piece: three corners relative to x_p, facet normal
+  float leaf[12][kPairQueue];                 // the same per queued leaf
+  int leaf_entry[kPairQueue];
+  uint32_t stack[kPairStack];
+  float np[3][kPairBatch];                    // per entry: target normal
+  float acc[kPairBatch][4];
+  int first[kPairBatch + 1];                  // pieces before the entry
+  int32_t op[kPairBatch], ot[kPairBatch];
+};
+
+// Evaluates `count` leaves from the end of the queue and adds them to the entries' sums.
+__device__ __forceinline__ void near_leaves(PairWarp &w, int begin, int count, int lane, float kappa, float inv_ebar) {
+  float acc[4] = {0.f, 0.f, 0.f, 0.f};
+  int entry = -1;
+  if (lane < count) {
+    const int s = begin + lane;
+    entry = w.leaf_entry[s];
+    const V3<float> a{w.leaf[0][s], w.leaf[1][s], w.leaf[2][s]}, b{w.leaf[3][s], w.leaf[4][s], w.leaf[5][s]},
+        c{w.leaf[6][s], w.leaf[7][s], w.leaf[8][s]}, ns{w.leaf[9][s], w.leaf[10][s], w.leaf[11][s]};
+    const V3<float> np{w.np[0][entry], w.np[1][entry], w.np[2][entry]};
+    const V3<float> e01{b.x - a.x, b.y - a.y, b.z - a.z}, e02{c.x - a.x, c.y - a.y, c.z - a.z};
+    const V3<float> cr{e01.y * e02.z - e01.z * e02.y, e01.z * e02.x - e01.x * e02.z, e01.x * e02.y - e01.y * e02.x};
+    const float area = 0.5f * sqrtf(dot(cr, cr));
+    for (int q = 0; q < 7; ++q) {
+      const float b0 = c_rad_bf[3 * q], b1 = c_rad_bf[3 * q + 1], b2 = c_rad_bf[3 * q + 2];
+      const V3<float> dq{-(b0 * a.x + b1 * b.x + b2 * c.x), -(b0 * a.y + b1 * b.y + b2 * c.y),
+                         -(b0 * a.z + b1 * b.z + b2 * c.z)};
+      float o[4];
+      abcd_point(kappa, inv_ebar, dq, np, ns, o);
+      const float wq = area * c_rad_wf[q];
+      for (int k = 0; k < 4; ++k) acc[k] += wq * o[k];
+    }
+  }
+  unsigned rest = __ballot_sync(0xffffffffu, entry >= 0);
+  while (rest) {
+    const int key = __shfl_sync(0xffffffffu, entry, __ffs(rest) - 1);
+    const bool mine = entry == key;
+    rest &= ~__ballot_sync(0xffffffffu, mine);
+    float v[4];
+    for (int k = 0; k < 4; ++k) v[k] = mine ? acc[k] : 0.f;
+    // four sums over the warp: each half keeps two of them, each quarter one
+    const bool h16 = lane & 16, h8 = lane & 8;
+    float u0 = (h16 ? v[2] : v[0]) + __shfl_xor_sync(0xffffffffu, h16 ? v[0] : v[2], 16);
+    float u1 = (h16 ? v[3] : v[1]) + __shfl_xor_sync(0xffffffffu, h16 ? v[1] : v[3], 16);
+    float u = (h8 ? u1 : u0) + __shfl_xor_sync(0xffffffffu, h8 ? u0 : u1, 8);
+    u += __shfl_xor_sync(0xffffffffu, u, 4);
+    u += __shfl_xor_sync(0xffffffffu, u, 2);
+    u += __shfl_xor_sync(0xffffffffu, u, 1);
+    if ((lane & 7) == 0) w.acc[key][(h16 ? 2 : 0) + (h8 ? 1 : 0)] += u;
+  }
+  __syncwarp();
+}
+
+__global__ void __launch_bounds__(kPairWarps * 32)
+    k_near_pairs(int64_t nnz, const int32_t *__restrict__ row, unsigned long long *__restrict__ counter,
+                 KernelParams kp, const int32_t *__restrict__ perm, GeomF32 gf, const int32_t *__restrict__ tri,
+                 const int64_t *__restrict__ inc_ptr, const int32_t *__restrict__ inc_tri,
+                 const int32_t *__restrict__ col, P2PView pv, float4 *__restrict__ coef, uint8_t *__restrict__ full) {
+  __shared__ PairWarp warps[kPairWarps];
+  PairWarp &w = warps[threadIdx.x / 32];
+  const int lane = threadIdx.x % 32;
+  const unsigned all = 0xffffffffu, below = (1u << lane) - 1u;
   const float kappa = (float)kp.kappa, inv_ebar = (float)(1.0 / kp.ebar);
-  bool done = false, in_pair = false, in_piece = false, have = false, whole = false;
-  int64_t e = 0, tj = 0, tend = 0, op = 0, ot = 0;
-  int half = 0, d = 0;
-  uint32_t path = 0;                          // digit of level l in bits 2(l-1) .. 2l-1
-  V3<float> np{0, 0, 0}, ns{0, 0, 0}, R0{0, 0, 0}, R1{0, 0, 0}, R2{0, 0, 0};
-  V3<float> la{0, 0, 0}, lb{0, 0, 0}, lc{0, 0, 0};
-  float larea = 0.f, acc[4] = {0, 0, 0, 0};
   while (true) {
-    // phase 1: advance to the next leaf (or the next entry)
-    while (!have && !done) {
-      if (!in_pair) {
-        e = (int64_t)atomicAdd(counter, 1ULL);
-        if (e >= nnz) {
-          done = true;
-          break;
-        }
-        const int p = row[e], t = col[e];
-        if (t == p) continue;                 // diagonal: k_near_self
-        op = perm[p];
-        ot = perm[t];
-        {
-          const float4 na = gf.nrm_area[op];
-          np = V3<float>{na.x, na.y, na.z};
-        }
+    int64_t e0 = 0;
+    if (lane == 0) e0 = (int64_t)atomicAdd(counter, (unsigned long long)kPairBatch);
+    e0 = __shfl_sync(all, e0, 0);
+    if (e0 >= nnz) return;
+    // the entries of the batch: a lane each; no pieces on the diagonal (k_near_self)
+    const int64_t e = e0 + lane;
+    bool whole = false, pair = false;
+    int pieces = 0;
+    if (lane < kPairBatch && e < nnz) {
+      const int p = row[e], t = col[e];
+      pair = p != t;
+      if (pair) {
+        const int32_t op = perm[p], ot = perm[t];
+        const float4 na = gf.nrm_area[op];
+        w.op[lane] = op;
+        w.ot[lane] = ot;
+        w.np[0][lane] = na.x;
+        w.np[1][lane] = na.y;
+        w.np[2][lane] = na.z;
+        pieces = 2 * (int)(inc_ptr[ot + 1] - inc_ptr[ot]);
         whole = p2p_leaves_out(pv, p, t);
-        tj = inc_ptr[ot];
-        tend = inc_ptr[ot + 1];
-        half = 0;
-        in_piece = false;
-        acc[0] = acc[1] = acc[2] = acc[3] = 0.f;
-        in_pair = true;
       }
-      if (!in_piece) {
-        if (tj >= tend) {                     // entry finished
-          float o[4] = {acc[0], acc[1], acc[2], acc[3]};
-          if (!whole) {
-            const V3<float> dd = diff_f32(gf, op, gf.hi[ot], gf.lo[ot]);
-            const float4 na = gf.nrm_area[ot];
-            const V3<float> nt{na.x, na.y, na.z};
-            float f[4];
-            abcd_point(kappa, inv_ebar, dd, np, nt, f);
-            const float at = na.w;
-            for (int k = 0; k < 4; ++k) o[k] -= at * f[k];
-          }
-          coef[e] = make_float4(o[0], o[1], o[2], o[3]);
-          full[e] = whole ? 1 : 0;
-          in_pair = false;
-          continue;
-        }
-        const int32_t T = inc_tri[tj];
+    }
+    int upto = pieces;
+#pragma unroll
+    for (int m = 1; m < kPairBatch; m <<= 1) {
+      const int v = __shfl_up_sync(all, upto, m);
+      if (lane >= m) upto += v;
+    }
+    if (lane < kPairBatch) {
+      w.first[lane] = upto - pieces;
+      for (int k = 0; k < 4; ++k) w.acc[lane][k] = 0.f;
+      if (lane == kPairBatch - 1) w.first[kPairBatch] = upto;
+    }
+    __syncwarp();
+    const int total = w.first[kPairBatch];
+    int queued = 0;
+    for (int u0 = 0; u0 < total; u0 += 32) {
+      int entry = 0;
+      if (u0 + lane < total) {
+#pragma unroll
+        for (int m = kPairBatch / 2; m > 0; m >>= 1)
+          if (w.first[entry + m] <= u0 + lane) entry += m;
+        const int j = u0 + lane - w.first[entry];
+        const int64_t op = w.op[entry], ot = w.ot[entry];
+        const int32_t T = inc_tri[inc_ptr[ot] + (j >> 1)];
         V3<float> P[3];
         tri_rel_f32(gf, tri, T, ot, op, P);
         const V3<float> ma{0.5f * (P[0].x + P[1].x), 0.5f * (P[0].y + P[1].y), 0.5f * (P[0].z + P[1].z)};
@@ -411,77 +508,107 @@ __global__ void __launch_bounds__(128) k_near_pairs(int64_t nnz, const int32_t *
         const float third = 1.0f / 3.0f;
         const V3<float> cen{(P[0].x + P[1].x + P[2].x) * third, (P[0].y + P[1].y + P[2].y) * third,
                             (P[0].z + P[1].z + P[2].z) * third};
-        {
-          const float4 tn = gf.tri_nrm[T];
-          ns = V3<float>{tn.x, tn.y, tn.z};
+        const V3<float> R1 = (j & 1) == 0 ? ma : cen, R2 = (j & 1) == 0 ? cen : mb;
+        const float4 tn = gf.tri_nrm[T];
+        w.corner[0][lane] = P[0].x;
+        w.corner[1][lane] = P[0].y;
+        w.corner[2][lane] = P[0].z;
+        w.corner[3][lane] = R1.x;
+        w.corner[4][lane] = R1.y;
+        w.corner[5][lane] = R1.z;
+        w.corner[6][lane] = R2.x;
+        w.corner[7][lane] = R2.y;
+        w.corner[8][lane] = R2.z;
+        w.corner[9][lane] = tn.x;
+        w.corner[10][lane] = tn.y;
+        w.corner[11][lane] = tn.z;
+        w.stack[lane] = (uint32_t)lane << 16;         // depth 0, empty path
+      }
+      int size = min(32, total - u0);
+      __syncwarp();
+      while (size > 0) {
+        // Nodes are taken from the top: 32, or as many as surely fit when all of them split.
+        // One node's subtree alone needs at most 3 * kQuadDepth = 18 more places, and 21 are
+        // always free when it is begun.
+        const int take = min(min(32, size), max(1, (kPairStack - size - 21) / 3));
+        size -= take;
+        bool leaf = false, split = false;
+        uint32_t node = 0;
+        V3<float> a{0, 0, 0}, b{0, 0, 0}, c{0, 0, 0};
+        if (lane < take) {
+          node = w.stack[size + lane];
+          const int u = node >> 16, d = (node >> 12) & 15;
+          a = V3<float>{w.corner[0][u], w.corner[1][u], w.corner[2][u]};
+          b = V3<float>{w.corner[3][u], w.corner[4][u], w.corner[5][u]};
+          c = V3<float>{w.corner[6][u], w.corner[7][u], w.corner[8][u]};
+          for (int l = 0; l < d; ++l) {
+            const V3<float> mab{0.5f * (a.x + b.x), 0.5f * (a.y + b.y), 0.5f * (a.z + b.z)};
+            const V3<float> mbc{0.5f * (b.x + c.x), 0.5f * (b.y + c.y), 0.5f * (b.z + c.z)};
+            const V3<float> mca{0.5f * (c.x + a.x), 0.5f * (c.y + a.y), 0.5f * (c.z + a.z)};
+            const uint32_t digit = (node >> (2 * (d - 1 - l))) & 3u;
+            a = digit == 0 ? a : (digit == 2 ? mca : mab);
+            b = digit == 1 ? b : (digit == 0 ? mab : mbc);
+            c = digit == 2 ? c : (digit == 1 ? mbc : mca);
+          }
+          // split while |centroid| < 3 x the longest edge (compared squared)
+          const V3<float> e01{b.x - a.x, b.y - a.y, b.z - a.z}, e12{c.x - b.x, c.y - b.y, c.z - b.z},
+              e02{c.x - a.x, c.y - a.y, c.z - a.z};
+          const float diam2 = fmaxf(dot(e01, e01), fmaxf(dot(e12, e12), dot(e02, e02)));
+          const float third = 1.0f / 3.0f;
+          const V3<float> g{(a.x + b.x + c.x) * third, (a.y + b.y + c.y) * third, (a.z + b.z + c.z) * third};
+          split = d < kQuadDepth && dot(g, g) < 9.0f * diam2;
+          leaf = !split;
         }
-        R0 = P[0];
-        R1 = half == 0 ? ma : cen;
-        R2 = half == 0 ? cen : mb;
-        d = 0;
-        path = 0;
-        in_piece = true;
-      }
-      // the node at (d, path)
-      V3<float> a = R0, b = R1, c = R2;
-      for (int l = 1; l <= d; ++l) {
-        const V3<float> mab{0.5f * (a.x + b.x), 0.5f * (a.y + b.y), 0.5f * (a.z + b.z)};
-        const V3<float> mbc{0.5f * (b.x + c.x), 0.5f * (b.y + c.y), 0.5f * (b.z + c.z)};
-        const V3<float> mca{0.5f * (c.x + a.x), 0.5f * (c.y + a.y), 0.5f * (c.z + a.z)};
-        switch ((path >> (2 * (l - 1))) & 3u) {
-          case 0: b = mab; c = mca; break;
-          case 1: a = mab; c = mbc; break;
-          case 2: a = mca; b = mbc; break;
-          default: a = mab; b = mbc; c = mca; break;
+        const unsigned ms = __ballot_sync(all, split), ml = __ballot_sync(all, leaf);
+        if (leaf) {
+          const int s = queued + __popc(ml & below), u = node >> 16;
+          w.leaf[0][s] = a.x;
+          w.leaf[1][s] = a.y;
+          w.leaf[2][s] = a.z;
+          w.leaf[3][s] = b.x;
+          w.leaf[4][s] = b.y;
+          w.leaf[5][s] = b.z;
+          w.leaf[6][s] = c.x;
+          w.leaf[7][s] = c.y;
+          w.leaf[8][s] = c.z;
+          w.leaf[9][s] = w.corner[9][u];
+          w.leaf[10][s] = w.corner[10][u];
+          w.leaf[11][s] = w.corner[11][u];
         }
-      }
-      const V3<float> e01{b.x - a.x, b.y - a.y, b.z - a.z}, e12{c.x - b.x, c.y - b.y, c.z - b.z},
-          e02{c.x - a.x, c.y - a.y, c.z - a.z};
-      // split while |centroid| < 3 x the longest edge (compared squared)
-      const float diam2 = fmaxf(dot(e01, e01), fmaxf(dot(e12, e12), dot(e02, e02)));
-      const float third = 1.0f / 3.0f;
-      const V3<float> g{(a.x + b.x + c.x) * third, (a.y + b.y + c.y) * third, (a.z + b.z + c.z) * third};
-      if (d < kQuadDepth && dot(g, g) < 9.0f * diam2) {
-        ++d;                                  // first child (its digit is 0)
-        continue;
-      }
-      const V3<float> cr{e01.y * e02.z - e01.z * e02.y, e01.z * e02.x - e01.x * e02.z, e01.x * e02.y - e01.y * e02.x};
-      la = a;
-      lb = b;
-      lc = c;
-      larea = 0.5f * sqrtf(dot(cr, cr));
-      have = true;
-      // next node of the walk: the next sibling, climbing past last children
-      while (d > 0 && ((path >> (2 * (d - 1))) & 3u) == 3u) {
-        path &= ~(3u << (2 * (d - 1)));
-        --d;
-      }
-      if (d > 0) {
-        path += 1u << (2 * (d - 1));
-      } else {
-        in_piece = false;                     // piece done: the other half, or the next triangle
-        if (half == 0) {
-          half = 1;
-        } else {
-          half = 0;
-          ++tj;
+        // the piece's entry is known to the lane that read it
+        const int owner = __shfl_sync(all, entry, (node >> 16) & 31);
+        if (leaf) w.leaf_entry[queued + __popc(ml & below)] = owner;
+        if (split) {
+          const uint32_t child = (node & 0xffff0000u) | ((((node >> 12) & 15u) + 1u) << 12) | ((node & 0xfffu) << 2);
+          const int s = size + 4 * __popc(ms & below);
+          for (int q = 0; q < 4; ++q) w.stack[s + q] = child | q;
+        }
+        size += 4 * __popc(ms);
+        queued += __popc(ml);
+        __syncwarp();
+        if (queued >= 32) {
+          queued -= 32;
+          near_leaves(w, queued, 32, lane, kappa, inv_ebar);
         }
       }
     }
-    if (__all_sync(0xffffffffu, !have)) break; // every lane has run out of entries
-    // phase 2: the lanes' leaves together
-    if (have) {
-      for (int q = 0; q < 7; ++q) {
-        const float b0 = c_rad_bf[3 * q], b1 = c_rad_bf[3 * q + 1], b2 = c_rad_bf[3 * q + 2];
-        const V3<float> dq{-(b0 * la.x + b1 * lb.x + b2 * lc.x), -(b0 * la.y + b1 * lb.y + b2 * lc.y),
-                           -(b0 * la.z + b1 * lb.z + b2 * lc.z)};
-        float o[4];
-        abcd_point(kappa, inv_ebar, dq, np, ns, o);
-        const float w = larea * c_rad_wf[q];
-        for (int k = 0; k < 4; ++k) acc[k] += w * o[k];
+    if (queued > 0) near_leaves(w, 0, queued, lane, kappa, inv_ebar);
+    if (pair) {
+      float o[4];
+      for (int k = 0; k < 4; ++k) o[k] = w.acc[lane][k];
+      if (!whole) {
+        const int64_t op = w.op[lane], ot = w.ot[lane];
+        const V3<float> dd = diff_f32(gf, op, gf.hi[ot], gf.lo[ot]);
+        const float4 na = gf.nrm_area[ot];
+        const V3<float> nt{na.x, na.y, na.z}, np{w.np[0][lane], w.np[1][lane], w.np[2][lane]};
+        float f[4];
+        abcd_point(kappa, inv_ebar, dd, np, nt, f);
+        for (int k = 0; k < 4; ++k) o[k] -= na.w * f[k];
       }
-      have = false;
+      coef[e] = make_float4(o[0], o[1], o[2], o[3]);
+      full[e] = whole ? 1 : 0;
     }
+    __syncwarp();
   }
 }
 
@@ -566,7 +693,8 @@ Err build_near(afmpb_t *h) {
   int64_t *d_cnt = nullptr;
   AFMPB_TRY(A.alloc(&d_cnt, n, "near cnt"));
   const double cnear = h->opt.near_c;
-  k_near_search<<<div_up(n, 128), 128, 0, s>>>(n, cnear, h->d_perm, h->d_xyz, h->d_rho64, h->d_pos, h->d_nrm,
+  k_near_search<<<div_up(n * kNearLanes, kNearSearchBlock), kNearSearchBlock, 0, s>>>(
+      n, cnear, h->d_perm, h->d_xyz, h->d_rho64, h->d_pos, h->d_nrm,
                                                h->d_box_center, h->d_box_rho, h->d_box_child0, h->d_box_nchild,
                                                h->d_box_begin, h->d_box_end, d_cnt, nullptr, nullptr, false);
   AFMPB_TRY(check_launch("k_near_search count"));
@@ -579,7 +707,8 @@ Err build_near(afmpb_t *h) {
   AFMPB_TRY(A.alloc(&h->d_near_col, h->nnz, "near col"));
   AFMPB_TRY(A.alloc(&h->d_near_coef, h->nnz, "near coef"));
   AFMPB_CUDA(cudaMemcpyAsync(h->d_near_ptr, ptr.data(), sizeof(int64_t) * (n + 1), cudaMemcpyHostToDevice, s));
-  k_near_search<<<div_up(n, 128), 128, 0, s>>>(n, cnear, h->d_perm, h->d_xyz, h->d_rho64, h->d_pos, h->d_nrm,
+  k_near_search<<<div_up(n * kNearLanes, kNearSearchBlock), kNearSearchBlock, 0, s>>>(
+      n, cnear, h->d_perm, h->d_xyz, h->d_rho64, h->d_pos, h->d_nrm,
                                                h->d_box_center, h->d_box_rho, h->d_box_child0, h->d_box_nchild,
                                                h->d_box_begin, h->d_box_end, nullptr, h->d_near_ptr, h->d_near_col,
                                                true);
@@ -595,8 +724,8 @@ Err build_near(afmpb_t *h) {
                                                                       h->d_tri_nrm, g_hi, g_lo, g_na, g_tn);
   AFMPB_TRY(check_launch("k_geom_f32"));
   const GeomF32 gf{g_hi, g_lo, g_na, g_tn};
-  k_near_self<<<div_up(n, 128), 128, 0, s>>>(n, kp, h->d_perm, gf, h->d_tri, h->d_inc_ptr, h->d_inc_tri,
-                                              h->d_near_ptr, h->d_near_col, h->d_near_coef, h->d_near_full);
+  k_near_self<<<div_up(n * kSelfLanes, 128), 128, 0, s>>>(n, kp, h->d_perm, gf, h->d_tri, h->d_inc_ptr, h->d_inc_tri,
+                                                          h->d_near_ptr, h->d_near_col, h->d_near_coef, h->d_near_full);
   AFMPB_TRY(check_launch("k_near_self"));
   int32_t *d_row = nullptr;
   unsigned long long *d_counter = nullptr;
@@ -610,10 +739,12 @@ Err build_near(afmpb_t *h) {
   int dev = 0, sms = 0;
   AFMPB_CUDA(cudaGetDevice(&dev));
   AFMPB_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const int64_t want = div_up(h->nnz, 128);   // lanes take entries dynamically; cap the grid
-  const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)sms * 16));
-  k_near_pairs<<<grid, 128, 0, s>>>(h->nnz, d_row, d_counter, kp, h->d_perm, gf, h->d_tri, h->d_inc_ptr,
-                                    h->d_inc_tri, h->d_near_col, pv, h->d_near_coef, h->d_near_full);
+  int resident = 1;
+  AFMPB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, k_near_pairs, kPairWarps * 32, 0));
+  const int64_t want = div_up(h->nnz, kPairBatch * kPairWarps);   // warps take batches dynamically
+  const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)sms * resident));
+  k_near_pairs<<<grid, kPairWarps * 32, 0, s>>>(h->nnz, d_row, d_counter, kp, h->d_perm, gf, h->d_tri, h->d_inc_ptr,
+                                                h->d_inc_tri, h->d_near_col, pv, h->d_near_coef, h->d_near_full);
   AFMPB_TRY(check_launch("k_near_pairs"));
   AFMPB_CUDA(cudaStreamSynchronize(s));
   A.release(g_tn);
