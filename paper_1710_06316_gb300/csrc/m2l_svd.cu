@@ -29,10 +29,9 @@ namespace afmpb {
 namespace {
 
 constexpr int kGramTile = 32;       // Gram matrix tile (32 x 32 per CTA)
-constexpr int kRowsPerCta = 8;      // rows of T = K_o Q (and of C) per CTA
+constexpr int kGramTables = 4;      // tables per launch of the Gram kernels
 constexpr int kChunkBoxes = 16;     // boxes per compress / expand CTA (a multiple of 4; 16 against 32:
                                     // expand 32 -> 27 us on the 163,842-node sphere)
-constexpr int kMaxN3 = kMaxOrder * kMaxOrder * kMaxOrder;
 constexpr int kMaxRank = 192;       // largest compressed size (M2L staging in shared memory)
 
 struct NodesD {
@@ -52,9 +51,15 @@ __device__ __forceinline__ double m2l_entry(const NodesD &nd, int N, int3 o, int
   return v;
 }
 
-__global__ void k_table_f64(int N, int noffs, const int3 *__restrict__ offs, NodesD nd, double kw, double invw,
+struct TableScale {                 // per table: kappa w (negative: Laplace) and 1 / w
+  double kw[kGramTables], invw[kGramTables];
+};
+
+__global__ void k_table_f64(int N, int noffs, const int3 *__restrict__ offs, NodesD nd, TableScale ts,
                             double *__restrict__ K) {
   const int N3 = N * N * N;
+  const double kw = ts.kw[blockIdx.y], invw = ts.invw[blockIdx.y];
+  K += (size_t)blockIdx.y * noffs * N3 * N3;
   const int64_t tot = (int64_t)noffs * N3 * N3;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < tot; e += (int64_t)gridDim.x * blockDim.x) {
     const int o = (int)(e / ((int64_t)N3 * N3));
@@ -63,30 +68,14 @@ __global__ void k_table_f64(int N, int noffs, const int3 *__restrict__ offs, Nod
   }
 }
 
-// The same table in FP32 (for C_o = Q^T K_o Q, which the products use in FP32 and BF16).
-__global__ void k_table_f32(int N, int noffs, const int3 *__restrict__ offs, NodesD nd, double kw, double invw,
-                            float *__restrict__ K) {
-  const int N3 = N * N * N;
-  const int64_t tot = (int64_t)noffs * N3 * N3;
-  const float fkw = (float)kw, finvw = (float)invw, c = (float)kInv4Pi;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < tot; e += (int64_t)gridDim.x * blockDim.x) {
-    const int o = (int)(e / ((int64_t)N3 * N3));
-    const int rem = (int)(e % ((int64_t)N3 * N3));
-    const int i = rem / N3, k = rem % N3;
-    const int3 of = offs[o];
-    const float dx = (float)(nd.x[i / (N * N)] - 2.0 * of.x - nd.x[k / (N * N)]);
-    const float dy = (float)(nd.x[(i / N) % N] - 2.0 * of.y - nd.x[(k / N) % N]);
-    const float dz = (float)(nd.x[i % N] - 2.0 * of.z - nd.x[k % N]);
-    const float r = sqrtf(dx * dx + dy * dy + dz * dz);
-    float v = c / r;
-    if (fkw >= 0.0f) v = expf(-fkw * r) * v * finvw;
-    K[e] = v;
-  }
-}
-
-// H_r = K_r K_r^T for one offset per orbit of the cube's symmetry group (blockIdx.z = r).
+// H_r = K_r K_r^T for one offset r per orbit of the cube's symmetry group (blockIdx.z: table
+// and r).
+// The FP64 pipe bounds it, so only the tiles on and above the diagonal are formed, and
+// mirrored (entry (j, i) has the same products in the same order): 0.34 -> 0.17 ms a table
+// of order 6, four tables a launch.
 __global__ void __launch_bounds__(256) k_gram_rep(int N3, const double *__restrict__ K, double *__restrict__ H) {
   __shared__ double Ki[kGramTile][kGramTile + 1], Kj[kGramTile][kGramTile + 1];
+  if (blockIdx.y < blockIdx.x) return;
   const int i0 = blockIdx.x * kGramTile, j0 = blockIdx.y * kGramTile;
   const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
   double acc[2][2] = {{0, 0}, {0, 0}};
@@ -112,72 +101,139 @@ __global__ void __launch_bounds__(256) k_gram_rep(int N3, const double *__restri
   for (int a = 0; a < 2; ++a)
     for (int b = 0; b < 2; ++b) {
       const int i = i0 + ty + 16 * a, j = j0 + tx + 16 * b;
-      if (i < N3 && j < N3) Hr[(size_t)i * N3 + j] = acc[a][b];
+      if (i < N3 && j < N3) {
+        Hr[(size_t)i * N3 + j] = acc[a][b];
+        if (j0 > i0) Hr[(size_t)j * N3 + i] = acc[a][b];
+      }
     }
 }
 
 // Gram = sum over all offsets of K_o K_o^T, from the orbit representatives: an offset g.o
 // of the orbit of r has K_{g.o} = P_g K_r P_g^T (the kernel depends on |x - y| only and the
 // Chebyshev grid is symmetric), so the orbit contributes (|orbit| / 48) sum_g P_g H_r P_g^T,
-// entry (i, j) of which is H_r(perm_g(i), perm_g(j)) summed over the 48 elements g.
+// entry (i, j) of which is H_r(perm_g(i), perm_g(j)) summed over the 48 elements g.  Formed
+// for i <= j and mirrored, as the H_r are.
+// A thread sums the 48 terms of an entry for one r (threadIdx.y), and the first row of
+// threads adds these in order (one thread for all r: 0.12 ms a table, waiting for its loads;
+// 0.045 so, four tables a launch).
+constexpr int kSymCols = 32;
+
 __global__ void k_gram_sym(int N3, int nrep, const double *__restrict__ H, const double *__restrict__ wrep,
                            const int32_t *__restrict__ perm, double *__restrict__ gram) {
-  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (e >= (int64_t)N3 * N3) return;
-  const int i = (int)(e / N3), j = (int)(e % N3);
-  double sum = 0.0;
-  for (int r = 0; r < nrep; ++r) {
-    const double *Hr = H + (size_t)r * N3 * N3;
+  extern __shared__ double part[];             // [nrep][kSymCols]
+  const int i = blockIdx.y, j = blockIdx.x * kSymCols + threadIdx.x;
+  if ((blockIdx.x + 1) * kSymCols <= i) return;
+  const size_t NN = (size_t)N3 * N3;
+  if (j >= i && j < N3) {
+    const double *Hr = H + ((size_t)blockIdx.z * nrep + threadIdx.y) * NN;
     double t = 0.0;
+#pragma unroll 8
     for (int g = 0; g < 48; ++g) t += Hr[(size_t)perm[g * N3 + i] * N3 + perm[g * N3 + j]];
-    sum += wrep[r] * t;
-  }
-  gram[e] = sum;
-}
-
-// T[o][i][b] = sum_k K_o(i, k) Q(k, b)        (Q: [N3][R]; FP32: the operators C_o are used
-// in FP32 and BF16 by the products, while the basis Q itself comes from the FP64 Gram matrix)
-__global__ void __launch_bounds__(128) k_kq(int N3, int R, const float *__restrict__ K, const float *__restrict__ Q,
-                                            float *__restrict__ T) {
-  __shared__ float Ks[kRowsPerCta][kMaxN3];
-  const int o = blockIdx.x, i0 = blockIdx.y * kRowsPerCta;
-  const int rows = min(kRowsPerCta, N3 - i0);
-  for (int e = threadIdx.x; e < kRowsPerCta * N3; e += blockDim.x) {
-    const int r = e / N3, k = e % N3;
-    Ks[r][k] = r < rows ? K[((size_t)o * N3 + i0 + r) * N3 + k] : 0.0f;
+    part[threadIdx.y * kSymCols + threadIdx.x] = t;
   }
   __syncthreads();
-  for (int b = threadIdx.x; b < R; b += blockDim.x) {
-    float acc[kRowsPerCta] = {};
-    for (int k = 0; k < N3; ++k) {
-      const float q = Q[(size_t)k * R + b];
+  if (threadIdx.y != 0 || j < i || j >= N3) return;
+  double sum = 0.0;
+  for (int r = 0; r < nrep; ++r) sum += wrep[r] * part[r * kSymCols + threadIdx.x];
+  gram += blockIdx.z * NN;
+  gram[(size_t)i * N3 + j] = sum;
+  gram[(size_t)j * N3 + i] = sum;
+}
+
+// Operators in FP32 (the products use them in FP32 and BF16; the basis Q itself comes from
+// the FP64 Gram matrix).  T[o][i][b] = sum_k K_o(i, k) Q(k, b), Q: [N3][R].  A CTA takes
+// kOpRows rows i of one offset and up to 64 columns b; it forms the rows of K_o itself, from
+// the N x N coordinate differences of each axis, and a thread sums 4 x 4 entries over k in
+// order.  (With K_o written out by a kernel of its own, FP64 differences for every entry and
+// half of the threads idle at R = 64, the two took 0.62 ms a table; 0.145 so.)
+constexpr int kOpRows = 32, kOpCols = 64, kOpSlab = 32;
+
+// four rows x four columns += A[., c] B[c, .] for the `cnt` rows c of a slab, in order
+__device__ __forceinline__ void op_tile(const float *a, int lda, const float *b, int ldb, int cnt, float2 (&acc)[4][2]) {
+#pragma unroll 4
+  for (int c = 0; c < cnt; ++c) {
+    const float4 x = *reinterpret_cast<const float4 *>(a + c * lda), y = *reinterpret_cast<const float4 *>(b + c * ldb);
+    const float xv[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
-      for (int r = 0; r < kRowsPerCta; ++r) acc[r] = fmaf(Ks[r][k], q, acc[r]);
+    for (int i = 0; i < 4; ++i) {
+      acc[i][0] = __ffma2_rn(make_float2(xv[i], xv[i]), make_float2(y.x, y.y), acc[i][0]);
+      acc[i][1] = __ffma2_rn(make_float2(xv[i], xv[i]), make_float2(y.z, y.w), acc[i][1]);
     }
-    for (int r = 0; r < rows; ++r) T[((size_t)o * N3 + i0 + r) * R + b] = acc[r];
   }
 }
 
-// C[o][a][b] = sum_i Q(i, a) T[o][i][b], stored FP32
-__global__ void __launch_bounds__(128) k_qtt(int N3, int R, const float *__restrict__ Q, const float *__restrict__ T,
+// rows [c0, c0 + cnt) x columns [b0, b0 + kOpCols) of a matrix with R columns, zero beyond
+__device__ __forceinline__ void op_slab(const float *__restrict__ src, int R, int c0, int cnt, int b0, float *dst) {
+  for (int e = threadIdx.x; e < kOpSlab * kOpCols; e += blockDim.x) {
+    const int c = e / kOpCols, b = e % kOpCols;
+    dst[e] = c < cnt && b0 + b < R ? src[(size_t)(c0 + c) * R + b0 + b] : 0.0f;
+  }
+}
+
+__global__ void __launch_bounds__(128) k_kq(int N, int R, const int3 *__restrict__ offs, NodesD nd, double kw, double invw,
+                                            const float *__restrict__ Q, float *__restrict__ T) {
+  extern __shared__ __align__(16) float osm[];
+  const int N3 = N * N * N;
+  float *Ks = osm;                                     // [N3][kOpRows]
+  float *Qs = osm + (size_t)N3 * kOpRows;              // [kOpSlab][kOpCols]
+  __shared__ float diff[3][kMaxOrder][kMaxOrder];      // coordinate differences by axis
+  const int i0 = blockIdx.y * kOpRows, b0 = blockIdx.z * kOpCols;
+  const int3 of = offs[blockIdx.x];
+  for (int e = threadIdx.x; e < 3 * N * N; e += blockDim.x) {
+    const int ax = e / (N * N), t = (e / N) % N, s = e % N;
+    const int oa = ax == 0 ? of.x : (ax == 1 ? of.y : of.z);
+    diff[ax][t][s] = (float)(nd.x[t] - 2.0 * oa - nd.x[s]);
+  }
+  __syncthreads();
+  const float fkw = (float)kw, finvw = (float)invw, c = (float)kInv4Pi;
+  for (int e = threadIdx.x; e < N3 * kOpRows; e += blockDim.x) {
+    const int k = e / kOpRows, i = i0 + e % kOpRows;
+    float v = 0.0f;
+    if (i < N3) {
+      const float dx = diff[0][i / (N * N)][k / (N * N)], dy = diff[1][(i / N) % N][(k / N) % N], dz = diff[2][i % N][k % N];
+      const float r = sqrtf(dx * dx + dy * dy + dz * dz);
+      v = c / r;
+      if (fkw >= 0.0f) v = expf(-fkw * r) * v * finvw;
+    }
+    Ks[e] = v;
+  }
+  const int r4 = (threadIdx.x / (kOpCols / 4)) * 4, c4 = (threadIdx.x % (kOpCols / 4)) * 4;
+  float2 acc[4][2] = {};
+  for (int k0 = 0; k0 < N3; k0 += kOpSlab) {
+    const int cnt = min(kOpSlab, N3 - k0);
+    __syncthreads();
+    op_slab(Q, R, k0, cnt, b0, Qs);
+    __syncthreads();
+    op_tile(Ks + (size_t)k0 * kOpRows + r4, kOpRows, Qs + c4, kOpCols, cnt, acc);
+  }
+  if (b0 + c4 < R)                                     // R is a multiple of 16
+    for (int i = 0; i < 4; ++i)
+      if (i0 + r4 + i < N3)
+        *reinterpret_cast<float4 *>(T + ((size_t)blockIdx.x * N3 + i0 + r4 + i) * R + b0 + c4) =
+            make_float4(acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y);
+}
+
+// C[o][a][b] = sum_i Q(i, a) T[o][i][b], 64 x 64 entries of one offset per CTA, 4 x 4 per thread
+__global__ void __launch_bounds__(256) k_qtt(int N3, int R, const float *__restrict__ Q, const float *__restrict__ T,
                                              float *__restrict__ C) {
-  __shared__ float Qs[kRowsPerCta][kMaxN3];
-  const int o = blockIdx.x, a0 = blockIdx.y * kRowsPerCta;
-  const int rows = min(kRowsPerCta, R - a0);
-  for (int e = threadIdx.x; e < kRowsPerCta * N3; e += blockDim.x) {
-    const int r = e / N3, i = e % N3;
-    Qs[r][i] = r < rows ? Q[(size_t)i * R + a0 + r] : 0.0f;
+  __shared__ __align__(16) float Qs[kOpSlab * kOpCols], Ts[kOpSlab * kOpCols];
+  const int a0 = blockIdx.y * kOpCols, b0 = blockIdx.z * kOpCols;
+  const float *To = T + (size_t)blockIdx.x * N3 * R;
+  const int r4 = (threadIdx.x / (kOpCols / 4)) * 4, c4 = (threadIdx.x % (kOpCols / 4)) * 4;
+  float2 acc[4][2] = {};
+  for (int k0 = 0; k0 < N3; k0 += kOpSlab) {
+    const int cnt = min(kOpSlab, N3 - k0);
+    __syncthreads();
+    op_slab(Q, R, k0, cnt, a0, Qs);
+    op_slab(To, R, k0, cnt, b0, Ts);
+    __syncthreads();
+    op_tile(Qs + r4, kOpCols, Ts + c4, kOpCols, cnt, acc);
   }
-  __syncthreads();
-  for (int b = threadIdx.x; b < R; b += blockDim.x) {
-    float acc[kRowsPerCta] = {};
-    for (int i = 0; i < N3; ++i) {
-      const float t = T[((size_t)o * N3 + i) * R + b];
-#pragma unroll
-      for (int r = 0; r < kRowsPerCta; ++r) acc[r] = fmaf(Qs[r][i], t, acc[r]);
-    }
-    for (int r = 0; r < rows; ++r) C[((size_t)o * R + a0 + r) * R + b] = acc[r];
-  }
+  if (b0 + c4 < R)
+    for (int i = 0; i < 4; ++i)
+      if (a0 + r4 + i < R)
+        *reinterpret_cast<float4 *>(C + ((size_t)blockIdx.x * R + a0 + r4 + i) * R + b0 + c4) =
+            make_float4(acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y);
 }
 
 // Asynchronous global -> shared copies (cp.async); src_bytes = 0 writes zeros.
@@ -530,24 +586,34 @@ Err build_m2l_svd(afmpb_t *h, bool *compressed) {
   AFMPB_TRY(A.alloc(&d_reps, reps.size(), "svd orbit offsets"));
   AFMPB_TRY(A.alloc(&d_wrep, wrep.size(), "svd orbit weights"));
   AFMPB_TRY(A.alloc(&d_perm, perm.size(), "svd point permutations"));
-  AFMPB_TRY(A.alloc(&d_H, (size_t)nrep * N3 * N3, "svd orbit grams"));
-  AFMPB_TRY(A.alloc(&d_K, (size_t)kNumOffsets * N3 * N3, "svd K64"));
-  AFMPB_TRY(A.alloc(&d_gram, (size_t)N3 * N3, "svd gram"));
+  const size_t gram_tables = std::min(kGramTables, ntab);
+  AFMPB_TRY(A.alloc(&d_H, gram_tables * nrep * N3 * N3, "svd orbit grams"));
+  AFMPB_TRY(A.alloc(&d_K, gram_tables * nrep * N3 * N3, "svd K64"));
+  AFMPB_TRY(A.alloc(&d_gram, gram_tables * N3 * N3, "svd gram"));
   AFMPB_CUDA(cudaMemcpyAsync(d_reps, reps.data(), sizeof(int3) * reps.size(), cudaMemcpyHostToDevice, s));
   AFMPB_CUDA(cudaMemcpyAsync(d_wrep, wrep.data(), sizeof(double) * wrep.size(), cudaMemcpyHostToDevice, s));
   AFMPB_CUDA(cudaMemcpyAsync(d_perm, perm.data(), sizeof(int32_t) * perm.size(), cudaMemcpyHostToDevice, s));
   AFMPB_CUDA(cudaMemcpyAsync(d_offs, offs.data(), sizeof(int3) * offs.size(), cudaMemcpyHostToDevice, s));
   // Gram matrices and their eigen-decompositions
   std::vector<std::vector<double>> gram(ntab, std::vector<double>((size_t)N3 * N3));
-  const dim3 ggrid((N3 + kGramTile - 1) / kGramTile, (N3 + kGramTile - 1) / kGramTile, nrep);
-  for (int t = 0; t < ntab; ++t) {
-    k_table_f64<<<256, 256, 0, s>>>(n, nrep, d_reps, nd, tab_kw[t], tab_invw[t], d_K);
+  for (int t = 0; t < ntab; t += kGramTables) {
+    const int nt = std::min(kGramTables, ntab - t);
+    TableScale ts{};
+    for (int k = 0; k < nt; ++k) {
+      ts.kw[k] = tab_kw[t + k];
+      ts.invw[k] = tab_invw[t + k];
+    }
+    const unsigned tiles = (N3 + kGramTile - 1) / kGramTile;
+    k_table_f64<<<dim3(256, nt), 256, 0, s>>>(n, nrep, d_reps, nd, ts, d_K);
     AFMPB_TRY(check_launch("k_table_f64 orbits"));
-    k_gram_rep<<<ggrid, 256, 0, s>>>(N3, d_K, d_H);
+    k_gram_rep<<<dim3(tiles, tiles, nt * nrep), 256, 0, s>>>(N3, d_K, d_H);
     AFMPB_TRY(check_launch("k_gram_rep"));
-    k_gram_sym<<<div_up((int64_t)N3 * N3, 256), 256, 0, s>>>(N3, nrep, d_H, d_wrep, d_perm, d_gram);
+    k_gram_sym<<<dim3((N3 + kSymCols - 1) / kSymCols, N3, nt), dim3(kSymCols, nrep), sizeof(double) * nrep * kSymCols, s>>>(
+        N3, nrep, d_H, d_wrep, d_perm, d_gram);
     AFMPB_TRY(check_launch("k_gram_sym"));
-    AFMPB_CUDA(cudaMemcpyAsync(gram[t].data(), d_gram, sizeof(double) * N3 * N3, cudaMemcpyDeviceToHost, s));
+    for (int k = 0; k < nt; ++k)
+      AFMPB_CUDA(cudaMemcpyAsync(gram[t + k].data(), d_gram + (size_t)k * N3 * N3, sizeof(double) * N3 * N3,
+                                 cudaMemcpyDeviceToHost, s));
   }
   AFMPB_CUDA(cudaStreamSynchronize(s));
   A.release(d_H);
@@ -600,7 +666,7 @@ Err build_m2l_svd(afmpb_t *h, bool *compressed) {
   AFMPB_TRY(A.alloc(&h->d_Q, (size_t)ntab * N3 * R, "svd Q"));
   AFMPB_TRY(A.alloc(&h->d_QT, (size_t)ntab * R * N3, "svd QT"));
   AFMPB_TRY(A.alloc(&h->d_C, (size_t)ntab * kNumOffsets * R * R, "svd C"));
-  float *d_Kf = reinterpret_cast<float *>(d_K), *d_T = nullptr;   // the FP64 table buffer is free now
+  float *d_T = nullptr;
   AFMPB_TRY(A.alloc(&d_T, (size_t)kNumOffsets * N3 * R, "svd T"));
   std::vector<float> qf((size_t)ntab * N3 * R), qtf((size_t)ntab * R * N3);
   for (int t = 0; t < ntab; ++t)
@@ -612,14 +678,15 @@ Err build_m2l_svd(afmpb_t *h, bool *compressed) {
       }
   AFMPB_CUDA(cudaMemcpyAsync(h->d_Q, qf.data(), sizeof(float) * qf.size(), cudaMemcpyHostToDevice, s));
   AFMPB_CUDA(cudaMemcpyAsync(h->d_QT, qtf.data(), sizeof(float) * qtf.size(), cudaMemcpyHostToDevice, s));
+  const int op_smem = (int)(sizeof(float) * ((size_t)N3 * kOpRows + kOpSlab * kOpCols));
+  const int cblk = (R + kOpCols - 1) / kOpCols;
+  AFMPB_TRY(raise_smem_limit((const void *)k_kq, op_smem));
   for (int t = 0; t < ntab; ++t) {
     const float *Qt = h->d_Q + (size_t)t * N3 * R;
-    k_table_f32<<<1024, 256, 0, s>>>(n, kNumOffsets, d_offs, nd, tab_kw[t], tab_invw[t], d_Kf);
-    AFMPB_TRY(check_launch("k_table_f32"));
-    k_kq<<<dim3(kNumOffsets, (N3 + kRowsPerCta - 1) / kRowsPerCta), 128, 0, s>>>(N3, R, d_Kf, Qt, d_T);
+    k_kq<<<dim3(kNumOffsets, (N3 + kOpRows - 1) / kOpRows, cblk), 128, op_smem, s>>>(n, R, d_offs, nd, tab_kw[t],
+                                                                                   tab_invw[t], Qt, d_T);
     AFMPB_TRY(check_launch("k_kq"));
-    k_qtt<<<dim3(kNumOffsets, (R + kRowsPerCta - 1) / kRowsPerCta), 128, 0, s>>>(
-        N3, R, Qt, d_T, h->d_C + (size_t)t * kNumOffsets * R * R);
+    k_qtt<<<dim3(kNumOffsets, cblk, cblk), 256, 0, s>>>(N3, R, Qt, d_T, h->d_C + (size_t)t * kNumOffsets * R * R);
     AFMPB_TRY(check_launch("k_qtt"));
   }
   // compress / expand work: chunks of up to kChunkBoxes boxes of one level, on the levels
