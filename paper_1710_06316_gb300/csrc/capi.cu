@@ -59,15 +59,11 @@ void destroy_handle(afmpb_t *h) {
   if (h->side2) cudaStreamDestroy(h->side2);
   if (h->ev_fork2) cudaEventDestroy(h->ev_fork2);
   if (h->ev_join2) cudaEventDestroy(h->ev_join2);
+  if (h->ev_zero) cudaEventDestroy(h->ev_zero);
   if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
   delete h;
 }
 
-// Captures the product for one parts mask.  With io == true the graph also holds the
-// gather of the caller's x and the scatter into the caller's y (kernel nodes whose pointer
-// arguments afmpb_matvec_parts updates in place for new buffers), so that a product is a
-// single graph launch: a plain kernel launch right before the far-field graph cost ~0.3 ms
-// of start-up on a 163,842-node product.
 // P2P runs beside the far-field chain (fork onto the low-priority side stream) for meshes
 // up to this size; above it the two run one after the other.  Measured products, mixed
 // precision, overlapped vs serial: 164k nodes 0.65 vs 0.73 ms, 200k 1.11 vs 1.46 ms, 2.1M
@@ -117,6 +113,11 @@ Err enqueue_product_far(afmpb_t *h, cudaStream_t cap, int parts, float *y) {
   return e;
 }
 
+// Captures the product for one parts mask.  With io == true the graph also holds the
+// gather of the caller's x and the scatter into the caller's y (kernel nodes whose pointer
+// arguments afmpb_matvec_parts updates in place for new buffers), so that a product is a
+// single graph launch: a plain kernel launch right before the far-field graph cost ~0.3 ms
+// of start-up on a 163,842-node product.
 Err capture_product(afmpb_t *h, int parts, bool io = false, const float *x = nullptr, float *y = nullptr) {
   // The far-field chain (a long sequence of short, latency-bound launches) is captured
   // from a high-priority stream and P2P from a low-priority one: the kernel nodes keep the
@@ -232,12 +233,13 @@ Err create_impl(afmpb_t *h, const afmpb_mesh *mesh, const afmpb_charges *ch) {
     int lo = 0, hi = 0;
     AFMPB_CUDA(cudaDeviceGetStreamPriorityRange(&lo, &hi));
     AFMPB_CUDA(cudaStreamCreateWithPriority(&h->side, cudaStreamNonBlocking, lo));   // P2P: lowest
-    AFMPB_CUDA(cudaStreamCreateWithPriority(&h->side2, cudaStreamNonBlocking, hi));  // P2L: with the chain
+    AFMPB_CUDA(cudaStreamCreateWithPriority(&h->side2, cudaStreamNonBlocking, hi));  // zeroing, P2L: with the chain
   }
   AFMPB_CUDA(cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming));
   AFMPB_CUDA(cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming));
   AFMPB_CUDA(cudaEventCreateWithFlags(&h->ev_fork2, cudaEventDisableTiming));
   AFMPB_CUDA(cudaEventCreateWithFlags(&h->ev_join2, cudaEventDisableTiming));
+  AFMPB_CUDA(cudaEventCreateWithFlags(&h->ev_zero, cudaEventDisableTiming));
   AFMPB_CUDA(cudaEventCreate(&h->ev_t0));
   AFMPB_CUDA(cudaEventCreate(&h->ev_t1));
   auto lap = [&](int i) {
@@ -902,8 +904,9 @@ afmpb_status afmpb_profile_product(afmpb_t *h, int reps, void *flush, size_t flu
       kernels += launches[i];
     }
     // the captured product runs the near correction as a kernel of its own after P2P and
-    // assembles y in L2P, where the stages above run k_combine and k_scatter
-    out->kernels_per_product = kernels - 1;
+    // assembles y in L2P, where the stages above run k_combine and k_scatter; the kernel that
+    // zeroes the local expansions is timed with the first stage of the far field
+    out->kernels_per_product = kernels;
     // graph replays (the path afmpb_matvec takes), same flush between repetitions
     cudaEvent_t a = nullptr, b = nullptr;
     cudaEventCreate(&a);

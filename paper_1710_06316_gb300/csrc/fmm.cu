@@ -99,6 +99,7 @@ __global__ void __launch_bounds__(32 * kP2MWarps) k_p2m(int nleaf, const int4 *_
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int l0 = (blockIdx.x * kP2MWarps + warp) * P::Leaves;
   if (l0 >= nleaf) return;                              // whole warps
+  after_previous();
   float *buf = sm[warp];
   const int sub = lane / P::G, half = lane % P::G / N, k = lane % N;   // this lane's weights
   const int ssub = lane / CH, snode = lane % CH;                       // the node that it stages
@@ -245,6 +246,7 @@ __global__ void __launch_bounds__(kAxisThreads<N>) k_m2m(const int32_t *__restri
   int child[8];
   load_children(par_child, child);
   stage_m2m_ops<N>(sS);
+  after_previous();
   const int m = threadIdx.x;
   const bool act = m < N3;
   const int i = m / (N * N), j = (m / N) % N, k = m % N;
@@ -303,6 +305,7 @@ __global__ void __launch_bounds__(kAxisThreads<N>) k_l2l(const int32_t *__restri
   int child[8];
   load_children(par_child, child);
   stage_m2m_ops<N>(sS);
+  after_previous();
   const int m = threadIdx.x;
   const bool act = m < N3;
   const int i = m / (N * N), j = (m / N) % N, k = m % N;
@@ -1030,6 +1033,17 @@ Err init_cheb_tables() {
   return Err{};
 }
 
+// L and the compressed locals, beside the upward pass.  A kernel, since a memset node has no
+// priority and its blocks wait behind those of P2P (products of 163,842 nodes 416 us so, 400
+// with the kernel); few blocks, which leave room to the chain (608 in place of 76: a protein
+// surface of 191,944 nodes 570 against 561 us; 24: 570).
+constexpr int kZeroBlocks = 76;
+
+__global__ void __launch_bounds__(256) k_zero(int64_t na, float2 *__restrict__ a, int64_t nb, float2 *__restrict__ b) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < na + nb; i += (int64_t)gridDim.x * blockDim.x)
+    (i < na ? a[i] : b[i - na]) = make_float2(0.f, 0.f);
+}
+
 template <int N>
 Err launch_far(afmpb_t *h, cudaStream_t s, StageTimer *tm, int parts, const FarOut *out) {
   constexpr int N3 = N * N * N;
@@ -1049,24 +1063,35 @@ Err launch_far(afmpb_t *h, cudaStream_t s, StageTimer *tm, int parts, const FarO
     return check_launch("k_p2l");
   };
   if (parts & kFarUp) {
-  AFMPB_CUDA(cudaMemsetAsync(h->d_L, 0, sizeof(float) * (size_t)T.nbox * 2 * N3, s));
-  if (p2l_beside) {
+  // (in the chain the two memsets cost a product of 2,562 nodes 6 us of 51)
+  const bool beside = !tm && h->side2;
+  cudaStream_t z = beside ? h->side2 : s;
+  if (beside) {
     AFMPB_CUDA(cudaEventRecord(h->ev_fork2, s));
-    AFMPB_CUDA(cudaStreamWaitEvent(h->side2, h->ev_fork2, 0));
-    AFMPB_TRY(launch_p2l(h->side2));
-    AFMPB_CUDA(cudaEventRecord(h->ev_join2, h->side2));
+    AFMPB_CUDA(cudaStreamWaitEvent(z, h->ev_fork2, 0));
   }
-  k_p2m<N><<<div_up(T.nleaf, kP2MWarps * P2MShape<N>::Leaves), 32 * kP2MWarps, 0, s>>>(T.nleaf, h->d_leaf_rec, inv_w0, h->d_pos,
-                                                                 h->d_nrm, h->d_xs, inv_ebar, h->d_M);
-  AFMPB_TRY(check_launch("k_p2m"));
+  {
+    const int64_t nl = (int64_t)T.nbox * N3, nc = compressed ? (int64_t)T.nbox * h->m2l_rank : 0;
+    k_zero<<<(unsigned)std::min<int64_t>(div_up(nl + nc, 4 * 256), kZeroBlocks), 256, 0, z>>>(
+        nl, reinterpret_cast<float2 *>(h->d_L), nc, reinterpret_cast<float2 *>(h->d_Lc));
+    AFMPB_TRY(check_launch("k_zero"));
+  }
+  if (beside) AFMPB_CUDA(cudaEventRecord(h->ev_zero, z));
+  if (p2l_beside) {
+    AFMPB_TRY(launch_p2l(z));
+    AFMPB_CUDA(cudaEventRecord(h->ev_join2, z));
+  }
+  AFMPB_TRY(launch_next(beside, "k_p2m", k_p2m<N>, div_up(T.nleaf, kP2MWarps * P2MShape<N>::Leaves), 32 * kP2MWarps, 0, s, T.nleaf,
+                        h->d_leaf_rec, inv_w0, h->d_pos, h->d_nrm, h->d_xs, inv_ebar, h->d_M));
   if (tm) tm->mark("p2m", 1);
   for (int level = T.nlevel - 2; level >= 2; --level) {
     const int p0 = T.par_start[level], np = T.par_start[level + 1] - p0;
     if (np == 0) continue;
-    k_m2m<N><<<dim3(np, 2), kAxisThreads<N>, 0, s>>>(h->d_par + p0, h->d_par_child + 8 * (size_t)p0, h->d_M);
-    AFMPB_TRY(check_launch("k_m2m"));
+    AFMPB_TRY(launch_next(true, "k_m2m", k_m2m<N>, dim3(np, 2), kAxisThreads<N>, 0, s, h->d_par + p0,
+                          h->d_par_child + 8 * (size_t)p0, h->d_M));
   }
   if (tm) tm->mark("m2m", std::max(0, T.nlevel - 3));
+  if (beside) AFMPB_CUDA(cudaStreamWaitEvent(s, h->ev_zero, 0));
   }
   if (compressed && p2l_beside) {
     AFMPB_TRY(enqueue_m2l_svd(h, s, tm, kFarUp | kFarM2L));
@@ -1090,13 +1115,18 @@ Err launch_far(afmpb_t *h, cudaStream_t s, StageTimer *tm, int parts, const FarO
   }
   if (tm && !compressed) tm->mark("m2l", h->m2l_groups.empty() ? 0 : 1);
   if (!(parts & kFarDown)) return Err{};
-  if (h->n_xbox > 0 && !p2l_beside) AFMPB_TRY(launch_p2l(s));
+  bool chained = compressed ? h->m2l_nchunks > 0 : !h->m2l_groups.empty() && (parts & kFarM2L) && !plane_wave;
+  if (h->n_xbox > 0 && !p2l_beside) {
+    AFMPB_TRY(launch_p2l(s));
+    chained = true;
+  }
   if (tm) tm->mark("p2l", h->n_xbox > 0 ? 1 : 0);
   for (int level = 2; level + 1 < T.nlevel; ++level) {
     const int p0 = T.par_start[level], np = T.par_start[level + 1] - p0;
     if (np == 0) continue;
-    k_l2l<N><<<dim3(np, 2), kAxisThreads<N>, 0, s>>>(h->d_par + p0, h->d_par_child + 8 * (size_t)p0, h->d_L);
-    AFMPB_TRY(check_launch("k_l2l"));
+    AFMPB_TRY(launch_next(chained, "k_l2l", k_l2l<N>, dim3(np, 2), kAxisThreads<N>, 0, s, h->d_par + p0,
+                          h->d_par_child + 8 * (size_t)p0, h->d_L));
+    chained = true;
   }
   if (tm) tm->mark("l2l", std::max(0, T.nlevel - 3));
   const int nblk = div_up(h->n, kL2PNodes);

@@ -269,8 +269,8 @@ struct afmpb_t {
   cudaStream_t stream = nullptr;   // handle stream (user's or own)
   bool own_stream = false;
   cudaStream_t side = nullptr;     // second stream: P2P beside the far-field chain
-  cudaStream_t side2 = nullptr;    // third stream: P2L beside the upward pass and the M2L
-  cudaEvent_t ev_fork2 = nullptr, ev_join2 = nullptr;
+  cudaStream_t side2 = nullptr;    // third stream: zeroed expansions and P2L beside the upward pass and the M2L
+  cudaEvent_t ev_fork2 = nullptr, ev_join2 = nullptr, ev_zero = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   cudaEvent_t ev_t0 = nullptr, ev_t1 = nullptr;
 
@@ -590,6 +590,35 @@ inline Err current_exception_err() {
     return make_err(AFMPB_EINTERNAL, "unknown host exception");
   }
 }
+
+// Launch of a kernel of a chain.  chained: its only predecessor in the stream is a kernel (no
+// copy, no event of another stream); then it may begin once that one's blocks have ended, and
+// waits for what they wrote in after_previous(), which every such kernel calls before it
+// touches anything that another kernel writes.  (At least one block waits, so a kernel ends
+// after all kernels before it.)  Blocks that begin before that (a trigger at the top of each
+// kernel) hold room that P2P uses: products of 12k nodes 89 -> 95 us, of 163,842 415 -> 424.
+template <class... P, class... A>
+Err launch_next(bool chained, const char *what, void (*k)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t s, A &&...a) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = chained ? 1 : 0;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k, P(std::forward<A>(a))...);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return make_err(AFMPB_ECUDA, std::string(what) + ": " + cudaGetErrorString(e));
+  }
+  return Err{};
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ void after_previous() { cudaGridDependencySynchronize(); }
+#endif
 
 inline Err check_launch(const char *what) {
   cudaError_t e = cudaGetLastError();

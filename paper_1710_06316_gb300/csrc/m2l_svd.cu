@@ -274,6 +274,7 @@ __global__ void __launch_bounds__(512) k_box_basis(int K, int ncol, const int4 *
                                                    const float *__restrict__ A, const float *__restrict__ X,
                                                    float *__restrict__ Y, __nv_bfloat16 *__restrict__ Y16) {
   extern __shared__ __align__(16) float sm[];
+  after_previous();
   float *Xs = sm;                                      // [K][kChunkBoxes]
   float *As = sm + (size_t)K * kChunkBoxes;            // [kStages][kSlabRows][ncol]
   const int4 ch = chunks[blockIdx.x];                  // first box, count, level
@@ -384,15 +385,15 @@ size_t basis_smem(int K, int ncol) {
 }
 
 template <bool ACCUM>
-Err launch_box_basis(cudaStream_t s, dim3 grid, int K, int ncol, const int4 *chunks, const int *level_table,
+Err launch_box_basis(bool chained, cudaStream_t s, dim3 grid, int K, int ncol, const int4 *chunks, const int *level_table,
                      const int *table_rank, int yuk_min, const float *A, const float *X, float *Y,
                      __nv_bfloat16 *Y16 = nullptr) {
   const size_t smem = basis_smem(K, ncol);
   // a thread to each tile: at most 512 (compress: rank <= kMaxRank; expand: n^3 <= 512)
   constexpr int TB = ACCUM ? 4 : 2;
   const int nthr = ((kChunkBoxes / TB) * (ncol / 4) + 31) / 32 * 32;
-  k_box_basis<TB, ACCUM><<<grid, nthr, smem, s>>>(K, ncol, chunks, level_table, table_rank, yuk_min, A, X, Y, Y16);
-  return check_launch(ACCUM ? "k_box_basis expand" : "k_box_basis compress");
+  return launch_next(chained, ACCUM ? "k_box_basis expand" : "k_box_basis compress", k_box_basis<TB, ACCUM>, grid, nthr, smem, s,
+                     K, ncol, chunks, level_table, table_rank, yuk_min, A, X, Y, Y16);
 }
 
 template <bool ACCUM>
@@ -729,14 +730,13 @@ Err build_m2l_svd(afmpb_t *h, bool *compressed) {
 Err enqueue_m2l_svd(afmpb_t *h, cudaStream_t s, StageTimer *tm, int parts) {
   const int R = h->m2l_rank, N3 = h->ncoef;
   const auto &T = h->shape;
-  if (parts & kFarUp) AFMPB_CUDA(cudaMemsetAsync(h->d_Lc, 0, sizeof(float) * (size_t)T.nbox * 2 * R, s));
   if (h->m2l_nchunks == 0) return Err{};
   const dim3 cgrid((unsigned)h->m2l_nchunks, 2);
   if (parts & kFarUp) {
-    AFMPB_TRY(launch_box_basis<false>(s, cgrid, N3, R, h->d_m2l_chunks, h->d_level_table, h->d_table_rank,
+    AFMPB_TRY(launch_box_basis<false>(false, s, cgrid, N3, R, h->d_m2l_chunks, h->d_level_table, h->d_table_rank,
                                        h->m2l_yuk_levels, h->d_Q, h->d_M, h->d_Mc,
                                        reinterpret_cast<__nv_bfloat16 *>(h->d_Mc16)));
-    if (tm) tm->mark("compress", 1);             // Lc memset (not a kernel) + basis change
+    if (tm) tm->mark("compress", 1);
   }
   if (!(parts & kFarM2L)) {
   } else if (h->opt.precision == 1) {
@@ -753,7 +753,7 @@ Err enqueue_m2l_svd(afmpb_t *h, cudaStream_t s, StageTimer *tm, int parts) {
   }
   if (tm && (parts & kFarM2L)) tm->mark("m2l", 1);
   if (!(parts & kFarDown)) return Err{};
-  AFMPB_TRY(launch_box_basis<true>(s, cgrid, R, N3, h->d_m2l_chunks, h->d_level_table, h->d_table_rank,
+  AFMPB_TRY(launch_box_basis<true>((parts & kFarM2L) != 0, s, cgrid, R, N3, h->d_m2l_chunks, h->d_level_table, h->d_table_rank,
                                    h->m2l_yuk_levels, h->d_QT, h->d_Lc, h->d_L));
   if (tm) tm->mark("expand", 1);
   return Err{};

@@ -146,6 +146,7 @@ __global__ void __launch_bounds__(kTsThreads) k_m2l_ts(int R, int nitems_arg, co
                                                       const int *__restrict__ d_nitems,
                                                       const TSReq *__restrict__ reqs) {
   extern __shared__ __align__(128) uint8_t smem[];
+  after_previous();
   const int nitems = kBatch ? *d_nitems : nitems_arg;
   auto runs_of = [&](const TSItem &it) -> const int4 * { return kBatch ? reqs[it.req].runs : runs_1; };
   auto masks_of = [&](const TSItem &it) -> const uint4 * { return kBatch ? reqs[it.req].masks : masks_1; };
@@ -653,14 +654,10 @@ Err enqueue_m2l_ts(afmpb_t *h, cudaStream_t s) {
   const auto *mc = reinterpret_cast<const __nv_bfloat16 *>(h->d_Mc16);
   const auto *tl = reinterpret_cast<const __nv_bfloat16 *>(h->d_ts_tiles);
   if (ts_stages(R) == 4)
-    k_m2l_ts<4, false><<<grid, kTsThreads, ts_smem_bytes(R), s>>>(R, h->ts_nitems, h->d_ts_items, h->d_ts_runs,
-                                                                  h->d_ts_masks, h->d_ts_ent, h->d_ts_box, mc, tl, h->d_Lc, h->d_tc_flag,
-                                                                  nullptr, nullptr);
-  else
-    k_m2l_ts<2, false><<<grid, kTsThreads, ts_smem_bytes(R), s>>>(R, h->ts_nitems, h->d_ts_items, h->d_ts_runs,
-                                                                  h->d_ts_masks, h->d_ts_ent, h->d_ts_box, mc, tl, h->d_Lc, h->d_tc_flag,
-                                                                  nullptr, nullptr);
-  return check_launch("k_m2l_ts");
+    return launch_next(true, "k_m2l_ts", k_m2l_ts<4, false>, grid, kTsThreads, ts_smem_bytes(R), s, R, h->ts_nitems, h->d_ts_items,
+                       h->d_ts_runs, h->d_ts_masks, h->d_ts_ent, h->d_ts_box, mc, tl, h->d_Lc, h->d_tc_flag, nullptr, nullptr);
+  return launch_next(true, "k_m2l_ts", k_m2l_ts<2, false>, grid, kTsThreads, ts_smem_bytes(R), s, R, h->ts_nitems, h->d_ts_items,
+                       h->d_ts_runs, h->d_ts_masks, h->d_ts_ent, h->d_ts_box, mc, tl, h->d_Lc, h->d_tc_flag, nullptr, nullptr);
 }
 
 // The items of the running problems of a batch, in their order: one block scans the

@@ -563,6 +563,7 @@ __global__ void __launch_bounds__(kRedThreads) k_gs_first(int64_t len, int64_t c
                                                           const float *__restrict__ ys, double *__restrict__ w,
                                                           double *part, int stride, double *__restrict__ hcol,
                                                           const int *__restrict__ guard) {
+  after_previous();
   if (guard && *guard == 0) return;
   __shared__ double tile[kGsTile];
   const int nv = gm[0] + 1;
@@ -590,6 +591,7 @@ __global__ void __launch_bounds__(kRedThreads) k_gs_second(int64_t len, int64_t 
                                                            double *__restrict__ w, double *part, int stride,
                                                            double *__restrict__ hcol, double *__restrict__ hcol2,
                                                            const int *__restrict__ guard) {
+  after_previous();
   if (guard && *guard == 0) return;
   __shared__ double tile[kGsTile];
   const int nv = gm[0] + 1;
@@ -665,6 +667,7 @@ __global__ void __launch_bounds__(kRedThreads) k_gs_norm(int64_t len, int64_t ch
                                                          double *__restrict__ g, double *__restrict__ res,
                                                          const double *__restrict__ tol, int batch,
                                                          cudaGraphConditionalHandle loop, const int *__restrict__ guard) {
+  after_previous();
   if (guard && *guard == 0) return;
   __shared__ double sh[32];
   const int j = gm[0], nv = j + 1;
@@ -703,6 +706,7 @@ __global__ void __launch_bounds__(kRedThreads) k_gs_norm(int64_t len, int64_t ch
 __global__ void k_gs_normalize(int64_t n, const int *__restrict__ gm, const double *__restrict__ w,
                                const double *__restrict__ hcol, double *__restrict__ V, int64_t n2,
                                float2 *__restrict__ xs, const int *__restrict__ guard) {
+  after_previous();
   if (guard && *guard == 0) return;
   const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (p >= n) return;
@@ -766,14 +770,15 @@ Err enqueue_step_tail(afmpb_t *h, int m, cudaStream_t cap, const int *act, bool 
     const int64_t chunk = ((n2 + 1183) / 1184 + kGsTile - 1) / kGsTile * kGsTile;
     const int nb = div_up(n2, chunk), stride = m + 2;
     int *gm = h->d_gm_int;
-    k_gs_first<<<nb, kRedThreads, 0, cap>>>(n2, chunk, gm, h->d_V, n2, h->d_ys, h->d_w, h->d_part, stride, h->d_hcol, act);
-    k_gs_second<<<nb, kRedThreads, 0, cap>>>(n2, chunk, gm, h->d_V, n2, h->d_w, h->d_part, stride, h->d_hcol, h->d_hcol2,
-                                             act);
-    k_gs_norm<<<nb, kRedThreads, 0, cap>>>(n2, chunk, gm, m, h->d_V, n2, h->d_w, h->d_part, stride, h->d_hcol, h->d_hcol2,
-                                           h->d_H, h->d_cs, h->d_sn, h->d_g, h->d_scal + 2, h->d_scal + 4,
-                                           batch ? 1 : 0, loop, act);
-    k_gs_normalize<<<div_up(n, 256), 256, 0, cap>>>(n, gm, h->d_w, h->d_hcol, h->d_V, n2, h->d_xs, act);
-    return check_launch("arnoldi step (fused)");
+    AFMPB_TRY(launch_next(true, "k_gs_first", k_gs_first, nb, kRedThreads, 0, cap, n2, chunk, gm, h->d_V, n2, h->d_ys, h->d_w,
+                          h->d_part, stride, h->d_hcol, act));
+    AFMPB_TRY(launch_next(true, "k_gs_second", k_gs_second, nb, kRedThreads, 0, cap, n2, chunk, gm, h->d_V, n2, h->d_w, h->d_part,
+                          stride, h->d_hcol, h->d_hcol2, act));
+    AFMPB_TRY(launch_next(true, "k_gs_norm", k_gs_norm, nb, kRedThreads, 0, cap, n2, chunk, gm, m, h->d_V, n2, h->d_w, h->d_part,
+                          stride, h->d_hcol, h->d_hcol2, h->d_H, h->d_cs, h->d_sn, h->d_g, h->d_scal + 2, h->d_scal + 4,
+                          batch ? 1 : 0, loop, act));
+    return launch_next(true, "k_gs_normalize", k_gs_normalize, div_up(n, 256), 256, 0, cap, n, gm, h->d_w, h->d_hcol, h->d_V, n2,
+                       h->d_xs, act);
   }
   const int *gm = h->d_gm_int;
   int *gmw = h->d_gm_int;
@@ -1085,14 +1090,16 @@ Err build_batch_graph(afmpb_t *const *hs, int k, const int *ms, bool fuse_m2l, c
   AFMPB_TRY(G.stream(&cap, hi));
   AFMPB_TRY(G.stream(&sp, lo));            // P2P fills the SMs the far-field chains leave free
   AFMPB_TRY(G.stream(&sm, hi));
-  std::vector<cudaStream_t> si(k);
-  std::vector<cudaEvent_t> ev_a(k), ev_b(k), ev_e(k);
+  std::vector<cudaStream_t> si(k), sz(k);
+  std::vector<cudaEvent_t> ev_h(k), ev_a(k), ev_b(k), ev_e(k);
   cudaEvent_t ev_fork = nullptr, ev_p = nullptr, ev_m = nullptr;
   AFMPB_TRY(G.event(&ev_fork));
   AFMPB_TRY(G.event(&ev_p));
   AFMPB_TRY(G.event(&ev_m));
   for (int i = 0; i < k; ++i) {
     AFMPB_TRY(G.stream(&si[i], hi));
+    AFMPB_TRY(G.stream(&sz[i], hi));
+    AFMPB_TRY(G.event(&ev_h[i]));
     AFMPB_TRY(G.event(&ev_a[i]));
     AFMPB_TRY(G.event(&ev_b[i]));
     AFMPB_TRY(G.event(&ev_e[i]));
@@ -1106,8 +1113,10 @@ Err build_batch_graph(afmpb_t *const *hs, int k, const int *ms, bool fuse_m2l, c
       const int *act = h->d_gm_int + 4;
       AFMPB_CUDA(cudaStreamWaitEvent(si[i], ev_fork, 0));
       AFMPB_TRY(enqueue_step_head(h, si[i], act));
-      AFMPB_CUDA(cudaMemsetAsync(h->d_phi_near, 0, sizeof(float4) * h->n, si[i]));
-      AFMPB_CUDA(cudaEventRecord(ev_a[i], si[i]));
+      AFMPB_CUDA(cudaEventRecord(ev_h[i], si[i]));
+      AFMPB_CUDA(cudaStreamWaitEvent(sz[i], ev_h[i], 0));
+      AFMPB_CUDA(cudaMemsetAsync(h->d_phi_near, 0, sizeof(float4) * h->n, sz[i]));   // beside the chain
+      AFMPB_CUDA(cudaEventRecord(ev_a[i], sz[i]));
       AFMPB_TRY(enqueue_far(h, si[i], nullptr, fuse_m2l ? kFarUp : kFarUp | kFarM2L));
       AFMPB_CUDA(cudaEventRecord(ev_b[i], si[i]));
     }

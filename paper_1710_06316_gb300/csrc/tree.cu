@@ -428,9 +428,7 @@ __global__ void k_x_route(int nbox, const int64_t *__restrict__ xptr, const int3
 // Point-to-point source boxes of a leaf: list 1, the list-4 boxes of itself and its
 // ancestors that are summed directly, and the leaves under each list-3 box (node positions
 // are stored relative to their own leaf, so P2P sources are leaves).  fill == false counts
-// boxes, source nodes, pairs and the block's relative cost (tiles of up to kP2PThreads
-// targets, each thread slice walking its share of the sources, plus the staging of every
-// source per tile, in quarter units).
+// boxes and pairs.
 __global__ void k_p2p_lists(int nleaf, const int32_t *__restrict__ leaves, const int32_t *__restrict__ bbeg,
                             const int32_t *__restrict__ bend, const int32_t *__restrict__ parent,
                             const int32_t *__restrict__ child0, const int32_t *__restrict__ nchild,
@@ -438,8 +436,7 @@ __global__ void k_p2p_lists(int nleaf, const int32_t *__restrict__ leaves, const
                             const int64_t *__restrict__ xptr, const int32_t *__restrict__ xidx,
                             const uint8_t *__restrict__ x_direct, const int64_t *__restrict__ wptr,
                             const int32_t *__restrict__ widx, int64_t *__restrict__ cnt, int64_t *__restrict__ pairs,
-                            uint64_t *__restrict__ cost, const int64_t *__restrict__ pptr, int32_t *__restrict__ pidx,
-                            bool fill) {
+                            const int64_t *__restrict__ pptr, int32_t *__restrict__ pidx, bool fill) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nleaf) return;
   const int b = leaves[i];
@@ -466,12 +463,8 @@ __global__ void k_p2p_lists(int nleaf, const int32_t *__restrict__ leaves, const
     }
   }
   if (fill) return;
-  const int64_t nt = bend[b] - bbeg[b];
   cnt[i] = nb;
-  pairs[i] = nt * src;
-  const int64_t tile = max((int64_t)1, min(nt, (int64_t)kP2PThreads));
-  const int64_t slices = kP2PThreads / tile, ntiles = (nt + tile - 1) / tile;
-  cost[i] = (uint64_t)(ntiles * (4 * ((src + slices - 1) / slices) + src + 256));
+  pairs[i] = (int64_t)(bend[b] - bbeg[b]) * src;
 }
 
 // Blocks' time of a unit of nt targets and `total` staged sources, in cycles of a scheduler
@@ -1103,22 +1096,17 @@ Err build_tree(afmpb_t *h) {
   }
 
   // ---- point-to-point source boxes per leaf (ascending: near-field setup looks a box up
-  //      by binary search), the P2P pair count and the blocks' longest-first order
+  //      by binary search) and the P2P pair count
   {
     const int nl = T.nleaf;
     int64_t *cnt = nullptr, *pairs_l = nullptr, *d_pairs = nullptr;
-    uint64_t *cost = nullptr, *cost_sorted = nullptr;
-    int32_t *iota = nullptr;
     AFMPB_TRY(A.alloc(&cnt, nl + 1, "p2p counts"));
     AFMPB_TRY(A.alloc(&pairs_l, nl, "p2p pairs"));
     AFMPB_TRY(A.alloc(&d_pairs, 1, "p2p pair total"));
-    AFMPB_TRY(A.alloc(&cost, nl, "p2p cost"));
-    AFMPB_TRY(A.alloc(&cost_sorted, nl, "p2p cost sorted"));
-    AFMPB_TRY(A.alloc(&iota, nl, "leaf iota"));
     AFMPB_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int64_t) * (nl + 1), s));
     k_p2p_lists<<<div_up(nl, 64), 64, 0, s>>>(nl, h->d_leaves, bbeg, bend, bparent, bchild0, bnchild, d_uptr,
                                               h->d_u_idx, d_xptr, h->d_x_idx, d_xdirect, d_wptr, h->d_w_idx, cnt,
-                                              pairs_l, cost, nullptr, nullptr, false);
+                                              pairs_l, nullptr, nullptr, false);
     AFMPB_TRY(check_launch("k_p2p_lists count"));
     int64_t n_p = 0;
     AFMPB_TRY(csr_ptr(h, cnt, nl, &h->d_p2p_ptr, &n_p, "p2p_ptr"));
@@ -1129,7 +1117,7 @@ Err build_tree(afmpb_t *h) {
     h->n_p2p_src = n_p;
     k_p2p_lists<<<div_up(nl, 64), 64, 0, s>>>(nl, h->d_leaves, bbeg, bend, bparent, bchild0, bnchild, d_uptr,
                                               h->d_u_idx, d_xptr, h->d_x_idx, d_xdirect, d_wptr, h->d_w_idx, nullptr,
-                                              nullptr, nullptr, h->d_p2p_ptr, h->d_p2p_idx, true);
+                                              nullptr, h->d_p2p_ptr, h->d_p2p_idx, true);
     AFMPB_TRY(check_launch("k_p2p_lists fill"));
     AFMPB_TRY(sort_rows(h, h->d_p2p_idx, n_p, h->d_p2p_ptr, h->d_p2p_ptr + 1, nl, "p2p sort"));
     AFMPB_TRY(cub_call(h, "p2p pairs", [&](void *t, size_t &bytes) {
@@ -1138,8 +1126,7 @@ Err build_tree(afmpb_t *h) {
     int64_t pairs = 0;
     AFMPB_TRY(read_one(&pairs, d_pairs, s));
     T.n_p2p_pairs = pairs - h->n;     // the diagonal t == p is skipped
-    for (void *q : {(void *)cnt, (void *)pairs_l, (void *)d_pairs, (void *)cost, (void *)cost_sorted, (void *)iota})
-      A.release(q);
+    for (void *q : {(void *)cnt, (void *)pairs_l, (void *)d_pairs}) A.release(q);
   }
   A.release(d_xdirect);
   T.n_u = n_uall;
