@@ -428,10 +428,10 @@ def fp32_peak_tflops(sm_max_mhz, sms):
 
 
 # FP32 operations per source-target pair in the P2P kernel (p2p_pair2, one lane of each
-# packed operation), counted from its source with an FMA as 2 flop: 44 FP32 arithmetic
-# operations (6 adds, 20 multiplies, 18 FMAs) = 62 flop, besides the compare and select of
-# the skip test and one rsqrt and one exp2 on the special-function unit.
-P2P_FLOP_PER_PAIR = 62
+# packed operation), counted from its source with an FMA as 2 flop: 35 FP32 arithmetic
+# operations (3 adds, 13 multiplies, 19 FMAs) = 54 flop, besides the skip test of near source
+# boxes and one rsqrt and one exp2 on the special-function unit.
+P2P_FLOP_PER_PAIR = 54
 
 
 def ncu_traffic(kernel):

@@ -119,8 +119,7 @@ std::tuple<int, int, int, int, int> cache_key(int precision, int order, double k
 }  // namespace
 
 // Tile shapes on the finished handle: the P2P work units (cut for resident blocks per SM x
-// units per block),
-// then the M2L offsets per item, each by timing the kernel itself.  The product graphs are
+// units per block), then the M2L offsets per item, each by timing the kernel itself.  The product graphs are
 // captured again afterwards (they hold the launch shapes).
 Err autotune_tiles(afmpb_t *h, afmpb_autotune_report *rep) {
   constexpr int kReps = 5;

@@ -3,7 +3,7 @@
 // Each problem keeps its own handle: tree, operators, expansions and Krylov state.  What a
 // batch adds is one P2P launch and one tensor-core M2L launch per Arnoldi step for all of
 // them.  The P2P units of every problem are merged into one list, ordered by cost across
-// problems (unit.req = problem), so the resident blocks deal out the union longest-first;
+// problems (unit.req = problem), so that the union is launched longest first, a block per unit;
 // the target-stationary M2L items are concatenated (TSItem.req = problem).  Per-problem
 // descriptors give the kernels each problem's arrays and its stop flag (gm[4] of its
 // step state), so a problem that has converged stops costing P2P and M2L work.

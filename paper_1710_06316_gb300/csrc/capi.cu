@@ -66,9 +66,9 @@ void destroy_handle(afmpb_t *h) {
 
 // P2P runs beside the far-field chain (fork onto the low-priority side stream) for meshes
 // up to this size; above it the two run one after the other.  Measured products, mixed
-// precision, overlapped vs serial: 164k nodes 0.65 vs 0.73 ms, 200k 1.11 vs 1.46 ms, 2.1M
-// 13.9 vs 14.3 ms, 10.5M 69.3 vs 62.0 ms (there the concurrent form contends for L2 with
-// working sets far above it).
+// precision, beside vs one after the other: 168k nodes 0.668 vs 0.862 ms, 1.0M 3.18 vs 3.25,
+// 2.5M 9.03 vs 9.11, 5.0M 15.57 vs 15.60, 10.5M 40.5 vs 40.3 ms (each fills the chip by
+// itself there, and beside each other they contend for L2).
 constexpr int64_t kOverlapMaxNodes = 4000000;
 
 // The kernel of the caller-buffer graph that writes y: the far chain's last one, or the

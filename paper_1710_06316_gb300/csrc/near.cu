@@ -376,7 +376,7 @@ __device__ __forceinline__ bool p2p_leaves_out(const P2PView &pv, int p, int t) 
 // is set.
 //
 // The FP32 pipe bounds the quadrature (7 points of ~80 operations per leaf of a piece's
-// subdivision), and entries differ widely: 8 to 500 leaves on a protein surface, 74 on
+// subdivision), and entries differ widely: 8 to 500 leaves on a protein surface, 34 on
 // average.  So a warp takes kPairBatch entries at a time from a global counter and shares
 // their leaves evenly:
 //   - a lane per entry reads the pair, a lane per piece (32 at a time) its corners;
@@ -384,7 +384,7 @@ __device__ __forceinline__ bool p2p_leaves_out(const P2PView &pv, int p, int t) 
 //     bits a level, from the top) with depth and piece, and splits or joins a queue of leaves;
 //   - whenever 32 leaves are queued, a lane evaluates each, and the warp adds their sums
 //     entry by entry in a fixed order.
-// (A lane to an entry, each walking its own tree: 4.56 ms for the 332,000 entries of
+// (A lane to an entry, each walking its own tree: 4.56 ms for the 962,000 entries of
 // 20,838 nodes, 1.38 so; a warp then ran as long as its largest entry.)
 constexpr int kPairBatch = 16, kPairWarps = 4;
 constexpr int kPairQueue = 64;                // leaves; fewer than 32 wait while 32 nodes are read
