@@ -19,6 +19,8 @@
 #include <algorithm>
 #include <array>
 #include <cmath>
+#include <exception>
+#include <new>
 #include <thread>
 
 #include "internal.cuh"
@@ -624,15 +626,29 @@ Err build_m2l_svd(afmpb_t *h, bool *compressed) {
   std::vector<std::vector<double>> lam(ntab, std::vector<double>(N3)), zt(ntab, std::vector<double>((size_t)N3 * N3));
   std::vector<int> rc(ntab, 0);
   {
+    const auto eig = [&](int t) {                // no exception leaves a thread
+      try {
+        rc[t] = sym_eig_desc(N3, gram[t].data(), lam[t].data(), zt[t].data());
+      } catch (const std::bad_alloc &) {
+        rc[t] = -2;
+      }
+    };
     std::vector<std::thread> pool;
-    for (int t = 0; t < ntab; ++t)
-      pool.emplace_back([&, t] { rc[t] = sym_eig_desc(N3, gram[t].data(), lam[t].data(), zt[t].data()); });
+    pool.reserve(ntab);
+    int started = 0;
+    try {
+      for (; started < ntab; ++started) pool.emplace_back(eig, started);
+    } catch (const std::exception &) {           // no further thread to be had: the rest here
+    }
+    for (int t = started; t < ntab; ++t) eig(t);
     for (auto &th : pool) th.join();
   }
   int rmax = 1;
   std::vector<int> rank(ntab);
-  for (int t = 0; t < ntab; ++t)
+  for (int t = 0; t < ntab; ++t) {
+    if (rc[t] == -2) return make_err(AFMPB_ENOMEM, "M2L compression: no host memory for the eigensolver");
     if (rc[t] != 0) return make_err(AFMPB_EINTERNAL, "M2L compression: eigensolver did not converge");
+  }
   for (int t = 0; t < ntab; ++t) {
     // Singular values of the stacked operators are the square roots of the eigenvalues.
     // The cut is relative to the larger of the table's own largest singular value and
