@@ -647,6 +647,11 @@ constexpr int kP2PRegBlocks = kP2PResident;
 // (3 e2 = 3 e1 + e (kr)^2, and (kr)^2 p2 = k^2 P) the four sums are
 //   PhiL += (p2/eps_bar + c)/r,              dn PhiL += (1/eps_bar) [m + (1 - eps_bar) c Q]/r^3,
 //   PhiY += e (k1 p2 + c)/r,                 dn PhiY += e (k1 m - k^2 P Q)/r^3.
+// For eps_bar < 1 the bracket of dn PhiL would cancel down to eps_bar c Q under a factor
+// 1/eps_bar (eps_in 80, eps_out 2: 15 times the rounding of its terms), so there
+//   u = S - (3 p2 + eps_bar c) Q,  dn PhiL += (1/eps_bar) u/r^3,  m = u + (eps_bar - 1) c Q,
+// where both parts of m have one sign as the bracket's have for eps_bar >= 1: one operation
+// more, in loops of their own (kLow).
 // The FP32 pipe bounds the kernel, so the count of its operations per pair is what this
 // form is for: 35 (43 in the order the formulas are printed in), 38 where the pair's
 // distance has to be tested, 25 and 27 without salt (k = 0: e = k1 = 1 and no exp2).
@@ -689,20 +694,23 @@ struct P2PConst {
   float2 kappa;          // k
   float2 nkl2e;          // -k log2(e)
   float2 kappa2;         // k^2
-  float2 omce;           // 1 - eps_bar
+  float2 wc;             // 1 - eps_bar (kLow: eps_bar - 1)
+};
+
+struct P2PSums {
+  float2 sL, nD, sY, dY; // a target's four sums (see p2p_pair2)
 };
 
 // sources: a = (-x0, -x1, -y0, -y1), b = (-z0, -z1, c0, c1), c = (gnx0, gnx1, gny0, gny1),
 // d = (gnz0, gnz1, w0, w1); positions in the target leaf's frame.  kTest: w = skip radius,
 // and pairs inside it contribute nothing here (the near CSR carries their whole near-rule
-// value; t == p is among them).  Otherwise no pair can be inside it and w = (1 - eps_bar) c.
+// value; t == p is among them).  Otherwise no pair can be inside it and w = wc c.
 // Sums: sL, sY as above; nD = eps_bar dn PhiL; dY.  Without salt the two kernels differ in
 // eps_bar alone and the product takes their difference: the parts with and without it are
 // summed apart, sL = sum p2/r, sY = sum c/r, nD = sum (S - 3 p2 Q)/r^3, dY = sum c Q/r^3.
-template <bool kTest, bool kSalt>
+template <bool kTest, bool kSalt, bool kLow>
 __device__ __forceinline__ void p2p_pair2(const P2PTarget &t, const float4 &a, const float4 &b, const float4 &c,
-                                          const float4 &d, const P2PConst &k, float2 &sL, float2 &nD, float2 &sY,
-                                          float2 &dY) {
+                                          const float4 &d, const P2PConst &k, P2PSums &s) {
   const float2 dx = __fadd2_rn(t.x, make_float2(a.x, a.y));
   const float2 dy = __fadd2_rn(t.y, make_float2(a.z, a.w));
   const float2 dz = __fadd2_rn(t.z, make_float2(b.x, b.y));
@@ -724,33 +732,53 @@ __device__ __forceinline__ void p2p_pair2(const P2PTarget &t, const float4 &a, c
   const float2 p2 = __fmul2_rn(P, ri2);
   const float2 G3 = __fmul2_rn(ri, ri2);
   if (!kSalt) {
-    sL = __ffma2_rn(ri, p2, sL);
-    sY = __ffma2_rn(ri, cc, sY);
-    nD = __ffma2_rn(G3, __ffma2_rn(__fmul2_rn(p2, Q), dup2(-3.0f), S), nD);
-    dY = __ffma2_rn(G3, __fmul2_rn(cc, Q), dY);
+    s.sL = __ffma2_rn(ri, p2, s.sL);
+    s.sY = __ffma2_rn(ri, cc, s.sY);
+    s.nD = __ffma2_rn(G3, __ffma2_rn(__fmul2_rn(p2, Q), dup2(-3.0f), S), s.nD);
+    s.dY = __ffma2_rn(G3, __fmul2_rn(cc, Q), s.dY);
     return;
   }
-  const float2 h = __ffma2_rn(p2, dup2(3.0f), cc);
-  const float2 m = __ffma2_rn(make_float2(-h.x, -h.y), Q, S);
-  const float2 dc = kTest ? __fmul2_rn(cc, k.omce) : make_float2(d.z, d.w);
-  nD = __ffma2_rn(G3, __ffma2_rn(dc, Q, m), nD);
-  sL = __ffma2_rn(ri, __ffma2_rn(k.inv_e, p2, cc), sL);
+  const float2 h = __ffma2_rn(p2, dup2(3.0f), kLow ? __fmul2_rn(cc, dup2(1.0f / k.inv_e.x)) : cc);
+  const float2 u = __ffma2_rn(make_float2(-h.x, -h.y), Q, S);
+  const float2 dc = kTest ? __fmul2_rn(cc, k.wc) : make_float2(d.z, d.w);
+  const float2 v = __ffma2_rn(dc, Q, u);
+  const float2 m = kLow ? v : u;
+  s.nD = __ffma2_rn(G3, kLow ? u : v, s.nD);
+  s.sL = __ffma2_rn(ri, __ffma2_rn(k.inv_e, p2, cc), s.sL);
   const float2 rr = __fmul2_rn(r2, ri);
   const float2 arg = __fmul2_rn(rr, k.nkl2e);
   const float2 ex = make_float2(ex2_approx(arg.x), ex2_approx(arg.y));
   const float2 k1 = __ffma2_rn(rr, k.kappa, dup2(1.0f));
   const float2 ei = __fmul2_rn(ex, ri);
-  sY = __ffma2_rn(ei, __ffma2_rn(k1, p2, cc), sY);
+  s.sY = __ffma2_rn(ei, __ffma2_rn(k1, p2, cc), s.sY);
   const float2 V = __fmul2_rn(__fmul2_rn(P, Q), k.kappa2);
-  dY = __ffma2_rn(__fmul2_rn(ei, ri2), __ffma2_rn(k1, m, make_float2(-V.x, -V.y)), dY);
+  s.dY = __ffma2_rn(__fmul2_rn(ei, ri2), __ffma2_rn(k1, m, make_float2(-V.x, -V.y)), s.dY);
 }
 
 // The sums of one target, (PhiL, dn PhiL, PhiY, dn PhiY) without the 1/(4 pi), from its
 // accumulators.
-__device__ __forceinline__ float4 p2p_sums(bool salt, float inv_e, float2 sL, float2 nD, float2 sY, float2 dY) {
-  const float a = sL.x + sL.y, b = nD.x + nD.y, c = sY.x + sY.y, d = dY.x + dY.y;
+__device__ __forceinline__ float4 p2p_sums(bool salt, float inv_e, const P2PSums &s) {
+  const float a = s.sL.x + s.sL.y, b = s.nD.x + s.nD.y, c = s.sY.x + s.sY.y, d = s.dY.x + s.dY.y;
   if (salt) return make_float4(a, inv_e * b, c, d);
   return make_float4(fmaf(inv_e, a, c), fmaf(inv_e, b, -d), a + c, b - d);
+}
+
+// A thread's share of a staged chunk: pairs e, e + slices, ... of its tested part (below
+// ntest), then of the others, for both of its targets.
+template <bool kSalt, bool kLow>
+__device__ __forceinline__ void p2p_chunk(int e, int slices, int ntest, int npairs, const float4 *sa, const float4 *sb,
+                                          const float4 *sc, const float4 *sd, const P2PTarget &tg, const P2PTarget &tg2,
+                                          const P2PConst &kc, P2PSums &acc, P2PSums &acc2) {
+  for (; e < ntest; e += slices) {
+    const float4 qa = sa[e], qb = sb[e], qc = sc[e], qd = sd[e];
+    p2p_pair2<true, kSalt, kLow>(tg, qa, qb, qc, qd, kc, acc);
+    p2p_pair2<true, kSalt, kLow>(tg2, qa, qb, qc, qd, kc, acc2);
+  }
+  for (; e < npairs; e += slices) {
+    const float4 qa = sa[e], qb = sb[e], qc = sc[e], qd = sd[e];
+    p2p_pair2<false, kSalt, kLow>(tg, qa, qb, qc, qd, kc, acc);
+    p2p_pair2<false, kSalt, kLow>(tg2, qa, qb, qc, qd, kc, acc2);
+  }
 }
 
 // A unit that covers its leaf's whole source list stores; a part of a split leaf adds.
@@ -799,9 +827,9 @@ __device__ __forceinline__ void p2p_body(const P2PUnit *__restrict__ units,
     kc.kappa = dup2(kap);
     kc.nkl2e = dup2(-1.4426950408889634f * kap);
     kc.kappa2 = dup2(kap * kap);
-    kc.omce = dup2(1.0f - 1.0f / inv_e);
+    kc.wc = dup2(inv_e > 1.0f ? 1.0f / inv_e - 1.0f : 1.0f - 1.0f / inv_e);
   }
-  const bool salt = kc.kappa.x > 0.0f;
+  const bool salt = kc.kappa.x > 0.0f, low = kc.inv_e.x > 1.0f;
   const int4 rec = P2P_ARG(leaf_rec)[unit.x];
   const int tb = rec.y, te = rec.z;
   // each thread takes two targets, t and t + tile, against the same sources
@@ -827,8 +855,7 @@ __device__ __forceinline__ void p2p_body(const P2PUnit *__restrict__ units,
       tg2.nx = dup2(nq.x); tg2.ny = dup2(nq.y); tg2.nz = dup2(nq.z);
       tg2.rs = dup2(p2p_skip_radius(P2P_ARG(skip_scale), nq.w));
     }
-    float2 sL = dup2(0.f), nD = dup2(0.f), sY = dup2(0.f), dY = dup2(0.f);
-    float2 sL2 = dup2(0.f), nD2 = dup2(0.f), sY2 = dup2(0.f), dY2 = dup2(0.f);
+    P2PSums acc{}, acc2{};
     for (int c0 = 0; c0 < total; c0 += kP2PChunk) {
       const int cnt = min(kP2PChunk, total - c0);
       const int npairs = (cnt + 1) >> 1;
@@ -863,7 +890,7 @@ __device__ __forceinline__ void p2p_body(const P2PUnit *__restrict__ units,
           fb[ln] = -pz; fb[2 + ln] = cw;
           fc[ln] = g * q.x; fc[2 + ln] = g * q.y;
           fd[ln] = g * q.z;
-          fd[2 + ln] = tested ? p2p_skip_radius(P2P_ARG(skip_scale), q.w) : cw * kc.omce.x;
+          fd[2 + ln] = tested ? p2p_skip_radius(P2P_ARG(skip_scale), q.w) : cw * kc.wc.x;
           // the odd slot after the last source of either part: its neighbour's place, no
           // weight, and in the tested part a radius that leaves it out
           if (ln == 0 && (j + 1 == nf || j + 1 == total)) {
@@ -877,34 +904,13 @@ __device__ __forceinline__ void p2p_body(const P2PUnit *__restrict__ units,
       }
       __syncthreads();
       if (act) {
-        int e = si;
-        if (salt) {
-          for (; e < ntest; e += slices) {
-            const float4 qa = sa[e], qb = sb[e], qc = sc[e], qd = sd[e];
-            p2p_pair2<true, true>(tg, qa, qb, qc, qd, kc, sL, nD, sY, dY);
-            p2p_pair2<true, true>(tg2, qa, qb, qc, qd, kc, sL2, nD2, sY2, dY2);
-          }
-          for (; e < npairs; e += slices) {
-            const float4 qa = sa[e], qb = sb[e], qc = sc[e], qd = sd[e];
-            p2p_pair2<false, true>(tg, qa, qb, qc, qd, kc, sL, nD, sY, dY);
-            p2p_pair2<false, true>(tg2, qa, qb, qc, qd, kc, sL2, nD2, sY2, dY2);
-          }
-        } else {
-          for (; e < ntest; e += slices) {
-            const float4 qa = sa[e], qb = sb[e], qc = sc[e], qd = sd[e];
-            p2p_pair2<true, false>(tg, qa, qb, qc, qd, kc, sL, nD, sY, dY);
-            p2p_pair2<true, false>(tg2, qa, qb, qc, qd, kc, sL2, nD2, sY2, dY2);
-          }
-          for (; e < npairs; e += slices) {
-            const float4 qa = sa[e], qb = sb[e], qc = sc[e], qd = sd[e];
-            p2p_pair2<false, false>(tg, qa, qb, qc, qd, kc, sL, nD, sY, dY);
-            p2p_pair2<false, false>(tg2, qa, qb, qc, qd, kc, sL2, nD2, sY2, dY2);
-          }
-        }
+        if (!salt) p2p_chunk<false, false>(si, slices, ntest, npairs, sa, sb, sc, sd, tg, tg2, kc, acc, acc2);
+        else if (!low) p2p_chunk<true, false>(si, slices, ntest, npairs, sa, sb, sc, sd, tg, tg2, kc, acc, acc2);
+        else p2p_chunk<true, true>(si, slices, ntest, npairs, sa, sb, sc, sd, tg, tg2, kc, acc, acc2);
       }
     }
-    red[threadIdx.x] = p2p_sums(salt, kc.inv_e.x, sL, nD, sY, dY);
-    red[kP2PThreads + threadIdx.x] = p2p_sums(salt, kc.inv_e.x, sL2, nD2, sY2, dY2);
+    red[threadIdx.x] = p2p_sums(salt, kc.inv_e.x, acc);
+    red[kP2PThreads + threadIdx.x] = p2p_sums(salt, kc.inv_e.x, acc2);
     __syncthreads();                                           // the sums are there, the last chunk is free
     if (si == 0 && t < te) {
       const float s = (float)kInv4Pi;
