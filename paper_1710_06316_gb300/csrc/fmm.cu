@@ -1178,10 +1178,6 @@ Err enqueue_far(afmpb_t *h, cudaStream_t s, StageTimer *tm, int parts, const Far
   }
 }
 
-// kappa as the P2P pass takes it: k^2 enters it, so a value whose screening is complete
-// (e^-kr = 0 for every r above 1e-13) is cut to where k^2 and its products stay finite.
-static float p2p_kappa(const afmpb_t *h) { return (float)std::min(h->kappa, 1e15); }
-
 const void *far_out_kernel(int order) {
   switch (order) {
     case 2: return (const void *)k_l2p<2, 2>;
@@ -1201,7 +1197,7 @@ Err enqueue_p2p(afmpb_t *h, cudaStream_t s) {
   AFMPB_CUDA(cudaMemsetAsync(h->d_phi_near, 0, sizeof(float4) * h->n, s));   // split leaves add into it
   if (h->p2p_nunits == 0) return Err{};
   k_p2p<<<h->p2p_nunits, kP2PThreads, 0, s>>>(h->d_p2p_units, h->d_leaf_rec, h->d_p2p_src, h->d_p2p_slot, h->d_pos,
-                                     h->d_nrm, h->d_xs, (float)(1.0 / h->ebar), p2p_kappa(h),
+                                     h->d_nrm, h->d_xs, (float)(1.0 / h->ebar), (float)h->kappa_p2p,
                                      (float)(kP2PSkip * h->opt.near_c), h->d_phi_near);
   return check_launch("k_p2p");
 }
@@ -1217,7 +1213,7 @@ P2PReq p2p_req_of(const afmpb_t *h, const int *active) {
   q.phi = h->d_phi_near;
   q.active = active;
   q.inv_ebar = (float)(1.0 / h->ebar);
-  q.kappa = p2p_kappa(h);
+  q.kappa = (float)h->kappa_p2p;
   q.skip_scale = (float)(kP2PSkip * h->opt.near_c);
   return q;
 }

@@ -827,6 +827,26 @@ Err build_p2p_units(afmpb_t *h) {
   return Err{};
 }
 
+// kappa as the P2P pass takes it.  (kr)^2 enters it, which must not overflow where e^-kr has
+// long vanished, so a kappa that screens every evaluated pair completely (e^-200 is no FP32
+// number; P2P leaves out distances up to kP2PSkip near_c times two patch radii) is cut to the
+// value that just does.  Below kappa w0 = 1e4 no square is near the range's end, and the
+// smallest radius is not read.
+static Err set_p2p_kappa(afmpb_t *h) {
+  h->kappa_p2p = std::min(h->kappa, 1e15);
+  if (h->laplace_only || h->kappa * h->shape.w0 <= 1e4) return Err{};
+  double *d_min = nullptr, rho = 0;
+  AFMPB_TRY(h->arena.alloc(&d_min, 1, "smallest patch radius"));
+  AFMPB_TRY(cub_call(h, "smallest patch radius", [&](void *t, size_t &bytes) {
+    return cub::DeviceReduce::Min(t, bytes, h->d_rho64, d_min, (int)h->n, h->stream);
+  }));
+  AFMPB_TRY(read_one(&rho, d_min, h->stream));
+  h->arena.release(d_min);
+  const double d = 2.0 * kP2PSkip * h->opt.near_c * rho;
+  if (h->kappa * d > 200.0) h->kappa_p2p = 200.0 / d;
+  return Err{};
+}
+
 Err build_tree(afmpb_t *h) {
   const int64_t n = h->n;
   cudaStream_t s = h->stream;
@@ -1252,6 +1272,7 @@ Err build_tree(afmpb_t *h) {
                                                                 kP2PSkip * h->opt.near_c, h->d_p2p_test);
   AFMPB_TRY(check_launch("k_p2p_test"));
   A.release(d_ext);
+  AFMPB_TRY(set_p2p_kappa(h));
   AFMPB_TRY(build_p2p_units(h));
   A.release(d_cnt1);
   A.release(d_cnt2);

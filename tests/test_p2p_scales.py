@@ -1,6 +1,7 @@
 """The point-to-point sums away from a solvated protein's constants: dielectric contrast below
-one (a droplet of the polar medium).  Reference: the pair terms in float64, each with its own
-rounding bound, so that an error that grows with the contrast shows."""
+one (a droplet of the polar medium), and complete screening.  Reference: the pair terms in
+float64, each with its own rounding bound, so that an error that grows with the contrast
+shows."""
 import numpy as np
 import pytest
 
@@ -46,3 +47,17 @@ def test_charge_sums_at_low_contrast(eps_out):
     q = np.abs(mol.q) / (4 * np.pi * eps_out)
     bound = np.concatenate([(eps * q / r).sum(1), (eps * q / r ** 2).sum(1)])
     assert np.all(np.abs(b - ref) <= bound), np.max(np.abs(b - ref) / bound)
+
+@pytest.mark.parametrize("kappa,radius", [(1e20, 2.0), (1e20, 2000.0), (1e12, 2e4), (50.0, 2.0)])
+def test_pairs_at_complete_screening(kappa, radius):
+    """Screening lengths far below every distance (the limit of a conducting solvent): the
+    screened sums vanish, whatever the mesh's unit."""
+    import paper_1710_06316_gb300 as pb
+    mol = synthetic.born_ion(subdiv=2, radius=radius, kappa=kappa)
+    o = oracle.Oracle.for_molecule(mol)
+    x = synthetic.random_unknowns(mol.n_nodes, 4).astype(np.float32).astype(np.float64)
+    with pb.Handle.for_molecule(mol, order=4, leaf_cap=4096) as h:
+        y = far_parts(h, x)
+        ref, bound = pair_sums(mol, o, whole_matrix(h), x)
+    assert np.all(np.isfinite(y))
+    assert np.all(np.abs(y - ref) <= bound), np.max(np.abs(y - ref) / bound)
