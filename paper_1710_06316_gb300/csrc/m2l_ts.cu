@@ -43,6 +43,9 @@ namespace afmpb {
 constexpr int kTsRows = 128;                   // target boxes per block (MMA M, TMEM lanes)
 constexpr int kTsThreads = 288;                // 4 gather warps, 4 epilogue warps, 1 MMA warp
 constexpr int kTsMaxR = 112;                   // largest compressed rank this kernel takes
+// Operand stages: two, so that two CTAs fit an SM at rank 64 (94 us on the 163,842-node sphere
+// against 122 us with four stages, a warp to each, on one CTA per SM).
+constexpr int kTsStages = 2;
 constexpr int kTsItemRuns = 32;                // most runs (offsets) in one item
 constexpr int kTsItemEnt = 768;                // most entries (translated pairs) in one item
 // Levels with at least this many boxes are blocked by octant: eight part-filled blocks of
@@ -134,7 +137,7 @@ __device__ __forceinline__ void red_add_v4(float *addr, float a, float b, float 
 // With kBatch the items of several problems share the launch: item.req names the problem
 // whose runs, entries, multipoles, tables and local expansions (reqs[item.req]) it uses,
 // and the item count is read from *d_nitems (a list compacted to the running problems).
-template <int NS, bool kBatch>
+template <bool kBatch>
 __global__ void __launch_bounds__(kTsThreads) k_m2l_ts(int R, int nitems_arg, const TSItem *__restrict__ items,
                                                       const int4 *__restrict__ runs_1,
                                                       const uint4 *__restrict__ masks_1,
@@ -145,6 +148,7 @@ __global__ void __launch_bounds__(kTsThreads) k_m2l_ts(int R, int nitems_arg, co
                                                       float *__restrict__ Lc_1, int *__restrict__ err_flag,
                                                       const int *__restrict__ d_nitems,
                                                       const TSReq *__restrict__ reqs) {
+  constexpr int NS = kTsStages;
   extern __shared__ __align__(128) uint8_t smem[];
   after_previous();
   const int nitems = kBatch ? *d_nitems : nitems_arg;
@@ -441,10 +445,7 @@ __global__ void __launch_bounds__(kTsThreads) k_m2l_ts(int R, int nitems_arg, co
 
 namespace {
 int ts_stage_bytes(int R) { return 2 * kTsRows * R * 2 + 2 * R * R * 2; }   // A hi, lo + B hi, lo
-// Two operand stages, two CTAs per SM (R <= 64): measured on the 163,842-node sphere,
-// 94 us against 122 us with four stages (a warp to each) on one CTA per SM
-int ts_stages(int) { return 2; }
-int ts_smem_bytes(int R) { return ts_stages(R) * ts_stage_bytes(R); }
+int ts_smem_bytes(int R) { return kTsStages * ts_stage_bytes(R); }
 }  // namespace
 
 bool m2l_ts_applies(const afmpb_t *h) { return h->m2l_rank > 0 && h->m2l_rank <= kTsMaxR && h->d_Mc16; }
@@ -566,13 +567,8 @@ Err build_m2l_ts(afmpb_t *h) {
   k_ts_tables<<<2048, 256, 0, s>>>(R, h->m2l_ntables, h->d_C, reinterpret_cast<__nv_bfloat16 *>(h->d_ts_tiles));
   AFMPB_TRY(check_launch("k_ts_tables"));
   AFMPB_TRY(alloc_wait_flag(h));
-  if (ts_stages(R) == 4) {
-    AFMPB_TRY(raise_smem_limit((const void *)k_m2l_ts<4, false>, ts_smem_bytes(R)));
-    AFMPB_TRY(raise_smem_limit((const void *)k_m2l_ts<4, true>, ts_smem_bytes(R)));
-  } else {
-    AFMPB_TRY(raise_smem_limit((const void *)k_m2l_ts<2, false>, ts_smem_bytes(R)));
-    AFMPB_TRY(raise_smem_limit((const void *)k_m2l_ts<2, true>, ts_smem_bytes(R)));
-  }
+  AFMPB_TRY(raise_smem_limit((const void *)k_m2l_ts<false>, ts_smem_bytes(R)));
+  AFMPB_TRY(raise_smem_limit((const void *)k_m2l_ts<true>, ts_smem_bytes(R)));
   AFMPB_CUDA(cudaStreamSynchronize(s));
   return Err{};
 }
@@ -653,10 +649,7 @@ Err enqueue_m2l_ts(afmpb_t *h, cudaStream_t s) {
   const unsigned grid = (unsigned)std::min(h->ts_nitems, per_sm * sms);
   const auto *mc = reinterpret_cast<const __nv_bfloat16 *>(h->d_Mc16);
   const auto *tl = reinterpret_cast<const __nv_bfloat16 *>(h->d_ts_tiles);
-  if (ts_stages(R) == 4)
-    return launch_next(true, "k_m2l_ts", k_m2l_ts<4, false>, grid, kTsThreads, ts_smem_bytes(R), s, R, h->ts_nitems, h->d_ts_items,
-                       h->d_ts_runs, h->d_ts_masks, h->d_ts_ent, h->d_ts_box, mc, tl, h->d_Lc, h->d_tc_flag, nullptr, nullptr);
-  return launch_next(true, "k_m2l_ts", k_m2l_ts<2, false>, grid, kTsThreads, ts_smem_bytes(R), s, R, h->ts_nitems, h->d_ts_items,
+  return launch_next(true, "k_m2l_ts", k_m2l_ts<false>, grid, kTsThreads, ts_smem_bytes(R), s, R, h->ts_nitems, h->d_ts_items,
                        h->d_ts_runs, h->d_ts_masks, h->d_ts_ent, h->d_ts_box, mc, tl, h->d_Lc, h->d_tc_flag, nullptr, nullptr);
 }
 
@@ -715,12 +708,8 @@ Err enqueue_m2l_ts_batch(const TSReq *d_reqs, const TSItem *d_items, int nitems,
   AFMPB_TRY(check_launch("k_ts_compact"));
   const int per_sm = std::max(1, std::min(2, (227 * 1024) / (ts_smem_bytes(R) + 16 * 1024)));
   const unsigned grid = (unsigned)std::min(nitems, per_sm * sms);
-  if (ts_stages(R) == 4)
-    k_m2l_ts<4, true><<<grid, kTsThreads, ts_smem_bytes(R), s>>>(R, 0, d_items_run, nullptr, nullptr, nullptr, nullptr,
-                                                                 nullptr, nullptr, nullptr, err_flag, d_count, d_reqs);
-  else
-    k_m2l_ts<2, true><<<grid, kTsThreads, ts_smem_bytes(R), s>>>(R, 0, d_items_run, nullptr, nullptr, nullptr, nullptr,
-                                                                 nullptr, nullptr, nullptr, err_flag, d_count, d_reqs);
+  k_m2l_ts<true><<<grid, kTsThreads, ts_smem_bytes(R), s>>>(R, 0, d_items_run, nullptr, nullptr, nullptr, nullptr, nullptr,
+                                                            nullptr, nullptr, err_flag, d_count, d_reqs);
   return check_launch("k_m2l_ts batch");
 }
 

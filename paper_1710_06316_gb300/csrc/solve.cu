@@ -700,8 +700,7 @@ Err enqueue_cycle_xs(afmpb_t *h, cudaStream_t s, const int *act) {
 
 Err enqueue_step_tail(afmpb_t *h, int m, cudaStream_t cap, const int *act, bool batch, cudaGraphConditionalHandle loop) {
   const int64_t n = h->n, n2 = 2 * n;
-  const int orth = h->opt.orth;
-  if (orth == 0) {
+  if (h->opt.orth == 0) {
     // a tile to a block, more of them above the partial sums' 1,184 blocks
     const int64_t chunk = ((n2 + 1183) / 1184 + kGsTile - 1) / kGsTile * kGsTile;
     const int nb = div_up(n2, chunk), stride = m + 2;
@@ -724,29 +723,17 @@ Err enqueue_step_tail(afmpb_t *h, int m, cudaStream_t cap, const int *act, bool 
   const int nb_el = div_up(n, 256), nb_el2 = div_up(n2, 256);
   const int nb_comb = std::min(nb_el2, 4 * 1184);
   k_from_ys<<<nb_el2, 256, 0, cap>>>(n2, h->d_ys, nullptr, h->d_w, act);
-  if (orth == 0) {      // classical Gram-Schmidt twice, then the norm: three reductions
-    k_multidot_j<<<nb, kRedThreads, 0, cap>>>(n2, gm, h->d_V, n2, h->d_w, h->d_part, stride, 0, first);
-    k_reduce_parts_j<<<m + 1, 256, 0, cap>>>(nb, gm, 0, h->d_part, stride, h->d_hcol, first);
-    k_sub_combo_j<<<nb_comb, 256, 0, cap>>>(n2, gm, h->d_V, n2, h->d_hcol, h->d_w, first);
-    k_multidot_j<<<nb, kRedThreads, 0, cap>>>(n2, gm, h->d_V, n2, h->d_w, h->d_part, stride, 0, first);
-    k_reduce_parts_j<<<m + 1, 256, 0, cap>>>(nb, gm, 0, h->d_part, stride, h->d_hcol2, first);
-    k_sub_combo_j<<<nb_comb, 256, 0, cap>>>(n2, gm, h->d_V, n2, h->d_hcol2, h->d_w, first);
-    k_add_small_j<<<1, 128, 0, cap>>>(gm, h->d_hcol2, h->d_hcol, first);
-    if (act) k_multidot_j<<<nb, kRedThreads, 0, cap>>>(n2, gm, h->d_V, n2, h->d_w, h->d_part, stride, 2, act);
-    else k_multidot<<<nb, kRedThreads, 0, cap>>>(n2, 1, h->d_w, 0, h->d_w, h->d_part, stride);
-    k_norm_to_j<<<1, 256, 0, cap>>>(nb, h->d_part, stride, gm, h->d_hcol, first);
-  } else {              // one fused reduction; a guarded second pass on loss of orthogonality
-    k_multidot_j<<<nb, kRedThreads, 0, cap>>>(n2, gm, h->d_V, n2, h->d_w, h->d_part, stride, 1, first);
-    k_reduce_parts_j<<<m + 2, 256, 0, cap>>>(nb, gm, 1, h->d_part, stride, h->d_hcol, first);
-    k_sub_combo_j<<<nb_comb, 256, 0, cap>>>(n2, gm, h->d_V, n2, h->d_hcol, h->d_w, first);
-    k_pythagoras_j<<<1, 1, 0, cap>>>(gmw, h->d_hcol, act);
-    k_multidot_j<<<nb, kRedThreads, 0, cap>>>(n2, gm, h->d_V, n2, h->d_w, h->d_part, stride, 0, guard);
-    k_reduce_parts_j<<<m + 1, 256, 0, cap>>>(nb, gm, 0, h->d_part, stride, h->d_hcol2, guard);
-    k_sub_combo_j<<<nb_comb, 256, 0, cap>>>(n2, gm, h->d_V, n2, h->d_hcol2, h->d_w, guard);
-    k_add_small_j<<<1, 128, 0, cap>>>(gm, h->d_hcol2, h->d_hcol, guard);
-    k_multidot_j<<<nb, kRedThreads, 0, cap>>>(n2, gm, h->d_V, n2, h->d_w, h->d_part, stride, 2, guard);
-    k_norm_to_j<<<1, 256, 0, cap>>>(nb, h->d_part, stride, gm, h->d_hcol, guard);
-  }
+  // one fused reduction; a guarded second pass on loss of orthogonality
+  k_multidot_j<<<nb, kRedThreads, 0, cap>>>(n2, gm, h->d_V, n2, h->d_w, h->d_part, stride, 1, first);
+  k_reduce_parts_j<<<m + 2, 256, 0, cap>>>(nb, gm, 1, h->d_part, stride, h->d_hcol, first);
+  k_sub_combo_j<<<nb_comb, 256, 0, cap>>>(n2, gm, h->d_V, n2, h->d_hcol, h->d_w, first);
+  k_pythagoras_j<<<1, 1, 0, cap>>>(gmw, h->d_hcol, act);
+  k_multidot_j<<<nb, kRedThreads, 0, cap>>>(n2, gm, h->d_V, n2, h->d_w, h->d_part, stride, 0, guard);
+  k_reduce_parts_j<<<m + 1, 256, 0, cap>>>(nb, gm, 0, h->d_part, stride, h->d_hcol2, guard);
+  k_sub_combo_j<<<nb_comb, 256, 0, cap>>>(n2, gm, h->d_V, n2, h->d_hcol2, h->d_w, guard);
+  k_add_small_j<<<1, 128, 0, cap>>>(gm, h->d_hcol2, h->d_hcol, guard);
+  k_multidot_j<<<nb, kRedThreads, 0, cap>>>(n2, gm, h->d_V, n2, h->d_w, h->d_part, stride, 2, guard);
+  k_norm_to_j<<<1, 256, 0, cap>>>(nb, h->d_part, stride, gm, h->d_hcol, guard);
   k_normalize_j<<<nb_el, 256, 0, cap>>>(n, h->d_w, h->d_hcol, gm, h->d_V, n2, act);
   k_givens_j<<<1, 1, 0, cap>>>(gm, m, h->d_hcol, h->d_H, h->d_cs, h->d_sn, h->d_g, h->d_scal + 2, act);
   if (batch) k_step_end_b<<<1, 1, 0, cap>>>(gmw, m, h->d_scal + 2, h->d_scal + 4);
