@@ -194,8 +194,8 @@ typedef struct {
     double ms_per_m2l_pair, ms_per_box, ms_rest;
     double ms_tuning;          /* host time of the calibration and the candidate trees   */
     /* Tile shapes, chosen on the handle built at best_cap by timing the kernels themselves:
-     * P2P work units cut for blocks per SM (4-6) x units per block (1-6), and the number of
-     * offsets per work item of the tensor-core M2L (8-32; 0 when that kernel is not used). */
+     * P2P work units per resident block (1-6; p2p_resident blocks per SM, a constant of the
+     * kernel), and offsets per work item of the tensor-core M2L (8-32; 0 when not used). */
     int p2p_resident, p2p_units_per_block, m2l_runs_per_item;
     double p2p_ms_default, p2p_ms_tuned;   /* P2P at the library defaults and at the choice  */
     double m2l_ms_default, m2l_ms_tuned;   /* the same for the M2L translations              */

@@ -12,8 +12,8 @@
 //   3. predicts the product time  t(s) = t_P2P(s) + b * pairs_V(s) + c * boxes(s) + t_rest
 //      and keeps the smallest.
 // Then, on the handle at the chosen capacity, the tile shapes of the two heaviest kernels
-// are picked by timing them: the size of the P2P work units (by the blocks per SM and the
-// units per block that it is cut for), and the number of offsets per work item of the tensor-core M2L.
+// are picked by timing them: the size of the P2P work units (units per resident block), and
+// the number of offsets per work item of the tensor-core M2L.
 // The choices are cached per (precision, order, screened or not, log2 of the node count),
 // so later handles of the same size class skip the tuning.
 #include <chrono>
@@ -85,7 +85,7 @@ Err time_candidate(afmpb_t *h, int cap, int reps, double *p2p_ms, int64_t *m2l_p
 
 std::mutex g_cache_mu;
 std::map<std::tuple<int, int, int, int, int>, int> g_cache;
-struct Tiles { int resident, units, runs; };
+struct Tiles { int units, runs; };
 std::map<std::tuple<int, int, int, int, int>, Tiles> g_tile_cache;
 
 // Mean time of `reps` launches of one stage on the handle's stream (after one warm-up).
@@ -118,33 +118,28 @@ std::tuple<int, int, int, int, int> cache_key(int precision, int order, double k
 
 }  // namespace
 
-// Tile shapes on the finished handle: the P2P work units (cut for resident blocks per SM x
-// units per block), then the M2L offsets per item, each by timing the kernel itself.  The product graphs are
-// captured again afterwards (they hold the launch shapes).
+// Tile shapes on the finished handle: the P2P units per resident block (the one number that
+// their size depends on), then the M2L offsets per item, each by timing the kernel itself.
+// The product graphs are captured again afterwards (they hold the launch shapes).
 Err autotune_tiles(afmpb_t *h, afmpb_autotune_report *rep) {
   constexpr int kReps = 5;
   auto p2p = [&]() { return enqueue_p2p(h, h->stream); };
   double ms = 0, best_ms = 0;
   AFMPB_TRY(time_stage(h, kReps, p2p, &best_ms));
   rep->p2p_ms_default = best_ms;
-  int best_r = h->p2p_resident, best_u = h->p2p_units_per_block;
+  int best_u = h->p2p_units_per_block;
   for (int u : {1, 2, 3, 4, 6}) {
     h->p2p_units_per_block = u;
-    for (int r : {4, 5, 6}) {
-      h->p2p_resident = r;
-      AFMPB_TRY(build_p2p_units(h));
-      AFMPB_TRY(time_stage(h, kReps, p2p, &ms));
-      if (ms < best_ms) {
-        best_ms = ms;
-        best_r = r;
-        best_u = u;
-      }
+    AFMPB_TRY(build_p2p_units(h));
+    AFMPB_TRY(time_stage(h, kReps, p2p, &ms));
+    if (ms < best_ms) {
+      best_ms = ms;
+      best_u = u;
     }
   }
-  h->p2p_resident = best_r;
   h->p2p_units_per_block = best_u;
   AFMPB_TRY(build_p2p_units(h));
-  rep->p2p_resident = best_r;
+  rep->p2p_resident = kP2PResident;
   rep->p2p_units_per_block = best_u;
   rep->p2p_ms_tuned = best_ms;
   if (m2l_ts_applies(h) && h->ts_nitems > 0) {
@@ -172,7 +167,7 @@ Err autotune_tiles(afmpb_t *h, afmpb_autotune_report *rep) {
 void autotune_cache_tiles(const afmpb_t *h) {
   std::lock_guard<std::mutex> lk(g_cache_mu);
   g_tile_cache[cache_key(h->opt.precision, h->order, h->kappa, h->n)] =
-      Tiles{h->p2p_resident, h->p2p_units_per_block, h->ts_runs_per_item};
+      Tiles{h->p2p_units_per_block, h->ts_runs_per_item};
 }
 
 // Applies the cached tile shapes of the handle's size class; false when there are none.
@@ -184,7 +179,6 @@ bool autotune_cached_tiles(afmpb_t *h) {
     if (it == g_tile_cache.end()) return false;
     t = it->second;
   }
-  h->p2p_resident = t.resident;
   h->p2p_units_per_block = t.units;
   h->ts_runs_per_item = t.runs;
   if (!build_p2p_units(h).ok()) return false;

@@ -316,7 +316,6 @@ struct afmpb_t {
   afmpb::P2PUnit *d_p2p_units = nullptr;   // [p2p_nunits] P2P work units, most pairs first
   int p2p_nunits = 0;
   double kappa_p2p = 0;            // kappa as P2P takes it (set with the tree)
-  int p2p_resident = afmpb::kP2PResident;            // P2P blocks per SM that the unit size is cut for (tile tuner)
   int p2p_units_per_block = afmpb::kP2PUnitsPerBlock;   // P2P unit size (tile tuner)
   int n_xbox = 0;                  // boxes whose list 4 goes to their local expansion (P2L)
   int32_t *d_xbox = nullptr;       // those boxes

@@ -784,7 +784,7 @@ Err build_p2p_units(afmpb_t *h) {
   AFMPB_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const int64_t pairs = h->shape.n_p2p_pairs + h->n;
   const int64_t budget =
-      std::max<int64_t>(4096, pairs / ((int64_t)h->p2p_resident * sms * std::max(1, h->p2p_units_per_block)));
+      std::max<int64_t>(4096, pairs / ((int64_t)kP2PResident * sms * std::max(1, h->p2p_units_per_block)));
   int64_t *cnt = nullptr;
   AFMPB_TRY(A.alloc(&cnt, nl + 1, "p2p unit counts"));
   AFMPB_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int64_t) * (nl + 1), s));
