@@ -18,11 +18,13 @@
 
 #include <algorithm>
 #include <array>
+#include <atomic>
 #include <cmath>
 #include <exception>
 #include <new>
 #include <thread>
 
+#include "host_threads.h"
 #include "internal.cuh"
 #include "symeig.h"
 
@@ -633,14 +635,18 @@ Err build_m2l_svd(afmpb_t *h, bool *compressed) {
         rc[t] = -2;
       }
     };
+    const HostThreads extra(ntab - 1);           // a table each, as far as granted
+    std::atomic<int> next{0};
+    const auto tables = [&] {
+      for (int t = next++; t < ntab; t = next++) eig(t);
+    };
     std::vector<std::thread> pool;
     pool.reserve(ntab);
-    int started = 0;
     try {
-      for (; started < ntab; ++started) pool.emplace_back(eig, started);
-    } catch (const std::exception &) {           // no further thread to be had: the rest here
+      for (int k = 0; k < extra.count(); ++k) pool.emplace_back(tables);
+    } catch (const std::exception &) {           // no further thread to be had
     }
-    for (int t = started; t < ntab; ++t) eig(t);
+    tables();
     for (auto &th : pool) th.join();
   }
   int rmax = 1;

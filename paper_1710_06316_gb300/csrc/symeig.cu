@@ -16,6 +16,7 @@
 #include <thread>
 #include <vector>
 
+#include "host_threads.h"
 #include "symeig.h"
 
 namespace afmpb {
@@ -148,8 +149,8 @@ void apply_columns(int n, int c0, int c1, const Record &rec, double *work, doubl
   for (int r = 0; r < n; ++r) std::copy(z + (size_t)r * w, z + (size_t)(r + 1) * w, zt + (size_t)r * n + c0);
 }
 
-// zt on up to four threads (the caller's among them; a thread that cannot be had leaves its
-// columns to it).
+// zt on up to four threads (the caller's among them; a thread that is not granted or cannot be
+// had leaves its columns to it).
 void apply_all(int n, const Record &rec, double *zt) {
   const int parts = n >= 128 ? 4 : 1;
   std::vector<double> work((size_t)(n + 1) * n);
@@ -157,11 +158,12 @@ void apply_all(int n, const Record &rec, double *zt) {
     const int c0 = n * t / parts, c1 = n * (t + 1) / parts;
     apply_columns(n, c0, c1, rec, work.data() + (size_t)(n + 1) * c0, zt);
   };
+  const HostThreads extra(parts - 1);
   std::vector<std::thread> pool;
   pool.reserve(parts);
   int started = 1;
   try {
-    for (; started < parts; ++started) pool.emplace_back(part, started);
+    for (; started <= extra.count(); ++started) pool.emplace_back(part, started);
   } catch (...) {
   }
   part(0);
