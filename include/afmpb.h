@@ -491,7 +491,7 @@ afmpb_status afmpb_server_destroy(afmpb_server_t *s);
  * and (b) from the arrays afmpb_get_tree and afmpb_get_near export, with the node ranges
  * cut between leaves so that the ranks' estimated work (targets x point-to-point sources +
  * near-field entries) is balanced.  No GPU is touched.  (The multi-GPU product kernels are
- * not part of this library: every GB300 machine here has one GPU.) */
+ * not part of this library, which runs one process on one GPU.) */
 typedef struct {
     int64_t n_nodes, n_boxes;
     const int32_t *box_range;    /* [n_boxes*2] node range in Morton order (a box's range

@@ -633,7 +633,7 @@ __global__ void __launch_bounds__(kL2PNodes) k_l2p(int64_t n, const int2 *__rest
 // ------------------------------------------------------------------------------------
 // P2P (lists 1 and 3): point (far-rule) sums over t != p, both kernels, both outputs.
 // ------------------------------------------------------------------------------------
-constexpr int kP2PChunk = 768;      // sources staged in shared memory at a time (8 CTAs/SM)
+constexpr int kP2PChunk = 768;      // sources staged in shared memory at a time (24 KB)
 constexpr int kP2PPairs = kP2PChunk / 2;
 constexpr int kP2PRegBlocks = kP2PResident;
 
@@ -1041,10 +1041,8 @@ Err init_cheb_tables() {
 
 // L and the compressed locals, beside the upward pass.  A kernel, since a memset node has no
 // priority and its blocks wait behind those of P2P (products of 163,842 nodes 416 us so, 400
-// with the kernel); few blocks, which leave room to the chain (608 in place of 76: a protein
-// surface of 191,944 nodes 570 against 561 us; 24: 570).
-constexpr int kZeroBlocks = 76;
-
+// with the kernel); half a block per SM, which leaves room to the chain (on 152 SMs 608 in
+// place of 76: a protein surface of 191,944 nodes 570 against 561 us; 24: 570).
 __global__ void __launch_bounds__(256) k_zero(int64_t na, float2 *__restrict__ a, int64_t nb, float2 *__restrict__ b) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < na + nb; i += (int64_t)gridDim.x * blockDim.x)
     (i < na ? a[i] : b[i - na]) = make_float2(0.f, 0.f);
@@ -1077,8 +1075,11 @@ Err launch_far(afmpb_t *h, cudaStream_t s, StageTimer *tm, int parts, const FarO
     AFMPB_CUDA(cudaStreamWaitEvent(z, h->ev_fork2, 0));
   }
   {
+    int dev = 0, sms = 0;
+    AFMPB_CUDA(cudaGetDevice(&dev));
+    AFMPB_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const int64_t nl = (int64_t)T.nbox * N3, nc = compressed ? (int64_t)T.nbox * h->m2l_rank : 0;
-    k_zero<<<(unsigned)std::min<int64_t>(div_up(nl + nc, 4 * 256), kZeroBlocks), 256, 0, z>>>(
+    k_zero<<<(unsigned)std::min(div_up(nl + nc, 4 * 256), std::max(1, sms / 2)), 256, 0, z>>>(
         nl, reinterpret_cast<float2 *>(h->d_L), nc, reinterpret_cast<float2 *>(h->d_Lc));
     AFMPB_TRY(check_launch("k_zero"));
   }

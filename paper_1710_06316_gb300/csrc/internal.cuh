@@ -169,7 +169,7 @@ struct TreeShape {
   std::vector<int> lvl_start;              // [nlevel + 1] box index ranges per level
   std::vector<int> par_start;              // [nlevel + 1] the same over the boxes with children
   double c0[3] = {0, 0, 0};                // root centre
-  double w0 = 1;                           // root half width (power of two)
+  double w0 = 1;                           // root half width
   int64_t n_u = 0, n_v = 0, n_w = 0, n_x = 0, n_p2p_pairs = 0;
 };
 
