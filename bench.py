@@ -434,9 +434,10 @@ def fp32_peak_tflops(sm_max_mhz, sms):
 P2P_FLOP_PER_PAIR = 54
 
 
-def ncu_traffic(kernel):
-    """Per-launch DRAM bytes from the committed ncu summary, if the source files of that
-    kernel (listed on its line) are unchanged since the capture."""
+def ncu_traffic(kernel, workload):
+    """Per-launch DRAM bytes from the committed ncu summary, if it was captured on this
+    workload (nodes, P2P pairs, order, precision) and the source files of that kernel
+    (listed on its line) are unchanged since."""
     p = os.path.join(ROOT, "profiles", "ncu_traffic.txt")
     if not os.path.exists(p):
         return None
@@ -444,7 +445,7 @@ def ncu_traffic(kernel):
     src = os.path.join(ROOT, "paper_1710_06316_gb300", "csrc")
     for line in open(p):
         t = line.split()
-        if len(t) >= 4 and not line.startswith("#") and t[0] == kernel:
+        if len(t) >= 5 and not line.startswith("#") and t[0] == kernel and t[4] == workload:
             h = hashlib.sha1()
             for f in t[3].split(","):
                 h.update(open(os.path.join(src, f), "rb").read())
@@ -502,7 +503,7 @@ def rooflines(prof, info, n, order, peaks, kind, precision, sms):
         if "useful_achieved" in e:
             e["useful_frac"] = round(e["useful_achieved"] / e["peak"], 4)
             e["useful_achieved"] = round(e["useful_achieved"], 3)
-        e["traffic"] = ncu_traffic(k)
+        e["traffic"] = ncu_traffic(k, "%d/%d/%d/%d" % (n, info["n_p2p_pairs"], order, precision))
     dom = max(out, key=lambda k: out[k]["ms_per_launch"])
     head = dict(out[dom], stage=dom, sms=sms,
                 stage_ms={k: round(v[0], 5) for k, v in stages.items()})

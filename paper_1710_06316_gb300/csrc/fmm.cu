@@ -651,7 +651,7 @@ constexpr int kP2PRegBlocks = kP2PResident;
 // 1/eps_bar (eps_in 80, eps_out 2: 15 times the rounding of its terms), so there
 //   u = S - (3 p2 + eps_bar c) Q,  dn PhiL += (1/eps_bar) u/r^3,  m = u + (eps_bar - 1) c Q,
 // where both parts of m have one sign as the bracket's have for eps_bar >= 1: one operation
-// more, in loops of their own (kLow).
+// more, in loops of their own (kLow; products of 163,842 nodes 394 us above, 393 below).
 // The FP32 pipe bounds the kernel, so the count of its operations per pair is what this
 // form is for: 35 (43 in the order the formulas are printed in), 38 where the pair's
 // distance has to be tested, 25 and 27 without salt (k = 0: e = k1 = 1 and no exp2).
