@@ -513,7 +513,10 @@ __global__ void __launch_bounds__(256) k_p2l(const int32_t *__restrict__ xbox, c
 // L2P: evaluate both local expansions and their normal derivatives at leaf targets.
 // One thread per node in Morton order, whatever leaf it is in: every lane has a node (a CTA
 // per leaf left 28 of 64 lanes idle on leaves of 36).  A CTA's nodes span a few leaves,
-// whose weights are staged in shared memory a few leaves at a time.  Each sum runs in
+// whose weights are staged in shared memory; where they span more than kL2PLeaves leaves, a
+// thread reads its leaf's weights from L2 instead.  (Staged round after round, for a few nodes
+// each time, L2P took 53 us on 642 nodes in leaves of three and 45 us on 163,842 in leaves of
+// ten; 12 and 27 us so.)  Each sum runs in
 // ascending order of its points: the gradient of a nearly constant field is a small
 // difference, and a sum in another order moves it by more than the rest of the product's
 // rounding (which rules out packed pairs along z; pairs along y or of value and derivative
@@ -527,7 +530,8 @@ __global__ void __launch_bounds__(256) k_p2l(const int32_t *__restrict__ xbox, c
 // (kOut == 2: caller order) or y[t] (kOut == 1).  That takes the combine and the scatter
 // (two launches and their passes over memory) off the end of the product.
 // ------------------------------------------------------------------------------------
-constexpr int kL2PLeaves = 6;
+constexpr int kL2PLeaves = 6;       // leaves staged
+constexpr int kL2PResident = 4;     // blocks per SM: registers for many of a thread's loads in flight
 
 // (phi, grad phi) of a local expansion at a node, the gradient in box half widths.
 template <int N>
@@ -567,7 +571,7 @@ __device__ __forceinline__ float4 l2p_eval(const float *Lk, const float (&sx)[N]
 }
 
 template <int N, int kOut>
-__global__ void __launch_bounds__(kL2PNodes) k_l2p(int64_t n, const int2 *__restrict__ blk,
+__global__ void __launch_bounds__(kL2PNodes, kL2PResident) k_l2p(int64_t n, const int2 *__restrict__ blk,
                                                    const int4 *__restrict__ leaf_rec, float inv_w0,
                                                    const float4 *__restrict__ pos, const float4 *__restrict__ nrm,
                                                    const float *__restrict__ L, float4 *__restrict__ phi,
@@ -592,22 +596,8 @@ __global__ void __launch_bounds__(kL2PNodes) k_l2p(int64_t n, const int2 *__rest
       if (kOut == 2) o = perm[t];
     }
   }
-  for (int l0 = lr.x; l0 <= lr.y; l0 += kL2PLeaves) {
-    const int nl = min(kL2PLeaves, lr.y + 1 - l0);
-    if (l0 > lr.x) __syncthreads();
-    if (threadIdx.x < nl) srec[threadIdx.x] = leaf_rec[l0 + threadIdx.x];
-    __syncthreads();
-#pragma unroll 4
-    for (int e = threadIdx.x; e < nl * N3; e += kL2PNodes) {     // two weights at a time
-      const int l = e / N3;
-      reinterpret_cast<float2 *>(&sL[0][0])[e] =
-          reinterpret_cast<const float2 *>(L + (size_t)srec[l].x * 2 * N3)[e - l * N3];
-    }
-    __syncthreads();
-    int l = 0;
-    while (l + 1 < nl && t >= srec[l].z) ++l;
-    if (!node || t < srec[l].y || t >= srec[l].z) continue;
-    const float invw = inv_width(inv_w0, srec[l].w);
+  auto eval = [&](const float *w, int level) {          // this thread's node, from its leaf's weights
+    const float invw = inv_width(inv_w0, level);
     float sx[N], dsx[N], sy[N], dsy[N];
     float sz[N], dsz[N];
     cheb_basis<N>(p.z * invw, sz, dsz);
@@ -616,7 +606,7 @@ __global__ void __launch_bounds__(kL2PNodes) k_l2p(int64_t n, const int2 *__rest
     float2 out[2];
 #pragma unroll 1
     for (int kt = 0; kt < 2; ++kt) {
-      const float4 v = l2p_eval<N>(&sL[l][kt * N3], sx, dsx, sy, dsy, sz, dsz);
+      const float4 v = l2p_eval<N>(w + kt * N3, sx, dsx, sy, dsy, sz, dsz);
       const float2 u = make_float2(v.x, (q.x * v.y + q.y * v.z + q.z * v.w) * invw);
       if (kt == 0) out[0] = u;
       else out[1] = u;
@@ -627,7 +617,33 @@ __global__ void __launch_bounds__(kL2PNodes) k_l2p(int64_t n, const int2 *__rest
     } else {
       phi[t] = make_float4(out[0].x, out[0].y, out[1].x, out[1].y);
     }
+  };
+  if (lr.y - lr.x >= kL2PLeaves) {                      // small leaves
+    if (!node) return;
+    int lo = lr.x, hi = lr.y;                           // the leaf whose nodes end after t
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if (leaf_rec[mid].z > t) hi = mid;
+      else lo = mid + 1;
+    }
+    const int4 rec = leaf_rec[lo];
+    eval(L + (size_t)rec.x * 2 * N3, rec.w);
+    return;
   }
+  const int nl = lr.y + 1 - lr.x;
+  if (threadIdx.x < nl) srec[threadIdx.x] = leaf_rec[lr.x + threadIdx.x];
+  __syncthreads();
+#pragma unroll 4
+  for (int e = threadIdx.x; e < nl * N3; e += kL2PNodes) {       // two weights at a time
+    const int l = e / N3;
+    reinterpret_cast<float2 *>(&sL[0][0])[e] =
+        reinterpret_cast<const float2 *>(L + (size_t)srec[l].x * 2 * N3)[e - l * N3];
+  }
+  __syncthreads();
+  if (!node) return;
+  int l = 0;
+  while (l + 1 < nl && t >= srec[l].z) ++l;
+  eval(&sL[l][0], srec[l].w);
 }
 
 // ------------------------------------------------------------------------------------
