@@ -69,39 +69,51 @@ __device__ __forceinline__ float2 dup2(float a) { return make_float2(a, a); }
 // ------------------------------------------------------------------------------------
 // P2M: leaf sources -> Laplace and Yukawa multipole weights.
 //   A[ijk] += c Sx[i] (Sy[j] Sz[k]),  B[ijk] += dSx[i] (g_x Sy Sz) + Sx[i] (g_y dSy Sz + g_z Sy dSz)
-// A leaf takes 2 N lanes of a warp (so N = 6 puts two leaves in a warp, N = 8 two, N = 4
-// four): lane (half, k) holds the weights (., j, k) of both sums for half of the j, so that
-// a node's factors are read once per N N / 2 weights, and the x direction runs on packed
-// FP32 pairs.  Each weight adds its leaf's nodes in order.  Instruction issue bounds it: a
-// thread per (j, k) with N weights took 3.3 times the instructions and left 28 of 64 lanes
-// idle at N = 6 (35.8 us on the 163,842-node sphere, alone).
+// Lane (part, k) holds the weights (., j, k) of both sums for JL of the j, so that a node's
+// factors are read once per N JL weights, and the x direction runs on packed FP32 pairs.
+// Each weight adds its leaf's nodes in order.  Two shapes, with the same sums:
+//   * many leaves (kWide false): half of the j to a lane, 2 N lanes to a leaf, so N = 6 puts
+//     two leaves in a warp, N = 8 two, N = 4 four.  Instruction issue bounds it: a thread per
+//     (j, k) with N weights took 3.3 times the instructions and left 28 of 64 lanes idle at
+//     N = 6 (35.8 us on the 163,842-node sphere, alone).
+//   * few leaves at odd orders (kWide), where the other shape stages 6, 10 or 16 nodes of a leaf
+//     at a time and has lanes without a last j: a warp to a leaf, all lanes staging its nodes,
+//     and one or two j to a lane.  The chain of a leaf's nodes bounds it: order 3 on 10,242
+//     nodes 42 us in the other shape, 20 so, 163,842 nodes 57 / 29; order 5 on 642 nodes 24 / 14.
 // ------------------------------------------------------------------------------------
 constexpr int kP2MWarps = 4;        // warps per CTA
-
+// kWide at odd orders, up to this many warps of the other shape per SM (at even orders it gains
+// a few us of P2M and nothing in a product).
+constexpr int kP2MWideWarps = 12;
 template <int N>
+constexpr bool kP2MHasWide = N % 2 == 1;
+
+template <int N, bool kWide>
 struct P2MShape {
-  static constexpr int H = (N + 1) / 2;               // packed pairs along x; j of a lane
-  static constexpr int G = 2 * N;                     // lanes of a leaf
-  static constexpr int Leaves = 32 / G;               // leaves of a warp
+  static constexpr int H = (N + 1) / 2;               // packed pairs along x
+  static constexpr int JL = !kWide ? H : N * N <= 32 ? 1 : 2;   // j of a lane
+  static constexpr int G = (N + JL - 1) / JL * N;     // lanes of a leaf
+  static constexpr int Leaves = kWide ? 1 : 32 / G;   // leaves of a warp
   static constexpr int CH = 32 / Leaves;              // nodes of a leaf staged at a time
+  static_assert(G <= 32, "a leaf's lanes are of one warp");
   // a node's row: Sx (2 H), dSx (2 H), (Sy, Sy, dSy, dSy) per j, (Sz, dSz) per k, (c, gx, gy, gz)
   static constexpr int oY = 4 * H, oZ = oY + 4 * N, oW = (oZ + 2 * N + 3) & ~3, Row = oW + 4;
 };
 
-template <int N>
+template <int N, bool kWide>
 __global__ void __launch_bounds__(32 * kP2MWarps) k_p2m(int nleaf, const int4 *__restrict__ leaf_rec,
                                                         float inv_w0, const float4 *__restrict__ pos,
                                                         const float4 *__restrict__ nrm, const float2 *__restrict__ xs,
                                                         float inv_ebar, float *__restrict__ M) {
-  using P = P2MShape<N>;
-  constexpr int N3 = N * N * N, H = P::H, CH = P::CH;
+  using P = P2MShape<N, kWide>;
+  constexpr int N3 = N * N * N, H = P::H, JL = P::JL, CH = P::CH;
   __shared__ __align__(16) float sm[kP2MWarps][32 * P::Row];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int l0 = (blockIdx.x * kP2MWarps + warp) * P::Leaves;
   if (l0 >= nleaf) return;                              // whole warps
   after_previous();
   float *buf = sm[warp];
-  const int sub = lane / P::G, half = lane % P::G / N, k = lane % N;   // this lane's weights
+  const int sub = lane / P::G, part = lane % P::G / N, k = lane % N;   // this lane's weights
   const int ssub = lane / CH, snode = lane % CH;                       // the node that it stages
   const int4 none = make_int4(0, 0, 0, 0);
   const int4 rec = sub < P::Leaves && l0 + sub < nleaf ? leaf_rec[l0 + sub] : none;
@@ -109,9 +121,9 @@ __global__ void __launch_bounds__(32 * kP2MWarps) k_p2m(int nleaf, const int4 *_
   const int nodes = rec.z - rec.y, snodes = srec.z - srec.y;
   const int most = __reduce_max_sync(0xffffffffu, nodes);
   const float invw = inv_width(inv_w0, srec.w);
-  float2 A[H][H], B[H][H];
+  float2 A[JL][H], B[JL][H];
 #pragma unroll
-  for (int j = 0; j < H; ++j)
+  for (int j = 0; j < JL; ++j)
 #pragma unroll
     for (int i = 0; i < H; ++i) A[j][i] = B[j][i] = make_float2(0.f, 0.f);
   float4 pn = make_float4(0.f, 0.f, 0.f, 0.f), qn = pn;  // the next chunk's node, read ahead
@@ -164,9 +176,9 @@ __global__ void __launch_bounds__(32 * kP2MWarps) k_p2m(int nleaf, const int4 *_
       const float2 sz = dup2(z.x), dsz = dup2(z.y);
       const float2 wc = dup2(w.x), wx = dup2(w.y), wy = dup2(w.z), wz = dup2(w.w);
 #pragma unroll
-      for (int jj = 0; jj < H; ++jj) {
-        const int j = half * H + jj;                    // the second half of an odd N has one j less
-        if (N % 2 && j >= N) continue;
+      for (int jj = 0; jj < JL; ++jj) {
+        const int j = part * JL + jj;                   // the last part of an odd N has one j less
+        if (N % JL && j >= N) continue;
         const float4 y = *reinterpret_cast<const float4 *>(row + P::oY + 4 * j);
         const float2 sy = make_float2(y.x, y.y), dsy = make_float2(y.z, y.w);
         const float2 yz = __fmul2_rn(sy, sz);
@@ -184,9 +196,9 @@ __global__ void __launch_bounds__(32 * kP2MWarps) k_p2m(int nleaf, const int4 *_
   if (sub >= P::Leaves || l0 + sub >= nleaf) return;
   float *out = M + (size_t)rec.x * 2 * N3 + k;
 #pragma unroll
-  for (int jj = 0; jj < H; ++jj) {
-    const int j = half * H + jj;
-    if (N % 2 && j >= N) continue;
+  for (int jj = 0; jj < JL; ++jj) {
+    const int j = part * JL + jj;
+    if (N % JL && j >= N) continue;
 #pragma unroll
     for (int i = 0; i < N; ++i) {
       const float a = (i & 1) ? A[jj][i / 2].y : A[jj][i / 2].x, v = (i & 1) ? B[jj][i / 2].y : B[jj][i / 2].x;
@@ -1090,10 +1102,10 @@ Err launch_far(afmpb_t *h, cudaStream_t s, StageTimer *tm, int parts, const FarO
     AFMPB_CUDA(cudaEventRecord(h->ev_fork2, s));
     AFMPB_CUDA(cudaStreamWaitEvent(z, h->ev_fork2, 0));
   }
+  int dev = 0, sms = 0;
+  AFMPB_CUDA(cudaGetDevice(&dev));
+  AFMPB_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   {
-    int dev = 0, sms = 0;
-    AFMPB_CUDA(cudaGetDevice(&dev));
-    AFMPB_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const int64_t nl = (int64_t)T.nbox * N3, nc = compressed ? (int64_t)T.nbox * h->m2l_rank : 0;
     k_zero<<<(unsigned)std::min(div_up(nl + nc, 4 * 256), std::max(1, sms / 2)), 256, 0, z>>>(
         nl, reinterpret_cast<float2 *>(h->d_L), nc, reinterpret_cast<float2 *>(h->d_Lc));
@@ -1104,7 +1116,9 @@ Err launch_far(afmpb_t *h, cudaStream_t s, StageTimer *tm, int parts, const FarO
     AFMPB_TRY(launch_p2l(z));
     AFMPB_CUDA(cudaEventRecord(h->ev_join2, z));
   }
-  AFMPB_TRY(launch_next(beside, "k_p2m", k_p2m<N>, div_up(T.nleaf, kP2MWarps * P2MShape<N>::Leaves), 32 * kP2MWarps, 0, s, T.nleaf,
+  const bool wide = kP2MHasWide<N> && T.nleaf <= kP2MWideWarps * P2MShape<N, false>::Leaves * sms;
+  AFMPB_TRY(launch_next(beside, "k_p2m", wide ? k_p2m<N, kP2MHasWide<N>> : k_p2m<N, false>,
+                        div_up(T.nleaf, kP2MWarps * (wide ? 1 : P2MShape<N, false>::Leaves)), 32 * kP2MWarps, 0, s, T.nleaf,
                         h->d_leaf_rec, inv_w0, h->d_pos, h->d_nrm, h->d_xs, inv_ebar, h->d_M));
   if (tm) tm->mark("p2m", 1);
   for (int level = T.nlevel - 2; level >= 2; --level) {
