@@ -66,6 +66,7 @@ void destroy_handle(afmpb_t *h) {
   if (h->ev_fork2) cudaEventDestroy(h->ev_fork2);
   if (h->ev_join2) cudaEventDestroy(h->ev_join2);
   if (h->ev_zero) cudaEventDestroy(h->ev_zero);
+  if (h->ev_p2p) cudaEventDestroy(h->ev_p2p);
   if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
   delete h;
 }
@@ -76,6 +77,20 @@ void destroy_handle(afmpb_t *h) {
 // 2.5M 9.03 vs 9.11, 5.0M 15.57 vs 15.60, 10.5M 40.5 vs 40.3 ms (each fills the chip by
 // itself there, and beside each other they contend for L2).
 constexpr int64_t kOverlapMaxNodes = 4000000;
+
+// The FP32 translations of order 4 (full form, k_m2l: atomics from a few waves of blocks) wait
+// for P2P on small meshes where they outweigh it: blocks that start between P2P's end up
+// unevenly spread.  Products beside P2P and after it: 20,838 nodes in leaves of up to 8 nodes
+// 790 and 669 us, 48 nodes 255 and 220, 24 nodes 292 and 290; 10,242 nodes 375 and 330 (8), 111
+// and 110 (48); 2,562 nodes 65 and 59 (24).  Above that size, or with fewer than 2 translations
+// to 1000 pairs, the one or the other wins by the mesh (163,842 nodes 847 and 916 us at 48, 634
+// and 724 at 192), at other orders neither.
+constexpr int64_t kM2LAloneNodes = 30000;
+
+bool m2l_after_p2p(const afmpb_t *h) {
+  return h->order == 4 && h->m2l_rank == 0 && h->opt.precision == 0 && h->opt.m2l_method != AFMPB_M2L_PLANE_WAVE &&
+         h->n <= kM2LAloneNodes && 500 * h->n_m2l_pairs >= h->shape.n_p2p_pairs;
+}
 
 // The kernel of the caller-buffer graph that writes y: the far chain's last one, or the
 // scatter where the product has no far part.
@@ -112,6 +127,10 @@ Err enqueue_product_far(afmpb_t *h, cudaStream_t cap, int parts, float *y) {
     out.join = h->ev_join;
   }
   Err e = enqueue_p2p(h, s);
+  if (beside && m2l_after_p2p(h)) {
+    cudaEventRecord(h->ev_p2p, s);
+    out.before_m2l = h->ev_p2p;
+  }
   if (e.ok() && near) e = enqueue_near_fold(h, s);
   if (beside) cudaEventRecord(h->ev_join, h->side);
   if (e.ok()) e = enqueue_far(h, cap, nullptr, kFarAll, &out);
@@ -246,6 +265,7 @@ Err create_impl(afmpb_t *h, const afmpb_mesh *mesh, const afmpb_charges *ch) {
   AFMPB_CUDA(cudaEventCreateWithFlags(&h->ev_fork2, cudaEventDisableTiming));
   AFMPB_CUDA(cudaEventCreateWithFlags(&h->ev_join2, cudaEventDisableTiming));
   AFMPB_CUDA(cudaEventCreateWithFlags(&h->ev_zero, cudaEventDisableTiming));
+  AFMPB_CUDA(cudaEventCreateWithFlags(&h->ev_p2p, cudaEventDisableTiming));
   AFMPB_CUDA(cudaEventCreate(&h->ev_t0));
   AFMPB_CUDA(cudaEventCreate(&h->ev_t1));
   auto lap = [&](int i) {

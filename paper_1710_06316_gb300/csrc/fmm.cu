@@ -1137,6 +1137,7 @@ Err launch_far(afmpb_t *h, cudaStream_t s, StageTimer *tm, int parts, const FarO
   } else if (compressed) {
     AFMPB_TRY(enqueue_m2l_svd(h, s, tm, parts));  // marks compress, m2l, expand itself
   } else if (!h->m2l_groups.empty() && (parts & kFarM2L)) {
+    if (out && out->before_m2l) AFMPB_CUDA(cudaStreamWaitEvent(s, out->before_m2l, 0));
     if (plane_wave) {
       AFMPB_TRY(enqueue_m2l_pw(h, s));
     } else if (h->opt.precision == 1) {

@@ -270,7 +270,7 @@ struct afmpb_t {
   bool own_stream = false;
   cudaStream_t side = nullptr;     // second stream: P2P beside the far-field chain
   cudaStream_t side2 = nullptr;    // third stream: zeroed expansions and P2L beside the upward pass and the M2L
-  cudaEvent_t ev_fork2 = nullptr, ev_join2 = nullptr, ev_zero = nullptr;
+  cudaEvent_t ev_fork2 = nullptr, ev_join2 = nullptr, ev_zero = nullptr, ev_p2p = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   cudaEvent_t ev_t0 = nullptr, ev_t1 = nullptr;
 
@@ -451,6 +451,7 @@ constexpr int kFarUp = 1, kFarM2L = 2, kFarDown = 4, kFarAll = 7;
 // y in caller order, or d_ys when y is null.
 struct FarOut {
   cudaEvent_t join = nullptr;
+  cudaEvent_t before_m2l = nullptr;   // the full-form translations wait for it (P2P), if given
   bool fold = false;
   bool diag = true;          // with alpha x
   float *y = nullptr;
