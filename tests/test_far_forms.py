@@ -98,13 +98,13 @@ def sphere(subdiv, seed):
     return mol
 
 
-@pytest.mark.parametrize("order,leaf_cap", [(3, 90), (4, 90), (6, 90), (4, 45), (5, 45), (6, 45), (3, 2), (8, 12)])
+@pytest.mark.parametrize("order,leaf_cap", [(3, 90), (4, 90), (6, 90), (4, 58), (5, 58), (6, 58), (3, 2), (8, 12)])
 def test_blocks_of_few_and_of_many_leaves(order, leaf_cap):
     mol = sphere(4, order)
     spans = block_spans(check(mol, order, leaf_cap, leaf_cap), mol.n_nodes)[:-1]   # whole blocks
     if leaf_cap == 90:
         assert (spans <= 6).all()
-    elif leaf_cap == 45:
+    elif leaf_cap == 58:
         assert (spans <= 6).any() and (spans > 6).any()
     else:
         assert (spans > 6).all()
