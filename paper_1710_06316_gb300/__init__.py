@@ -262,8 +262,8 @@ def selftest_bounded_wait(spin_limit=1000) -> bool:
     return bool(e.value)
 
 
-def estimate_bytes(n_nodes, n_atoms, order=6, leaf_cap=0, restart=0, charge_fmm=0) -> int:
-    o = Options(leaf_cap=leaf_cap, restart=restart, charge_fmm=charge_fmm)
+def estimate_bytes(n_nodes, n_atoms, order=6, leaf_cap=0, restart=0, charge_fmm=0, precision=0, m2l_tol=0.0) -> int:
+    o = Options(leaf_cap=leaf_cap, restart=restart, charge_fmm=charge_fmm, precision=precision, m2l_tol=m2l_tol)
     return int(load().afmpb_estimate_bytes(int(n_nodes), int(n_atoms), int(order), C.byref(o)))
 
 

@@ -986,13 +986,21 @@ size_t afmpb_estimate_bytes(int64_t n_nodes, int64_t n_atoms, int fmm_order, con
   b += n * per_row * (4 + 16 + 1) + 8 * (n + 1);                                        // near CSR
   b += nbox * (2 * 2 * n3 * 4 + 64 + 27 * 4 + 200 * 4 * 2);                             // boxes, lists
   b += 316 * n3 * n3 * 4 * 14;                                                          // M2L tables
+  // full-form translations (orders up to 4, or m2l_tol < 0) on the tensor cores: tiles of a fixed
+  // size for the Laplace table and one per level; a surface's octree has about log4(n / cap) + 2
+  if (o && o->precision == 1 && (n3 <= 64 || o->m2l_tol < 0)) {
+    const double levels = std::ceil(std::log2(std::max(1.0, (double)n / cap)) / 2.0) + 4.0;
+    b += m2l_tc_tile_bytes((int)n3) * (size_t)std::min(levels, (double)kMaxLevel);
+  }
   b += (size_t)(m + 1) * 2 * n * 8 + 8 * 2 * n * 8;                                     // GMRES
   b += (size_t)std::max<int64_t>(n_atoms, 0) * 32 * 2;
   const int cfm = o ? o->charge_fmm : 0;
   if (n_atoms > 0 && (cfm == 2 || (cfm == 0 && (double)n_nodes * (double)n_atoms > AFMPB_CHARGE_FMM_PAIRS))) {
-    const size_t nu = n + (size_t)n_atoms;                                             // charge FMM
-    const size_t nbu = 3 * (nu / (size_t)std::max(cap / 2, 1) + 64);
-    b += nu * 160 + nbu * (2 * 2 * n3 * 4 + 64 + 27 * 4 + 200 * 4 * 2) + 316 * n3 * n3 * 4 * 14;
+    // charge FMM: an octree and expansions of its own order (8, leaves of 128 or more), one
+    // Laplace table (full form at most) and the scratch of its compression
+    const size_t nu = n + (size_t)n_atoms, n3u = 512;
+    const size_t nbu = 3 * (nu / (size_t)(std::max(cap, 128) / 2) + 64);
+    b += nu * 320 + nbu * (2 * 2 * n3u * 4 + 64 + 27 * 4 + 200 * 4 * 2) + 316 * n3u * n3u * 4;
   }
   return b + (64u << 20);
 }

@@ -470,6 +470,7 @@ Err enqueue_p2p_batch(const P2PReq *d_reqs, const P2PUnit *d_units, int nunits, 
 Err enqueue_near_fold(afmpb_t *h, cudaStream_t s);   // near SpMV into phi_near, after P2P
 Err enqueue_combine(afmpb_t *h, cudaStream_t s, int parts);
 Err enqueue_m2l_tc(afmpb_t *h, cudaStream_t s);       // tensor-core M2L (precision 1)
+size_t m2l_tc_tile_bytes(int n3);                     // its operand tiles of one full-form table
 Err build_m2l_tc(afmpb_t *h);
 // m2l_ts.cu: the target-stationary tensor-core M2L
 bool m2l_ts_applies(const afmpb_t *h);

@@ -272,6 +272,10 @@ namespace {
 constexpr int kTcSmem = (2 * kTcAElems + 2 * kTcBElems) * 2;
 }
 
+size_t m2l_tc_tile_bytes(int n3) {
+  return (size_t)kNumOffsets * ((n3 + kTcRows - 1) / kTcRows) * 2 * 2 * kTcAElems * sizeof(uint16_t);
+}
+
 Err build_m2l_tc(afmpb_t *h) {
   // R: compressed size (a multiple of 16) or n^3
   const int N3 = h->m2l_rank > 0 ? h->m2l_rank : h->ncoef;
